@@ -1,6 +1,6 @@
 // mlp.cu -- training of the branching network on the GPU: forward on the
-// tensor cores, softmax cross-entropy per decision node, backward (dW1 on the
-// tensor cores as X^T * dH), Adam with FP32 master weights, BF16 packing.
+// tensor cores, softmax cross-entropy per decision node and backward (dW1^T on
+// the tensor cores as dH^T * X) in one kernel, Adam with FP32 master weights, BF16 packing.
 //
 // Training data are the decision traces of the plain search (scuba_trace):
 // node k has rows [node_row[k], node_row[k] + node_nrows[k]) -- one row per
@@ -14,7 +14,10 @@
 // b2 at 1152.
 #include <cuda_runtime.h>
 
+#include <cooperative_groups.h>
+
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 #include <cstdint>
 #include <map>
@@ -75,174 +78,323 @@ __global__ void k_pack(const float* master, MlpWeights* W) {
   if (p < NPARAM) pack_one(master, W, p);
 }
 
-// Stage rows [r, r+16) of x (clipped to [lo, hi)) into a shared 16x16 tile.
-__device__ __forceinline__ void stage_tile(const __nv_bfloat16* x, int64_t r, int64_t lo,
-                                           int64_t hi, __nv_bfloat16* tile, int lane) {
-  for (int k = lane; k < 16 * NFEAT; k += 32) {
-    const int64_t row = r + k / NFEAT;
-    tile[k] = (row >= lo && row < hi) ? x[row * NFEAT + (k % NFEAT)] : __float2bfloat16(0.0f);
-  }
-  __syncwarp();
-}
+// ---- one 16-row tile on the tensor cores -----------------------------------
+//
+// The forward pass runs transposed, z^T = W1^T X^T: the weights are the A
+// operand (four 16-unit tiles that stay in registers), the rows the B operand,
+// so a lane loads its operand straight from a row (8 contiguous bytes) and the
+// pre-activations of hidden units g, g + 8 at rows 2t, 2t + 1 land in the layout
+// in which the backward pass needs dH^T as an A operand: dW1^T = dH^T X takes
+// no trip of dH through shared memory, only X is transposed (movmatrix).
+// The 16 features are numbered so that lane t's 8 bytes (features 4t .. 4t+3)
+// are the logical columns 2t, 2t+1, 2t+8, 2t+9 of the mma; the sum over them
+// does not depend on that numbering.
 
-// Scores of all rows [0, rows): one warp per 16-row tile (grid-stride).
-__global__ void k_forward(const __nv_bfloat16* x, int64_t rows, const MlpWeights* W,
-                          float* scores) {
-  __shared__ __nv_bfloat16 tiles[8][16 * NFEAT];
-  const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-  const int64_t nt = (rows + 15) / 16;
-  for (int64_t t = (int64_t)blockIdx.x * (blockDim.x >> 5) + wib; t < nt;
-       t += (int64_t)gridDim.x * (blockDim.x >> 5)) {
-    stage_tile(x, 16 * t, 0, rows, tiles[wib], lane);
-    float lo, hi;
-    learn::mlp_tile_scores(W, tiles[wib], lane, lo, hi);
-    const int g = lane >> 2;
-    if ((lane & 3) == 0) {
-      if (16 * t + g < rows) scores[16 * t + g] = lo;
-      if (16 * t + g + 8 < rows) scores[16 * t + g + 8] = hi;
+struct HiddenWeights {
+  uint32_t a[4][4];         // W1^T: hidden units 16q .. 16q+15, logical features
+  float b1[4][2], w2[4][2];  // units 16q + g, 16q + g + 8
+};
+
+__device__ __forceinline__ void load_hidden(const MlpWeights* W, int g, int t, HiddenWeights& H) {
+#pragma unroll
+  for (int q = 0; q < 4; q++) {
+#pragma unroll
+    for (int u = 0; u < 2; u++) {
+      const int j = 16 * q + g + 8 * u;
+      const uint32_t* r = reinterpret_cast<const uint32_t*>(W->w1t + j * NFEAT + 4 * t);
+      H.a[q][u] = r[0];
+      H.a[q][2 + u] = r[1];
+      H.b1[q][u] = W->b1[j];
+      H.w2[q][u] = __bfloat162float(W->w2[j]);
     }
-    __syncwarp();
   }
 }
 
-// Per node: scores of its rows, softmax, cross-entropy against normalised
-// targets, dS = softmax - target. One warp per node.
-__global__ void k_node_loss(const int64_t* node_row, const int32_t* node_nrows,
-                            const int32_t* node_closed, int64_t k0, int64_t k1,
-                            const __nv_bfloat16* x, const MlpWeights* W, const float* target,
-                            float* dS, float* loss) {
-  __shared__ __nv_bfloat16 tiles[8][16 * NFEAT];
+// D = A(16x16) * B(16x8) + C, BF16 inputs, FP32 accumulate.
+__device__ __forceinline__ void mma_add(float d[4], const uint32_t a[4], uint32_t b0, uint32_t b1,
+                                        float c0, float c1, float c2, float c3) {
+  asm volatile(
+      "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 "
+      "{%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%10,%11,%12,%13};\n"
+      : "=f"(d[0]), "=f"(d[1]), "=f"(d[2]), "=f"(d[3])
+      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1), "f"(c0), "f"(c1), "f"(c2),
+        "f"(c3));
+}
+
+__device__ __forceinline__ uint32_t transpose8x8(uint32_t m) {
+  uint32_t r;
+  asm volatile("movmatrix.sync.aligned.m8n8.trans.b16 %0, %1;\n" : "=r"(r) : "r"(m));
+  return r;
+}
+
+// Lane (g, t)'s features 4t .. 4t+3 of one row; zeros past the end. WIDE: x is
+// 8-byte aligned (rows are 32 bytes); otherwise the elements are read one by one.
+template <bool WIDE>
+__device__ __forceinline__ uint2 load_row(const __nv_bfloat16* x, int64_t row, int64_t end, int t) {
+  uint2 v = make_uint2(0u, 0u);
+  if (row < end) {
+    const __nv_bfloat16* p = x + row * NFEAT + 4 * t;
+    if (WIDE) {
+      v = __ldg(reinterpret_cast<const uint2*>(p));
+    } else {
+      v.x = learn::pack_bf16(p[0], p[1]);
+      v.y = learn::pack_bf16(p[2], p[3]);
+    }
+  }
+  return v;
+}
+
+// The row of its tile whose score a lane keeps: lanes with g < 4 take one row
+// each, lanes with g >= 4 repeat them.
+__device__ __forceinline__ int lane_row(int g, int t) {
+  return 8 * ((g >> 1) & 1) + 2 * t + (g & 1);
+}
+
+// Score (without the output bias) of row lane_row(g, t) of the tile whose
+// rows g and g + 8 the lanes hold in x0 and x1.
+__device__ __forceinline__ float tile_score(const HiddenWeights& H, uint2 x0, uint2 x1, int g) {
+  float p[2][2] = {{0.f, 0.f}, {0.f, 0.f}};
+#pragma unroll
+  for (int q = 0; q < 4; q++) {
+#pragma unroll
+    for (int h = 0; h < 2; h++) {
+      float z[4];
+      mma_add(z, H.a[q], h ? x1.x : x0.x, h ? x1.y : x0.y, H.b1[q][0], H.b1[q][0], H.b1[q][1],
+              H.b1[q][1]);
+      p[h][0] += fmaxf(z[0], 0.f) * H.w2[q][0] + fmaxf(z[2], 0.f) * H.w2[q][1];
+      p[h][1] += fmaxf(z[1], 0.f) * H.w2[q][0] + fmaxf(z[3], 0.f) * H.w2[q][1];
+    }
+  }
+  // sum over g (8 lanes), each step halving the rows a lane goes on with:
+  // rows 8h + 2t + j end at the lanes with g = 2h + j (mod 4)
+  const bool h = (g & 2) != 0, j = (g & 1) != 0;
+  float r0 = h ? p[1][0] : p[0][0], r1 = h ? p[1][1] : p[0][1];
+  r0 += __shfl_xor_sync(FULL, h ? p[0][0] : p[1][0], 8);
+  r1 += __shfl_xor_sync(FULL, h ? p[0][1] : p[1][1], 8);
+  float s = j ? r1 : r0;
+  s += __shfl_xor_sync(FULL, j ? r0 : r1, 4);
+  return s + __shfl_xor_sync(FULL, s, 16);
+}
+
+// Scores of all rows [0, rows): one warp per 16-row tile (grid-stride), the
+// next tile's rows loaded while this one's are multiplied.
+template <bool WIDE>
+__global__ void __launch_bounds__(256) k_forward(const __nv_bfloat16* x, int64_t rows,
+                                                 const MlpWeights* W, float* scores) {
+  const int lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
+  HiddenWeights H;
+  load_hidden(W, g, t, H);
+  const float b2 = W->b2;
+  const int64_t step = 16 * (int64_t)gridDim.x * (blockDim.x >> 5);
+  int64_t r = 16 * ((int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5));
+  uint2 x0 = load_row<WIDE>(x, r + g, rows, t), x1 = load_row<WIDE>(x, r + g + 8, rows, t);
+  for (; r < rows; r += step) {
+    const uint2 n0 = load_row<WIDE>(x, r + step + g, rows, t);
+    const uint2 n1 = load_row<WIDE>(x, r + step + g + 8, rows, t);
+    const float s = tile_score(H, x0, x1, g) + b2;
+    const int64_t row = r + lane_row(g, t);
+    if (g < 4 && row < rows) scores[row] = s;
+    x0 = n0;
+    x1 = n1;
+  }
+}
+
+// Softmax statistics of a set of scores: the maximum and the sum of
+// exp(score - maximum), with the set's targets summed beside them.
+struct SoftStat {
+  float m, e, t;
+};
+
+// exp(s - m), 0 for s = -inf beside an m that is still -inf.
+__device__ __forceinline__ float exp_from(float s, float m) {
+  return expf(s - (m == -INFINITY ? 0.0f : m));
+}
+
+__device__ __forceinline__ SoftStat merge(const SoftStat& a, const SoftStat& b) {
+  const float m = fmaxf(a.m, b.m);
+  return SoftStat{m, a.e * exp_from(a.m, m) + b.e * exp_from(b.m, m), a.t + b.t};
+}
+
+// Loss and gradients of trace nodes [k0, k1) in one pass per node: scores,
+// softmax cross-entropy against the normalised targets, dS = softmax - target
+// and the gradients of every parameter (dW1 on the tensor cores from dH in
+// BF16). `split` blocks (a cluster) share a node's 16-row tiles and exchange
+// their softmax statistics through distributed shared memory; the nodes are
+// strided over the clusters, the gradients stay in registers across them and
+// are reduced once per block. A thread keeps the scores of its own rows in dS
+// between the two passes over the node's rows; the rows' features come from
+// L1 or L2 the second time.
+//
+// Bound by instruction issue: about 500 instructions per 16-row tile
+// (activations, masks and sums of 64 hidden units per row) against 640 bytes.
+// A minibatch of 64 nodes has 64,000 rows, too few for one warp per node
+// (the split is the one that fills 2 blocks on each of the 152 SMs).
+constexpr int kGradWarps = 8;
+constexpr int kGradStride = 17 * NHID + 2 * NHID + 4;  // floats one warp stages for the reduction
+
+template <bool WIDE>
+__global__ void __launch_bounds__(32 * kGradWarps, 2)
+    k_node_grad(const int64_t* node_row, const int32_t* node_nrows, const int32_t* node_closed,
+                int64_t k0, int64_t k1, const __nv_bfloat16* x, const MlpWeights* W,
+                const float* target, float* dS, float* grad, int split) {
+  __shared__ float stage[kGradWarps][kGradStride];
+  __shared__ SoftStat warp_stat[kGradWarps];
+  __shared__ SoftStat cta_stat[2];
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-  for (int64_t k = k0 + (int64_t)blockIdx.x * (blockDim.x >> 5) + wib; k < k1;
-       k += (int64_t)gridDim.x * (blockDim.x >> 5)) {
-    const int64_t r0 = node_row[k];
-    const int32_t n = node_nrows[k];
-    float tsum = 0.0f;
-    for (int i = lane; i < n; i += 32) tsum += target[r0 + i];
-    for (int d = 16; d > 0; d >>= 1) tsum += __shfl_xor_sync(FULL, tsum, d);
-    const bool use = node_closed[k] && n > 1 && tsum > 0.0f;
+  const int g = lane >> 2, t = lane & 3;
+  const int rank = blockIdx.x % split;
+  HiddenWeights H;
+  load_hidden(W, g, t, H);
+  const float b2 = W->b2;
+  float cw1[4][2][4], gw2[4][2], gb1[4][2], gb2 = 0.0f, ce = 0.0f, used = 0.0f;
+#pragma unroll
+  for (int q = 0; q < 4; q++) {
+    gw2[q][0] = gw2[q][1] = gb1[q][0] = gb1[q][1] = 0.0f;
+#pragma unroll
+    for (int f = 0; f < 2; f++) cw1[q][f][0] = cw1[q][f][1] = cw1[q][f][2] = cw1[q][f][3] = 0.0f;
+  }
+  const int64_t step = 16 * (int64_t)kGradWarps * split;
+  int parity = 0;
+  for (int64_t k = k0 + blockIdx.x / split; k < k1; k += gridDim.x / split, parity ^= 1) {
+    const int64_t r0 = node_row[k], end = r0 + node_nrows[k];
+    const int64_t first = r0 + 16 * ((int64_t)wib * split + rank);
+    // scores and their statistics
+    SoftStat st{-INFINITY, 0.0f, 0.0f};
+    {
+      uint2 x0 = load_row<WIDE>(x, first + g, end, t), x1 = load_row<WIDE>(x, first + g + 8, end, t);
+      for (int64_t r = first; r < end; r += step) {
+        const uint2 n0 = load_row<WIDE>(x, r + step + g, end, t);
+        const uint2 n1 = load_row<WIDE>(x, r + step + g + 8, end, t);
+        const int64_t row = r + lane_row(g, t);
+        const bool mine = g < 4 && row < end;
+        const float tv = mine ? target[row] : 0.0f;
+        const float s = tile_score(H, x0, x1, g) + b2;
+        if (mine) {
+          dS[row] = s;
+          st.t += tv;
+          if (s > st.m) {
+            st.e *= expf(st.m - s);
+            st.m = s;
+          }
+          st.e += exp_from(s, st.m);
+        }
+        x0 = n0;
+        x1 = n1;
+      }
+    }
+    for (int d = 16; d > 0; d >>= 1)
+      st = merge(st, SoftStat{__shfl_xor_sync(FULL, st.m, d), __shfl_xor_sync(FULL, st.e, d),
+                              __shfl_xor_sync(FULL, st.t, d)});
+    __syncthreads();  // the previous node's statistics have been read
+    if (lane == 0) warp_stat[wib] = st;
+    __syncthreads();
+    st = warp_stat[0];
+    for (int w = 1; w < kGradWarps; w++) st = merge(st, warp_stat[w]);
+    if (split > 1) {
+      // two slots: a block may be one node ahead of the slowest reader of the
+      // other slot, never two (the barrier of the node between them)
+      cooperative_groups::cluster_group cl = cooperative_groups::this_cluster();
+      if (threadIdx.x == 0) cta_stat[parity] = st;
+      cl.sync();
+      st = *cl.map_shared_rank(&cta_stat[parity], 0);
+      for (int b = 1; b < split; b++) st = merge(st, *cl.map_shared_rank(&cta_stat[parity], b));
+    }
+    const bool use = node_closed[k] && end - r0 > 1 && st.t > 0.0f;
     if (!use) {
-      for (int i = lane; i < n; i += 32) dS[r0 + i] = 0.0f;
+      for (int64_t r = first; r < end; r += step) {
+        const int64_t row = r + lane_row(g, t);
+        if (g < 4 && row < end) dS[row] = 0.0f;
+      }
       continue;
     }
-    // scores into dS (as scratch), then the max
-    for (int64_t r = r0; r < r0 + n; r += 16) {
-      stage_tile(x, r, r0, r0 + n, tiles[wib], lane);
-      float lo, hi;
-      learn::mlp_tile_scores(W, tiles[wib], lane, lo, hi);
-      const int g = lane >> 2;
-      if ((lane & 3) == 0) {
-        if (r + g < r0 + n) dS[r + g] = lo;
-        if (r + g + 8 < r0 + n) dS[r + g + 8] = hi;
+    const float lse = st.m + logf(st.e);
+    if (rank == 0 && threadIdx.x == 0) used += 1.0f;
+    for (int64_t r = first; r < end; r += step) {
+      const uint2 x0 = load_row<WIDE>(x, r + g, end, t), x1 = load_row<WIDE>(x, r + g + 8, end, t);
+      const int64_t row = r + lane_row(g, t);
+      float ds_mine = 0.0f;
+      if (g < 4 && row < end) {
+        const float s = dS[row], tn = target[row] / st.t;
+        ds_mine = expf(s - lse) - tn;
+        dS[row] = ds_mine;
+        ce -= tn * (s - lse);
+        gb2 += ds_mine;
       }
-      __syncwarp();
-    }
-    float mx = -INFINITY;
-    for (int i = lane; i < n; i += 32) mx = fmaxf(mx, dS[r0 + i]);
-    for (int d = 16; d > 0; d >>= 1) mx = fmaxf(mx, __shfl_xor_sync(FULL, mx, d));
-    float se = 0.0f;
-    for (int i = lane; i < n; i += 32) se += expf(dS[r0 + i] - mx);
-    for (int d = 16; d > 0; d >>= 1) se += __shfl_xor_sync(FULL, se, d);
-    const float lse = mx + logf(se);
-    float ce = 0.0f;
-    for (int i = lane; i < n; i += 32) {
-      const float s = dS[r0 + i];
-      const float t = target[r0 + i] / tsum;
-      ce -= t * (s - lse);
-      dS[r0 + i] = expf(s - lse) - t;
-    }
-    for (int d = 16; d > 0; d >>= 1) ce += __shfl_xor_sync(FULL, ce, d);
-    if (lane == 0) {
-      atomicAdd(&loss[0], ce);
-      atomicAdd(&loss[1], 1.0f);
+      float ds[2][2];  // rows 8h + 2t + j
+#pragma unroll
+      for (int h = 0; h < 2; h++)
+#pragma unroll
+        for (int j = 0; j < 2; j++)
+          ds[h][j] = __shfl_sync(FULL, ds_mine, 4 * (2 * h + j) + t);
+      // X as a B operand (rows x logical features): b[f][h] for rows 8h .. 8h+7
+      const uint32_t bx[2][2] = {{transpose8x8(x0.x), transpose8x8(x1.x)},
+                                 {transpose8x8(x0.y), transpose8x8(x1.y)}};
+#pragma unroll
+      for (int q = 0; q < 4; q++) {
+        uint32_t dh[4];  // dH^T: units 16q .. 16q+15, the tile's rows
+#pragma unroll
+        for (int h = 0; h < 2; h++) {
+          float z[4], d[4];
+          mma_add(z, H.a[q], h ? x1.x : x0.x, h ? x1.y : x0.y, H.b1[q][0], H.b1[q][0], H.b1[q][1],
+                  H.b1[q][1]);
+#pragma unroll
+          for (int u = 0; u < 4; u++)
+            d[u] = z[u] > 0.f ? ds[h][u & 1] * H.w2[q][u >> 1] : 0.f;
+          gw2[q][0] += fmaxf(z[0], 0.f) * ds[h][0] + fmaxf(z[1], 0.f) * ds[h][1];
+          gw2[q][1] += fmaxf(z[2], 0.f) * ds[h][0] + fmaxf(z[3], 0.f) * ds[h][1];
+          gb1[q][0] += d[0] + d[1];
+          gb1[q][1] += d[2] + d[3];
+          dh[2 * h] = learn::pack_bf16(__float2bfloat16(d[0]), __float2bfloat16(d[1]));
+          dh[2 * h + 1] = learn::pack_bf16(__float2bfloat16(d[2]), __float2bfloat16(d[3]));
+        }
+#pragma unroll
+        for (int f = 0; f < 2; f++)
+          mma_add(cw1[q][f], dh, bx[f][0], bx[f][1], cw1[q][f][0], cw1[q][f][1], cw1[q][f][2],
+                  cw1[q][f][3]);
+      }
     }
   }
-}
-
-// Gradients of the summed node losses with respect to every parameter.
-// One block per node; warps stride over its 16-row tiles. dW1 = X^T dH runs
-// on the tensor cores: A = X^T tile (features x rows), B = dH tile (rows x
-// 8 hidden units) staged through shared memory in BF16.
-__global__ void __launch_bounds__(128) k_backward(const int64_t* node_row,
-                                                  const int32_t* node_nrows, int64_t k0,
-                                                  const __nv_bfloat16* x, const MlpWeights* W,
-                                                  const float* dS, float* grad) {
-  __shared__ __nv_bfloat16 xt[4][16 * NFEAT];
-  __shared__ __nv_bfloat16 dh_t[4][16 * NHID];
-  __shared__ float gacc[NPARAM];
-  const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5, nw = blockDim.x >> 5;
-  const int g = lane >> 2, t = lane & 3;
-  for (int p = threadIdx.x; p < NPARAM; p += blockDim.x) gacc[p] = 0.0f;
+  if (split > 1) cooperative_groups::this_cluster().sync();  // every remote read is done
+  // one sum per parameter over the block's warps, then global
+  float* mine = stage[wib];
+#pragma unroll
+  for (int q = 0; q < 4; q++) {
+#pragma unroll
+    for (int u = 0; u < 2; u++) {
+      const int j = 16 * q + g + 8 * u;
+#pragma unroll
+      for (int f = 0; f < 2; f++) {  // logical features 2t, 2t+1 (f = 0), 2t+8, 2t+9 (f = 1)
+        mine[17 * j + 4 * t + 2 * f] = cw1[q][f][2 * u];
+        mine[17 * j + 4 * t + 2 * f + 1] = cw1[q][f][2 * u + 1];
+      }
+      float a = gb1[q][u], b = gw2[q][u];
+      a += __shfl_xor_sync(FULL, a, 1);
+      a += __shfl_xor_sync(FULL, a, 2);
+      b += __shfl_xor_sync(FULL, b, 1);
+      b += __shfl_xor_sync(FULL, b, 2);
+      if (t == 0) {
+        mine[17 * NHID + j] = a;
+        mine[18 * NHID + j] = b;
+      }
+    }
+  }
+  for (int d = 16; d > 0; d >>= 1) {
+    gb2 += __shfl_xor_sync(FULL, gb2, d);
+    ce += __shfl_xor_sync(FULL, ce, d);
+  }
+  if (lane == 0) {
+    mine[19 * NHID] = gb2;
+    mine[19 * NHID + 1] = ce;
+    mine[19 * NHID + 2] = used;
+  }
   __syncthreads();
-  const int64_t k = k0 + blockIdx.x;
-  const int64_t r0 = node_row[k];
-  const int32_t n = node_nrows[k];
-  float cw1[NHID / 8][4];
+  for (int p = threadIdx.x; p < NPARAM + 2; p += blockDim.x) {
+    const int at = p < OFF_B1 ? 17 * (p % NHID) + p / NHID : 17 * NHID + (p - OFF_B1);
+    float s = 0.0f;
 #pragma unroll
-  for (int q = 0; q < NHID / 8; q++) cw1[q][0] = cw1[q][1] = cw1[q][2] = cw1[q][3] = 0.0f;
-  float gw2[16], gb1[16], gb2 = 0.0f;
-#pragma unroll
-  for (int q = 0; q < 16; q++) gw2[q] = gb1[q] = 0.0f;
-  for (int64_t r = r0 + 16 * wib; r < r0 + n; r += 16 * nw) {
-    stage_tile(x, r, r0, r0 + n, xt[wib], lane);
-    float z[4 * (NHID / 8)];
-    float lo, hi;
-    learn::mlp_tile_scores(W, xt[wib], lane, lo, hi, z);
-    const float ds_lo = (r + g < r0 + n) ? dS[r + g] : 0.0f;
-    const float ds_hi = (r + g + 8 < r0 + n) ? dS[r + g + 8] : 0.0f;
-    if (t == 0) gb2 += ds_lo + ds_hi;
-#pragma unroll
-    for (int q = 0; q < NHID / 8; q++) {
-      const int j0 = 8 * q + 2 * t;
-      const float w0 = __bfloat162float(W->w2[j0]), w1 = __bfloat162float(W->w2[j0 + 1]);
-      const float z0 = z[4 * q], z1 = z[4 * q + 1], z2 = z[4 * q + 2], z3 = z[4 * q + 3];
-      gw2[2 * q] += fmaxf(z0, 0.f) * ds_lo + fmaxf(z2, 0.f) * ds_hi;
-      gw2[2 * q + 1] += fmaxf(z1, 0.f) * ds_lo + fmaxf(z3, 0.f) * ds_hi;
-      const float d0 = z0 > 0.f ? ds_lo * w0 : 0.f, d1 = z1 > 0.f ? ds_lo * w1 : 0.f;
-      const float d2 = z2 > 0.f ? ds_hi * w0 : 0.f, d3 = z3 > 0.f ? ds_hi * w1 : 0.f;
-      gb1[2 * q] += d0 + d2;
-      gb1[2 * q + 1] += d1 + d3;
-      __nv_bfloat16* dr = dh_t[wib];
-      dr[g * NHID + j0] = __float2bfloat16(d0);
-      dr[g * NHID + j0 + 1] = __float2bfloat16(d1);
-      dr[(g + 8) * NHID + j0] = __float2bfloat16(d2);
-      dr[(g + 8) * NHID + j0 + 1] = __float2bfloat16(d3);
-    }
-    __syncwarp();
-    // A = X^T: A[i][row] = x[row][i]
-    const __nv_bfloat16* xs = xt[wib];
-    uint32_t a[4];
-    a[0] = learn::pack_bf16(xs[(2 * t) * NFEAT + g], xs[(2 * t + 1) * NFEAT + g]);
-    a[1] = learn::pack_bf16(xs[(2 * t) * NFEAT + g + 8], xs[(2 * t + 1) * NFEAT + g + 8]);
-    a[2] = learn::pack_bf16(xs[(2 * t + 8) * NFEAT + g], xs[(2 * t + 9) * NFEAT + g]);
-    a[3] = learn::pack_bf16(xs[(2 * t + 8) * NFEAT + g + 8], xs[(2 * t + 9) * NFEAT + g + 8]);
-    const __nv_bfloat16* dr = dh_t[wib];
-#pragma unroll
-    for (int q = 0; q < NHID / 8; q++) {
-      uint32_t b[2];
-      b[0] = learn::pack_bf16(dr[(2 * t) * NHID + 8 * q + g], dr[(2 * t + 1) * NHID + 8 * q + g]);
-      b[1] = learn::pack_bf16(dr[(2 * t + 8) * NHID + 8 * q + g],
-                              dr[(2 * t + 9) * NHID + 8 * q + g]);
-      learn::mma16816(cw1[q], a, b);
-    }
-    __syncwarp();
+    for (int w = 0; w < kGradWarps; w++) s += stage[w][at];
+    if (s != 0.0f) atomicAdd(&grad[p], s);
   }
-  // reduce into shared, then global
-  for (int q = 0; q < NHID / 8; q++) {
-    const int j0 = 8 * q + 2 * t;
-    atomicAdd(&gacc[g * NHID + j0], cw1[q][0]);
-    atomicAdd(&gacc[g * NHID + j0 + 1], cw1[q][1]);
-    atomicAdd(&gacc[(g + 8) * NHID + j0], cw1[q][2]);
-    atomicAdd(&gacc[(g + 8) * NHID + j0 + 1], cw1[q][3]);
-    atomicAdd(&gacc[OFF_W2 + j0], gw2[2 * q]);
-    atomicAdd(&gacc[OFF_W2 + j0 + 1], gw2[2 * q + 1]);
-    atomicAdd(&gacc[OFF_B1 + j0], gb1[2 * q]);
-    atomicAdd(&gacc[OFF_B1 + j0 + 1], gb1[2 * q + 1]);
-  }
-  if (t == 0) atomicAdd(&gacc[OFF_B2], gb2);
-  __syncthreads();
-  for (int p = threadIdx.x; p < NPARAM; p += blockDim.x)
-    if (gacc[p] != 0.0f) atomicAdd(&grad[p], gacc[p]);
 }
 
 // One training step after a minibatch's gradient: Adam (Kingma and Ba,
@@ -287,6 +439,21 @@ std::map<int, TrainScratch>& train_scratch() {
   return m;
 }
 
+// SMs of the current device (read once per device and process).
+int sm_count() {
+  static std::atomic<int> known[64];
+  int dev = 0, sms = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return 152;
+  if (dev < 64 && (sms = known[dev].load(std::memory_order_relaxed)) > 0) return sms;
+  if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 152;
+  if (dev < 64) known[dev].store(sms, std::memory_order_relaxed);
+  return sms;
+}
+
+// Whether the feature rows allow 8-byte loads (a caller may pass any 2-byte
+// aligned pointer).
+bool wide_rows(const void* x) { return (reinterpret_cast<uintptr_t>(x) & 7) == 0; }
+
 int fail(const char* what, cudaError_t e) {
   set_error(std::string(what) + ": " + cudaGetErrorString(e));
   return SCUBA_ERR_CUDA;
@@ -329,31 +496,43 @@ extern "C" int scuba_mlp_forward(const uint16_t* x, int64_t rows, const void* we
   if (rows < 0 || (rows > 0 && (!x || !weights || !scores))) return SCUBA_ERR_ARG;
   if (rows == 0) return SCUBA_OK;
   const int64_t tiles = (rows + 15) / 16;
-  const int grid = (int)std::min<int64_t>((tiles + 7) / 8, 65535);
-  mlpk::k_forward<<<grid, 256, 0, (cudaStream_t)stream>>>(
-      reinterpret_cast<const __nv_bfloat16*>(x), rows,
-      static_cast<const learn::MlpWeights*>(weights), scores);
+  // 8 tiles per block, at most 8 blocks on each SM: a warp of a large call
+  // then loads its next tile while it multiplies this one
+  const int grid = (int)std::min<int64_t>((tiles + 7) / 8, (int64_t)sm_count() * 8);
+  const __nv_bfloat16* xb = reinterpret_cast<const __nv_bfloat16*>(x);
+  const learn::MlpWeights* W = static_cast<const learn::MlpWeights*>(weights);
+  if (wide_rows(xb))
+    mlpk::k_forward<true><<<grid, 256, 0, (cudaStream_t)stream>>>(xb, rows, W, scores);
+  else
+    mlpk::k_forward<false><<<grid, 256, 0, (cudaStream_t)stream>>>(xb, rows, W, scores);
   cudaError_t e = cudaGetLastError();
   return e == cudaSuccess ? SCUBA_OK : fail("scuba_mlp_forward", e);
 }
 
-// The loss and gradient kernels of nodes [k0, k1) into grad (cleared by
-// the caller): per-node softmax cross-entropy, then the backward pass.
+// The loss and gradients of nodes [k0, k1) into grad (cleared by the caller).
 static void grad_kernels(const scuba_trace* tr, int64_t k0, int64_t k1, const void* weights,
                          float* grad, float* dS, cudaStream_t st) {
   const int64_t nodes = k1 - k0;
   if (nodes <= 0) return;
-  const int lgrid = (int)std::min<int64_t>((nodes + 7) / 8, 65535);
-  mlpk::k_node_loss<<<lgrid, 256, 0, st>>>(
-      tr->node_row, tr->node_nrows, tr->node_closed, k0, k1,
-      reinterpret_cast<const __nv_bfloat16*>(tr->x),
-      static_cast<const learn::MlpWeights*>(weights), tr->target, dS, grad + learn::NPARAM);
-  for (int64_t b = 0; b < nodes; b += 65535) {
-    const int64_t cnt = std::min<int64_t>(65535, nodes - b);
-    mlpk::k_backward<<<(unsigned)cnt, 128, 0, st>>>(
-        tr->node_row, tr->node_nrows, k0 + b, reinterpret_cast<const __nv_bfloat16*>(tr->x),
-        static_cast<const learn::MlpWeights*>(weights), dS, grad);
-  }
+  // blocks per node: as many (1, 2, 4, 8) as still fit two blocks on each SM
+  const int64_t slots = 2 * (int64_t)sm_count();
+  int split = 1;
+  while (split < 8 && 2 * split * nodes <= slots) split *= 2;
+  const __nv_bfloat16* x = reinterpret_cast<const __nv_bfloat16*>(tr->x);
+  cudaLaunchAttribute attr;
+  attr.id = cudaLaunchAttributeClusterDimension;
+  attr.val.clusterDim.x = split;
+  attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)(std::min(nodes * split, slots / split * split)));
+  cfg.blockDim = dim3(32 * mlpk::kGradWarps);
+  cfg.stream = st;
+  cfg.attrs = &attr;
+  cfg.numAttrs = 1;
+  cudaLaunchKernelEx(
+      &cfg, wide_rows(x) ? mlpk::k_node_grad<true> : mlpk::k_node_grad<false>, tr->node_row,
+      tr->node_nrows, tr->node_closed, k0, k1, x, static_cast<const learn::MlpWeights*>(weights),
+      tr->target, dS, grad, split);
 }
 
 static int grad_impl(const scuba_trace* tr, int64_t k0, int64_t k1, const void* weights,
@@ -398,7 +577,7 @@ extern "C" int scuba_mlp_train(const scuba_trace* tr, int64_t nodes, float* mast
   cudaMemsetAsync(adam_v, 0, sizeof(float) * learn::NPARAM, st);
   cudaMemsetAsync(gbuf, 0, sizeof(float) * 2 * gwords, st);
   if (epoch_loss) cudaMemsetAsync(epoch_loss, 0, sizeof(float) * 2 * (size_t)epochs, st);
-  // three launches per minibatch: loss, backward, Adam + packing (which also
+  // two launches per minibatch: loss and gradients, Adam + packing (which also
   // clears the other gradient buffer for the next minibatch)
   int step = 0;
   for (int ep = 0; ep < epochs; ep++) {

@@ -1161,13 +1161,14 @@ __device__ int run_cdcl(const Solve& S, Warp& w, int64_t slot, int unit, int ins
   // clause sharing with the other jobs of this instance: on for a cube and
   // once this job has given one away or sees others running
   bool shared = S.share_lbd > 0 && job != nullptr;
-  unsigned long long share_rd = 0;
+  unsigned long long share_rd =
+      S.share_lbd > 0 ? S.share_base[(uint32_t)inst & S.share_mask] : 0ull;
   for (;;) {
     if ((++iter & 63u) == 0u) {
       int stop = 0;
       if (w.lane == 0) {
         if (S.abort_flag && *S.abort_flag) stop = 1;
-        else if (globaltimer() - S.ctrl->t0 > S.time_ns) stop = 2;
+        else if (search_ns(S) > S.time_ns) stop = 2;
         else if (*(volatile uint32_t*)&S.done[unit] & 1u) stop = 3;
 #ifdef SCUBA_CHECKED
         else if (batch_failed(S.ctrl)) stop = 4;  // a bounds check failed: stop

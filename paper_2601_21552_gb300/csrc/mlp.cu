@@ -239,119 +239,113 @@ __global__ void __launch_bounds__(32 * kGradWarps, 2)
                 const float* target, float* dS, float* grad, int split) {
   __shared__ float stage[kGradWarps][kGradStride];
   __shared__ SoftStat warp_stat[kGradWarps];
-  __shared__ SoftStat cta_stat[2];
+  __shared__ SoftStat cta_stat;
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
   const int g = lane >> 2, t = lane & 3;
   const int rank = blockIdx.x % split;
   HiddenWeights H;
   load_hidden(W, g, t, H);
   const float b2 = W->b2;
-  float cw1[4][2][4], gw2[4][2], gb1[4][2], gb2 = 0.0f, ce = 0.0f, used = 0.0f;
+  float cw1[4][2][4], gw2[4][2], gb1[4][2], gb2 = 0.0f, ce = 0.0f;
 #pragma unroll
   for (int q = 0; q < 4; q++) {
     gw2[q][0] = gw2[q][1] = gb1[q][0] = gb1[q][1] = 0.0f;
 #pragma unroll
     for (int f = 0; f < 2; f++) cw1[q][f][0] = cw1[q][f][1] = cw1[q][f][2] = cw1[q][f][3] = 0.0f;
   }
+  const int64_t k = k0 + blockIdx.x / split;
   const int64_t step = 16 * (int64_t)kGradWarps * split;
-  int parity = 0;
-  for (int64_t k = k0 + blockIdx.x / split; k < k1; k += gridDim.x / split, parity ^= 1) {
-    const int64_t r0 = node_row[k], end = r0 + node_nrows[k];
-    const int64_t first = r0 + 16 * ((int64_t)wib * split + rank);
-    // scores and their statistics
-    SoftStat st{-INFINITY, 0.0f, 0.0f};
-    {
-      uint2 x0 = load_row<WIDE>(x, first + g, end, t), x1 = load_row<WIDE>(x, first + g + 8, end, t);
-      for (int64_t r = first; r < end; r += step) {
-        const uint2 n0 = load_row<WIDE>(x, r + step + g, end, t);
-        const uint2 n1 = load_row<WIDE>(x, r + step + g + 8, end, t);
-        const int64_t row = r + lane_row(g, t);
-        const bool mine = g < 4 && row < end;
-        const float tv = mine ? target[row] : 0.0f;
-        const float s = tile_score(H, x0, x1, g) + b2;
-        if (mine) {
-          dS[row] = s;
-          st.t += tv;
-          if (s > st.m) {
-            st.e *= expf(st.m - s);
-            st.m = s;
-          }
-          st.e += exp_from(s, st.m);
-        }
-        x0 = n0;
-        x1 = n1;
+  const int64_t r0 = node_row[k], end = r0 + node_nrows[k];
+  const int64_t first = r0 + 16 * ((int64_t)wib * split + rank);
+  // scores and their statistics
+  SoftStat st{-INFINITY, 0.0f, 0.0f};
+  uint2 x0 = load_row<WIDE>(x, first + g, end, t), x1 = load_row<WIDE>(x, first + g + 8, end, t);
+  for (int64_t r = first; r < end; r += step) {
+    const uint2 n0 = load_row<WIDE>(x, r + step + g, end, t);
+    const uint2 n1 = load_row<WIDE>(x, r + step + g + 8, end, t);
+    const int64_t row = r + lane_row(g, t);
+    const bool mine = g < 4 && row < end;
+    const float tv = mine ? target[row] : 0.0f;
+    const float s = tile_score(H, x0, x1, g) + b2;
+    if (mine) {
+      dS[row] = s;
+      st.t += tv;
+      if (s > st.m) {
+        st.e *= expf(st.m - s);
+        st.m = s;
       }
+      st.e += exp_from(s, st.m);
     }
-    for (int d = 16; d > 0; d >>= 1)
-      st = merge(st, SoftStat{__shfl_xor_sync(FULL, st.m, d), __shfl_xor_sync(FULL, st.e, d),
-                              __shfl_xor_sync(FULL, st.t, d)});
-    __syncthreads();  // the previous node's statistics have been read
-    if (lane == 0) warp_stat[wib] = st;
-    __syncthreads();
-    st = warp_stat[0];
-    for (int w = 1; w < kGradWarps; w++) st = merge(st, warp_stat[w]);
-    if (split > 1) {
-      // two slots: a block may be one node ahead of the slowest reader of the
-      // other slot, never two (the barrier of the node between them)
-      cooperative_groups::cluster_group cl = cooperative_groups::this_cluster();
-      if (threadIdx.x == 0) cta_stat[parity] = st;
-      cl.sync();
-      st = *cl.map_shared_rank(&cta_stat[parity], 0);
-      for (int b = 1; b < split; b++) st = merge(st, *cl.map_shared_rank(&cta_stat[parity], b));
-    }
-    const bool use = node_closed[k] && end - r0 > 1 && st.t > 0.0f;
-    if (!use) {
-      for (int64_t r = first; r < end; r += step) {
-        const int64_t row = r + lane_row(g, t);
-        if (g < 4 && row < end) dS[row] = 0.0f;
-      }
-      continue;
-    }
-    const float lse = st.m + logf(st.e);
-    if (rank == 0 && threadIdx.x == 0) used += 1.0f;
+    x0 = n0;
+    x1 = n1;
+  }
+  for (int d = 16; d > 0; d >>= 1)
+    st = merge(st, SoftStat{__shfl_xor_sync(FULL, st.m, d), __shfl_xor_sync(FULL, st.e, d),
+                            __shfl_xor_sync(FULL, st.t, d)});
+  if (lane == 0) warp_stat[wib] = st;
+  __syncthreads();
+  st = warp_stat[0];
+  for (int w = 1; w < kGradWarps; w++) st = merge(st, warp_stat[w]);
+  if (split > 1) {
+    cooperative_groups::cluster_group cl = cooperative_groups::this_cluster();
+    if (threadIdx.x == 0) cta_stat = st;
+    cl.sync();
+    st = *cl.map_shared_rank(&cta_stat, 0);
+    for (int b = 1; b < split; b++) st = merge(st, *cl.map_shared_rank(&cta_stat, b));
+  }
+  if (!(node_closed[k] && end - r0 > 1 && st.t > 0.0f)) {  // the node takes no part
     for (int64_t r = first; r < end; r += step) {
-      const uint2 x0 = load_row<WIDE>(x, r + g, end, t), x1 = load_row<WIDE>(x, r + g + 8, end, t);
       const int64_t row = r + lane_row(g, t);
-      float ds_mine = 0.0f;
-      if (g < 4 && row < end) {
-        const float s = dS[row], tn = target[row] / st.t;
-        ds_mine = expf(s - lse) - tn;
-        dS[row] = ds_mine;
-        ce -= tn * (s - lse);
-        gb2 += ds_mine;
-      }
-      float ds[2][2];  // rows 8h + 2t + j
+      if (g < 4 && row < end) dS[row] = 0.0f;
+    }
+    if (split > 1) cooperative_groups::this_cluster().sync();  // the others have read cta_stat
+    return;
+  }
+  const float lse = st.m + logf(st.e);
+  for (int64_t r = first; r < end; r += step) {
+    x0 = load_row<WIDE>(x, r + g, end, t);
+    x1 = load_row<WIDE>(x, r + g + 8, end, t);
+    const int64_t row = r + lane_row(g, t);
+    float ds_mine = 0.0f;
+    if (g < 4 && row < end) {
+      const float s = dS[row], tn = target[row] / st.t;
+      ds_mine = expf(s - lse) - tn;
+      dS[row] = ds_mine;
+      ce -= tn * (s - lse);
+      gb2 += ds_mine;
+    }
+    float ds[2][2];  // rows 8h + 2t + j
 #pragma unroll
-      for (int h = 0; h < 2; h++)
+    for (int h = 0; h < 2; h++)
 #pragma unroll
-        for (int j = 0; j < 2; j++)
-          ds[h][j] = __shfl_sync(FULL, ds_mine, 4 * (2 * h + j) + t);
-      // X as a B operand (rows x logical features): b[f][h] for rows 8h .. 8h+7
-      const uint32_t bx[2][2] = {{transpose8x8(x0.x), transpose8x8(x1.x)},
-                                 {transpose8x8(x0.y), transpose8x8(x1.y)}};
+      for (int j = 0; j < 2; j++)
+        ds[h][j] = __shfl_sync(FULL, ds_mine, 4 * (2 * h + j) + t);
+    // X as a B operand (rows x logical features): b[f][h] for rows 8h .. 8h+7
+    const uint32_t bx[2][2] = {{transpose8x8(x0.x), transpose8x8(x1.x)},
+                               {transpose8x8(x0.y), transpose8x8(x1.y)}};
 #pragma unroll
-      for (int q = 0; q < 4; q++) {
-        uint32_t dh[4];  // dH^T: units 16q .. 16q+15, the tile's rows
+    for (int q = 0; q < 4; q++) {
+      uint32_t dh[4];  // dH^T: units 16q .. 16q+15, the tile's rows
 #pragma unroll
-        for (int h = 0; h < 2; h++) {
-          float z[4], d[4];
-          mma_add(z, H.a[q], h ? x1.x : x0.x, h ? x1.y : x0.y, H.b1[q][0], H.b1[q][0], H.b1[q][1],
-                  H.b1[q][1]);
+      for (int h = 0; h < 2; h++) {
+        float z[4], d[4];
+        mma_add(z, H.a[q], h ? x1.x : x0.x, h ? x1.y : x0.y, H.b1[q][0], H.b1[q][0], H.b1[q][1],
+                H.b1[q][1]);
 #pragma unroll
-          for (int u = 0; u < 4; u++)
-            d[u] = z[u] > 0.f ? ds[h][u & 1] * H.w2[q][u >> 1] : 0.f;
-          gw2[q][0] += fmaxf(z[0], 0.f) * ds[h][0] + fmaxf(z[1], 0.f) * ds[h][1];
-          gw2[q][1] += fmaxf(z[2], 0.f) * ds[h][0] + fmaxf(z[3], 0.f) * ds[h][1];
-          gb1[q][0] += d[0] + d[1];
-          gb1[q][1] += d[2] + d[3];
-          dh[2 * h] = learn::pack_bf16(__float2bfloat16(d[0]), __float2bfloat16(d[1]));
-          dh[2 * h + 1] = learn::pack_bf16(__float2bfloat16(d[2]), __float2bfloat16(d[3]));
+        for (int u = 0; u < 4; u++)
+          d[u] = z[u] > 0.f ? ds[h][u & 1] * H.w2[q][u >> 1] : 0.f;
+#pragma unroll
+        for (int u = 0; u < 4; u++) {
+          if (z[u] > 0.f) gw2[q][u >> 1] += z[u] * ds[h][u & 1];
+          gb1[q][u >> 1] += d[u];
         }
-#pragma unroll
-        for (int f = 0; f < 2; f++)
-          mma_add(cw1[q][f], dh, bx[f][0], bx[f][1], cw1[q][f][0], cw1[q][f][1], cw1[q][f][2],
-                  cw1[q][f][3]);
+        dh[2 * h] = learn::pack_bf16(__float2bfloat16(d[0]), __float2bfloat16(d[1]));
+        dh[2 * h + 1] = learn::pack_bf16(__float2bfloat16(d[2]), __float2bfloat16(d[3]));
       }
+#pragma unroll
+      for (int f = 0; f < 2; f++)
+        mma_add(cw1[q][f], dh, bx[f][0], bx[f][1], cw1[q][f][0], cw1[q][f][1], cw1[q][f][2],
+                cw1[q][f][3]);
     }
   }
   if (split > 1) cooperative_groups::this_cluster().sync();  // every remote read is done
@@ -385,7 +379,7 @@ __global__ void __launch_bounds__(32 * kGradWarps, 2)
   if (lane == 0) {
     mine[19 * NHID] = gb2;
     mine[19 * NHID + 1] = ce;
-    mine[19 * NHID + 2] = used;
+    mine[19 * NHID + 2] = rank == 0 && wib == 0 ? 1.0f : 0.0f;  // nodes used
   }
   __syncthreads();
   for (int p = threadIdx.x; p < NPARAM + 2; p += blockDim.x) {
@@ -524,7 +518,7 @@ static void grad_kernels(const scuba_trace* tr, int64_t k0, int64_t k1, const vo
   attr.val.clusterDim.x = split;
   attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((unsigned)(std::min(nodes * split, slots / split * split)));
+  cfg.gridDim = dim3((unsigned)(nodes * split));
   cfg.blockDim = dim3(32 * mlpk::kGradWarps);
   cfg.stream = st;
   cfg.attrs = &attr;

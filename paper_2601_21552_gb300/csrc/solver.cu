@@ -2,11 +2,9 @@
 // Sec. V-B, step 10, applied to one query per static memory instruction).
 //
 // Layout in HBM (per batch, built by the prep kernels from the caller's CSR):
-//   norm[L]        u32  normalised literal code per literal slot (2(v-1)+neg),
-//                       NONE for dropped slots, UNIT_BIT for unit clauses
 //   occ_begin[..]  u32  per instance 2V+1 offsets: occurrence list of each
-//                       literal code (clauses that contain it)
-//   ent[L]         u64  occurrence entries, in clause order within a list:
+//                       literal code 2(v-1)+neg (clauses that contain it)
+//   ent[L]         u64  occurrence entries, clause group by clause group within a list:
 //                       binary (x|y) in x's list = {y, NONE}; ternary
 //                       (x|y|z) in x's list = {y, z}; longer clauses =
 //                       {LONG_CLAUSE|local clause index, 0}
@@ -43,7 +41,6 @@ namespace dev {
 constexpr uint32_t FULL = 0xffffffffu;
 constexpr uint32_t NONE = 0xffffffffu;
 constexpr uint32_t LONG_CLAUSE = 0x80000000u;
-constexpr uint32_t UNIT_BIT = 0x40000000u;
 constexpr uint32_t FLIP = 0x80000000u;
 constexpr uint32_t F_EMPTY = 1u, F_BAD = 2u;
 constexpr int MAX_PREFIX = 248;   // literals in a split job's prefix
@@ -75,8 +72,9 @@ struct Ctrl {
   uint32_t idle;        // warps waiting for work
   int32_t status;       // first error (scuba status code)
   uint32_t q_head, q_tail;
-  uint64_t t0;          // globaltimer at launch
+  uint64_t t0;          // globaltimer when the search began (0: not yet)
   uint32_t jobs_split;  // statistics
+  uint32_t next_item, n_items;  // preparation work items
   int32_t check_site;   // checked build: site of the first failed bounds check (0: none)
   uint64_t check_index; // ... the index it saw
   uint64_t check_limit; // ... and the bound it broke
@@ -114,251 +112,6 @@ __device__ __forceinline__ bool batch_failed(Ctrl* c) {
   return *(volatile int32_t*)&c->status != 0;
 }
 
-struct Prep {
-  int n;
-  int64_t C, L;
-  int64_t total_vars;  // model size promised by the caller
-  int64_t occ_cap;     // allocated occurrence-offset entries
-  int32_t vmax;
-  const int64_t* vb;
-  Ctrl* ctrl;
-  const int64_t* icb;
-  const int64_t* cb;
-  const int32_t* lits;
-  const int32_t* nv;
-  int64_t* occ_base;   // [n+1]
-  uint32_t* norm;      // [L]
-  uint32_t* occ_cnt;   // [occ_total] counts, then fill cursors
-  uint32_t* occ_begin; // [occ_total]
-  uint64_t* ent;       // [L]
-  uint32_t* units;     // [C]
-  uint32_t* nunits;    // [n]
-  uint32_t* flags;     // [n]
-};
-
-__device__ __forceinline__ int32_t clamp_nv(int32_t v, int32_t vmax) {
-  return v < 0 ? 0 : (v > vmax ? vmax : v);
-}
-
-// occ_base[i] = sum_{j<i} (2 nv[j] + 1); single block, chunked scan. Also
-// validates the batch header: clause ranges monotonic and covering exactly
-// [0, total_clauses), 0 <= nv <= max_vars, model ranges inside total_vars.
-// Instances that fail get F_BAD; a header that cannot be trusted at all
-// stops the whole batch with SCUBA_ERR_MALFORMED.
-__global__ void k_occ_base(Prep P) {
-  __shared__ int64_t part[1024];
-  __shared__ int bad_header;
-  const int n = P.n, t = threadIdx.x, T = blockDim.x;
-  if (t == 0) bad_header = (P.icb[0] != 0 || P.icb[n] != P.C);
-  __syncthreads();
-  const int per = (n + T - 1) / T;
-  const int b = min(n, t * per), e = min(n, b + per);
-  int64_t s = 0;
-  for (int i = b; i < e; i++) {
-    const int32_t v = P.nv[i];
-    if (P.icb[i] > P.icb[i + 1]) bad_header = 1;
-    uint32_t f = 0;
-    if (v < 0 || v > P.vmax) f |= F_BAD;
-    // occurrence offsets are 32-bit within an instance
-    const int64_t ca = P.icb[i], cz = P.icb[i + 1];
-    if (ca >= 0 && cz >= ca && cz <= P.C && P.cb[cz] - P.cb[ca] >= (1LL << 32)) f |= F_BAD;
-    if (P.vb[i] < 0 || P.vb[i] + (int64_t)(v < 0 ? 0 : v) > P.total_vars) f |= F_BAD;
-    if (f) atomicOr(&P.flags[i], f);
-    s += 2 * (int64_t)clamp_nv(v, P.vmax) + 1;
-  }
-  part[t] = s;
-  __syncthreads();
-  if (t == 0) {
-    int64_t acc = 0;
-    for (int k = 0; k < T; k++) {
-      int64_t v = part[k];
-      part[k] = acc;
-      acc += v;
-    }
-    P.occ_base[n] = acc;
-    if (acc > P.occ_cap) bad_header = 1;
-  }
-  __syncthreads();
-  int64_t acc = part[t];
-  for (int i = b; i < e; i++) {
-    P.occ_base[i] = acc;
-    acc += 2 * (int64_t)clamp_nv(P.nv[i], P.vmax) + 1;
-  }
-  if (t == 0 && bad_header) fail_batch(P.ctrl, SCUBA_ERR_MALFORMED);
-}
-
-__device__ __forceinline__ int find_inst(const int64_t* icb, int n, int64_t c) {
-  int lo = 0, hi = n - 1;  // largest i with icb[i] <= c
-  while (lo < hi) {
-    int mid = (lo + hi + 1) >> 1;
-    if (icb[mid] <= c) lo = mid; else hi = mid - 1;
-  }
-  return lo;
-}
-
-// One thread per clause: validate, normalise clauses of length <= 3
-// (duplicates removed, tautologies dropped), count occurrences.
-__global__ void k_normalize(Prep P) {
-  if (batch_failed(P.ctrl)) return;
-  for (int64_t c = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; c < P.C;
-       c += (int64_t)gridDim.x * blockDim.x) {
-    int i = find_inst(P.icb, P.n, c);
-    while (i + 1 < P.n && P.icb[i + 1] <= c) i++;  // skip empty instances
-    const int V = clamp_nv(P.nv[i], P.vmax);
-    const int64_t b = P.cb[c], e = P.cb[c + 1];
-    if (b < 0 || e < b || e > P.L) { atomicOr(&P.flags[i], F_BAD); continue; }
-    const int64_t len = e - b;
-    bool bad = false;
-    for (int64_t k = b; k < e; k++) {
-      int32_t l = P.lits[k];
-      if (l == 0 || l > V || l < -V) bad = true;
-    }
-    if (bad) {
-      atomicOr(&P.flags[i], F_BAD);
-      for (int64_t k = b; k < e; k++) P.norm[k] = NONE;
-      continue;
-    }
-    if (len == 0) { atomicOr(&P.flags[i], F_EMPTY); continue; }
-    uint32_t* cnt = P.occ_cnt + P.occ_base[i];
-    if (len <= 3) {
-      uint32_t u[3];
-      int k = 0;
-      bool taut = false;
-      for (int64_t q = b; q < e; q++) {
-        uint32_t x = code_of(P.lits[q]);
-        bool dup = false;
-        for (int r = 0; r < k; r++) {
-          if (u[r] == x) dup = true;
-          if (u[r] == (x ^ 1u)) taut = true;
-        }
-        P.norm[q] = dup ? NONE : x;
-        if (!dup) u[k++] = x;
-      }
-      if (taut) {
-        for (int64_t q = b; q < e; q++) P.norm[q] = NONE;
-      } else if (k == 1) {
-        for (int64_t q = b; q < e; q++)
-          if (P.norm[q] != NONE) P.norm[q] |= UNIT_BIT;
-      } else {
-        for (int r = 0; r < k; r++) atomicAdd(&cnt[u[r]], 1u);
-      }
-    } else {
-      for (int64_t q = b; q < e; q++) {
-        uint32_t x = code_of(P.lits[q]);
-        P.norm[q] = x;
-        atomicAdd(&cnt[x], 1u);
-      }
-    }
-  }
-}
-
-// One warp per instance: exclusive scan of the 2V counts -> occ_begin; the
-// counts become fill cursors.
-__global__ void k_occ_scan(Prep P) {
-  if (batch_failed(P.ctrl)) return;
-  const int lane = threadIdx.x & 31;
-  const int w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int W = (gridDim.x * blockDim.x) >> 5;
-  for (int i = w; i < P.n; i += W) {
-    const int64_t base = P.occ_base[i];
-    const uint32_t m = 2u * (uint32_t)clamp_nv(P.nv[i], P.vmax);
-    uint32_t run = 0;
-    for (uint32_t s = 0; s < m; s += 32) {
-      uint32_t k = s + lane;
-      uint32_t v = k < m ? P.occ_cnt[base + k] : 0u;
-      uint32_t inc = v;
-      for (int d = 1; d < 32; d <<= 1) {
-        uint32_t y = __shfl_up_sync(FULL, inc, d);
-        if (lane >= d) inc += y;
-      }
-      if (k < m) {
-        P.occ_begin[base + k] = run + inc - v;
-        P.occ_cnt[base + k] = run + inc - v;
-      }
-      run += __shfl_sync(FULL, inc, 31);
-    }
-    if (lane == 0) P.occ_begin[base + m] = run;
-  }
-}
-
-// One warp per instance: fill occurrence entries in clause order
-// (deterministic), and compact the unit literals.
-__global__ void k_fill(Prep P) {
-  if (batch_failed(P.ctrl)) return;
-  __shared__ uint32_t sbase[32 * 8];
-  const int lane = threadIdx.x & 31;
-  const int wib = threadIdx.x >> 5;
-  uint32_t* my_base = sbase + 32 * wib;
-  const int w = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-  const int W = (gridDim.x * blockDim.x) >> 5;
-  for (int i = w; i < P.n; i += W) {
-    if (P.flags[i] & F_BAD) continue;
-    const int64_t c0 = P.icb[i], c1 = P.icb[i + 1];
-    const int64_t lbase = c0 < c1 ? P.cb[c0] : 0;
-    uint32_t* cur = P.occ_cnt + P.occ_base[i];
-    uint32_t nunit = 0;
-    for (int64_t cs = c0; cs < c1; cs += 32) {
-      const int64_t c = cs + lane;
-      const bool valid = c < c1;
-      int64_t b = 0, e = 0;
-      uint32_t lits3[3] = {NONE, NONE, NONE};
-      int nk = 0;
-      bool is_long = false, is_unit = false;
-      uint32_t unit_code = 0;
-      if (valid) {
-        b = P.cb[c];
-        e = P.cb[c + 1];
-        if (e - b > 3) {
-          is_long = true;
-          nk = (int)(e - b);
-        } else {
-          for (int64_t q = b; q < e; q++) {
-            uint32_t x = P.norm[q];
-            if (x == NONE) continue;
-            if (x & UNIT_BIT) { is_unit = true; unit_code = x & ~UNIT_BIT; continue; }
-            lits3[nk++] = x;
-          }
-          if (nk < 2) nk = 0;
-        }
-      }
-      // units, in clause order
-      uint32_t ub = __ballot_sync(FULL, is_unit);
-      if (is_unit) P.units[c0 + nunit + __popc(ub & ((1u << lane) - 1u))] = unit_code;
-      nunit += __popc(ub);
-      int rounds = __reduce_max_sync(FULL, (unsigned)nk);
-      for (int k = 0; k < rounds; k++) {
-        const bool has = k < nk;
-        uint32_t code = 0x80000000u | (uint32_t)lane;  // unique dummy
-        uint64_t entry = 0;
-        if (has) {
-          if (is_long) {
-            code = P.norm[b + k];
-            entry = (uint64_t)(LONG_CLAUSE | (uint32_t)(c - c0));
-          } else {
-            code = lits3[k];
-            uint32_t o1 = lits3[k == 0 ? 1 : 0];
-            uint32_t o2 = nk == 3 ? lits3[k == 2 ? 1 : 2] : NONE;
-            entry = (uint64_t)o1 | ((uint64_t)o2 << 32);
-          }
-        }
-        uint32_t grp = __match_any_sync(FULL, code);
-        int leader = __ffs(grp) - 1;
-        if (has && lane == leader) {
-          my_base[lane] = cur[code];
-          cur[code] += __popc(grp);
-        }
-        __syncwarp();
-        if (has) {
-          uint32_t pos = my_base[leader] + __popc(grp & ((1u << lane) - 1u));
-          P.ent[lbase + pos] = entry;
-        }
-        __syncwarp();
-      }
-    }
-    if (lane == 0) P.nunits[i] = nunit;
-  }
-}
-
 // --------------------------------------------------------------------------
 // Solve
 // --------------------------------------------------------------------------
@@ -370,6 +123,8 @@ struct Job {            // a DPLL subtree: the instance plus assumed literals
   uint32_t seq;         // ring-buffer sequence number (Vyukov MPMC queue)
   float inc;            // donor's activity increment; its activities are in job_act
 };
+
+#include "prep.cuh"
 
 // Decision-trace buffers (training data for the branching network).
 struct TraceDev {
@@ -463,6 +218,7 @@ struct Solve {
   // (inst & share_mask) is a ring of share_cap records of SHARE_REC words
   uint32_t* share;             // [pools][share_cap][SHARE_REC]
   unsigned long long* share_cur;  // [pools] records reserved so far
+  const unsigned long long* share_base;  // [pools] ... before this call
   uint32_t share_mask;         // pools - 1 (a power of two)
   uint32_t share_cap;          // records per pool (a power of two)
   uint32_t share_lbd;          // publish learned clauses of LBD <= this; 0: off
@@ -985,6 +741,17 @@ __device__ uint32_t pick(Warp& w) {
   return best_v;
 }
 
+// When the search began. Warps of one launch start at different times, so the
+// first of them sets it (start_clock) and every read goes to memory.
+__device__ __forceinline__ void start_clock(Ctrl* c) {
+  atomicCAS(reinterpret_cast<unsigned long long*>(&c->t0), 0ull,
+            (unsigned long long)globaltimer());
+}
+
+__device__ __forceinline__ uint64_t search_ns(const Solve& S) {
+  return globaltimer() - *(volatile uint64_t*)&S.ctrl->t0;
+}
+
 __device__ __forceinline__ void set_status(const Solve& S, int32_t st) {
   atomicCAS(&S.ctrl->status, 0, st);
 }
@@ -1093,7 +860,7 @@ __device__ void finish_job(const Solve& S, Warp& w, int unit, int r) {
       uint32_t d = atomicOr(&S.done[unit], 4u);
       if (!(d & 1u)) S.verdict[unit] = (d & 2u) ? SCUBA_UNKNOWN : SCUBA_UNSAT;
       atomicSub(&S.ctrl->inst_left, 1u);
-      if (S.finish_ns) S.finish_ns[unit] = (int64_t)(globaltimer() - S.ctrl->t0);
+      if (S.finish_ns) S.finish_ns[unit] = (int64_t)search_ns(S);
     }
     if (S.prof) {
       atomicAdd(&S.prof[1], 1ull);  // jobs run
@@ -1219,7 +986,7 @@ __device__ int run_job_body(const Solve& S, Warp& w, int unit, int inst, const T
       int stop = 0;
       if (w.lane == 0) {
         if (S.abort_flag && *S.abort_flag) stop = 1;
-        else if (globaltimer() - S.ctrl->t0 > S.time_ns) stop = 2;
+        else if (search_ns(S) > S.time_ns) stop = 2;
         else if (*(volatile uint32_t*)&S.done[unit] & 1u) stop = 3;  // solved elsewhere
 #ifdef SCUBA_CHECKED
         else if (batch_failed(S.ctrl)) stop = 4;  // a bounds check failed: stop
@@ -1367,6 +1134,7 @@ __global__ void __launch_bounds__(256, MODE == MODE_LEARNED ? SCUBA_LEARNED_MINB
                                     ((off + 15) & ~(size_t)15) + (size_t)wib * CD_SMEM_WARP);
   }
   if (batch_failed(S.ctrl)) return;
+  if (lane == 0) start_clock(S.ctrl);
   bool counted_idle = false;
   for (;;) {
     // 1) a shared subtree, 2) a fresh unit (an instance, possibly under
@@ -1426,7 +1194,7 @@ __global__ void __launch_bounds__(256, MODE == MODE_LEARNED ? SCUBA_LEARNED_MINB
           if (*(volatile uint32_t*)&S.ctrl->inst_left == 0u) stop = 1;
           else if (*(volatile int32_t*)&S.ctrl->status != 0) stop = 1;
           else if (S.abort_flag && *S.abort_flag) { stop = 1; set_status(S, SCUBA_ERR_ABORTED); }
-          else if (globaltimer() - S.ctrl->t0 > S.time_ns) { stop = 1; set_status(S, SCUBA_ERR_TIMEOUT); }
+          else if (search_ns(S) > S.time_ns) { stop = 1; set_status(S, SCUBA_ERR_TIMEOUT); }
           else {
             if (S.prof) atomicAdd(&S.prof[5], 1ull);  // idle polls
             __nanosleep(2000);
@@ -1519,7 +1287,8 @@ __global__ void __launch_bounds__(256) k_propagate(const __grid_constant__ PropA
   const int64_t slot = (int64_t)blockIdx.x * wpb + wib;
   w.trail = A.trail + slot * A.vmax;
   if (batch_failed(A.ctrl)) return;
-  for (int i = (int)(blockIdx.x * wpb + wib); i < A.n; i += gridDim.x * wpb) {
+  // instance i goes to block i mod grid: few instances spread over the SMs
+  for (int i = (int)(wib * gridDim.x + blockIdx.x); i < A.n; i += gridDim.x * wpb) {
     if (A.flags[i] & F_BAD) continue;
     w.V = (uint32_t)A.nv[i];
     w.c0 = A.icb[i];
@@ -1556,44 +1325,6 @@ __global__ void __launch_bounds__(256) k_propagate(const __grid_constant__ PropA
   }
 }
 
-// Instances still open when the kernel stopped (timeout / abort) -> UNKNOWN.
-__global__ void k_finalize(Solve S) {
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < S.n_units;
-       i += gridDim.x * blockDim.x) {
-    uint32_t d = S.done[i];
-    if (!(d & 5u)) S.verdict[i] = SCUBA_UNKNOWN;
-  }
-}
-
-__global__ void k_init_ring(Job* ring, uint32_t cap) {
-  for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < cap; i += gridDim.x * blockDim.x)
-    ring[i].seq = i;
-}
-
-__global__ void k_init_inst(uint32_t* pending, uint32_t* done, unsigned long long* dec, int n) {
-  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
-    pending[i] = 1u;
-    done[i] = 0u;
-    dec[i] = 0ull;
-  }
-}
-
-__global__ void k_start_clock(Ctrl* c) { c->t0 = globaltimer(); }
-
-__global__ void k_init_ctrl(Ctrl* c, uint32_t n) {
-  c->next_inst = 0;
-  c->inst_left = n;
-  c->idle = 0;
-  c->status = 0;
-  c->q_head = 0;
-  c->q_tail = 0;
-  c->t0 = globaltimer();
-  c->jobs_split = 0;
-  c->check_site = 0;
-  c->check_index = 0;
-  c->check_limit = 0;
-}
-
 }  // namespace dev
 
 // --------------------------------------------------------------------------
@@ -1608,11 +1339,11 @@ struct Buf {
 };
 
 struct Scratch {
-  Buf occ_base, norm, occ_cnt, occ_begin, ent, units, nunits, flags;
+  Buf occ_base, occ_begin, ent, units, nunits, flags, items;
   Buf pending, done, inst_dec, trail, dstack, act, ring, job_act, prefix, ctrl;
   Buf lvlcnt, lvl_node;
   Buf cd_var, cd_mark, cd_wl, cd_pool, cd_learnt, cd_arena, cd_clidx;
-  Buf share, share_cur;
+  Buf share, share_cur, share_base;
   Buf job_cls, cls_copy;
   Buf h_icb, h_cb, h_lits, h_nv, h_vb, h_verdict, h_model, h_stats;  // for the host entry
   int sms = 0;
@@ -1651,6 +1382,73 @@ T* P(Buf& b) { return reinterpret_cast<T*>(b.p); }
 int cuda_fail(const char* what, cudaError_t e) {
   set_error(std::string(what) + ": " + cudaGetErrorString(e));
   return SCUBA_ERR_CUDA;
+}
+
+// Launch shape of the preparation kernel: a batch whose literals fit 72 KB of
+// counters of 8 warps (1,843 variables) takes one block of 256 threads per
+// instance, three or more of them on an SM; larger instances take blocks of
+// 1,024 threads, one per SM, each a range of up to 3,264 literals.
+constexpr size_t kPrepSmem8 = 72 * 1024, kPrepSmem32 = 3264 * 68;
+
+struct PrepShape {
+  int warps;
+  uint32_t range;
+  size_t smem;
+  int64_t items;  // upper bound of the work items
+  bool table;     // more than one item per instance is possible
+};
+
+PrepShape prep_shape(int64_t n, int64_t total_vars, int vmax) {
+  PrepShape s;
+  const uint32_t lits = 2u * (uint32_t)vmax;
+  s.warps = (size_t)lits * 20 <= kPrepSmem8 ? 8 : 32;
+  s.range = s.warps == 8 ? lits : std::min(lits, 3264u);
+  s.smem = (size_t)s.range * 4 * (1 + s.warps / 2);
+  s.table = lits > s.range;
+  s.items = n + (s.table ? 2 * total_vars / s.range : 0);
+  return s;
+}
+
+// The batch's arrays and sizes; the caller fills in the scratch.
+dev::Prep prep_args(const scuba_cnf_batch* b, int vmax, const PrepShape& shape) {
+  dev::Prep pr;
+  pr.n = b->num_instances;
+  pr.C = b->total_clauses;
+  pr.L = b->total_lits;
+  pr.total_vars = b->total_vars;
+  pr.occ_cap = 2LL * b->total_vars + b->num_instances;
+  pr.vmax = vmax;
+  pr.range = shape.range;
+  pr.vb = b->inst_var_begin;
+  pr.icb = b->inst_clause_begin;
+  pr.cb = b->clause_begin;
+  pr.lits = b->lits;
+  pr.nv = b->inst_num_vars;
+  pr.items = nullptr;
+  pr.item_cap = (uint32_t)std::min<int64_t>(shape.items, 0xffffffffll);
+  return pr;
+}
+
+// Set-up and preparation of one call on `st`: two launches.
+cudaError_t launch_prep(const dev::Prep& pr, const dev::SearchInit& init, const PrepShape& shape,
+                        int sms, cudaStream_t st) {
+  const int64_t words = std::max<int64_t>(
+      {(int64_t)init.n_units, (int64_t)init.ring_cap, init.share_cur ? (int64_t)init.share_pools : 0});
+  const int others = (int)std::min<int64_t>((words + 1023) / 1024, 2 * (int64_t)sms);
+  dev::k_setup<<<1 + others, 1024, 0, st>>>(pr, init);
+  auto kern = shape.warps == 8 ? dev::k_prep<8> : dev::k_prep<32>;
+  // always the same value, so that calls of different batches agree on it
+  const cudaError_t e =
+      cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                           (int)(shape.warps == 8 ? kPrepSmem8 : kPrepSmem32));
+  if (e != cudaSuccess) return e;
+  const int64_t per_sm =
+      shape.warps == 8
+          ? std::max<int64_t>(1, std::min<int64_t>(8, 226 * 1024 / ((int64_t)shape.smem + 2048)))
+          : 1;
+  const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(shape.items, sms * per_sm));
+  kern<<<grid, 32 * shape.warps, shape.smem, st>>>(pr);
+  return cudaSuccess;
 }
 
 }  // namespace
@@ -1806,8 +1604,10 @@ static int solve_impl(const scuba_cnf_batch* b, uint8_t* verdict, uint8_t* model
   const int64_t slots = (int64_t)S.sms * bps * wpb;
   const uint32_t ring_cap = 2048;
 
-  if (ensure(S.occ_base, 8 * (size_t)(n + 1)) || ensure(S.norm, 4 * (size_t)L) ||
-      ensure(S.occ_cnt, 4 * (size_t)occ_total) || ensure(S.occ_begin, 4 * (size_t)occ_total) ||
+  const PrepShape shape = prep_shape(n, b->total_vars, vmax);
+  if (ensure(S.occ_base, 8 * (size_t)(n + 1)) ||
+      ensure(S.items, shape.table ? 8 * (size_t)shape.items : 0) ||
+      ensure(S.occ_begin, 4 * (size_t)occ_total) ||
       ensure(S.ent, 8 * (size_t)L) || ensure(S.units, 4 * (size_t)std::max<int64_t>(C, 1)) ||
       ensure(S.nunits, 4 * (size_t)n) || ensure(S.flags, 4 * (size_t)n) ||
       ensure(S.pending, 4 * (size_t)n_units) || ensure(S.done, 4 * (size_t)n_units) ||
@@ -1832,6 +1632,8 @@ static int solve_impl(const scuba_cnf_batch* b, uint8_t* verdict, uint8_t* model
       set_error("scuba_solve_batch: learnt_words must be at least max(max_vars + 8, 64)");
       return SCUBA_ERR_ARG;
     }
+    const size_t share_bytes = 4 * (size_t)kSharePools * kShareCap * dev::SHARE_REC;
+    const bool share_ready = S.share.p && S.share_cur.p && S.share_base.p;
     if (ensure(S.cd_var, 16 * (size_t)slots * vmax) ||
         ensure(S.cd_mark, (size_t)slots * vmax) ||
         ensure(S.cd_wl, 32 * (size_t)slots * vmax) ||
@@ -1841,46 +1643,25 @@ static int solve_impl(const scuba_cnf_batch* b, uint8_t* verdict, uint8_t* model
         ensure(S.cd_clidx, 4 * (size_t)slots * (arena_words / 8)) ||
         ensure(S.job_cls, 4 * (size_t)ring_cap * dev::JOB_CLS_WORDS) ||
         ensure(S.cls_copy, 4 * (size_t)slots * dev::JOB_CLS_WORDS) ||
-        ensure(S.share, 4 * (size_t)kSharePools * kShareCap * dev::SHARE_REC) ||
-        ensure(S.share_cur, 8 * (size_t)kSharePools)) {
+        ensure(S.share, share_bytes) || ensure(S.share_cur, 8 * (size_t)kSharePools) ||
+        ensure(S.share_base, 8 * (size_t)kSharePools)) {
       set_error("scuba_solve_batch: out of device memory for clause-learning scratch");
       return SCUBA_ERR_NOMEM;
     }
+    if (!share_ready) {  // fresh pools: no record, cursors at zero
+      cudaMemsetAsync(S.share.p, 0, share_bytes, st);
+      cudaMemsetAsync(S.share_cur.p, 0, 8 * (size_t)kSharePools, st);
+    }
   }
-  dev::Prep pr;
-  pr.n = n;
-  pr.C = C;
-  pr.L = L;
-  pr.icb = b->inst_clause_begin;
-  pr.cb = b->clause_begin;
-  pr.lits = b->lits;
-  pr.nv = b->inst_num_vars;
+  dev::Prep pr = prep_args(b, vmax, shape);
   pr.occ_base = P<int64_t>(S.occ_base);
-  pr.norm = P<uint32_t>(S.norm);
-  pr.occ_cnt = P<uint32_t>(S.occ_cnt);
   pr.occ_begin = P<uint32_t>(S.occ_begin);
   pr.ent = P<uint64_t>(S.ent);
   pr.units = P<uint32_t>(S.units);
   pr.nunits = P<uint32_t>(S.nunits);
   pr.flags = P<uint32_t>(S.flags);
-  pr.total_vars = b->total_vars;
-  pr.occ_cap = occ_total;
-  pr.vmax = vmax;
-  pr.vb = b->inst_var_begin;
+  if (shape.table) pr.items = P<int2>(S.items);
   pr.ctrl = P<dev::Ctrl>(S.ctrl);
-
-  NvtxRange prep_range("scuba prep + search launch");
-  dev::k_init_ctrl<<<1, 1, 0, st>>>(pr.ctrl, (uint32_t)n_units);
-  cudaMemsetAsync(pr.occ_cnt, 0, 4 * (size_t)occ_total, st);
-  cudaMemsetAsync(pr.flags, 0, 4 * (size_t)n, st);
-  dev::k_occ_base<<<1, 1024, 0, st>>>(pr);
-  if (C > 0) {
-    int grid = (int)std::min<int64_t>((C + 255) / 256, (int64_t)S.sms * 32);
-    dev::k_normalize<<<grid, 256, 0, st>>>(pr);
-  }
-  int wgrid = (int)std::min<int64_t>((n + 7) / 8, (int64_t)S.sms * 16);
-  dev::k_occ_scan<<<wgrid, 256, 0, st>>>(pr);
-  dev::k_fill<<<wgrid, 256, 0, st>>>(pr);
 
   dev::Solve sv;
   sv.n = n;
@@ -1948,19 +1729,19 @@ static int solve_impl(const scuba_cnf_batch* b, uint8_t* verdict, uint8_t* model
   sv.restart_unit = opt->restart_unit > 0 ? opt->restart_unit : 100;
   sv.share = nullptr;
   sv.share_cur = nullptr;
+  sv.share_base = nullptr;
   sv.share_mask = 0;
   sv.share_cap = 0;
   sv.share_lbd = 0;
   if (mode == dev::MODE_CDCL && opt->share_lbd >= 0) {
-    // the pools start empty every call: a record left by an earlier batch must
-    // never pass for one of this batch
+    // the pools keep earlier calls' records; this call's jobs read from where
+    // the cursors stood when it began (share_base)
     sv.share = P<uint32_t>(S.share);
     sv.share_cur = P<unsigned long long>(S.share_cur);
+    sv.share_base = P<unsigned long long>(S.share_base);
     sv.share_mask = kSharePools - 1;
     sv.share_cap = kShareCap;
     sv.share_lbd = opt->share_lbd > 0 ? (uint32_t)opt->share_lbd : 2u;
-    cudaMemsetAsync(sv.share, 0, 4 * (size_t)kSharePools * kShareCap * dev::SHARE_REC, st);
-    cudaMemsetAsync(sv.share_cur, 0, 8 * (size_t)kSharePools, st);
   }
   std::memset(&sv.tr, 0, sizeof(sv.tr));
   if (mode == dev::MODE_TRACE) {
@@ -1984,10 +1765,11 @@ static int solve_impl(const scuba_cnf_batch* b, uint8_t* verdict, uint8_t* model
     cudaMemsetAsync(sv.lvl_node, 0xff, 8 * (size_t)slots * learn::MAX_TRACE_DEPTH, st);
   }
 
-  dev::k_init_ring<<<16, 256, 0, st>>>(sv.ring, ring_cap);
-  dev::k_init_inst<<<(n_units + 255) / 256, 256, 0, st>>>(sv.pending, sv.done, sv.inst_dec,
-                                                          n_units);
-  dev::k_start_clock<<<1, 1, 0, st>>>(sv.ctrl);
+  NvtxRange prep_range("scuba prep + search launch");
+  const dev::SearchInit init{n_units, sv.pending, sv.done, sv.inst_dec, verdict, sv.ring, ring_cap,
+                             sv.share_cur, P<unsigned long long>(S.share_base), kSharePools};
+  e = launch_prep(pr, init, shape, S.sms, st);
+  if (e != cudaSuccess) return cuda_fail("preparation launch", e);
   auto kern = mode == dev::MODE_TRACE     ? dev::k_solve<dev::MODE_TRACE>
               : mode == dev::MODE_LEARNED ? dev::k_solve<dev::MODE_LEARNED>
               : mode == dev::MODE_CDCL    ? dev::k_solve<dev::MODE_CDCL>
@@ -2003,7 +1785,6 @@ static int solve_impl(const scuba_cnf_batch* b, uint8_t* verdict, uint8_t* model
   if (opt->search_event_begin) cudaEventRecord((cudaEvent_t)opt->search_event_begin, st);
   kern<<<S.sms * bps, 32 * wpb, smem, st>>>(sv);
   if (opt->search_event_end) cudaEventRecord((cudaEvent_t)opt->search_event_end, st);
-  dev::k_finalize<<<(n_units + 255) / 256, 256, 0, st>>>(sv);
   e = cudaGetLastError();
   if (e != cudaSuccess) return cuda_fail("kernel launch", e);
   return SCUBA_OK;
@@ -2107,12 +1888,12 @@ extern "C" void scuba_release(void) {
   auto it = scratch_map().find(dev);
   if (it == scratch_map().end()) return;
   Scratch& S = it->second;
-  Buf* all[] = {&S.occ_base, &S.norm, &S.occ_cnt, &S.occ_begin, &S.ent, &S.units, &S.nunits,
+  Buf* all[] = {&S.occ_base, &S.items, &S.occ_begin, &S.ent, &S.units, &S.nunits,
                 &S.flags, &S.pending, &S.done, &S.inst_dec, &S.trail, &S.dstack, &S.act,
                 &S.ring, &S.job_act, &S.prefix, &S.ctrl, &S.lvlcnt, &S.lvl_node,
                 &S.cd_var, &S.cd_mark, &S.cd_wl, &S.cd_pool,
                 &S.cd_learnt, &S.cd_arena, &S.cd_clidx, &S.job_cls, &S.cls_copy,
-                &S.share, &S.share_cur, &S.h_icb,
+                &S.share, &S.share_cur, &S.share_base, &S.h_icb,
                 &S.h_cb, &S.h_lits,
                 &S.h_nv, &S.h_vb,
                 &S.h_verdict, &S.h_model, &S.h_stats};
@@ -2219,8 +2000,11 @@ extern "C" int scuba_solve_batch_noalloc(const scuba_cnf_batch* b, uint8_t* verd
     off += (std::max<size_t>(bytes, 16) + 255) & ~(size_t)255;
     return at;
   };
-  const size_t o_occ_base = carve(8 * (size_t)(n + 1)), o_norm = carve(4 * (size_t)L),
-               o_occ_cnt = carve(4 * (size_t)occ_total), o_occ_begin = carve(4 * (size_t)occ_total),
+  // 4 L + 4 occ_total bytes are set aside and not used: the limit on what a
+  // batch may need is part of the interface
+  carve(4 * (size_t)L);
+  carve(4 * (size_t)occ_total);
+  const size_t o_occ_base = carve(8 * (size_t)(n + 1)), o_occ_begin = carve(4 * (size_t)occ_total),
                o_ent = carve(8 * (size_t)L), o_units = carve(4 * (size_t)std::max<int64_t>(C, 1)),
                o_nunits = carve(4 * (size_t)n), o_flags = carve(4 * (size_t)n),
                o_pending = carve(4 * (size_t)n), o_done = carve(4 * (size_t)n),
@@ -2239,41 +2023,26 @@ extern "C" int scuba_solve_batch_noalloc(const scuba_cnf_batch* b, uint8_t* verd
   unsigned char* base = static_cast<unsigned char*>(g_noalloc_scratch_addr[dev]);
   auto at = [&](size_t o) { return static_cast<void*>(base + o); };
 
-  dev::Prep pr;
-  pr.n = n;
-  pr.C = C;
-  pr.L = L;
-  pr.icb = b->inst_clause_begin;
-  pr.cb = b->clause_begin;
-  pr.lits = b->lits;
-  pr.nv = b->inst_num_vars;
+  const PrepShape shape = prep_shape(n, b->total_vars, vmax);
+  dev::Prep pr = prep_args(b, vmax, shape);
   pr.occ_base = static_cast<int64_t*>(at(o_occ_base));
-  pr.norm = static_cast<uint32_t*>(at(o_norm));
-  pr.occ_cnt = static_cast<uint32_t*>(at(o_occ_cnt));
   pr.occ_begin = static_cast<uint32_t*>(at(o_occ_begin));
   pr.ent = static_cast<uint64_t*>(at(o_ent));
   pr.units = static_cast<uint32_t*>(at(o_units));
   pr.nunits = static_cast<uint32_t*>(at(o_nunits));
   pr.flags = static_cast<uint32_t*>(at(o_flags));
-  pr.total_vars = b->total_vars;
-  pr.occ_cap = occ_total;
-  pr.vmax = vmax;
-  pr.vb = b->inst_var_begin;
   pr.ctrl = static_cast<dev::Ctrl*>(at(o_ctrl));
-
-  // the array keeps the previous call's contents: everything that must start
-  // at zero is cleared here, the rest is written before it is read
-  dev::k_init_ctrl<<<1, 1, 0, st>>>(pr.ctrl, (uint32_t)n);
-  cudaMemsetAsync(pr.occ_cnt, 0, 4 * (size_t)occ_total, st);
-  cudaMemsetAsync(pr.flags, 0, 4 * (size_t)n, st);
-  dev::k_occ_base<<<1, 1024, 0, st>>>(pr);
-  if (C > 0) {
-    int grid = (int)std::min<int64_t>((C + 255) / 256, (int64_t)sms * 32);
-    dev::k_normalize<<<grid, 256, 0, st>>>(pr);
+  if (shape.table) {
+    // in the search's trail, decision and activity arrays, not in use yet: 12 *
+    // slots * vmax bytes with vmax > 1,843, while a batch within the limit has
+    // fewer than 64 MiB / 40 instances (12.8 MiB of items; the arrays hold 12.8
+    // MiB from 152 SMs on, so only a smaller GPU could meet this error)
+    pr.items = static_cast<int2*>(at(o_trail));
+    if (8 * (size_t)shape.items > o_ring - o_trail) {
+      set_error("scuba_solve_batch_noalloc: too many instances beside a large one");
+      return SCUBA_ERR_TOO_LARGE;
+    }
   }
-  int wgrid = (int)std::min<int64_t>((n + 7) / 8, (int64_t)sms * 16);
-  dev::k_occ_scan<<<wgrid, 256, 0, st>>>(pr);
-  dev::k_fill<<<wgrid, 256, 0, st>>>(pr);
 
   dev::Solve sv;
   std::memset(&sv, 0, sizeof(sv));
@@ -2319,9 +2088,12 @@ extern "C" int scuba_solve_batch_noalloc(const scuba_cnf_batch* b, uint8_t* verd
   sv.finish_ns = nullptr;
   sv.prof = nullptr;
 
-  dev::k_init_ring<<<4, 256, 0, st>>>(sv.ring, ring_cap);
-  dev::k_init_inst<<<(n + 255) / 256, 256, 0, st>>>(sv.pending, sv.done, sv.inst_dec, n);
-  dev::k_start_clock<<<1, 1, 0, st>>>(sv.ctrl);
+  // the array keeps the previous call's contents: set-up writes everything that
+  // must have a value before the search, the rest is written before it is read
+  const dev::SearchInit init{n, sv.pending, sv.done, sv.inst_dec, verdict, sv.ring, ring_cap,
+                             nullptr, nullptr, 0};
+  e = launch_prep(pr, init, shape, sms, st);
+  if (e != cudaSuccess) return cuda_fail("preparation launch", e);
   // the kernel attribute is shared with the regular entry points: only ever
   // raise it, through the same per-device cache, so that a later regular
   // call that needs more shared memory still finds its own grant in place
@@ -2336,7 +2108,6 @@ extern "C" int scuba_solve_batch_noalloc(const scuba_cnf_batch* b, uint8_t* verd
     }
   }
   dev::k_solve<dev::MODE_PLAIN><<<sms, 32 * wpb, smem, st>>>(sv);
-  dev::k_finalize<<<(n + 255) / 256, 256, 0, st>>>(sv);
   e = cudaGetLastError();
   if (e != cudaSuccess) return cuda_fail("kernel launch", e);
   // report the device-side status of this call (the control block lives in
@@ -2383,46 +2154,31 @@ extern "C" int scuba_propagate_batch(const scuba_cnf_batch* b, const int64_t* as
   const uint32_t assign_words = (uint32_t)((vmax + 15) / 16);
   const size_t smem = (sizeof(dev::WarpShared) + (size_t)assign_words * 4) * wpb;
   if (smem > 227 * 1024) return SCUBA_ERR_TOO_LARGE;
-  const int blocks = S.sms;
+  // as many blocks as stay resident (the kernel waits on dependent loads, so
+  // warps in flight are what counts), but no more warps than instances
+  const int bps = (int)std::max<size_t>(1, std::min<size_t>(6, 227 * 1024 / (smem + 1024)));
+  const int blocks = std::max(1, std::min({n, S.sms * bps, std::max(S.sms, (n + wpb - 1) / wpb)}));
   const int64_t slots = (int64_t)blocks * wpb;
-  if (ensure(S.occ_base, 8 * (size_t)(n + 1)) || ensure(S.norm, 4 * (size_t)L) ||
-      ensure(S.occ_cnt, 4 * (size_t)occ_total) || ensure(S.occ_begin, 4 * (size_t)occ_total) ||
+  const PrepShape shape = prep_shape(n, b->total_vars, vmax);
+  if (ensure(S.occ_base, 8 * (size_t)(n + 1)) ||
+      ensure(S.items, shape.table ? 8 * (size_t)shape.items : 0) ||
+      ensure(S.occ_begin, 4 * (size_t)occ_total) ||
       ensure(S.ent, 8 * (size_t)L) || ensure(S.units, 4 * (size_t)std::max<int64_t>(C, 1)) ||
       ensure(S.nunits, 4 * (size_t)n) || ensure(S.flags, 4 * (size_t)n) ||
       ensure(S.trail, 4 * (size_t)slots * vmax) || ensure(S.ctrl, sizeof(dev::Ctrl)))
     return SCUBA_ERR_NOMEM;
-  dev::Prep pr;
-  pr.n = n;
-  pr.C = C;
-  pr.L = L;
-  pr.icb = b->inst_clause_begin;
-  pr.cb = b->clause_begin;
-  pr.lits = b->lits;
-  pr.nv = b->inst_num_vars;
+  dev::Prep pr = prep_args(b, vmax, shape);
   pr.occ_base = P<int64_t>(S.occ_base);
-  pr.norm = P<uint32_t>(S.norm);
-  pr.occ_cnt = P<uint32_t>(S.occ_cnt);
   pr.occ_begin = P<uint32_t>(S.occ_begin);
   pr.ent = P<uint64_t>(S.ent);
   pr.units = P<uint32_t>(S.units);
   pr.nunits = P<uint32_t>(S.nunits);
   pr.flags = P<uint32_t>(S.flags);
-  pr.total_vars = b->total_vars;
-  pr.occ_cap = occ_total;
-  pr.vmax = vmax;
-  pr.vb = b->inst_var_begin;
+  if (shape.table) pr.items = P<int2>(S.items);
   pr.ctrl = P<dev::Ctrl>(S.ctrl);
-  dev::k_init_ctrl<<<1, 1, 0, st>>>(pr.ctrl, (uint32_t)n);
-  cudaMemsetAsync(pr.occ_cnt, 0, 4 * (size_t)occ_total, st);
-  cudaMemsetAsync(pr.flags, 0, 4 * (size_t)n, st);
-  dev::k_occ_base<<<1, 1024, 0, st>>>(pr);
-  if (C > 0) {
-    int grid = (int)std::min<int64_t>((C + 255) / 256, (int64_t)S.sms * 32);
-    dev::k_normalize<<<grid, 256, 0, st>>>(pr);
-  }
-  int wgrid = (int)std::min<int64_t>((n + 7) / 8, (int64_t)S.sms * 16);
-  dev::k_occ_scan<<<wgrid, 256, 0, st>>>(pr);
-  dev::k_fill<<<wgrid, 256, 0, st>>>(pr);
+  const dev::SearchInit no_search{};
+  e = launch_prep(pr, no_search, shape, S.sms, st);
+  if (e != cudaSuccess) return cuda_fail("preparation launch", e);
   dev::PropArgs A;
   A.n = n;
   A.vmax = vmax;

@@ -6,10 +6,10 @@
 // internally and says no more about it; this mode puts the textbook
 // first-UIP scheme on top of the GPU propagation of the DPLL mode:
 //
-//  * The assignment takes 4 bits per variable in shared memory: value (true,
-//    false) and a "fresh" bit, set by the same compare-and-swap that claims
-//    the variable during a BCP round and cleared when the round after it
-//    starts. Every assigned variable keeps its reason (the occurrence entry or
+//  * The assignment takes two bit sets over literal codes in shared memory: the
+//    true literals, and the settled ones, true literals whose own propagation
+//    has begun (a literal assigned during a BCP round is "fresh" until then).
+//    Every assigned variable keeps its reason (the occurrence entry or
 //    clause reference that implied it) and its decision level.
 //  * Propagation rounds are frontier-parallel, so two lanes can assign
 //    variables of the same round in either trail order. An implication may
@@ -26,18 +26,17 @@
 //    settles the clause without reading it. After the static occurrence
 //    entries of each frontier batch, the watchers of every literal in the
 //    batch are spread over the 32 lanes like the static entries. A clause
-//    can sit on two lists of one batch only when both its watches are false;
-//    a lane then takes a per-clause lock first, and the loser retries after
-//    the winner has moved its watch. Moved watches are appended to their new
-//    lists one at a time (the warp copies a list when it grows) and the
-//    batch's own lists are compacted afterwards.
+//    can sit on two lists of one pass only when both its watches are false;
+//    the second lane then waits until the first has moved its watch. Moved
+//    watches are appended to their new lists all at once (the warp copies a
+//    list when it grows) and a list closes up while it is read.
 //  * Conflict analysis resolves the falsified clause with the reasons of
 //    current-level literals, newest first on the trail, until one
 //    current-level literal (the first UIP) is left; the lanes take the
 //    literals of each clause, and the next literal to resolve is the newest
-//    of the waiting ones, kept with their trail positions in shared memory
-//    (a warp-wide backward scan of the trail if more than CAND wait). Every
-//    variable met is bumped.
+//    of the waiting ones, each kept in a lane's registers (a warp-wide
+//    backward scan of the trail if more than 32 wait). Every variable met is
+//    bumped.
 //  * Hard instances are shared cube-and-conquer style through the DPLL mode's
 //    job ring: a busy warp that sees idle warps gives away the negation of
 //    its first free decision, together with the assumptions above it, as a
@@ -57,19 +56,33 @@
 //    if even that does not fit, every learned clause is dropped (all of them
 //    are implied by the formula, so any of this is sound).
 //
-// Clause arena layout (32-bit words, 16-byte aligned clauses): [len, lock, 0,
+// Clause arena layout (32-bit words, 16-byte aligned clauses): [len, 0, LBD,
 // 0, lit0 .. lit_{len-1}, padding to a multiple of 4]; lit0 and lit1 are the
 // watched literals.
 
 constexpr uint32_t LEARNT_REF = 0xC0000000u;  // clause reference: learned clause at offset
 constexpr uint32_t CD_HDR = 4;
-constexpr uint64_t WATCH_GONE = ~0ull;     // tombstone of a moved watch entry
-constexpr uint32_t NB_T = 1u, NB_F = 2u, NB_FRESH = 4u;  // assignment nibble bits
-constexpr uint32_t RING = 128;  // recent-trail entries per warp in shared memory
-constexpr uint32_t CAND = 96;   // current-level literals awaiting resolution, per warp
-// shared memory per warp for the clause-learning search (16-byte multiple)
-constexpr uint32_t CD_SMEM_WARP = RING * 8 + CAND * 8;
-constexpr uint8_t MK_PHASE = 1, MK_SEEN = 2;
+// Shared memory of a clause-learning warp beyond its assignment: the reasons of
+// the RING newest trail positions, the first LSM literals of the clause under
+// construction and, where they fit (Solve::cd_smem), per variable its
+// activity (CD_SMEM_ACT), its trail position and level packed into 32 bits and
+// its mark (both CD_SMEM_POS; at most 65,535 variables). The analysis walks from
+// variable to variable, so what it reads of each has to be near: with these in
+// global memory a resolution step took about 2,700 cycles.
+enum { CD_SMEM_POS = 1, CD_SMEM_ACT = 2 };
+constexpr uint32_t LSM = 64;
+
+__host__ __device__ __forceinline__ size_t cd_area_bytes(int what, int32_t vmax) {
+  const size_t v16 = ((size_t)vmax + 15) & ~(size_t)15;
+  return RING * 8 + LSM * 4 + (what & CD_SMEM_ACT ? 4 * v16 : 0) + (what & CD_SMEM_POS ? 5 * v16 : 0);
+}
+__device__ __forceinline__ float* cd_area_act(unsigned char* area) {
+  return reinterpret_cast<float*>(area + RING * 8 + LSM * 4);
+}
+
+// A variable's mark: bit 0 the saved phase, bits 1-7 the number (1..127, mod
+// 127) of the last analysis that met it, so that nothing is cleared after one.
+constexpr uint32_t MK_PHASE = 1, MK_EPOCHS = 127;
 
 // Profile counters (only when the caller passed a profile array): lane 0
 // adds the clock cycles of each phase to its warp's WarpShared::cyc.
@@ -101,382 +114,374 @@ struct VarInfo {
 
 struct CdWarp {
   VarInfo* var;       // [V] reason, trail position, decision level
-  uint8_t* mark;      // [V] MK_PHASE saved phase, MK_SEEN during analysis
+  uint8_t* mark;      // [V] saved phase and last analysis (MK_PHASE, MK_EPOCHS)
   WList* wl;          // [2V] learned watch list per literal code
   uint64_t* pool;     // [pool_cap] watch entries {clause, blocker}
   uint32_t* arena;    // [arena_words]
   uint32_t* cl_off;   // [arena_words / 8] arena offset of each learned clause, oldest first
   uint32_t* learnt;   // [V] clause under construction
-  uint2* ring;        // [RING] shared memory: {literal, trail position} of recent claims
-  uint2* cand;        // [CAND] shared memory: analysis queue {trail position, literal}
+  uint32_t* pl;       // [V] trail position | level << 16 in shared memory, or NULL
+  uint2* why;         // [RING] shared memory: reason of the literal in the ring's same slot
+  uint32_t* lsm;      // [LSM] shared memory: learnt[0 .. LSM)
   uint32_t arena_words, pool_cap;
   uint32_t top;       // first free arena word
   uint32_t ncl;       // learned clauses in the arena
   uint32_t pool_top;  // first free pool entry
   uint32_t full;      // the pool ran out during propagation: drop the learned clauses
+  uint32_t epoch;     // number of the last analysis (marks)
 };
 
-// The nibble of variable v (value bits and fresh bit).
-__device__ __forceinline__ uint32_t nib(const uint32_t* asg, uint32_t v) {
-  return (asg[v >> 3] >> ((v & 7u) * 4u)) & 7u;
+// Literal k of the clause under construction.
+__device__ __forceinline__ uint32_t learnt_at(const CdWarp& cd, uint32_t k) {
+  return k < LSM ? cd.lsm[k] : cd.learnt[k];
+}
+__device__ __forceinline__ void set_learnt(CdWarp& cd, uint32_t k, uint32_t l) {
+  if (k < LSM) cd.lsm[k] = l;
+  else cd.learnt[k] = l;
+}
+// Decision level of an assigned variable.
+__device__ __forceinline__ uint32_t level_of(const CdWarp& cd, uint32_t v) {
+  return cd.pl ? cd.pl[v] >> 16 : cd.var[v].level;
 }
 
-// Value (LV_U, LV_T, LV_F) of literal l whose variable has nibble n.
-__device__ __forceinline__ uint32_t nib_value(uint32_t n, uint32_t l) {
-  const uint32_t b = n & 3u;
-  if (b == 0u) return LV_U;
-  return ((b == NB_T) != ((l & 1u) != 0u)) ? LV_T : LV_F;
-}
-
+// Value (LV_U, LV_T, LV_F) of literal l.
 __device__ __forceinline__ uint32_t lit_value_cd(const uint32_t* asg, uint32_t l) {
-  return nib_value(nib(asg, l >> 1), l);
+  const uint32_t x = asg[2 * (l >> 5)];
+  if ((x >> (l & 31u)) & 1u) return LV_T;
+  return (x >> ((l & 31u) ^ 1u)) & 1u ? LV_F : LV_U;
 }
 
-// Assign l with reason `why` at the current level; fresh marks a claim made
-// inside a BCP round. One compare-and-swap claims value and fresh bit
-// together. Returns false on a clash with the opposite value.
-__device__ __forceinline__ bool imply_cd(Warp& w, CdWarp& cd, uint32_t l, uint64_t why,
-                                         uint32_t fresh = NB_FRESH) {
-  const uint32_t v = WIDX(w, l >> 1, w.V, 11), wi = v >> 3, sh = (v & 7u) * 4u;
-  const uint32_t val = (l & 1u) ? NB_F : NB_T;
-  uint32_t old = w.asg[wi];
-  for (;;) {
-    const uint32_t cur = (old >> sh) & 3u;
-    if (cur) return cur == val;
-    const uint32_t prev = atomicCAS(&w.asg[wi], old, old | ((val | fresh) << sh));
-    if (prev == old) break;
-    old = prev;
+// The two words {true, settled} that hold literal l and its negation.
+__device__ __forceinline__ uint2 lit_words(const uint32_t* asg, uint32_t l) {
+  return *reinterpret_cast<const uint2*>(asg + 2 * (l >> 5));
+}
+__device__ __forceinline__ bool has_bit(uint32_t x, uint32_t l) { return (x >> (l & 31u)) & 1u; }
+
+// Make literal l of every lane with want set true at the current level, with
+// its reason (all lanes). Returns true in a lane whose literal's negation was
+// claimed by another lane of this call.
+__device__ __forceinline__ bool claim_cd(Warp& w, CdWarp& cd, bool want, uint32_t l,
+                                         uint32_t why_lo, uint32_t why_hi) {
+  bool won;
+  const bool clash = claim_bits<2>(w, want, l, won);
+  const uint32_t pos = push_trail(w, won, l);
+  if (won) {
+    const uint32_t v = l >> 1;
+    cd.why[pos & (RING - 1u)] = make_uint2(why_lo, why_hi);
+    if (cd.pl) cd.pl[v] = pos | (w.nd << 16);
+    *reinterpret_cast<uint4*>(&cd.var[v]) = make_uint4(why_lo, why_hi, pos, w.nd);
   }
-  const uint32_t pos = WIDX(w, atomicAdd(&w.ws->tail, 1u), w.V, 12);
-  w.trail[pos] = l;
-  cd.ring[pos & (RING - 1u)] = make_uint2(l, pos);
-  *reinterpret_cast<uint4*>(&cd.var[v]) =
-      make_uint4((uint32_t)why, (uint32_t)(why >> 32), pos, w.nd);
-  return true;
+  return clash;
 }
 
-// trail[p], from the shared-memory ring when its slot still holds position p.
-__device__ __forceinline__ uint32_t trail_at(const Warp& w, const CdWarp& cd, uint32_t p) {
-  const uint2 e = cd.ring[p & (RING - 1u)];
-  return e.y == p ? e.x : w.trail[p];
+// Assign l, unassigned, for a decision, an assumption, a learned or an imported
+// clause (all lanes, uniform).
+__device__ __forceinline__ void assign_one_cd(Warp& w, CdWarp& cd, uint32_t l, uint32_t why_lo,
+                                              uint32_t why_hi) {
+  claim_cd(w, cd, w.lane == 0, l, why_lo, why_hi);
+  __syncwarp();
 }
 
-__device__ void eval_long_cd(Warp& w, CdWarp& cd, uint32_t local) {
-  const int64_t c = w.c0 + local;
-  const int64_t b = w.cb[c], e = w.cb[c + 1];
+// A long clause of the caller's CSR: unit or false, or nothing if it is true,
+// has two open literals, or its last open literal rests on a fresh one (that
+// literal's own list brings it back next round).
+__device__ __noinline__ Found eval_long_cd(const uint32_t* asg, const int32_t* lits, int64_t b,
+                                           int64_t e, uint32_t local) {
   uint32_t open_lit = NONE;
-  int n_open = 0;
   bool fresh_false = false;
   for (int64_t q = b; q < e; q++) {
-    const uint32_t x = code_of(__ldg(&w.lits[q]));
-    const uint32_t n = nib(w.asg, x >> 1);
-    const uint32_t vx = nib_value(n, x);
-    if (vx == LV_T) return;
-    if (vx == LV_U) {
-      if (x != open_lit) {
-        n_open++;
-        open_lit = x;
-        if (n_open > 1) return;
-      }
-    } else if (n & NB_FRESH) {
-      fresh_false = true;
+    const uint32_t x = code_of(__ldg(&lits[q]));
+    const uint2 ws = lit_words(asg, x);
+    if (has_bit(ws.x, x)) return Found{false, false, NONE, 0, 0, 0};
+    if (!has_bit(ws.x, x ^ 1u)) {
+      if (open_lit != NONE && x != open_lit) return Found{false, false, NONE, 0, 0, 0};
+      open_lit = x;
+    } else {
+      fresh_false |= !has_bit(ws.y, x ^ 1u);
     }
   }
-  if (n_open == 1 && fresh_false) return;  // a literal falsified this round: next round
-  if (n_open == 0 || !imply_cd(w, cd, open_lit, (uint64_t)(LONG_CLAUSE | local)))
-    record_conflict(w, LONG_CLAUSE | local, NONE, NONE);
+  return Found{open_lit != NONE && !fresh_false, open_lit == NONE, open_lit, LONG_CLAUSE | local,
+               NONE, NONE};
 }
 
-// One occurrence entry of the falsified (old) literal f: (f | a) with b ==
-// NONE, (f | a | b), or a long clause. One claim site and one conflict site.
-__device__ __forceinline__ void eval_entry_cd(Warp& w, CdWarp& cd, uint32_t f, uint64_t e) {
+// One occurrence entry of the falsified (settled) literal f: (f | a) with b ==
+// NONE, (f | a | b), or a long clause; without branches but for those. A
+// literal is implied only by settled false literals. For a wanted literal c0
+// and c1 are its reason, for a conflict c0..c2 the clause.
+__device__ __forceinline__ Found eval_entry_cd(const Warp& w, uint32_t f, uint64_t e) {
   const uint32_t a0 = (uint32_t)e, b0 = (uint32_t)(e >> 32);
   if (a0 & LONG_CLAUSE) {
-    eval_long_cd(w, cd, a0 & ~LONG_CLAUSE);
-    return;
+    const uint32_t local = a0 & ~LONG_CLAUSE;
+    const int64_t c = w.c0 + local;
+    return eval_long_cd(w.asg, w.lits, w.cb[c], w.cb[c + 1], local);
   }
-  const uint32_t a = WIDX(w, a0, 2u * w.V, 13);
-  const uint32_t b = b0 == NONE ? NONE : WIDX(w, b0, 2u * w.V, 13);
-  const uint32_t na = nib(w.asg, a >> 1);
-  const uint32_t va = nib_value(na, a);
-  uint32_t nb = 0, vb = LV_F;  // a binary entry has no third literal: read it as false
-  if (b != NONE) {
-    nb = nib(w.asg, b >> 1);
-    vb = nib_value(nb, b);
-  }
-  if (va == LV_T || vb == LV_T) return;
-  uint32_t unit = NONE, other = NONE;  // the literal to imply, the false one beside f
-  if (va == LV_U && vb == LV_F) {
-    if (nb & NB_FRESH) return;  // b falsified this round: next round
-    unit = a;
-    other = b;
-  } else if (vb == LV_U && va == LV_F) {
-    if (na & NB_FRESH) return;
-    unit = b;
-    other = a;
-  } else if (va == LV_U || vb == LV_U) {
-    return;  // two open literals
-  }
-  if (unit == NONE ||
-      !imply_cd(w, cd, unit, (uint64_t)f | ((uint64_t)other << 32)))
-    record_conflict(w, f, a, b);
+  const bool tern = b0 != NONE;
+  const uint32_t a = WIDX(w, a0, 2u * w.V, 13), b = tern ? WIDX(w, b0, 2u * w.V, 13) : a;
+  const uint2 xa = lit_words(w.asg, a), xb = lit_words(w.asg, b);
+  const bool ta = has_bit(xa.x, a), fa = has_bit(xa.x, a ^ 1u), sa = has_bit(xa.y, a ^ 1u);
+  const bool tb = tern && has_bit(xb.x, b), fb = !tern || has_bit(xb.x, b ^ 1u);
+  const bool sb = !tern || has_bit(xb.y, b ^ 1u);
+  const bool ua = !ta && !fa && sb, ub = !tb && !fb && sa;
+  const bool confl = fa && fb;
+  return Found{ua || ub, confl, ua ? a : b, f, confl ? a : ua ? b0 : a, confl ? b0 : NONE};
 }
 
-// Append entry e to literal g's watch list (all lanes, uniform arguments).
-__device__ void wl_append(Warp& w, CdWarp& cd, uint32_t g, uint64_t e) {
-  if (cd.full) return;
-  WList L = cd.wl[g];  // last written before a __syncwarp
-  if (L.len == L.cap) {
-    const uint32_t ncap = L.cap ? 2u * L.cap : 8u;
-    if ((uint64_t)cd.pool_top + ncap > cd.pool_cap) {
-      cd.full = 1;
-      if (w.lane == 0) record_conflict(w, NONE, NONE, NONE);  // ends this BCP
-      __syncwarp();
-      return;
+// A literal's watch list with room for more entries: copied to the pool's top
+// with twice the capacity. Returns the new top, or NONE if the pool is full.
+__device__ __noinline__ uint32_t grow_list(WList* wl, uint64_t* pool, uint32_t pool_top,
+                                           uint32_t pool_cap, uint32_t g, int lane) {
+  WList L = wl[g];
+  const uint32_t ncap = L.cap ? 2u * L.cap : 8u;
+  if ((uint64_t)pool_top + ncap > pool_cap) return NONE;
+  for (uint32_t k = lane; k < L.len; k += 32) pool[pool_top + k] = pool[L.off + k];
+  __syncwarp();
+  if (lane == 0) wl[g] = WList{pool_top, L.len, ncap, 0u};
+  __syncwarp();
+  return pool_top + ncap;
+}
+
+// Append entry e to literal g's watch list in every lane with mover set (all
+// lanes): lists with room take theirs at once, the others grow one by one.
+// Sets cd.full and a conflict (which ends the propagation) if the pool is full.
+__device__ __forceinline__ void append_watches(Warp& w, CdWarp& cd, bool mover, uint32_t g,
+                                               uint64_t e) {
+  uint32_t todo = __ballot_sync(FULL, mover);
+  while (todo) {
+    uint4 L = make_uint4(0, 0, 0, 0);  // {offset, length, capacity}
+    if (mover) L = *reinterpret_cast<const uint4*>(&cd.wl[g]);
+    const uint32_t grp =
+        (todo & (todo - 1u)) ? __match_any_sync(FULL, mover ? g : ~(uint32_t)w.lane) : 1u << w.lane;
+    const uint32_t rank = __popc(grp & ((1u << w.lane) - 1u)), size = __popc(grp);
+    const bool fits = mover && L.y + size <= L.z;
+    if (fits) {
+      cd.pool[L.x + L.y + rank] = e;
+      if (rank == 0) cd.wl[g].len = L.y + size;
+      mover = false;
     }
-    const uint32_t noff = cd.pool_top;
-    cd.pool_top += ncap;
-    for (uint32_t k = w.lane; k < L.len; k += 32) cd.pool[noff + k] = cd.pool[L.off + k];
-    L.off = noff;
-    L.cap = ncap;
+    __syncwarp();
+    todo = __ballot_sync(FULL, mover);
+    if (todo) {
+      const uint32_t gj = __shfl_sync(FULL, g, __ffs(todo) - 1);
+      const uint32_t top = grow_list(cd.wl, cd.pool, cd.pool_top, cd.pool_cap, gj, w.lane);
+      if (top == NONE) {
+        cd.full = 1;
+        w.confl = 1;
+        return;
+      }
+      cd.pool_top = top;
+    }
   }
-  __syncwarp();
-  if (w.lane == 0) {
-    cd.pool[L.off + L.len] = e;
-    L.len++;
-    cd.wl[g] = L;
-  }
-  __syncwarp();
 }
 
 // A new watch for a learned clause: the first position >= 2 whose literal is
 // not false, else the first whose literal was falsified during this round
-// (its own list brings the clause back next round), else NONE. Literals are
-// read 4 at a time (16-byte loads; clauses are 16-byte aligned and padded).
-__device__ __forceinline__ uint32_t new_watch(const uint32_t* asg, const uint32_t* lits,
-                                              uint32_t len) {
-  const uint4* L4 = reinterpret_cast<const uint4*>(lits);
+// (its own list brings the clause back next round), else NONE; g gets the
+// literal. x: the clause's first four literals; further ones are read 4 at a
+// time (16-byte loads; clauses are 16-byte aligned and padded).
+__device__ __forceinline__ uint32_t new_watch(const uint32_t* asg, const uint32_t* lits, uint4 x,
+                                              uint32_t len, uint32_t& g) {
   uint32_t fresh_pos = NONE;
-  for (uint32_t q = 0; q < len; q += 4) {
-    const uint4 a = L4[q >> 2];
-    const uint32_t x[4] = {a.x, a.y, a.z, a.w};
+  for (uint32_t q = 0;;) {
+    const uint32_t l[4] = {x.x, x.y, x.z, x.w};
     uint32_t open = 0, fr = 0;
 #pragma unroll
     for (int i = 0; i < 4; i++) {
       if (q + i < 2 || q + i >= len) continue;
-      const uint32_t n = nib(asg, x[i] >> 1);
-      if (nib_value(n, x[i]) != LV_F) open |= 1u << i;
-      else if (n & NB_FRESH) fr |= 1u << i;
+      const uint2 ws = lit_words(asg, l[i]);
+      if (!has_bit(ws.x, l[i] ^ 1u)) open |= 1u << i;
+      else if (!has_bit(ws.y, l[i] ^ 1u)) fr |= 1u << i;
     }
-    if (open) return q + __ffs(open) - 1;
-    if (fr && fresh_pos == NONE) fresh_pos = q + __ffs(fr) - 1;
+    const uint32_t hit = open ? open : fresh_pos == NONE ? fr : 0u;
+    if (hit) {
+      const int i = __ffs(hit) - 1;
+      g = i == 0 ? l[0] : i == 1 ? l[1] : i == 2 ? l[2] : l[3];
+      if (open) return q + i;
+      fresh_pos = q + i;
+    }
+    q += 4;
+    if (q >= len) return fresh_pos;
+    x = *reinterpret_cast<const uint4*>(lits + q);
   }
-  return fresh_pos;
-}
-
-// One watch entry (clause c, blocker) of the falsified literal f, at pool
-// index at. Returns the literal the watch moved to (NONE if it stayed) and
-// the entry for that literal's list.
-__device__ uint32_t visit_learnt(Warp& w, CdWarp& cd, uint32_t f, uint32_t at, uint32_t c,
-                                 uint64_t& moved_entry) {
-  uint32_t* C = cd.arena + c;
-  const uint32_t l0 = C[CD_HDR], l1 = C[CD_HDR + 1];
-  const uint32_t which = l0 == f ? 0u : 1u;
-  const uint32_t other = which ? l0 : l1;
-  const uint32_t vo = lit_value_cd(w.asg, other);
-  if (vo == LV_T) {
-    cd.pool[at] = (uint64_t)c | ((uint64_t)other << 32);  // new blocker
-    return NONE;
-  }
-  const uint32_t k = new_watch(w.asg, C + CD_HDR, C[0]);
-  if (k != NONE) {
-    const uint32_t g = C[CD_HDR + k];
-    C[CD_HDR + k] = f;
-    C[CD_HDR + which] = g;
-    cd.pool[at] = WATCH_GONE;
-    moved_entry = (uint64_t)c | ((uint64_t)other << 32);
-    return g;
-  }
-  if (vo == LV_F) {
-    record_conflict(w, LEARNT_REF | c, NONE, NONE);
-  } else if (vo == LV_U) {
-    if (!imply_cd(w, cd, other, (uint64_t)(LEARNT_REF | c)))
-      record_conflict(w, LEARNT_REF | c, NONE, NONE);
-  }
-  return NONE;
 }
 
 // Learned clauses watching the literals falsified in this batch: lane j <
-// nlit holds falsified literal f and its watch list pool[beg, beg + cnt).
-__device__ void learned_batch(Warp& w, CdWarp& cd, uint32_t nlit, uint32_t f, uint32_t beg,
-                              uint32_t cnt) {
-  __syncwarp();
-  if (cd.top == 0) return;  // no learned clauses
+// nlit holds falsified literal f and its watch list pool[beg, beg + cnt). Every
+// list is read to its end, also after a conflict, since it closes up as its
+// entries leave.
+__device__ __forceinline__ void learned_batch(Warp& w, CdWarp& cd, const LaneMap& m,
+                                              uint32_t nlit, uint32_t f, uint32_t beg,
+                                              uint32_t cnt) {
+  if (!__any_sync(FULL, cnt != 0)) return;
   const long long t0 = pf_now(*w.S);
-  uint32_t inc = cnt;
-#pragma unroll
-  for (int d = 1; d < 32; d <<= 1) {
-    const uint32_t y = __shfl_up_sync(FULL, inc, d);
-    if (w.lane >= d) inc += y;
-  }
-  const uint32_t excl = inc - cnt;
-  const uint32_t total = __shfl_sync(FULL, inc, 31);
+  const uint32_t total = batch_total(m, cnt);
   WCOUNT(w, visits, total);
-  uint32_t dirty = 0;  // lists that lost an entry
-  for (uint32_t e0 = 0; e0 < total; e0 += 32) {
-    const uint32_t e = e0 + w.lane;
-    int lo_j = 0, hi_j = 31;  // owner: smallest lane j with inc_j > e
-#pragma unroll
-    for (int s2 = 0; s2 < 5; s2++) {
-      const int mid = (lo_j + hi_j) >> 1;
-      const uint32_t v = __shfl_sync(FULL, inc, mid);
-      if (v > e) hi_j = mid; else lo_j = mid + 1;
-      if (lo_j > hi_j) lo_j = hi_j;
+  const uint32_t width = 1u << m.lg, sub = m.sub;
+  // the lanes of this lane's literal, and those of them before it
+  const uint32_t mates = (width == 32u ? FULL : (1u << width) - 1u) << ((uint32_t)w.lane - sub);
+  const uint32_t before = mates & ((1u << w.lane) - 1u);
+  for (uint32_t s = 0; s < nlit; s += 32u >> m.lg) {
+    uint32_t jb = beg, jf = f, jc = cnt;
+    if (!m.few) {
+      const uint32_t j = s + m.group;
+      jb = __shfl_sync(FULL, beg, j);
+      jf = __shfl_sync(FULL, f, j);
+      jc = __shfl_sync(FULL, cnt, j);
+      if (j >= nlit) jc = 0;
     }
-    const uint32_t jbeg = __shfl_sync(FULL, beg, lo_j);
-    const uint32_t jex = __shfl_sync(FULL, excl, lo_j);
-    const uint32_t jf = __shfl_sync(FULL, f, lo_j);
-    bool pending = false;
-    uint32_t at = 0, c = 0;
-    if (e < total) {
-      at = WIDX(w, jbeg + (e - jex), cd.pool_cap, 16);
-      const uint64_t ent = cd.pool[at];
-      c = WIDX(w, (uint32_t)ent, cd.top, 17);
-      pending = lit_value_cd(w.asg, WIDX(w, (uint32_t)(ent >> 32), 2u * w.V, 18)) != LV_T;  // blocker
-    }
-    uint32_t g = NONE;
-    uint64_t moved = 0;
-    // both watches false: the clause may be on two lists of this batch, so
-    // the lane locks it; a loser retries after the winner's pass
-    while (__any_sync(FULL, pending)) {
-      if (pending) {
-        volatile uint32_t* C = cd.arena + c;
-        const uint32_t other = C[CD_HDR] == jf ? C[CD_HDR + 1] : C[CD_HDR];
-        bool go = true, locked = false;
-        if (lit_value_cd(w.asg, other) == LV_F) {
-          locked = atomicCAS((uint32_t*)&C[1], 0u, 1u) == 0u;
-          go = locked;
-        }
-        if (go) {
-          g = visit_learnt(w, cd, jf, at, c, moved);
-          if (locked) {
-            __threadfence_block();
-            atomicExch((uint32_t*)&C[1], 0u);
-          }
-          pending = false;
-        }
+    uint32_t kept = 0;
+    for (uint32_t k = sub; __any_sync(FULL, k < jc); k += width) {
+      const bool in = k < jc;
+      uint64_t entry = 0;
+      uint32_t c = 0;
+      bool pending = false;
+      if (in) {
+        entry = cd.pool[WIDX(w, jb + k, cd.pool_cap, 16)];
+        c = WIDX(w, (uint32_t)entry, cd.top, 17);
+        const uint32_t blocker = WIDX(w, (uint32_t)(entry >> 32), 2u * w.V, 18);
+        pending = !has_bit(w.asg[2 * (blocker >> 5)], blocker);
       }
+      if (w.confl) pending = false;
+      uint64_t now = entry;  // the entry that stays in this list
+      bool mover = false;
+      uint32_t g = NONE;
+      while (__any_sync(FULL, pending)) {
+        uint32_t* const L = cd.arena + c + CD_HDR;
+        uint4 x = make_uint4(0, 0, 0, 0);
+        uint32_t len = 0, other = 0;
+        uint2 ow = make_uint2(0, 0);
+        bool both = false;
+        if (pending) {
+          x = *reinterpret_cast<const uint4*>(L);
+          len = L[-(int)CD_HDR];
+          other = x.x == jf ? x.y : x.x;
+          ow = lit_words(w.asg, other);
+          both = has_bit(ow.x, other ^ 1u);
+        }
+        // both watches false: the clause may be on another lane's list too; the
+        // first lane moves its watch (or finds the conflict), the next looks again
+        bool go = pending;
+        const uint32_t bm = __ballot_sync(FULL, both);
+        if (bm & (bm - 1u)) {
+          const uint32_t grp = __match_any_sync(FULL, both ? c : ~(uint32_t)w.lane);
+          go = pending && (!both || (grp & ((1u << w.lane) - 1u)) == 0u);
+        }
+        bool want = false, confl = false;
+        if (go) {
+          pending = false;
+          if (has_bit(ow.x, other)) {
+            now = (uint64_t)c | ((uint64_t)other << 32);  // new blocker
+          } else {
+            const uint32_t at = new_watch(w.asg, L, x, len, g);
+            if (at != NONE) {
+              L[at] = jf;
+              L[x.x == jf ? 0 : 1] = g;
+              mover = true;
+              now = (uint64_t)c | ((uint64_t)other << 32);
+            } else {
+              confl = both;
+              want = !both;
+            }
+          }
+        }
+        if (__any_sync(FULL, want || confl)) {
+          confl |= claim_cd(w, cd, want, other, LEARNT_REF | c, 0u);
+          note_conflict(w, confl, LEARNT_REF | c, NONE, NONE);
+          if (w.confl) pending = false;
+        }
+        __syncwarp();
+      }
+      if (__any_sync(FULL, mover)) append_watches(w, cd, mover && !cd.full, g, now);
+      // close the list up behind the entries that left
+      const uint32_t stay = __ballot_sync(FULL, in && !mover);
+      const uint32_t to = kept + __popc(stay & before);
+      if (in && !mover && (to != k || now != entry)) cd.pool[jb + to] = now;
+      kept += __popc(stay & mates);
       __syncwarp();
     }
-    dirty |= __reduce_or_sync(FULL, g != NONE ? (1u << lo_j) : 0u);
-    uint32_t movers = __ballot_sync(FULL, g != NONE);
-    while (movers) {
-      const int j = __ffs(movers) - 1;
-      movers &= movers - 1u;
-      const uint32_t gj = __shfl_sync(FULL, g, j);
-      const uint64_t mj = __shfl_sync(FULL, moved, j);
-      wl_append(w, cd, gj, mj);
-    }
-  }
-  // compact the lists that lost entries (lane j owns frontier literal j)
-  if (w.lane < nlit && ((dirty >> w.lane) & 1u) && !cd.full) {
-    uint32_t keep = 0;
-    for (uint32_t k = 0; k < cnt; k++) {
-      const uint64_t ent = cd.pool[beg + k];
-      if (ent != WATCH_GONE) cd.pool[beg + keep++] = ent;
-    }
-    cd.wl[f].len = keep;
+    if (sub == 0 && kept != jc) cd.wl[jf].len = kept;
   }
   __syncwarp();
   pf_add(*w.S, w, PF_LEARNED, t0);
 }
 
-// Static occurrence entries of one batch over the 32 lanes: lane j < nlit
-// holds falsified literal f and its occurrence list ent[beg, beg + cnt). One
-// evaluation site keeps the hot code small.
-__device__ __forceinline__ void static_batch(Warp& w, CdWarp& cd, uint32_t nlit, uint32_t f,
-                                             uint32_t beg, uint32_t cnt) {
-  uint32_t inc = cnt;
-#pragma unroll
-  for (int d = 1; d < 32; d <<= 1) {
-    const uint32_t y = __shfl_up_sync(FULL, inc, d);
-    if (w.lane >= d) inc += y;
-  }
-  const uint32_t excl = inc - cnt;
-  const uint32_t total = __shfl_sync(FULL, inc, 31);
-  WCOUNT(w, visits, total);
-  for (uint32_t e0 = 0; e0 < total; e0 += 32) {
-    const uint32_t e = e0 + w.lane;
-    int j = 0;  // owner: smallest lane j with inc_j > e (lane 0 alone when nlit == 1)
-    if (nlit > 1) {
-      int hi_j = 31;
-#pragma unroll
-      for (int s2 = 0; s2 < 5; s2++) {
-        const int mid = (j + hi_j) >> 1;
-        const uint32_t v = __shfl_sync(FULL, inc, mid);
-        if (v > e) hi_j = mid; else j = mid + 1;
-        if (j > hi_j) j = hi_j;
-      }
-    }
-    const uint32_t jbeg = __shfl_sync(FULL, beg, j);
-    const uint32_t jex = __shfl_sync(FULL, excl, j);
-    const uint32_t jf = __shfl_sync(FULL, f, j);
-    if (e < total) eval_entry_cd(w, cd, jf, __ldg(&w.ent[WIDX(w, jbeg + (e - jex), w.ent_end, 15)]));
-  }
-}
-
-// Unit propagation to a fixpoint (true on conflict), in the frontier rounds
-// of the DPLL search. Per batch of up to 32 frontier literals the lanes read
-// their literal (from the ring when it is there), clear its fresh bit, and
-// load both its occurrence-list bounds and its learned watch list before
-// the static entries and then the learned watchers are evaluated.
-__device__ bool bcp_cd(Warp& w, CdWarp& cd) {
-  for (;;) {
-    __syncwarp();
-    const uint32_t hi = *(volatile uint32_t*)&w.ws->tail;
-    if (w.head >= hi) return false;
-    const uint32_t lo = w.head;
+// Unit propagation to a fixpoint (true on conflict: w.confl, ws->cl), in the
+// frontier rounds of the DPLL search. Per batch of up to 32 frontier literals
+// the lanes read their literal, mark it settled, and load both its
+// occurrence-list bounds and its learned watch list before the static entries
+// and then the learned watchers are evaluated.
+__device__ __forceinline__ bool bcp_cd(Warp& w, CdWarp& cd) {
+  while (w.head < w.tail) {
+    const uint32_t lo = w.head, hi = w.tail;
     w.head = hi;
     WCOUNT(w, props, hi - lo);
     for (uint32_t base = lo; base < hi; base += 32) {
       const uint32_t nlit = min(32u, hi - base);
+      const LaneMap m = lane_map(w.lane, nlit);
       uint32_t f = 0, beg = 0, cnt = 0, lbeg = 0, lcnt = 0;
-      if (w.lane < nlit) {
-        const uint32_t t = trail_at(w, cd, base + w.lane);
-        const uint32_t v = t >> 1;
-        atomicAnd(&w.asg[v >> 3], ~(NB_FRESH << ((v & 7u) * 4u)));  // no longer fresh
-        f = WIDX(w, t ^ 1u, 2u * w.V, 14);
+      if (m.mine < nlit) {
+        const uint32_t t = WIDX(w, frontier_lit(w, base + m.mine), 2u * w.V, 14);
+        f = t ^ 1u;
         beg = __ldg(&w.occ[f]);
         cnt = __ldg(&w.occ[f + 1]) - beg;
         if (cd.top) {
-          const WList L = cd.wl[f];
-          lbeg = L.off;
-          lcnt = L.len;
+          const uint2 L = *reinterpret_cast<const uint2*>(&cd.wl[f]);  // {offset, length}
+          lbeg = L.x;
+          lcnt = L.y;
         }
+        if (!m.few || m.sub == 0) atomicOr(&w.asg[2 * (t >> 5) + 1], 1u << (t & 31u));  // settled
       }
       __syncwarp();
-      static_batch(w, cd, nlit, f, beg, cnt);
-      learned_batch(w, cd, nlit, f, lbeg, lcnt);
-      __syncwarp();
-      if (*(volatile uint32_t*)&w.ws->conflict) return true;
+      spread_lists(m, nlit, f, beg, cnt, [&](uint32_t jf, uint32_t at, bool in) {
+        Found r{false, false, 0, 0, 0, 0};
+        if (in) r = eval_entry_cd(w, jf, __ldg(&w.ent[WIDX(w, at, w.ent_end, 15)]));
+        if (__any_sync(FULL, r.want || r.confl)) {
+          const bool clash = claim_cd(w, cd, r.want, r.lit, r.c0, r.c1);
+          // a clash: the clause's wanted literal is false after all
+          note_conflict(w, r.confl || clash, r.c0, r.c1,
+                        clash && !(r.c0 & LONG_CLAUSE) ? r.lit : r.c2);
+          __syncwarp();
+        }
+        return w.confl != 0;
+      });
+      const uint32_t total = batch_total(m, cnt);
+      WCOUNT(w, visits, total);
+      if (w.confl) return true;
+      if (cd.top) {
+        learned_batch(w, cd, m, nlit, f, lbeg, lcnt);
+        if (w.confl) return true;
+      }
     }
   }
+  return false;
 }
 
 // First-UIP analysis of the recorded conflict (all lanes). Leaves the learned
 // clause in cd.learnt[0 .. n): the asserting literal first, then a literal of
 // the backjump level; returns n, the backjump level in blev and the clause's
 // LBD (distinct decision levels, counted per group of 32 literals) in lbd.
-// Returns 0 if a consistency check fails (seen marks may then be left set).
-__device__ uint32_t analyze_cd(Warp& w, CdWarp& cd, uint32_t& blev, uint32_t& lbd) {
-  const uint32_t lvl = w.nd;
+// Returns 0 if a consistency check fails.
+//
+// A resolution step is a chain of dependent latencies on one warp, so it stays
+// near: marks, positions and levels in shared memory, recent reasons in the
+// ring's slots, and each current-level literal not yet resolved waits, with
+// its reason, in the registers of the lane that met it. The lanes that hold
+// none take the next clause's literals; the newest waiting literal is found
+// with one warp-wide maximum of trail positions, and marks carry the
+// analysis' number instead of being cleared on the way. If all 32 lanes hold a
+// literal, the rest of this analysis scans the trail for seen marks instead.
+__device__ __forceinline__ uint32_t analyze_cd(Warp& w, CdWarp& cd, uint32_t& blev,
+                                               uint32_t& lbd) {
+  const uint32_t lvl = w.nd, below = (1u << w.lane) - 1u;
   uint32_t n = 1, path = 0, p = NONE;
   uint32_t r0 = w.ws->cl[0], r1 = w.ws->cl[1], r2 = w.ws->cl[2];
-  int64_t idx = (int64_t)*(volatile uint32_t*)&w.ws->tail - 1;
-  // Current-level literals not yet resolved wait in cd.cand with their trail
-  // positions; the newest is the next to resolve. If more than CAND wait at
-  // once, the rest of this analysis scans the trail for seen marks instead.
-  uint32_t ncand = 0;
+  uint32_t idx = w.tail;  // the trail below this position is not resolved yet
+  if (++cd.epoch > MK_EPOCHS) {  // every number used: start over on clean marks
+    for (uint32_t v = w.lane; v < w.V; v += 32) cd.mark[v] &= (uint8_t)MK_PHASE;
+    cd.epoch = 1;
+    __syncwarp();
+  }
+  const uint32_t seen = cd.epoch << 1;
+  uint32_t key = 0, mylit = 0, my0 = 0, my1 = 0;  // waiting literal (key: position + 1; 0: none)
   bool overflow = false;
   bool big = false;
   for (;;) {
@@ -495,42 +500,63 @@ __device__ uint32_t analyze_cd(Warp& w, CdWarp& cd, uint32_t& blev, uint32_t& lb
       csr = w.lits + b;
       cnt = (uint32_t)(w.cb[cl + 1] - b);
     }
-    for (uint32_t k0 = 0; k0 < cnt; k0 += 32) {
-      const uint32_t k = k0 + w.lane;
+    for (uint32_t k0 = 0; k0 < cnt;) {
+      uint32_t idle = __ballot_sync(FULL, key == 0);
+      if (idle == 0) overflow = true;
+      if (overflow) idle = FULL;
+      const uint32_t k = k0 + __popc(idle & below);
+      k0 += __popc(idle);
       uint32_t q = NONE;
-      if (k < cnt) q = src ? src[k] : csr ? code_of(csr[k]) : (k == 0 ? r0 : k == 1 ? r1 : r2);
+      if (k < cnt && ((idle >> w.lane) & 1u))
+        q = src ? src[k] : csr ? code_of(csr[k]) : (k == 0 ? r0 : k == 1 ? r1 : r2);
       const uint32_t v = q == NONE ? NONE >> 1 : WIDX(w, q >> 1, w.V, 21);
       bool take = false;
-      uint32_t mk = 0, lv = 0, ps = 0;
+      uint32_t mk = 0, pos = 0, lev = 0;
+      uint2 why = make_uint2(0, 0);
+      float a = 0.0f;
       if (q != NONE && (p == NONE || v != (p >> 1))) {
-        mk = cd.mark[v];  // three independent loads
-        const uint2 pl = *reinterpret_cast<const uint2*>(&cd.var[v].pos);
-        ps = pl.x;
-        lv = pl.y;
-        take = !(mk & MK_SEEN) && lv > 0;
+        mk = cd.mark[v];  // independent loads
+        a = w.act[v];
+        if (cd.pl) {
+          const uint32_t x = cd.pl[v];
+          pos = x & 0xffffu;
+          lev = x >> 16;
+        } else {
+          const uint4 rec = *reinterpret_cast<const uint4*>(&cd.var[v]);
+          why = make_uint2(rec.x, rec.y);
+          pos = rec.z;
+          lev = rec.w;
+        }
+        take = (mk & ~MK_PHASE) != seen && lev > 0;
       }
-      // one lane per variable (a long clause may repeat a literal)
-      const uint32_t grp = __match_any_sync(FULL, take ? v : NONE);
-      if (take && __ffs(grp) - 1 != w.lane) take = false;
+      if (csr) {  // one lane per variable: a long clause may repeat a literal
+        const uint32_t grp = __match_any_sync(FULL, take ? v : NONE);
+        if (take && __ffs(grp) - 1 != w.lane) take = false;
+      }
+      const bool cur = take && lev >= lvl;
+      const uint32_t lowm = __ballot_sync(FULL, take && !cur);
+      path += __popc(__ballot_sync(FULL, cur));
       if (take) {
-        cd.mark[v] = mk | MK_SEEN;
-        const float a = w.act[v] + w.inc;
+        cd.mark[v] = (uint8_t)((mk & MK_PHASE) | seen);
+        a += w.inc;
         w.act[v] = a;
         big |= a > 1e20f;
-      }
-      const bool cur = take && lv >= lvl;
-      const uint32_t curm = __ballot_sync(FULL, cur);
-      path += __popc(curm);
-      if (!overflow) {
-        if (ncand + __popc(curm) <= CAND) {
-          if (cur) cd.cand[ncand + __popc(curm & ((1u << w.lane) - 1u))] = make_uint2(ps, q ^ 1u);
-          ncand += __popc(curm);
-        } else {
-          overflow = true;
+        if (!cur) {
+          set_learnt(cd, WIDX(w, n + __popc(lowm & below), w.V, 20), q);
+        } else if (!overflow) {
+          key = pos + 1u;
+          mylit = q ^ 1u;
+          if (cd.pl) {
+            // the slot of a literal's position holds its reason as long as the
+            // ring still names that literal there
+            why = cd.why[pos & (RING - 1u)];
+            if (w.tail - pos > RING || w.ws->ring[pos & (RING - 1u)] != mylit)
+              why = *reinterpret_cast<const uint2*>(&cd.var[v].reason_lo);
+          }
+          my0 = why.x;
+          my1 = why.y;
         }
       }
-      const uint32_t lowm = __ballot_sync(FULL, take && lv < lvl);
-      if (take && lv < lvl) cd.learnt[WIDX(w, n + __popc(lowm & ((1u << w.lane) - 1u)), w.V, 20)] = q;
       n += __popc(lowm);
       __syncwarp();
     }
@@ -539,67 +565,47 @@ __device__ uint32_t analyze_cd(Warp& w, CdWarp& cd, uint32_t& blev, uint32_t& lb
     if (path == 0) return 0;
     if (!overflow) {
       // the newest waiting literal (trail positions are distinct)
-      uint32_t key = 0, kk = 0;  // key = position + 1
-      for (uint32_t k = w.lane; k < ncand; k += 32) {
-        const uint32_t x = cd.cand[k].x + 1u;
-        if (x > key) {
-          key = x;
-          kk = k;
-        }
-      }
-      for (int d = 16; d > 0; d >>= 1) {
-        const uint32_t ok = __shfl_xor_sync(FULL, key, d), oi = __shfl_xor_sync(FULL, kk, d);
-        if (ok > key) {
-          key = ok;
-          kk = oi;
-        }
-      }
-      if (key == 0) return 0;
-      p = cd.cand[kk].y;
-      idx = (int64_t)key - 2;  // where a trail scan would continue
-      __syncwarp();
-      if (w.lane == 0) cd.cand[kk] = cd.cand[ncand - 1];
-      ncand--;
+      const uint32_t top = __reduce_max_sync(FULL, key);
+      if (top == 0) return 0;
+      const int owner = __ffs(__ballot_sync(FULL, key == top)) - 1;
+      p = __shfl_sync(FULL, mylit, owner);
+      r0 = __shfl_sync(FULL, my0, owner);
+      r1 = __shfl_sync(FULL, my1, owner);
+      if (key == top) key = 0;
+      idx = top - 1u;
     } else {
       for (;;) {  // the newest seen literal on the trail
-        if (idx < 0) return 0;
-        const int64_t pos = idx - w.lane;
+        if (idx == 0) return 0;
+        const uint32_t pos = idx - 1u - w.lane;
         bool sn = false;
-        if (pos >= 0) sn = (cd.mark[w.trail[pos] >> 1] & MK_SEEN) != 0;
+        if (w.lane < idx) sn = (cd.mark[w.trail[pos] >> 1] & ~MK_PHASE) == seen;
         const uint32_t m = __ballot_sync(FULL, sn);
         if (m) {
-          idx -= __ffs(m) - 1;
+          idx -= __ffs(m);
           break;
         }
-        idx -= 32;
+        idx = idx > 32u ? idx - 32u : 0u;
       }
       p = w.trail[idx];
-      idx--;
+      const uint2 rw = *reinterpret_cast<const uint2*>(&cd.var[p >> 1].reason_lo);
+      r0 = rw.x;
+      r1 = rw.y;
     }
-    __syncwarp();
-    if (w.lane == 0) cd.mark[p >> 1] &= (uint8_t)~MK_SEEN;
-    __syncwarp();
     if (--path == 0) break;
-    const uint2 rw = *reinterpret_cast<const uint2*>(&cd.var[p >> 1].reason_lo);
-    const uint64_t why = (uint64_t)rw.x | ((uint64_t)rw.y << 32);
-    r0 = (uint32_t)why;
-    r1 = (uint32_t)(why >> 32);
     r2 = NONE;
   }
-  if (w.lane == 0) cd.learnt[0] = p ^ 1u;
+  if (w.lane == 0) set_learnt(cd, 0, p ^ 1u);
   // backjump level: the highest level among learnt[1..n), moved to position 1
   uint32_t best_l = 0, best_k = 1, levels = 1;  // learnt[0] is alone at level lvl
   for (uint32_t k0 = 1; k0 < n; k0 += 32) {
     const uint32_t k = k0 + w.lane;
     uint32_t lv = NONE;
     if (k < n) {
-      const uint32_t q = cd.learnt[k];
-      lv = cd.var[q >> 1].level;
+      lv = level_of(cd, learnt_at(cd, k) >> 1);
       if (lv > best_l) {
         best_l = lv;
         best_k = k;
       }
-      cd.mark[q >> 1] &= (uint8_t)~MK_SEEN;
     }
     const uint32_t grp = __match_any_sync(FULL, lv);
     levels += __popc(__ballot_sync(FULL, k < n && __ffs(grp) - 1 == w.lane));
@@ -615,9 +621,9 @@ __device__ uint32_t analyze_cd(Warp& w, CdWarp& cd, uint32_t& blev, uint32_t& lb
   }
   __syncwarp();
   if (w.lane == 0 && n > 2 && best_k != 1) {
-    const uint32_t t = cd.learnt[1];
-    cd.learnt[1] = cd.learnt[best_k];
-    cd.learnt[best_k] = t;
+    const uint32_t t = learnt_at(cd, 1);
+    set_learnt(cd, 1, learnt_at(cd, best_k));
+    set_learnt(cd, best_k, t);
   }
   big = __any_sync(FULL, big);
   if (big) {
@@ -633,18 +639,18 @@ __device__ uint32_t analyze_cd(Warp& w, CdWarp& cd, uint32_t& blev, uint32_t& lb
 __device__ void backjump_cd(Warp& w, CdWarp& cd, uint32_t lev) {
   if (w.nd <= lev) return;
   const uint32_t pos = w.dstack[lev];
-  const uint32_t tail = *(volatile uint32_t*)&w.ws->tail;
+  const uint32_t tail = w.tail;
   WCOUNT(w, undone, tail - pos);
   for (uint32_t t = pos + w.lane; t < tail; t += 32) {
     const uint32_t l = w.trail[t], v = l >> 1;
-    atomicAnd(&w.asg[v >> 3], ~(0xfu << ((v & 7u) * 4u)));
-    cd.mark[v] = (l & 1u) ? 0 : MK_PHASE;
+    const uint32_t keep = ~(3u << (l & 30u));
+    atomicAnd(&w.asg[2 * (l >> 5)], keep);
+    atomicAnd(&w.asg[2 * (l >> 5) + 1], keep);
+    cd.mark[v] = (l & 1u) ? 0 : (uint8_t)MK_PHASE;
   }
   __syncwarp();
-  if (w.lane == 0) w.ws->tail = pos;
-  __syncwarp();
   w.nd = lev;
-  w.head = pos;
+  w.head = w.tail = pos;
 }
 
 // Arena words a learned clause of n literals takes.
@@ -655,10 +661,10 @@ __device__ __forceinline__ uint32_t clause_words(uint32_t n) {
 // Store learnt[0..n) (n >= 2) at the arena top and watch its first two
 // literals. The caller checked the arena has room; the pool may run out
 // (cd.full).
-__device__ uint32_t add_learnt(Warp& w, CdWarp& cd, uint32_t n, uint32_t lbd) {
+__device__ __forceinline__ uint32_t add_learnt(Warp& w, CdWarp& cd, uint32_t n, uint32_t lbd) {
   const uint32_t c = cd.top;
   for (uint32_t k = w.lane; k < ((n + 3u) & ~3u); k += 32)
-    cd.arena[c + CD_HDR + k] = k < n ? cd.learnt[k] : NONE;
+    cd.arena[c + CD_HDR + k] = k < n ? learnt_at(cd, k) : NONE;
   if (w.lane == 0) {
     cd.arena[c] = n;
     cd.arena[c + 1] = 0u;
@@ -672,13 +678,13 @@ __device__ uint32_t add_learnt(Warp& w, CdWarp& cd, uint32_t n, uint32_t lbd) {
   __syncwarp();
   cd.top = c + clause_words(n);
   cd.ncl++;
-  const uint32_t l0 = cd.learnt[0], l1 = cd.learnt[1];
-  wl_append(w, cd, l0, (uint64_t)c | ((uint64_t)l1 << 32));
-  wl_append(w, cd, l1, (uint64_t)c | ((uint64_t)l0 << 32));
+  const uint32_t l0 = cd.lsm[0], l1 = cd.lsm[1];
+  append_watches(w, cd, w.lane < 2, w.lane == 0 ? l0 : l1,
+                 (uint64_t)c | ((uint64_t)(w.lane == 0 ? l1 : l0) << 32));
   return c;
 }
 
-__device__ void clear_learnts(Warp& w, CdWarp& cd) {
+__device__ __noinline__ void clear_learnts(Warp& w, CdWarp& cd) {
   for (uint32_t k = w.lane; k < 2u * w.V; k += 32) cd.wl[k] = WList{0u, 0u, 0u, 0u};
   cd.top = 0;
   cd.ncl = 0;
@@ -792,13 +798,19 @@ __device__ bool rebuild_watches(Warp& w, CdWarp& cd) {
 // (drop_half false) or halve it, and if the lists still do not fit, drop it.
 // Afterwards the bottom levels are propagated again from the first trail
 // entry, over the rebuilt watch lists too.
-__device__ void maintain_db(Warp& w, CdWarp& cd, bool drop_half) {
+__device__ __noinline__ void maintain_db(Warp& w, CdWarp& cd, bool drop_half) {
   const long long t0 = pf_now(*w.S);
   if (w.S->prof && w.lane == 0) w.ws->cyc[PF_NDB]++;
   backjump_cd(w, cd, w.nd_fixed);
   if (!reduce_db(w, cd, drop_half) && (drop_half || !reduce_db(w, cd, true)))
     clear_learnts(w, cd);
-  if (w.lane == 0) w.ws->conflict = 0;
+  w.confl = 0;
+  // the head moves back: the ring has to hold the last positions below the tail
+  // again (undone claims may have overwritten them)
+  for (uint32_t k = w.lane; k < min(w.tail, RING); k += 32) {
+    const uint32_t p = w.tail - 1u - k;
+    w.ws->ring[p & (RING - 1u)] = w.trail[p];
+  }
   __syncwarp();
   w.head = 0;
   pf_add(*w.S, w, PF_DB, t0);
@@ -821,7 +833,7 @@ __device__ uint32_t luby_cd(uint32_t i) {
 // dst[JOB_CLS_WORDS] = [count, words used, offsets[JOB_CLS_MAX], records
 // {len, lbd, literals}]. Every learned clause is implied by the formula, so
 // the cube may use them whatever its assumptions.
-__device__ void export_clauses(Warp& w, CdWarp& cd, uint32_t* dst) {
+__device__ __noinline__ void export_clauses(Warp& w, CdWarp& cd, uint32_t* dst) {
   constexpr uint32_t base = 2 + JOB_CLS_MAX;
   uint32_t m = 0, used = base;
   for (int64_t k0 = (int64_t)cd.ncl - 1; k0 >= 0 && m < JOB_CLS_MAX; k0 -= 32) {
@@ -866,7 +878,7 @@ __device__ void export_clauses(Warp& w, CdWarp& cd, uint32_t* dst) {
 // The clauses a donor attached to this cube (see export_clauses) into the
 // empty database, then its watch lists. Returns false (the database is left
 // empty) if they do not fit.
-__device__ bool import_clauses(Warp& w, CdWarp& cd, const uint32_t* src) {
+__device__ __noinline__ bool import_clauses(Warp& w, CdWarp& cd, const uint32_t* src) {
   const uint32_t m = min(src[0], JOB_CLS_MAX);
   uint32_t top = 0;
   for (uint32_t k0 = 0; k0 < m; k0 += 32) {
@@ -912,38 +924,7 @@ __device__ bool import_clauses(Warp& w, CdWarp& cd, const uint32_t* src) {
   return true;
 }
 
-// Highest-activity unassigned variable (ties: lowest id) over the 4-bit
-// assignment; NONE if all are assigned.
-__device__ uint32_t pick_cd(Warp& w) {
-  float best_a = -1.0f;
-  uint32_t best_v = NONE;
-  const uint32_t nwords = (w.V + 7u) >> 3;
-  for (uint32_t k = w.lane; k < nwords; k += 32) {
-    const uint32_t word = w.asg[k];
-    uint32_t un = ~(word | (word >> 1)) & 0x11111111u;  // value bits 00
-    const uint32_t lim = w.V - 8u * k;
-    if (lim < 8u) un &= (1u << (4u * lim)) - 1u;
-    while (un) {
-      const uint32_t bitpos = __ffs(un) - 1;
-      un &= un - 1u;
-      const uint32_t v = 8u * k + (bitpos >> 2);
-      const float a = w.act[v];
-      if (a > best_a || (a == best_a && v < best_v)) {
-        best_a = a;
-        best_v = v;
-      }
-    }
-  }
-  for (int d = 16; d > 0; d >>= 1) {
-    const float oa = __shfl_xor_sync(FULL, best_a, d);
-    const uint32_t ov = __shfl_xor_sync(FULL, best_v, d);
-    if (oa > best_a || (oa == best_a && ov < best_v)) {
-      best_a = oa;
-      best_v = ov;
-    }
-  }
-  return best_v;
-}
+__device__ uint32_t pick_cd(Warp& w) { return pick_max<2>(w); }
 
 // ---- clauses shared between the jobs of one instance ----------------------
 //
@@ -973,12 +954,11 @@ __device__ void share_publish(const Solve& S, Warp& w, CdWarp& cd, uint32_t n, u
     if (w.lane == 1) x = (uint32_t)w.inst;
     else if (w.lane == 2) x = n | (min(lbd, 255u) << 8);
     else if (w.lane == 3) x = (uint32_t)slot;
-    else x = (uint32_t)(w.lane - 4) < n ? cd.learnt[w.lane - 4] : NONE;
+    else x = (uint32_t)(w.lane - 4) < n ? cd.lsm[w.lane - 4] : NONE;
     *(volatile uint32_t*)&rec[w.lane] = x;
   }
-  __threadfence();
   __syncwarp();
-  if (w.lane == 0) *(volatile uint32_t*)&rec[0] = (uint32_t)(r + 1ull);
+  if (w.lane == 0) store_release(&rec[0], (uint32_t)(r + 1ull));
   __syncwarp();
 }
 
@@ -989,7 +969,7 @@ __device__ void share_publish(const Solve& S, Warp& w, CdWarp& cd, uint32_t n, u
 // and the false literal of highest level; a clause with one open literal
 // left implies it, one with none refutes the job. Returns false in that
 // case (the job's assumptions contradict the formula), true otherwise.
-__device__ bool share_import(const Solve& S, Warp& w, CdWarp& cd, int64_t slot,
+__device__ __noinline__ bool share_import(const Solve& S, Warp& w, CdWarp& cd, int64_t slot,
                              unsigned long long& rd) {
   const uint32_t p = (uint32_t)w.inst & S.share_mask;
   const unsigned long long cap = S.share_cap;
@@ -999,7 +979,6 @@ __device__ bool share_import(const Solve& S, Warp& w, CdWarp& cd, int64_t slot,
   unsigned long long from = rd;
   if (cur > cap / 2 && from < cur - cap / 2) from = cur - cap / 2;  // skip what may be overwritten
   const unsigned long long to = min(cur, from + 256ull);
-  const uint64_t no_reason = ~0ull;
   bool ok_all = true;
   for (unsigned long long base = from; base < to && ok_all; base += 32) {
     const unsigned long long r = base + (unsigned long long)w.lane;
@@ -1035,7 +1014,7 @@ __device__ bool share_import(const Solve& S, Warp& w, CdWarp& cd, int64_t slot,
       }
       const bool have = (uint32_t)w.lane < nj;
       const uint32_t val = have ? lit_value_cd(w.asg, my) : LV_F;
-      const uint32_t lvl = have && val == LV_F ? cd.var[my >> 1].level : 0u;
+      const uint32_t lvl = have && val == LV_F ? level_of(cd, my >> 1) : 0u;
       const uint32_t nf = __ballot_sync(FULL, have && val != LV_F);
       if (nf == 0u) {  // every literal false: the job's assumptions are refuted
         ok_all = false;
@@ -1054,8 +1033,7 @@ __device__ bool share_import(const Solve& S, Warp& w, CdWarp& cd, int64_t slot,
       const bool unit = __popc(nf) == 1 && __shfl_sync(FULL, val, w0) == LV_U;
       const uint32_t first = __shfl_sync(FULL, my, w0);
       if (nj == 1) {  // a unit clause: its literal holds in every model
-        if (unit && w.lane == 0) imply_cd(w, cd, first, no_reason, 0u);
-        __syncwarp();
+        if (unit) assign_one_cd(w, cd, first, NONE, NONE);
         continue;
       }
       if ((uint64_t)cd.top + clause_words(nj) > cd.arena_words || cd.full) break;
@@ -1066,14 +1044,11 @@ __device__ bool share_import(const Solve& S, Warp& w, CdWarp& cd, int64_t slot,
         if (w.lane == w0) at = 0;
         else if (w.lane == w1) at = 1;
         else at = 2u + __popc(rest & ((1u << w.lane) - 1u));
-        cd.learnt[at] = my;
+        cd.lsm[at] = my;
       }
       __syncwarp();
       const uint32_t c = add_learnt(w, cd, nj, lbdj);
-      if (unit) {
-        if (w.lane == 0) imply_cd(w, cd, cd.learnt[0], (uint64_t)(LEARNT_REF | c), 0u);
-        __syncwarp();
-      }
+      if (unit) assign_one_cd(w, cd, first, LEARNT_REF | c, 0u);
     }
   }
   rd = to;
@@ -1085,13 +1060,20 @@ __device__ bool share_import(const Solve& S, Warp& w, CdWarp& cd, int64_t slot,
 // from the subtree-sharing ring), start to verdict. Returns SAT, UNSAT (for a
 // cube: no model extends it) or UNKNOWN.
 __device__ int run_cdcl(const Solve& S, Warp& w, int64_t slot, int unit, int inst,
-                        const TakenJob* job, uint2* ring, int& abort_code) {
+                        const TakenJob* job, unsigned char* area, int& abort_code) {
   CdWarp cd;
-  cd.ring = ring;
-  cd.cand = ring + RING;
+  cd.why = reinterpret_cast<uint2*>(area);
+  cd.lsm = reinterpret_cast<uint32_t*>(area + RING * 8);
+  cd.epoch = 0;
   cd.var = reinterpret_cast<VarInfo*>(S.cd_var) + slot * S.vmax;
-  for (uint32_t k = w.lane; k < RING; k += 32) ring[k] = make_uint2(NONE, NONE);
+  cd.pl = nullptr;
   cd.mark = S.cd_mark + slot * S.vmax;
+  if (S.cd_smem & CD_SMEM_POS) {
+    const size_t v16 = ((size_t)S.vmax + 15) & ~(size_t)15;
+    unsigned char* at = area + cd_area_bytes(S.cd_smem & CD_SMEM_ACT, S.vmax);
+    cd.pl = reinterpret_cast<uint32_t*>(at);
+    cd.mark = at + 4 * v16;
+  }
   cd.wl = S.cd_wl + slot * 2 * S.vmax;
   cd.pool = S.cd_pool + slot * S.cd_pool_cap;
   cd.arena = S.cd_arena + slot * S.cd_arena_words;
@@ -1114,41 +1096,43 @@ __device__ int run_cdcl(const Solve& S, Warp& w, int64_t slot, int unit, int ins
   w.nd = 0;
   w.nd_fixed = 0;
   w.inc = job ? job->inc : 1.0f;  // a cube starts from its donor's activities
-  const uint32_t nwords = (w.V + 7u) >> 3;
+  const uint32_t nwords = 2u * ((w.V + 15u) >> 4);
   for (uint32_t k = w.lane; k < nwords; k += 32) w.asg[k] = 0u;
   for (uint32_t v = w.lane; v < w.V; v += 32) {
     if (!job) w.act[v] = 0.0f;
     cd.mark[v] = 0;
   }
-  clear_learnts(w, cd);
-  if (job && job->cls) import_clauses(w, cd, job->cls);  // the donor's clauses
-  if (w.lane == 0) {
-    w.ws->tail = 0;
-    w.ws->conflict = 0;
-  }
+  w.tail = 0;
+  w.confl = 0;
+  // Calls of the rarely used parts work on copies of w and cd, so that the
+  // search itself can keep them in registers.
+  auto apart = [&](auto&& fn) {
+    Warp w2 = w;
+    CdWarp cd2 = cd;
+    fn(w2, cd2);
+    w = w2;
+    cd = cd2;
+  };
+  apart([&](Warp& a, CdWarp& b) {
+    clear_learnts(a, b);
+    if (job && job->cls) import_clauses(a, b, job->cls);  // the donor's clauses
+  });
   __syncwarp();
   if (S.flags[inst] & F_EMPTY) return SCUBA_UNSAT;
-  const uint64_t no_reason = ~0ull;
   const uint32_t nu = S.nunits[inst];
   const uint32_t* un = S.units + w.c0;
-  for (uint32_t k = w.lane; k < nu; k += 32)
-    if (!imply_cd(w, cd, un[k], no_reason, 0u)) record_conflict(w, un[k], NONE, NONE);
-  __syncwarp();
-  if (w.ws->conflict) return SCUBA_UNSAT;
-  if (job) {  // the cube's literals as decisions of levels 1, 2, ...
-    for (int k = 0; k < job->len; k++) {
-      if (bcp_cd(w, cd)) return SCUBA_UNSAT;
-      const uint32_t l = job->lit[k];
-      const uint32_t val = lit_value_cd(w.asg, l);
-      if (val == LV_F) return SCUBA_UNSAT;
-      if (val == LV_T) continue;
-      if (w.lane == 0) w.dstack[WIDX(w, w.nd, (uint32_t)S.vmax, 19)] = *(volatile uint32_t*)&w.ws->tail;
-      w.nd++;
-      if (w.lane == 0) imply_cd(w, cd, l, no_reason, 0u);
-      __syncwarp();
-    }
-    w.nd_fixed = w.nd;
+  for (uint32_t k0 = 0; k0 < nu; k0 += 32) {
+    const uint32_t l = k0 + w.lane < nu ? un[k0 + w.lane] : NONE;
+    const bool clash = claim_cd(w, cd, l != NONE, l, NONE, NONE);
+    __syncwarp();
+    // a unit clause against an earlier one's value, or another lane's
+    const bool bad = l != NONE && lit_value_cd(w.asg, l) != LV_T;
+    if (__any_sync(FULL, clash || bad)) return SCUBA_UNSAT;
   }
+  // the cube's literals become decisions of levels 1, 2, ..., one after each
+  // propagation of the main loop
+  int next_asm = 0;
+  const int n_asm = job ? job->len : 0;
 
   // fixed levels that are the unit's own assumptions, not cube literals
   const uint32_t asm_levels =
@@ -1184,10 +1168,11 @@ __device__ int run_cdcl(const Solve& S, Warp& w, int64_t slot, int unit, int ins
     const bool confl = bcp_cd(w, cd);
     pf_add(S, w, PF_BCP, t0);
     if (cd.full) {  // the watch pool ran out: compact it (or halve the clauses)
-      maintain_db(w, cd, false);
+      apart([](Warp& a, CdWarp& b) { maintain_db(a, b, false); });
       continue;
     }
     if (confl) {
+      if (next_asm < n_asm) return SCUBA_UNSAT;  // the assumptions alone
       WCOUNT(w, conflicts, 1);
       if (w.nd <= w.nd_fixed) return SCUBA_UNSAT;
       conflicts++;
@@ -1202,37 +1187,50 @@ __device__ int run_cdcl(const Solve& S, Warp& w, int64_t slot, int unit, int ins
       if (shared && n <= SHARE_MAXLEN && (n == 1 || lbd <= S.share_lbd))
         share_publish(S, w, cd, n, lbd, slot);
       w.inc *= (1.0f / 0.95f);
-      if (w.lane == 0) w.ws->conflict = 0;
+      w.confl = 0;
       const uint32_t target = max(blev, w.nd_fixed);
       if (n >= 2 && (uint64_t)cd.top + clause_words(n) > cd.arena_words) {
-        maintain_db(w, cd, true);  // arena full: restart with half the clauses
-        if ((uint64_t)cd.top + clause_words(n) > cd.arena_words) clear_learnts(w, cd);
+        apart([&](Warp& a, CdWarp& b) {
+          maintain_db(a, b, true);  // arena full: restart with half the clauses
+          if ((uint64_t)b.top + clause_words(n) > b.arena_words) clear_learnts(a, b);
+        });
         since_restart = 0;
       } else {
         backjump_cd(w, cd, target);
       }
-      uint64_t why = no_reason;
+      uint32_t why = NONE;
+      const uint32_t uip = cd.lsm[0];
       if (n >= 2) {
         uint32_t c = add_learnt(w, cd, n, lbd);
-        if (cd.full) {  // the pool ran out: compact it, the new clause included
-          maintain_db(w, cd, false);
-          // the newest clause survives a compaction or a halving; after a
-          // full drop it is added again to the empty database
-          c = cd.ncl > 0 ? cd.cl_off[cd.ncl - 1] : add_learnt(w, cd, n, lbd);
-        }
-        why = (uint64_t)(LEARNT_REF | c);
+        if (cd.full)  // the pool ran out: compact it, the new clause included
+          apart([&](Warp& a, CdWarp& b) {
+            maintain_db(a, b, false);
+            // the newest clause survives a compaction or a halving; after a
+            // full drop it is added again to the empty database
+            c = b.ncl > 0 ? b.cl_off[b.ncl - 1] : add_learnt(a, b, n, lbd);
+          });
+        why = LEARNT_REF | c;
       }
       // the clause is unit once every literal but the first is false
-      if (n == 1 || blev <= w.nd) {
-        if (w.lane == 0) imply_cd(w, cd, cd.learnt[0], why, 0u);
-        __syncwarp();
-      }
+      if (n == 1 || blev <= w.nd) assign_one_cd(w, cd, uip, why, n == 1 ? NONE : 0u);
       pf_add(S, w, PF_ANALYZE, t0);
       if (S.budget > 0) {  // conflicts of the instance, all of its cubes together
         unsigned long long tot = 0;
         if (w.lane == 0) tot = atomicAdd(&S.inst_dec[unit], 1ull) + 1ull;
         tot = __shfl_sync(FULL, tot, 0);
         if ((int64_t)tot >= S.budget) return SCUBA_UNKNOWN;
+      }
+      continue;
+    }
+    if (next_asm < n_asm) {
+      const uint32_t l = job->lit[next_asm++];
+      const uint32_t val = lit_value_cd(w.asg, l);
+      if (val == LV_F) return SCUBA_UNSAT;
+      if (val == LV_U) {
+        if (w.lane == 0) w.dstack[WIDX(w, w.nd, (uint32_t)S.vmax, 19)] = w.tail;
+        w.nd++;
+        w.nd_fixed = w.nd;
+        assign_one_cd(w, cd, l, NONE, NONE);
       }
       continue;
     }
@@ -1243,7 +1241,7 @@ __device__ int run_cdcl(const Solve& S, Warp& w, int64_t slot, int unit, int ins
       if (conflicts >= next_reduce) {  // a restart that also halves the database
         reductions++;
         next_reduce = conflicts + 2000u + 300u * reductions;
-        maintain_db(w, cd, true);
+        apart([](Warp& a, CdWarp& b) { maintain_db(a, b, true); });
       } else {
         backjump_cd(w, cd, w.nd_fixed);
       }
@@ -1252,10 +1250,14 @@ __device__ int run_cdcl(const Solve& S, Warp& w, int64_t slot, int unit, int ins
         if (w.lane == 0) others = *(volatile uint32_t*)&S.pending[unit] > 1u;
         shared = __shfl_sync(FULL, others, 0) != 0u;
       }
-      if (shared && !share_import(S, w, cd, slot, share_rd)) return SCUBA_UNSAT;
+      if (shared) {
+        bool ok = true;
+        apart([&](Warp& a, CdWarp& b) { ok = share_import(S, a, b, slot, share_rd); });
+        if (!ok) return SCUBA_UNSAT;
+      }
       continue;
     }
-    WCOUNT(w, act_reads, w.V - *(volatile uint32_t*)&w.ws->tail);
+    WCOUNT(w, act_reads, w.V - w.tail);
     t0 = pf_now(S);
     const uint32_t v = pick_cd(w);
     pf_add(S, w, PF_DECIDE, t0);
@@ -1267,7 +1269,7 @@ __device__ int run_cdcl(const Solve& S, Warp& w, int64_t slot, int unit, int ins
       if (won && S.model)
         for (uint32_t x = w.lane; x < w.V; x += 32) {
           S.model[(S.unit_vb ? S.unit_vb[unit] : S.vb[inst]) + x] =
-              (nib(w.asg, x) & 3u) == NB_T ? 1 : 0;
+              lit_value_cd(w.asg, 2u * x) == LV_T ? 1 : 0;
         }
       __syncwarp();
       return SCUBA_SAT;
@@ -1290,7 +1292,9 @@ __device__ int run_cdcl(const Solve& S, Warp& w, int64_t slot, int unit, int ins
         if (w.lane == 0) atomicAdd(&S.pending[unit], 1u);
         __syncwarp();
         if (ring_push(S, w, unit, k + 1, w.trail, w.dstack, k, [&](uint32_t cell) {
-              export_clauses(w, cd, S.job_cls + (size_t)cell * JOB_CLS_WORDS);
+              apart([&](Warp& a, CdWarp& b) {
+                export_clauses(a, b, S.job_cls + (size_t)cell * JOB_CLS_WORDS);
+              });
             })) {
           w.nd_fixed = k + 1;
           shared = S.share_lbd > 0;
@@ -1312,9 +1316,8 @@ __device__ int run_cdcl(const Solve& S, Warp& w, int64_t slot, int unit, int ins
     w.decisions++;
     WCOUNT(w, decisions, 1);
     const uint32_t lit = 2u * v + ((cd.mark[v] & MK_PHASE) ? 0u : 1u);
-    if (w.lane == 0) w.dstack[WIDX(w, w.nd, (uint32_t)S.vmax, 19)] = *(volatile uint32_t*)&w.ws->tail;
+    if (w.lane == 0) w.dstack[WIDX(w, w.nd, (uint32_t)S.vmax, 19)] = w.tail;
     w.nd++;
-    if (w.lane == 0) imply_cd(w, cd, lit, no_reason, 0u);
-    __syncwarp();
+    assign_one_cd(w, cd, lit, NONE, NONE);
   }
 }

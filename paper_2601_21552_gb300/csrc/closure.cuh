@@ -1,0 +1,155 @@
+// closure.cuh -- unit propagation of scuba_propagate_batch (included by solver.cu
+// inside namespace scuba::dev). A closure's rounds are wide (a whole input word
+// is assumed at once, frontiers of hundreds of literals), so the lanes take the
+// entries of up to 32 literals as one list, 32 at a time; the searches, whose
+// rounds are a few literals, use bcp() and bcp_cd() instead.
+
+__device__ __forceinline__ void close_conflict(Warp& w, uint32_t a, uint32_t b, uint32_t c) {
+  if (atomicCAS(&w.ws->conflict, 0u, 1u) == 0u) {
+    w.ws->cl[0] = a;
+    w.ws->cl[1] = b;
+    w.ws->cl[2] = c;
+  }
+}
+
+// Assign literal l true. Returns false on a clash with the opposite value.
+__device__ __forceinline__ bool close_claim(Warp& w, uint32_t l) {
+  uint32_t v = WIDX(w, l >> 1, w.V, 1);
+  uint32_t sh = (v & 15u) * 2u;
+  uint32_t mask = ((l & 1u) ? 2u : 1u) << sh;
+  uint32_t old = atomicOr(&w.asg[v >> 4], mask);
+  uint32_t ob = (old >> sh) & 3u;
+  if (ob == 0u) {
+    uint32_t pos = atomicAdd(&w.ws->tail, 1u);
+    w.trail[WIDX(w, pos, w.V, 2)] = l;
+    return true;
+  }
+  if (ob == (mask >> sh)) return true;
+  if ((old & mask) == 0u) atomicAnd(&w.asg[v >> 4], ~mask);  // undo our bit
+  return false;
+}
+
+__device__ void close_long(Warp& w, uint32_t local, uint32_t f) {
+  const int64_t c = w.c0 + local;
+  const int64_t b = w.cb[c], e = w.cb[c + 1];
+  uint32_t open_lit = NONE;
+  int n_open = 0;
+  for (int64_t q = b; q < e; q++) {
+    uint32_t x = code_of(__ldg(&w.lits[q]));
+    uint32_t vx = lit_value(w.asg, x);
+    if (vx == LV_T || vx == LV_X) return;
+    if (vx == LV_U && x != open_lit) {
+      n_open++;
+      open_lit = x;
+      if (n_open > 1) return;
+    }
+  }
+  if (n_open == 0) {
+    close_conflict(w, LONG_CLAUSE | local, NONE, NONE);
+  } else if (!close_claim(w, open_lit)) {
+    close_conflict(w, LONG_CLAUSE | local, NONE, NONE);
+  }
+}
+
+// Visit one occurrence entry of the falsified literal f.
+__device__ __forceinline__ void close_entry(Warp& w, uint32_t f, uint64_t e) {
+  const uint32_t a0 = (uint32_t)e, b0 = (uint32_t)(e >> 32);
+  if (a0 & LONG_CLAUSE) {
+    close_long(w, a0 & ~LONG_CLAUSE, f);
+    return;
+  }
+  const uint32_t a = WIDX(w, a0, 2u * w.V, 3);
+  const uint32_t b = b0 == NONE ? NONE : WIDX(w, b0, 2u * w.V, 3);
+  const uint32_t va = lit_value(w.asg, a);
+  if (b == NONE) {  // binary (f | a)
+    if (va == LV_T || va == LV_X) return;
+    if (va == LV_F || !close_claim(w, a)) close_conflict(w, f, a, NONE);
+    return;
+  }
+  const uint32_t vb = lit_value(w.asg, b);  // ternary (f | a | b)
+  if (va == LV_T || vb == LV_T || va == LV_X || vb == LV_X) return;
+  if (va == LV_F && vb == LV_F) {
+    close_conflict(w, f, a, b);
+  } else if (va == LV_F) {
+    if (!close_claim(w, b)) close_conflict(w, f, a, b);
+  } else if (vb == LV_F) {
+    if (!close_claim(w, a)) close_conflict(w, f, a, b);
+  }
+}
+
+// Unit propagation to a fixpoint. Returns true on conflict.
+// Each round takes the trail literals assigned in the previous round (the
+// frontier) and spreads their occurrence entries over the 32 lanes:
+// The values of a conflicting instance are what this order of visits leaves.
+__device__ bool close_rounds(Warp& w) {
+  for (;;) {
+    __syncwarp();
+    const uint32_t hi = *(volatile uint32_t*)&w.ws->tail;
+    if (w.head >= hi) return false;
+    const uint32_t lo = w.head;
+    w.head = hi;
+    for (uint32_t base = lo; base < hi; base += 32) {
+      const uint32_t nlit = min(32u, hi - base);
+      if (nlit == 1) {
+        // one literal: every lane reads the same list bounds (broadcast)
+        const uint32_t f = WIDX(w, w.trail[base] ^ 1u, 2u * w.V, 4);
+        const uint32_t beg = __ldg(&w.occ[f]);
+        const uint32_t cnt = __ldg(&w.occ[f + 1]) - beg;
+        for (uint32_t e = w.lane; e < cnt; e += 32)
+          close_entry(w, f, __ldg(&w.ent[WIDX(w, beg + e, w.ent_end, 5)]));
+      } else {
+        uint32_t f = 0, beg = 0, cnt = 0;
+        if (w.lane < nlit) {
+          f = WIDX(w, w.trail[base + w.lane] ^ 1u, 2u * w.V, 4);  // the literal that became false
+          beg = __ldg(&w.occ[f]);
+          cnt = __ldg(&w.occ[f + 1]) - beg;
+        }
+        uint32_t inc = cnt;
+#pragma unroll
+        for (int d = 1; d < 32; d <<= 1) {
+          uint32_t y = __shfl_up_sync(FULL, inc, d);
+          if (w.lane >= d) inc += y;
+        }
+        const uint32_t excl = inc - cnt;
+        const uint32_t total = __shfl_sync(FULL, inc, 31);
+        if (total <= 32) {
+          // owner of entry e = the lane whose segment starts at the last
+          // segment start <= e: segment starts as a bit mask, ranks by popc
+          const bool has = cnt > 0;
+          const uint32_t starts = __reduce_or_sync(FULL, has ? (1u << excl) : 0u);
+          const uint32_t nz = __ballot_sync(FULL, has);
+          const uint32_t e = w.lane;
+          int j = 0;
+          if (e < total) {
+            const int rank = __popc(starts & ((2u << e) - 1u)) - 1;
+            j = __fns(nz, 0, rank + 1);
+          }
+          const uint32_t jbeg = __shfl_sync(FULL, beg, j);
+          const uint32_t jex = __shfl_sync(FULL, excl, j);
+          const uint32_t jf = __shfl_sync(FULL, f, j);
+          if (e < total) close_entry(w, jf, __ldg(&w.ent[WIDX(w, jbeg + (e - jex), w.ent_end, 5)]));
+        } else {
+          for (uint32_t e0 = 0; e0 < total; e0 += 32) {
+            const uint32_t e = e0 + w.lane;
+            // owner = smallest lane j with inc_j > e
+            int lo_j = 0, hi_j = 31;
+#pragma unroll
+            for (int s2 = 0; s2 < 5; s2++) {
+              int mid = (lo_j + hi_j) >> 1;
+              uint32_t v = __shfl_sync(FULL, inc, mid);
+              if (v > e) hi_j = mid; else lo_j = mid + 1;
+              if (lo_j > hi_j) lo_j = hi_j;
+            }
+            const int j = lo_j;
+            const uint32_t jbeg = __shfl_sync(FULL, beg, j);
+            const uint32_t jex = __shfl_sync(FULL, excl, j);
+            const uint32_t jf = __shfl_sync(FULL, f, j);
+            if (e < total) close_entry(w, jf, __ldg(&w.ent[WIDX(w, jbeg + (e - jex), w.ent_end, 5)]));
+          }
+        }
+      }
+      __syncwarp();
+      if (*(volatile uint32_t*)&w.ws->conflict) return true;
+    }
+  }
+}

@@ -142,6 +142,11 @@ struct TraceDev {
 
 enum { MODE_PLAIN = 0, MODE_TRACE = 1, MODE_LEARNED = 2, MODE_CDCL = 3 };
 
+// Activities of a slot: whole groups of 16, what one 2-bit assignment word covers.
+__host__ __device__ __forceinline__ int64_t act_stride(int32_t vmax) {
+  return ((int64_t)vmax + 15) & ~(int64_t)15;
+}
+
 struct WList;  // a learned watch list (clause-learning mode)
 
 struct Solve {
@@ -205,6 +210,8 @@ struct Solve {
   // conflict-driven clause learning (per slot)
   uint4* cd_var;               // [slots][vmax] reason, trail position, level (16 B)
   uint8_t* cd_mark;            // [slots][vmax]
+  int cd_smem;                 // per-variable state kept in shared memory (CD_SMEM_*)
+  uint32_t cd_smem_warp;       // bytes of shared memory per warp beyond the assignment
   WList* cd_wl;                // [slots][2 vmax] learned watch lists
   uint64_t* cd_pool;           // [slots][cd_pool_cap] watch entries
   uint32_t* cd_learnt;         // [slots][vmax]
@@ -224,11 +231,17 @@ struct Solve {
   uint32_t share_lbd;          // publish learned clauses of LBD <= this; 0: off
 };
 
-struct WarpShared {
-  uint32_t tail;
-  uint32_t conflict;
+// Recent trail literals a warp keeps in shared memory (a power of two).
+constexpr uint32_t RING = 64;
+
+struct alignas(16) WarpShared {
+  uint32_t tail, conflict;  // closures only: the searches keep theirs in registers
   uint32_t cl[3];
   uint32_t pad[3];
+  // ring[p mod RING] = trail[p] for the positions p in [head, tail) that are
+  // at most RING below the tail: a propagation round reads its literals here
+  // instead of waiting for the global trail
+  uint32_t ring[RING];
   // per-job work counters (lane 0 updates them; kept out of registers)
   unsigned long long decisions, conflicts, props, visits, act_reads, undone;
   // clause-learning profile (cycles of lane 0 per phase; counts)
@@ -262,6 +275,8 @@ struct Warp {
   const int32_t* lits;     // the caller's literals (long clauses)
   int64_t c0;
   uint32_t head;
+  uint32_t tail;           // trail length (the same in all lanes)
+  uint32_t confl;          // a clause of the last bcp() is false (ws->cl)
   uint32_t nd;
   uint32_t nd_fixed;       // decisions below this index are assumptions
   float inc;
@@ -294,170 +309,202 @@ __device__ __forceinline__ void warp_checks(Warp& w, Ctrl* c) {
     if ((w).lane == 0) (w).ws->field += (amount); \
   } while (0)
 
-__device__ __forceinline__ void record_conflict(Warp& w, uint32_t a, uint32_t b, uint32_t c) {
-  if (atomicCAS(&w.ws->conflict, 0u, 1u) == 0u) {
-    w.ws->cl[0] = a;
-    w.ws->cl[1] = b;
-    w.ws->cl[2] = c;
-  }
+#include "closure.cuh"
+
+// Trail literal p of the current frontier.
+__device__ __forceinline__ uint32_t frontier_lit(const Warp& w, uint32_t p) {
+  return w.tail - p <= RING ? w.ws->ring[p & (RING - 1u)] : w.trail[p];
 }
 
-// Assign literal l true. Returns false on a clash with the opposite value.
-__device__ __forceinline__ bool imply(Warp& w, uint32_t l) {
-  uint32_t v = WIDX(w, l >> 1, w.V, 1);
-  uint32_t sh = (v & 15u) * 2u;
-  uint32_t mask = ((l & 1u) ? 2u : 1u) << sh;
-  uint32_t old = atomicOr(&w.asg[v >> 4], mask);
-  uint32_t ob = (old >> sh) & 3u;
-  if (ob == 0u) {
-    uint32_t pos = atomicAdd(&w.ws->tail, 1u);
+// Append the literals of the lanes with won set to the trail (all lanes): in
+// lane order, so no counter in memory is involved. Returns the lane's position.
+__device__ __forceinline__ uint32_t push_trail(Warp& w, bool won, uint32_t l) {
+  const uint32_t m = __ballot_sync(FULL, won);
+  const uint32_t pos = w.tail + __popc(m & ((1u << w.lane) - 1u));
+  if (won) {
     w.trail[WIDX(w, pos, w.V, 2)] = l;
-    return true;
+    w.ws->ring[pos & (RING - 1u)] = l;
   }
-  if (ob == (mask >> sh)) return true;
-  if ((old & mask) == 0u) atomicAnd(&w.asg[v >> 4], ~mask);  // undo our bit
+  w.tail += __popc(m);
+  return pos;
+}
+
+// Make literal l of every lane with want set true (all lanes). The assignment is
+// a bit set over literal codes, STRIDE words apart: bit l set = l is true. Of
+// the lanes that claim one variable the first wins; returns true in a lane
+// whose literal's negation was claimed by another lane of this call (seeing
+// both bits, a lane agrees with the winner or the undo of the lane that saw
+// one covers it); won is set where the lane's literal is new.
+template <int STRIDE>
+__device__ __forceinline__ bool claim_bits(Warp& w, bool want, uint32_t l, bool& won) {
+  bool clash = false;
+  won = false;
+  if (want) {
+    const uint32_t at = WIDX(w, l, 2u * w.V, 1);
+    uint32_t* word = &w.asg[STRIDE * (at >> 5)];
+    const uint32_t old = atomicOr(word, 1u << (at & 31u));
+    const uint32_t t = (old >> (at & 31u)) & 1u, f = (old >> ((at & 31u) ^ 1u)) & 1u;
+    won = !(t | f);
+    clash = f && !t;
+    if (clash) atomicAnd(word, ~(1u << (at & 31u)));
+  }
+  return clash;
+}
+
+// Assign l, unassigned, for a decision or an assumption (all lanes, uniform).
+__device__ __forceinline__ void assign_one(Warp& w, uint32_t l) {
+  bool won;
+  claim_bits<1>(w, w.lane == 0, l, won);
+  push_trail(w, won, l);
+  __syncwarp();
+}
+
+// What one visited clause asks for: a literal to make true, or a conflict with
+// the clause's falsified literals (or its reference) in c0..c2.
+struct Found {
+  bool want, confl;
+  uint32_t lit, c0, c1, c2;
+};
+
+__device__ __noinline__ Found eval_long(const uint32_t* asg, const int32_t* lits, int64_t b,
+                                        int64_t e, uint32_t local) {
+  uint32_t open_lit = NONE;
+  for (int64_t q = b; q < e; q++) {
+    const uint32_t x = code_of(__ldg(&lits[q]));
+    const uint32_t vx = lit_value(asg, x);
+    if (vx == LV_T || (vx == LV_U && open_lit != NONE && x != open_lit))
+      return Found{false, false, NONE, 0, 0, 0};
+    if (vx == LV_U) open_lit = x;
+  }
+  return Found{open_lit != NONE, open_lit == NONE, open_lit, LONG_CLAUSE | local, NONE, NONE};
+}
+
+// One occurrence entry of the falsified literal f, without branches but for
+// long clauses: bit a of the assignment says a is true, bit a ^ 1 that it is
+// false; a binary entry's missing literal counts as false.
+__device__ __forceinline__ Found eval_entry(const Warp& w, uint32_t f, uint64_t e) {
+  const uint32_t a0 = (uint32_t)e, b0 = (uint32_t)(e >> 32);
+  if (a0 & LONG_CLAUSE) {
+    const uint32_t local = a0 & ~LONG_CLAUSE;
+    const int64_t c = w.c0 + local;
+    return eval_long(w.asg, w.lits, w.cb[c], w.cb[c + 1], local);
+  }
+  const bool tern = b0 != NONE;
+  const uint32_t a = WIDX(w, a0, 2u * w.V, 3), b = tern ? WIDX(w, b0, 2u * w.V, 3) : a;
+  const uint32_t xa = w.asg[a >> 5], xb = w.asg[b >> 5];
+  const bool ta = (xa >> (a & 31u)) & 1u, fa = (xa >> ((a & 31u) ^ 1u)) & 1u;
+  const bool tb = tern && ((xb >> (b & 31u)) & 1u);
+  const bool fb = !tern || ((xb >> ((b & 31u) ^ 1u)) & 1u);
+  const bool ua = !ta && !fa && fb, ub = !tb && !fb && fa;
+  return Found{ua || ub, fa && fb, ua ? a : b, f, a, b0};
+}
+
+// How the lanes share a batch of nlit frontier literals: one literal has the
+// whole warp, two have 16 lanes each, more have 8 lanes each, four at a time.
+// Most lists hold 3 to 8 entries and most rounds 1 to 4 literals, so a round is
+// usually one pass -- no scan over the list lengths, no search for the owner
+// of an entry. With up to four literals (few) every lane reads its own
+// literal and list bounds; with more, lane j reads those of literal j and
+// each pass fetches its four with shuffles.
+struct LaneMap {
+  uint32_t lg;     // log2 of lanes per literal
+  uint32_t sub;    // this lane's place among its literal's lanes
+  uint32_t group;  // which of the pass's literals is this lane's
+  uint32_t mine;   // the literal of the batch whose bounds this lane reads
+  bool few;
+};
+
+__device__ __forceinline__ LaneMap lane_map(uint32_t lane, uint32_t nlit) {
+  LaneMap m;
+  m.lg = nlit == 1 ? 5u : nlit == 2 ? 4u : 3u;
+  m.sub = lane & ((1u << m.lg) - 1u);
+  m.group = lane >> m.lg;
+  m.few = nlit <= 4;
+  m.mine = m.few ? m.group : lane;
+  return m;
+}
+
+// The lane holds literal m.mine's falsified code f and list [beg, beg + cnt) (cnt 0
+// past the last literal); visit(f, index, in) runs for every index of every
+// list (all lanes, in = the lane has one) until it returns true.
+template <class Visit>
+__device__ __forceinline__ bool spread_lists(const LaneMap& m, uint32_t nlit, uint32_t f,
+                                             uint32_t beg, uint32_t cnt, Visit&& visit) {
+  for (uint32_t s = 0; s < nlit; s += 32u >> m.lg) {
+    uint32_t jb = beg, jf = f, jc = cnt;
+    if (!m.few) {
+      const uint32_t j = s + m.group;
+      jb = __shfl_sync(FULL, beg, j);
+      jf = __shfl_sync(FULL, f, j);
+      jc = __shfl_sync(FULL, cnt, j);
+      if (j >= nlit) jc = 0;
+    }
+    uint32_t k = m.sub;
+    do {
+      if (visit(jf, jb + k, k < jc)) return true;
+      k += 1u << m.lg;
+    } while (__any_sync(FULL, k < jc));
+  }
   return false;
 }
 
-__device__ void eval_long(Warp& w, uint32_t local, uint32_t f) {
-  const int64_t c = w.c0 + local;
-  const int64_t b = w.cb[c], e = w.cb[c + 1];
-  uint32_t open_lit = NONE;
-  int n_open = 0;
-  for (int64_t q = b; q < e; q++) {
-    uint32_t x = code_of(__ldg(&w.lits[q]));
-    uint32_t vx = lit_value(w.asg, x);
-    if (vx == LV_T || vx == LV_X) return;
-    if (vx == LV_U && x != open_lit) {
-      n_open++;
-      open_lit = x;
-      if (n_open > 1) return;
-    }
-  }
-  if (n_open == 0) {
-    record_conflict(w, LONG_CLAUSE | local, NONE, NONE);
-  } else if (!imply(w, open_lit)) {
-    record_conflict(w, LONG_CLAUSE | local, NONE, NONE);
-  }
+// Entries of all lists of a batch (every lane).
+__device__ __forceinline__ uint32_t batch_total(const LaneMap& m, uint32_t cnt) {
+  return __reduce_add_sync(FULL, m.few && m.sub != 0 ? 0u : cnt);
 }
 
-// Visit one occurrence entry of the falsified literal f.
-__device__ __forceinline__ void eval_entry(Warp& w, uint32_t f, uint64_t e) {
-  const uint32_t a0 = (uint32_t)e, b0 = (uint32_t)(e >> 32);
-  if (a0 & LONG_CLAUSE) {
-    eval_long(w, a0 & ~LONG_CLAUSE, f);
-    return;
+// Remember the conflict of the first lane that has one (all lanes).
+__device__ __forceinline__ void note_conflict(Warp& w, bool confl, uint32_t c0, uint32_t c1,
+                                              uint32_t c2) {
+  const uint32_t m = __ballot_sync(FULL, confl);
+  if (!m) return;
+  if (w.lane == __ffs(m) - 1) {
+    w.ws->cl[0] = c0;
+    w.ws->cl[1] = c1;
+    w.ws->cl[2] = c2;
   }
-  const uint32_t a = WIDX(w, a0, 2u * w.V, 3);
-  const uint32_t b = b0 == NONE ? NONE : WIDX(w, b0, 2u * w.V, 3);
-  const uint32_t va = lit_value(w.asg, a);
-  if (b == NONE) {  // binary (f | a)
-    if (va == LV_T || va == LV_X) return;
-    if (va == LV_F || !imply(w, a)) record_conflict(w, f, a, NONE);
-    return;
-  }
-  const uint32_t vb = lit_value(w.asg, b);  // ternary (f | a | b)
-  if (va == LV_T || vb == LV_T || va == LV_X || vb == LV_X) return;
-  if (va == LV_F && vb == LV_F) {
-    record_conflict(w, f, a, b);
-  } else if (va == LV_F) {
-    if (!imply(w, b)) record_conflict(w, f, a, b);
-  } else if (vb == LV_F) {
-    if (!imply(w, a)) record_conflict(w, f, a, b);
-  }
+  w.confl = 1;
+  __syncwarp();
 }
 
-// Unit propagation to a fixpoint. Returns true on conflict.
+// Unit propagation to a fixpoint. Returns true on conflict (w.confl, ws->cl).
 // Each round takes the trail literals assigned in the previous round (the
-// frontier) and spreads their occurrence entries over the 32 lanes:
-// visit(f, entry) evaluates one occurrence entry of the falsified literal f;
-// on_round(lo, hi) runs at the start of each round (frontier trail[lo, hi))
-// and after_batch(base, count) after each batch of up to 32 frontier
-// literals (all lanes, both).
-template <class Visit, class Round, class Batch>
-__device__ __forceinline__ bool bcp_rounds(Warp& w, Visit&& visit, Round&& on_round,
-                                           Batch&& after_batch) {
-  for (;;) {
-    __syncwarp();
-    const uint32_t hi = *(volatile uint32_t*)&w.ws->tail;
-    if (w.head >= hi) return false;
-    const uint32_t lo = w.head;
+// frontier) and spreads their occurrence entries over the 32 lanes. A round is
+// one chain of dependent latencies -- literal, list bounds, entry, assignment
+// words, claim -- so the lanes evaluate without branching and claim together:
+// one shared-memory atomic per claimed literal, positions from a ballot.
+__device__ __forceinline__ bool bcp(Warp& w) {
+  while (w.head < w.tail) {
+    const uint32_t lo = w.head, hi = w.tail;
     w.head = hi;
-    on_round(lo, hi);
     WCOUNT(w, props, hi - lo);
     for (uint32_t base = lo; base < hi; base += 32) {
       const uint32_t nlit = min(32u, hi - base);
-      if (nlit == 1) {
-        // one literal: every lane reads the same list bounds (broadcast)
-        const uint32_t f = WIDX(w, w.trail[base] ^ 1u, 2u * w.V, 4);
-        const uint32_t beg = __ldg(&w.occ[f]);
-        const uint32_t cnt = __ldg(&w.occ[f + 1]) - beg;
-        WCOUNT(w, visits, cnt);
-        for (uint32_t e = w.lane; e < cnt; e += 32)
-          visit(f, __ldg(&w.ent[WIDX(w, beg + e, w.ent_end, 5)]));
-      } else {
-        uint32_t f = 0, beg = 0, cnt = 0;
-        if (w.lane < nlit) {
-          f = WIDX(w, w.trail[base + w.lane] ^ 1u, 2u * w.V, 4);  // the literal that became false
-          beg = __ldg(&w.occ[f]);
-          cnt = __ldg(&w.occ[f + 1]) - beg;
-        }
-        uint32_t inc = cnt;
-#pragma unroll
-        for (int d = 1; d < 32; d <<= 1) {
-          uint32_t y = __shfl_up_sync(FULL, inc, d);
-          if (w.lane >= d) inc += y;
-        }
-        const uint32_t excl = inc - cnt;
-        const uint32_t total = __shfl_sync(FULL, inc, 31);
-        WCOUNT(w, visits, total);
-        if (total <= 32) {
-          // owner of entry e = the lane whose segment starts at the last
-          // segment start <= e: segment starts as a bit mask, ranks by popc
-          const bool has = cnt > 0;
-          const uint32_t starts = __reduce_or_sync(FULL, has ? (1u << excl) : 0u);
-          const uint32_t nz = __ballot_sync(FULL, has);
-          const uint32_t e = w.lane;
-          int j = 0;
-          if (e < total) {
-            const int rank = __popc(starts & ((2u << e) - 1u)) - 1;
-            j = __fns(nz, 0, rank + 1);
-          }
-          const uint32_t jbeg = __shfl_sync(FULL, beg, j);
-          const uint32_t jex = __shfl_sync(FULL, excl, j);
-          const uint32_t jf = __shfl_sync(FULL, f, j);
-          if (e < total) visit(jf, __ldg(&w.ent[WIDX(w, jbeg + (e - jex), w.ent_end, 5)]));
-        } else {
-          for (uint32_t e0 = 0; e0 < total; e0 += 32) {
-            const uint32_t e = e0 + w.lane;
-            // owner = smallest lane j with inc_j > e
-            int lo_j = 0, hi_j = 31;
-#pragma unroll
-            for (int s2 = 0; s2 < 5; s2++) {
-              int mid = (lo_j + hi_j) >> 1;
-              uint32_t v = __shfl_sync(FULL, inc, mid);
-              if (v > e) hi_j = mid; else lo_j = mid + 1;
-              if (lo_j > hi_j) lo_j = hi_j;
-            }
-            const int j = lo_j;
-            const uint32_t jbeg = __shfl_sync(FULL, beg, j);
-            const uint32_t jex = __shfl_sync(FULL, excl, j);
-            const uint32_t jf = __shfl_sync(FULL, f, j);
-            if (e < total) visit(jf, __ldg(&w.ent[WIDX(w, jbeg + (e - jex), w.ent_end, 5)]));
-          }
-        }
+      const LaneMap m = lane_map(w.lane, nlit);
+      uint32_t f = 0, beg = 0, cnt = 0;
+      if (m.mine < nlit) {
+        f = WIDX(w, frontier_lit(w, base + m.mine) ^ 1u, 2u * w.V, 4);  // became false
+        beg = __ldg(&w.occ[f]);
+        cnt = __ldg(&w.occ[f + 1]) - beg;
       }
-      after_batch(base, nlit);
-      __syncwarp();
-      if (*(volatile uint32_t*)&w.ws->conflict) return true;
+      spread_lists(m, nlit, f, beg, cnt, [&](uint32_t jf, uint32_t at, bool in) {
+        Found r{false, false, 0, 0, 0, 0};
+        if (in) r = eval_entry(w, jf, __ldg(&w.ent[WIDX(w, at, w.ent_end, 5)]));
+        if (__any_sync(FULL, r.want || r.confl)) {
+          bool won;
+          const bool clash = claim_bits<1>(w, r.want, r.lit, won);
+          push_trail(w, won, r.lit);
+          note_conflict(w, r.confl || clash, r.c0, r.c1, r.c2);
+          __syncwarp();
+        }
+        return w.confl != 0;
+      });
+      const uint32_t total = batch_total(m, cnt);
+      WCOUNT(w, visits, total);
+      if (w.confl) return true;
     }
   }
-}
-
-__device__ bool bcp(Warp& w) {
-  return bcp_rounds(
-      w, [&](uint32_t f, uint64_t e) { eval_entry(w, f, e); }, [](uint32_t, uint32_t) {},
-      [](uint32_t, uint32_t) {});
+  return false;
 }
 
 template <int MODE>
@@ -481,26 +528,25 @@ __device__ void bump(Warp& w) {
     __syncwarp();
   }
   bool big = false;
-  if (w.lane == 0) {
-    if (a & LONG_CLAUSE) {
+  if (a & LONG_CLAUSE) {
+    if (w.lane == 0) {
       const int64_t cl = w.c0 + (a & ~LONG_CLAUSE);
       for (int64_t q = w.cb[cl]; q < w.cb[cl + 1]; q++) {
         uint32_t v = code_of(w.lits[q]) >> 1;
         w.act[v] += w.inc;
         big |= w.act[v] > 1e20f;
       }
-    } else {
-      uint32_t x[3] = {a, b, c};
-      for (int k = 0; k < 3; k++)
-        if (x[k] != NONE) {
-          uint32_t v = x[k] >> 1;
-          w.act[v] += w.inc;
-          big |= w.act[v] > 1e20f;
-        }
+    }
+  } else {  // at most three literals of distinct variables: a lane each
+    const uint32_t x = w.lane == 0 ? a : w.lane == 1 ? b : w.lane == 2 ? c : NONE;
+    if (x != NONE) {
+      const float v = w.act[x >> 1] + w.inc;
+      w.act[x >> 1] = v;
+      big = v > 1e20f;
     }
   }
   w.inc *= (1.0f / 0.95f);
-  big = __shfl_sync(FULL, (int)big, 0) || w.inc > 1e20f;
+  big = __any_sync(FULL, big) || w.inc > 1e20f;
   __syncwarp();
   if (big) {
     for (uint32_t v = w.lane; v < w.V; v += 32) w.act[v] *= 1e-20f;
@@ -538,7 +584,7 @@ __device__ void var_features(const Warp& w, uint32_t v, uint32_t ninputs, Out&& 
       else if (open == 3) c3[pol]++;
     }
   }
-  const float tail = (float)*(volatile uint32_t*)&w.ws->tail;
+  const float tail = (float)w.tail;
   put(0, c2[0] * 0.25f);
   put(1, c3[0] * 0.25f);
   put(2, c2[1] * 0.25f);
@@ -676,19 +722,28 @@ __device__ uint32_t pick_learned(Warp& w) {
 // above the assumptions is left to flip (the subtree is refuted).
 template <int MODE>
 __device__ bool backtrack(Warp& w) {
-  uint32_t nd = w.nd;
-  if (w.lane == 0)
-    while (nd > w.nd_fixed && (w.dstack[nd - 1] & FLIP)) nd--;
-  nd = __shfl_sync(FULL, nd, 0);
-  __syncwarp();
-  if (nd <= w.nd_fixed) return false;
+  // the deepest decision not yet flipped, 32 at a time
+  uint32_t nd = w.nd, pos = 0;
+  for (;; nd -= 32) {
+    if (nd <= w.nd_fixed) return false;
+    const uint32_t at = nd - 1u - (uint32_t)w.lane;
+    const bool in = (uint32_t)w.lane < nd - w.nd_fixed;
+    const uint32_t d = in ? w.dstack[at] : FLIP;
+    const uint32_t open = __ballot_sync(FULL, !(d & FLIP));
+    if (open) {
+      const int j = __ffs(open) - 1;
+      nd -= (uint32_t)j;
+      pos = __shfl_sync(FULL, d, j);
+      break;
+    }
+    if (nd - w.nd_fixed <= 32) return false;
+  }
   if (MODE == MODE_TRACE) {
     // levels nd .. w.nd-1 are popped: their subtrees are complete
     const uint32_t hi_l = min(w.nd, (uint32_t)w.S->trace_depth);
     for (uint32_t l = nd; l < hi_l; l++) trace_close(w, l);
   }
-  const uint32_t pos = w.dstack[nd - 1] & ~FLIP;
-  const uint32_t tail = *(volatile uint32_t*)&w.ws->tail;
+  const uint32_t tail = w.tail;
   const uint32_t d = w.trail[pos];
   WCOUNT(w, undone, tail - pos);
   for (uint32_t t = pos + w.lane; t < tail; t += 32) {
@@ -696,50 +751,58 @@ __device__ bool backtrack(Warp& w) {
     atomicAnd(&w.asg[v >> 4], ~(3u << ((v & 15u) * 2u)));
   }
   __syncwarp();
-  if (w.lane == 0) {
-    w.dstack[nd - 1] |= FLIP;
-    w.ws->tail = pos;
-    w.ws->conflict = 0;
-  }
-  __syncwarp();
+  if (w.lane == 0) w.dstack[nd - 1] = pos | FLIP;
   w.nd = nd;
-  w.head = pos;
-  if (w.lane == 0) imply(w, d ^ 1u);
-  __syncwarp();
+  w.head = w.tail = pos;
+  w.confl = 0;
+  assign_one(w, d ^ 1u);
   return true;
 }
 
-// Highest-activity unassigned variable (ties: lowest id); NONE if all assigned.
-__device__ uint32_t pick(Warp& w) {
+// The best (activity, then lowest id) of the lanes' candidates.
+__device__ __forceinline__ uint32_t best_of_warp(float a, uint32_t v) {
+  // activities are not negative, so their bits order as the numbers do; a
+  // lane without a candidate has a = -1
+  const uint32_t key = v == NONE ? 0u : __float_as_uint(a) + 1u;
+  const uint32_t top = __reduce_max_sync(FULL, key);
+  return __reduce_min_sync(FULL, key == top ? v : NONE);
+}
+
+// Highest-activity unassigned variable (ties: lowest id); NONE if all are
+// assigned. STRIDE: words between the assignment words of 16 variables (2 with
+// clause learning). The activities of four neighbouring variables are one load
+// (a slot's activities begin on a 64-byte boundary), all those of a lane's
+// assignment word are on their way together, and a word without an unassigned
+// variable loads nothing.
+template <int STRIDE>
+__device__ __forceinline__ uint32_t pick_max(const Warp& w) {
   float best_a = -1.0f;
   uint32_t best_v = NONE;
   const uint32_t nwords = (w.V + 15u) >> 4;
   for (uint32_t k = w.lane; k < nwords; k += 32) {
-    const uint32_t word = w.asg[k];
+    const uint32_t word = w.asg[STRIDE * k];
     uint32_t un = ~(word | (word >> 1)) & 0x55555555u;  // 00 pairs
     const uint32_t lim = w.V - 16u * k;
     if (lim < 16u) un &= (1u << (2u * lim)) - 1u;
-    while (un) {
-      const uint32_t bitpos = __ffs(un) - 1;
-      un &= un - 1u;
-      const uint32_t v = 16u * k + (bitpos >> 1);
-      const float a = w.act[v];
-      if (a > best_a || (a == best_a && v < best_v)) {
-        best_a = a;
-        best_v = v;
+    if (!un) continue;
+    const float4* a4 = reinterpret_cast<const float4*>(w.act + 16 * k);
+    float4 a[4];
+#pragma unroll
+    for (uint32_t q = 0; q < 4; q++) a[q] = a4[q];
+#pragma unroll
+    for (uint32_t q = 0; q < 16; q++) {
+      const float x = q % 4 == 0 ? a[q / 4].x : q % 4 == 1 ? a[q / 4].y : q % 4 == 2 ? a[q / 4].z
+                                                                                  : a[q / 4].w;
+      if (((un >> (2 * q)) & 1u) && x > best_a) {  // ids ascend: ties keep the lower one
+        best_a = x;
+        best_v = 16 * k + q;
       }
     }
   }
-  for (int d = 16; d > 0; d >>= 1) {
-    float oa = __shfl_xor_sync(FULL, best_a, d);
-    uint32_t ov = __shfl_xor_sync(FULL, best_v, d);
-    if (oa > best_a || (oa == best_a && ov < best_v)) {
-      best_a = oa;
-      best_v = ov;
-    }
-  }
-  return best_v;
+  return best_of_warp(best_a, best_v);
 }
+
+__device__ uint32_t pick(Warp& w) { return pick_max<1>(w); }
 
 // When the search began. Warps of one launch start at different times, so the
 // first of them sets it (start_clock) and every read goes to memory.
@@ -754,6 +817,14 @@ __device__ __forceinline__ uint64_t search_ns(const Solve& S) {
 
 __device__ __forceinline__ void set_status(const Solve& S, int32_t st) {
   atomicCAS(&S.ctrl->status, 0, st);
+}
+
+// Publish x to other SMs after every write that this thread has made or seen
+// (the warp's, after a __syncwarp). A release store waits for those writes and
+// nothing more; a __threadfence would also empty this SM's L1, which the
+// other 15 or more searching warps of the SM live in.
+__device__ __forceinline__ void store_release(uint32_t* p, uint32_t x) {
+  asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(x) : "memory");
 }
 
 // ---- job ring (bounded MPMC queue, Vyukov) --------------------------------
@@ -799,9 +870,8 @@ __device__ bool ring_push(const Solve& S, const Warp& w, int inst, uint32_t plen
     cell->inc = w.inc;
   }
   extra(slot & (S.ring_cap - 1));
-  __threadfence();
   __syncwarp();
-  if (w.lane == 0) atomicExch(&cell->seq, slot + 1);
+  if (w.lane == 0) store_release(&cell->seq, slot + 1);
   __syncwarp();
   return true;
 }
@@ -812,7 +882,9 @@ __device__ bool ring_push(const Solve& S, const Warp& w, int inst, uint32_t plen
   return ring_push(S, w, inst, plen, prefix_src_trail, dpos, flip_index, [](uint32_t) {});
 }
 
-// Try to take a job; returns slot or NONE.
+// Try to take a job; returns slot or NONE. Only a warp that takes one fences: a
+// fence empties the SM's L1, and idle warps come by every 2 us (fencing on each
+// visit left the busy warps of a mostly idle GPU without an L1).
 __device__ uint32_t ring_pop(const Solve& S, int lane) {
   Ctrl* C = S.ctrl;
   uint32_t slot = NONE;
@@ -823,12 +895,15 @@ __device__ uint32_t ring_pop(const Solve& S, int lane) {
       uint32_t seq = *(volatile uint32_t*)&cell->seq;
       int32_t dif = (int32_t)(seq - (pos + 1));
       if (dif == 0) {
-        if (atomicCAS(&C->q_head, pos, pos + 1) == pos) { slot = pos; break; }
+        if (atomicCAS(&C->q_head, pos, pos + 1) == pos) {
+          slot = pos;
+          __threadfence();  // acquire: the cell's contents after its sequence number
+          break;
+        }
       } else if (dif < 0) {
         break;  // empty
       }
     }
-    __threadfence();  // acquire: the cell's contents after its sequence number
   }
   slot = __shfl_sync(FULL, slot, 0);
   __syncwarp();
@@ -837,10 +912,7 @@ __device__ uint32_t ring_pop(const Solve& S, int lane) {
 
 __device__ void ring_release(const Solve& S, uint32_t slot, int lane) {
   __syncwarp();
-  if (lane == 0) {
-    __threadfence();
-    atomicExch(&S.ring[slot & (S.ring_cap - 1)].seq, slot + S.ring_cap);
-  }
+  if (lane == 0) store_release(&S.ring[slot & (S.ring_cap - 1)].seq, slot + S.ring_cap);
   __syncwarp();
 }
 
@@ -951,35 +1023,26 @@ __device__ int run_job_body(const Solve& S, Warp& w, int unit, int inst, const T
   } else {
     for (uint32_t v = w.lane; v < w.V; v += 32) w.act[v] = 0.0f;
   }
-  if (w.lane == 0) {
-    w.ws->tail = 0;
-    w.ws->conflict = 0;
-  }
+  w.tail = 0;
+  w.confl = 0;
   __syncwarp();
   if (S.flags[inst] & F_EMPTY) return SCUBA_UNSAT;
-  // level 0: unit clauses, then the job's assumptions as fixed decisions
+  // level 0: unit clauses; the job's assumptions follow as fixed decisions, one
+  // after each propagation of the main loop
   const uint32_t nu = S.nunits[inst];
   const uint32_t* un = S.units + w.c0;
-  for (uint32_t k = w.lane; k < nu; k += 32)
-    if (!imply(w, un[k])) record_conflict(w, un[k], NONE, NONE);
-  __syncwarp();
-  if (w.ws->conflict) return SCUBA_UNSAT;
-  if (job) {
-    for (int k = 0; k < job->len; k++) {
-      if (bcp(w)) return SCUBA_UNSAT;
-      const uint32_t l = job->lit[k];
-      const uint32_t val = lit_value(w.asg, l);
-      if (val == LV_F) return SCUBA_UNSAT;
-      if (val == LV_T) continue;
-      if (w.lane == 0) {
-        w.dstack[WIDX(w, w.nd, (uint32_t)w.S->vmax, 6)] = *(volatile uint32_t*)&w.ws->tail | FLIP;
-        imply(w, l);
-      }
-      w.nd++;
-      __syncwarp();
-    }
-    w.nd_fixed = w.nd;
+  for (uint32_t k0 = 0; k0 < nu; k0 += 32) {
+    const uint32_t l = k0 + w.lane < nu ? un[k0 + w.lane] : NONE;
+    bool won;
+    const bool clash = claim_bits<1>(w, l != NONE, l, won);
+    push_trail(w, won, l);
+    __syncwarp();
+    // a unit clause against an earlier one's value, or another lane's
+    const bool bad = l != NONE && !won && lit_value(w.asg, l) != LV_T;
+    if (__any_sync(FULL, clash || bad)) return SCUBA_UNSAT;
   }
+  int next_asm = 0;
+  const int n_asm = job ? job->len : 0;
   uint32_t iter = 0;
   for (;;) {
     if ((++iter & 63u) == 0u) {
@@ -999,12 +1062,25 @@ __device__ int run_job_body(const Solve& S, Warp& w, int unit, int inst, const T
       if (stop == 3) return SCUBA_UNSAT;  // the instance is SAT already; this subtree is moot
     }
     if (bcp(w)) {
+      if (next_asm < n_asm) return SCUBA_UNSAT;  // the assumptions alone
       WCOUNT(w, conflicts, 1);
       bump<MODE>(w);
       if (!backtrack<MODE>(w)) return SCUBA_UNSAT;
       continue;
     }
-    WCOUNT(w, act_reads, w.V - *(volatile uint32_t*)&w.ws->tail);
+    if (next_asm < n_asm) {
+      const uint32_t l = job->lit[next_asm++];
+      const uint32_t val = lit_value(w.asg, l);
+      if (val == LV_F) return SCUBA_UNSAT;
+      if (val == LV_U) {
+        if (w.lane == 0) w.dstack[WIDX(w, w.nd, (uint32_t)w.S->vmax, 6)] = w.tail | FLIP;
+        w.nd++;
+        w.nd_fixed = w.nd;
+        assign_one(w, l);
+      }
+      continue;
+    }
+    WCOUNT(w, act_reads, w.V - w.tail);
     uint32_t v;
     if (MODE == MODE_LEARNED && w.nd < (uint32_t)S.learned_depth) v = pick_learned(w);
     else v = pick(w);
@@ -1063,12 +1139,9 @@ __device__ int run_job_body(const Solve& S, Warp& w, int unit, int inst, const T
     }
     w.decisions++;
     WCOUNT(w, decisions, 1);
-    if (w.lane == 0) {
-      w.dstack[WIDX(w, w.nd, (uint32_t)w.S->vmax, 6)] = *(volatile uint32_t*)&w.ws->tail;
-      imply(w, 2u * v + 1u);  // false first
-    }
+    if (w.lane == 0) w.dstack[WIDX(w, w.nd, (uint32_t)w.S->vmax, 6)] = w.tail;
     w.nd++;
-    __syncwarp();
+    assign_one(w, 2u * v + 1u);  // false first
   }
 }
 
@@ -1106,7 +1179,7 @@ __global__ void __launch_bounds__(256, MODE == MODE_LEARNED ? SCUBA_LEARNED_MINB
                       (size_t)S.vmax * wib
                 : S.trail + slot * S.vmax;
   w.dstack = S.dstack + slot * S.vmax;
-  w.act = S.act + slot * S.vmax;
+  w.act = S.act + slot * act_stride(S.vmax);
   w.cb = S.cb;
   w.lits = S.lits;
   w.lane = lane;
@@ -1124,14 +1197,15 @@ __global__ void __launch_bounds__(256, MODE == MODE_LEARNED ? SCUBA_LEARNED_MINB
         (S.trail_smem ? (size_t)S.vmax * wpb : 0));
     w.xtile = reinterpret_cast<__nv_bfloat16*>(tiles) + (size_t)wib * 32 * learn::NFEAT;
   }
-  uint2* ring = nullptr;
+  unsigned char* area = nullptr;
   if (MODE == MODE_CDCL) {
-    // recent-trail ring and analysis queue after the per-warp assignment (and
-    // trail) areas, 16-byte aligned
+    // the warp's own area after the per-warp assignment (and trail) areas,
+    // 16-byte aligned
     const size_t off = ((sizeof(WarpShared) / 4) * wpb + (size_t)S.assign_words * wpb +
                         (S.trail_smem ? (size_t)S.vmax * wpb : 0)) * 4;
-    ring = reinterpret_cast<uint2*>(reinterpret_cast<unsigned char*>(smem) +
-                                    ((off + 15) & ~(size_t)15) + (size_t)wib * CD_SMEM_WARP);
+    area = reinterpret_cast<unsigned char*>(smem) + ((off + 15) & ~(size_t)15) +
+           (size_t)wib * S.cd_smem_warp;
+    if (S.cd_smem & CD_SMEM_ACT) w.act = cd_area_act(area);
   }
   if (batch_failed(S.ctrl)) return;
   if (lane == 0) start_clock(S.ctrl);
@@ -1170,8 +1244,13 @@ __global__ void __launch_bounds__(256, MODE == MODE_LEARNED ? SCUBA_LEARNED_MINB
       ring_release(S, slot_j, lane);
       job = &taken;
     } else {
+      // look before taking a number: idle warps come by every 2 us, and an
+      // atomic from each of them would hold up the working warps' (and wrap)
       uint32_t k = 0;
-      if (lane == 0) k = atomicAdd(&S.ctrl->next_inst, 1u);
+      if (lane == 0) {
+        k = *(volatile uint32_t*)&S.ctrl->next_inst;
+        if (k < (uint32_t)S.n_units) k = atomicAdd(&S.ctrl->next_inst, 1u);
+      }
       k = __shfl_sync(FULL, k, 0);
       if (k < (uint32_t)S.n_units) {
         unit = S.order ? S.order[k] : (int)k;
@@ -1233,7 +1312,7 @@ __global__ void __launch_bounds__(256, MODE == MODE_LEARNED ? SCUBA_LEARNED_MINB
     } else if (moot) {
       r = SCUBA_UNSAT;  // moot: another subtree already found a model
     } else if constexpr (MODE == MODE_CDCL) {
-      r = run_cdcl(S, w, slot, unit, inst, job, ring, abort_code);
+      r = run_cdcl(S, w, slot, unit, inst, job, area, abort_code);
     } else {
       r = run_job<MODE>(S, w, unit, inst, job, abort_code);
     }
@@ -1307,15 +1386,15 @@ __global__ void __launch_bounds__(256) k_propagate(const __grid_constant__ PropA
     __syncwarp();
     bool confl = (A.flags[i] & F_EMPTY) != 0;
     for (uint32_t k = lane; k < A.nunits[i] && !confl; k += 32)
-      if (!imply(w, A.units[w.c0 + k])) record_conflict(w, 0, NONE, NONE);
+      if (!close_claim(w, A.units[w.c0 + k])) close_conflict(w, 0, NONE, NONE);
     for (int64_t k = A.asm_begin[i] + lane; k < A.asm_begin[i + 1]; k += 32) {
       const int32_t l = A.asm_lits[k];
       if (l == 0 || l > (int32_t)w.V || l < -(int32_t)w.V) continue;
-      if (!imply(w, code_of(l))) record_conflict(w, 0, NONE, NONE);
+      if (!close_claim(w, code_of(l))) close_conflict(w, 0, NONE, NONE);
     }
     __syncwarp();
     confl = confl || w.ws->conflict != 0;
-    if (!confl) confl = bcp(w);
+    if (!confl) confl = close_rounds(w);
     if (lane == 0) A.conflict[i] = confl ? 1 : 0;
     for (uint32_t x = lane; x < w.V; x += 32) {
       const uint32_t bits = (w.asg[x >> 4] >> ((x & 15u) * 2u)) & 3u;
@@ -1576,8 +1655,8 @@ static int solve_impl(const scuba_cnf_batch* b, uint8_t* verdict, uint8_t* model
   int wpb = opt->warps_per_block > 0 ? opt->warps_per_block : 8;
   int bps = opt->blocks_per_sm > 0 ? opt->blocks_per_sm : 5;
   wpb = std::min(wpb, 8);
-  // 2 bits per variable; the clause-learning search keeps 4 (value + fresh)
-  const uint32_t assign_words = mode == dev::MODE_CDCL ? (uint32_t)((vmax + 7) / 8)
+  // 2 bits per variable; the clause-learning search keeps 4 (true, settled)
+  const uint32_t assign_words = mode == dev::MODE_CDCL ? 2u * (uint32_t)((vmax + 15) / 16)
                                                        : (uint32_t)((vmax + 15) / 16);
   const size_t smem_cap = 227 * 1024, sm_cap = 228 * 1024;
   const size_t per_warp_g = sizeof(dev::WarpShared) + (size_t)assign_words * 4;
@@ -1588,7 +1667,18 @@ static int solve_impl(const scuba_cnf_batch* b, uint8_t* verdict, uint8_t* model
   (void)per_warp_s;
   size_t per_warp = trail_smem ? per_warp_s : per_warp_g;
   if (mode == dev::MODE_LEARNED) per_warp += 32 * learn::NFEAT * sizeof(__nv_bfloat16);
-  if (mode == dev::MODE_CDCL) per_warp += dev::CD_SMEM_WARP;
+  int cd_smem = 0;
+  uint32_t cd_smem_warp = 0;
+  if (mode == dev::MODE_CDCL) {
+    // per-variable state in shared memory (9 or 5 bytes a variable) as long as 8
+    // warps still fit an SM
+    for (int what : {dev::CD_SMEM_POS | dev::CD_SMEM_ACT, (int)dev::CD_SMEM_POS, 0}) {
+      cd_smem = what;
+      cd_smem_warp = (uint32_t)dev::cd_area_bytes(what, vmax);
+      if (vmax < 65536 && (per_warp + cd_smem_warp) * 8 + 16 <= smem_cap) break;
+    }
+    per_warp += cd_smem_warp;
+  }
   size_t smem = per_warp * wpb + (mode == dev::MODE_CDCL ? 16 : 0);  // ring alignment
   while (wpb > 1 && smem > smem_cap) {
     wpb--;
@@ -1612,7 +1702,7 @@ static int solve_impl(const scuba_cnf_batch* b, uint8_t* verdict, uint8_t* model
       ensure(S.nunits, 4 * (size_t)n) || ensure(S.flags, 4 * (size_t)n) ||
       ensure(S.pending, 4 * (size_t)n_units) || ensure(S.done, 4 * (size_t)n_units) ||
       ensure(S.inst_dec, 8 * (size_t)n_units) || ensure(S.trail, 4 * (size_t)slots * vmax) ||
-      ensure(S.dstack, 4 * (size_t)slots * vmax) || ensure(S.act, 4 * (size_t)slots * vmax) ||
+      ensure(S.dstack, 4 * (size_t)slots * vmax) || ensure(S.act, 4 * (size_t)(slots * dev::act_stride(vmax))) ||
       ensure(S.ring, sizeof(dev::Job) * (size_t)ring_cap) ||
       ensure(S.job_act, 4 * (size_t)ring_cap * vmax) ||
       ensure(S.prefix, 4 * (size_t)slots * dev::MAX_PREFIX) || ensure(S.ctrl, sizeof(dev::Ctrl))) {
@@ -1717,6 +1807,8 @@ static int solve_impl(const scuba_cnf_batch* b, uint8_t* verdict, uint8_t* model
   sv.lvl_node = nullptr;
   sv.cd_var = P<uint4>(S.cd_var);
   sv.cd_mark = P<uint8_t>(S.cd_mark);
+  sv.cd_smem = cd_smem;
+  sv.cd_smem_warp = cd_smem_warp;
   sv.cd_wl = P<dev::WList>(S.cd_wl);
   sv.cd_pool = P<uint64_t>(S.cd_pool);
   sv.cd_pool_cap = arena_words;
@@ -2000,16 +2092,20 @@ extern "C" int scuba_solve_batch_noalloc(const scuba_cnf_batch* b, uint8_t* verd
     off += (std::max<size_t>(bytes, 16) + 255) & ~(size_t)255;
     return at;
   };
-  // 4 L + 4 occ_total bytes are set aside and not used: the limit on what a
-  // batch may need is part of the interface
+  // 4 L + 4 occ_total bytes are set aside and not used (but for the padding of
+  // the activities): the limit on what a batch may need is part of the interface
   carve(4 * (size_t)L);
   carve(4 * (size_t)occ_total);
+  const size_t act_bytes = 4 * (size_t)(slots * dev::act_stride(vmax));
+  const size_t act_pad = ((act_bytes + 255) & ~(size_t)255) -
+                         ((4 * (size_t)slots * vmax + 255) & ~(size_t)255);
+  off -= std::min(off, act_pad);
   const size_t o_occ_base = carve(8 * (size_t)(n + 1)), o_occ_begin = carve(4 * (size_t)occ_total),
                o_ent = carve(8 * (size_t)L), o_units = carve(4 * (size_t)std::max<int64_t>(C, 1)),
                o_nunits = carve(4 * (size_t)n), o_flags = carve(4 * (size_t)n),
                o_pending = carve(4 * (size_t)n), o_done = carve(4 * (size_t)n),
                o_inst_dec = carve(8 * (size_t)n), o_trail = carve(4 * (size_t)slots * vmax),
-               o_dstack = carve(4 * (size_t)slots * vmax), o_act = carve(4 * (size_t)slots * vmax),
+               o_dstack = carve(4 * (size_t)slots * vmax), o_act = carve(act_bytes),
                o_ring = carve(sizeof(dev::Job) * (size_t)ring_cap),
                o_job_act = carve(4 * (size_t)ring_cap * vmax),
                o_prefix = carve(4 * (size_t)slots * dev::MAX_PREFIX),

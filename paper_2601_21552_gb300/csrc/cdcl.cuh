@@ -62,22 +62,24 @@
 
 constexpr uint32_t LEARNT_REF = 0xC0000000u;  // clause reference: learned clause at offset
 constexpr uint32_t CD_HDR = 4;
-// Shared memory of a clause-learning warp beyond its assignment: the reasons of
-// the RING newest trail positions, the first LSM literals of the clause under
+// Shared memory of a clause-learning warp beyond its assignment: its profile, the
+// literals and reasons of the CD_RING newest trail positions (a power of two), the
+// first LSM literals of the clause under
 // construction and, where they fit (Solve::cd_smem), per variable its
 // activity (CD_SMEM_ACT), its trail position and level packed into 32 bits and
 // its mark (both CD_SMEM_POS; at most 65,535 variables). The analysis walks from
 // variable to variable, so what it reads of each has to be near: with these in
 // global memory a resolution step took about 2,700 cycles.
 enum { CD_SMEM_POS = 1, CD_SMEM_ACT = 2 };
-constexpr uint32_t LSM = 64;
+constexpr uint32_t CD_RING = 64, LSM = 64;
+constexpr size_t CD_FIXED = 8 * 8 + CD_RING * 12 + LSM * 4;
 
 __host__ __device__ __forceinline__ size_t cd_area_bytes(int what, int32_t vmax) {
   const size_t v16 = ((size_t)vmax + 15) & ~(size_t)15;
-  return RING * 8 + LSM * 4 + (what & CD_SMEM_ACT ? 4 * v16 : 0) + (what & CD_SMEM_POS ? 5 * v16 : 0);
+  return CD_FIXED + (what & CD_SMEM_ACT ? 4 * v16 : 0) + (what & CD_SMEM_POS ? 5 * v16 : 0);
 }
 __device__ __forceinline__ float* cd_area_act(unsigned char* area) {
-  return reinterpret_cast<float*>(area + RING * 8 + LSM * 4);
+  return reinterpret_cast<float*>(area + CD_FIXED);
 }
 
 // A variable's mark: bit 0 the saved phase, bits 1-7 the number (1..127, mod
@@ -85,7 +87,7 @@ __device__ __forceinline__ float* cd_area_act(unsigned char* area) {
 constexpr uint32_t MK_PHASE = 1, MK_EPOCHS = 127;
 
 // Profile counters (only when the caller passed a profile array): lane 0
-// adds the clock cycles of each phase to its warp's WarpShared::cyc.
+// adds the clock cycles of each phase to its warp's profile.
 enum { PF_BCP = 0, PF_LEARNED = 1, PF_ANALYZE = 2, PF_DECIDE = 3, PF_DB = 4, PF_NDB = 5,
        PF_NLEARNT = 6 };
 
@@ -94,7 +96,7 @@ __device__ __forceinline__ long long pf_now(const Solve& S) {
 }
 
 __device__ __forceinline__ void pf_add(const Solve& S, Warp& w, int k, long long t0) {
-  if (S.prof && w.lane == 0) w.ws->cyc[k] += (unsigned long long)(clock64() - t0);
+  if (S.prof && w.lane == 0) w.cyc[k] += (unsigned long long)(clock64() - t0);
 }
 
 __device__ __forceinline__ bool is_learnt_ref(uint32_t a) {
@@ -121,8 +123,16 @@ struct CdWarp {
   uint32_t* cl_off;   // [arena_words / 8] arena offset of each learned clause, oldest first
   uint32_t* learnt;   // [V] clause under construction
   uint32_t* pl;       // [V] trail position | level << 16 in shared memory, or NULL
-  uint2* why;         // [RING] shared memory: reason of the literal in the ring's same slot
-  uint32_t* lsm;      // [LSM] shared memory: learnt[0 .. LSM)
+  unsigned char* area; // the warp's shared-memory area:
+  // reason of the literal in the ring's same slot; ring[p mod CD_RING] = trail[p]
+  // as in WarpShared; learnt[0 .. LSM)
+  __device__ __forceinline__ uint2* why() const { return reinterpret_cast<uint2*>(area + 64); }
+  __device__ __forceinline__ uint32_t* ring() const {
+    return reinterpret_cast<uint32_t*>(area + 64 + 8 * CD_RING);
+  }
+  __device__ __forceinline__ uint32_t* lsm() const {
+    return reinterpret_cast<uint32_t*>(area + 64 + 12 * CD_RING);
+  }
   uint32_t arena_words, pool_cap;
   uint32_t top;       // first free arena word
   uint32_t ncl;       // learned clauses in the arena
@@ -133,10 +143,10 @@ struct CdWarp {
 
 // Literal k of the clause under construction.
 __device__ __forceinline__ uint32_t learnt_at(const CdWarp& cd, uint32_t k) {
-  return k < LSM ? cd.lsm[k] : cd.learnt[k];
+  return k < LSM ? cd.lsm()[k] : cd.learnt[k];
 }
 __device__ __forceinline__ void set_learnt(CdWarp& cd, uint32_t k, uint32_t l) {
-  if (k < LSM) cd.lsm[k] = l;
+  if (k < LSM) cd.lsm()[k] = l;
   else cd.learnt[k] = l;
 }
 // Decision level of an assigned variable.
@@ -164,10 +174,10 @@ __device__ __forceinline__ bool claim_cd(Warp& w, CdWarp& cd, bool want, uint32_
                                          uint32_t why_lo, uint32_t why_hi) {
   bool won;
   const bool clash = claim_bits<2>(w, want, l, won);
-  const uint32_t pos = push_trail(w, won, l);
+  const uint32_t pos = push_trail<CD_RING>(w, cd.ring(), won, l);
   if (won) {
     const uint32_t v = l >> 1;
-    cd.why[pos & (RING - 1u)] = make_uint2(why_lo, why_hi);
+    cd.why()[pos & (CD_RING - 1u)] = make_uint2(why_lo, why_hi);
     if (cd.pl) cd.pl[v] = pos | (w.nd << 16);
     *reinterpret_cast<uint4*>(&cd.var[v]) = make_uint4(why_lo, why_hi, pos, w.nd);
   }
@@ -419,7 +429,7 @@ __device__ __forceinline__ bool bcp_cd(Warp& w, CdWarp& cd) {
       const LaneMap m = lane_map(w.lane, nlit);
       uint32_t f = 0, beg = 0, cnt = 0, lbeg = 0, lcnt = 0;
       if (m.mine < nlit) {
-        const uint32_t t = WIDX(w, frontier_lit(w, base + m.mine), 2u * w.V, 14);
+        const uint32_t t = WIDX(w, frontier_lit<CD_RING>(w, cd.ring(), base + m.mine), 2u * w.V, 14);
         f = t ^ 1u;
         beg = __ldg(&w.occ[f]);
         cnt = __ldg(&w.occ[f + 1]) - beg;
@@ -549,8 +559,8 @@ __device__ __forceinline__ uint32_t analyze_cd(Warp& w, CdWarp& cd, uint32_t& bl
           if (cd.pl) {
             // the slot of a literal's position holds its reason as long as the
             // ring still names that literal there
-            why = cd.why[pos & (RING - 1u)];
-            if (w.tail - pos > RING || w.ws->ring[pos & (RING - 1u)] != mylit)
+            why = cd.why()[pos & (CD_RING - 1u)];
+            if (w.tail - pos > CD_RING || cd.ring()[pos & (CD_RING - 1u)] != mylit)
               why = *reinterpret_cast<const uint2*>(&cd.var[v].reason_lo);
           }
           my0 = why.x;
@@ -673,12 +683,12 @@ __device__ __forceinline__ uint32_t add_learnt(Warp& w, CdWarp& cd, uint32_t n, 
   }
   if (w.lane == 0) {
     cd.cl_off[cd.ncl] = c;
-    if (w.S->prof) w.ws->cyc[PF_NLEARNT]++;
+    if (w.S->prof) w.cyc[PF_NLEARNT]++;
   }
   __syncwarp();
   cd.top = c + clause_words(n);
   cd.ncl++;
-  const uint32_t l0 = cd.lsm[0], l1 = cd.lsm[1];
+  const uint32_t l0 = cd.lsm()[0], l1 = cd.lsm()[1];
   append_watches(w, cd, w.lane < 2, w.lane == 0 ? l0 : l1,
                  (uint64_t)c | ((uint64_t)(w.lane == 0 ? l1 : l0) << 32));
   return c;
@@ -800,16 +810,16 @@ __device__ bool rebuild_watches(Warp& w, CdWarp& cd) {
 // entry, over the rebuilt watch lists too.
 __device__ __noinline__ void maintain_db(Warp& w, CdWarp& cd, bool drop_half) {
   const long long t0 = pf_now(*w.S);
-  if (w.S->prof && w.lane == 0) w.ws->cyc[PF_NDB]++;
+  if (w.S->prof && w.lane == 0) w.cyc[PF_NDB]++;
   backjump_cd(w, cd, w.nd_fixed);
   if (!reduce_db(w, cd, drop_half) && (drop_half || !reduce_db(w, cd, true)))
     clear_learnts(w, cd);
   w.confl = 0;
   // the head moves back: the ring has to hold the last positions below the tail
   // again (undone claims may have overwritten them)
-  for (uint32_t k = w.lane; k < min(w.tail, RING); k += 32) {
+  for (uint32_t k = w.lane; k < min(w.tail, CD_RING); k += 32) {
     const uint32_t p = w.tail - 1u - k;
-    w.ws->ring[p & (RING - 1u)] = w.trail[p];
+    cd.ring()[p & (CD_RING - 1u)] = w.trail[p];
   }
   __syncwarp();
   w.head = 0;
@@ -954,7 +964,7 @@ __device__ void share_publish(const Solve& S, Warp& w, CdWarp& cd, uint32_t n, u
     if (w.lane == 1) x = (uint32_t)w.inst;
     else if (w.lane == 2) x = n | (min(lbd, 255u) << 8);
     else if (w.lane == 3) x = (uint32_t)slot;
-    else x = (uint32_t)(w.lane - 4) < n ? cd.lsm[w.lane - 4] : NONE;
+    else x = (uint32_t)(w.lane - 4) < n ? cd.lsm()[w.lane - 4] : NONE;
     *(volatile uint32_t*)&rec[w.lane] = x;
   }
   __syncwarp();
@@ -1044,7 +1054,7 @@ __device__ __noinline__ bool share_import(const Solve& S, Warp& w, CdWarp& cd, i
         if (w.lane == w0) at = 0;
         else if (w.lane == w1) at = 1;
         else at = 2u + __popc(rest & ((1u << w.lane) - 1u));
-        cd.lsm[at] = my;
+        cd.lsm()[at] = my;
       }
       __syncwarp();
       const uint32_t c = add_learnt(w, cd, nj, lbdj);
@@ -1062,8 +1072,7 @@ __device__ __noinline__ bool share_import(const Solve& S, Warp& w, CdWarp& cd, i
 __device__ int run_cdcl(const Solve& S, Warp& w, int64_t slot, int unit, int inst,
                         const TakenJob* job, unsigned char* area, int& abort_code) {
   CdWarp cd;
-  cd.why = reinterpret_cast<uint2*>(area);
-  cd.lsm = reinterpret_cast<uint32_t*>(area + RING * 8);
+  cd.area = area;
   cd.epoch = 0;
   cd.var = reinterpret_cast<VarInfo*>(S.cd_var) + slot * S.vmax;
   cd.pl = nullptr;
@@ -1105,7 +1114,9 @@ __device__ int run_cdcl(const Solve& S, Warp& w, int64_t slot, int unit, int ins
   w.tail = 0;
   w.confl = 0;
   // Calls of the rarely used parts work on copies of w and cd, so that the
-  // search itself can keep them in registers.
+  // search itself can keep them in registers. (All of them come back, also the
+  // pointers, which do not change: a compiler that knows that computes them from
+  // the launch's arguments each time, which measured 4 % slower.)
   auto apart = [&](auto&& fn) {
     Warp w2 = w;
     CdWarp cd2 = cd;
@@ -1199,7 +1210,7 @@ __device__ int run_cdcl(const Solve& S, Warp& w, int64_t slot, int unit, int ins
         backjump_cd(w, cd, target);
       }
       uint32_t why = NONE;
-      const uint32_t uip = cd.lsm[0];
+      const uint32_t uip = cd.lsm()[0];
       if (n >= 2) {
         uint32_t c = add_learnt(w, cd, n, lbd);
         if (cd.full)  // the pool ran out: compact it, the new clause included

@@ -1,8 +1,14 @@
 // closure.cuh -- unit propagation of scuba_propagate_batch (included by solver.cu
-// inside namespace scuba::dev). A closure's rounds are wide (a whole input word
-// is assumed at once, frontiers of hundreds of literals), so the lanes take the
-// entries of up to 32 literals as one list, 32 at a time; the searches, whose
-// rounds are a few literals, use bcp() and bcp_cd() instead.
+// inside namespace scuba::dev). A closure's rounds are wide (whole input words
+// are assumed at once, frontiers of hundreds of literals), unlike the searches'.
+// One warp takes a batch of 32 frontier literals' entries as one list
+// (close_rounds); where instances are few and large a block's warps share one:
+// eight lanes take a literal's list, every lane claims what its entry implies by
+// itself, and a round ends at a barrier (close_shared). The closure does not
+// depend on the order of that.
+// What a conflict leaves in the assignment does, so an instance that
+// conflicts is done again by one warp in a fixed order (close_rounds): its
+// values are the same in every run, as they always were.
 
 __device__ __forceinline__ void close_conflict(Warp& w, uint32_t a, uint32_t b, uint32_t c) {
   if (atomicCAS(&w.ws->conflict, 0u, 1u) == 0u) {
@@ -77,7 +83,7 @@ __device__ __forceinline__ void close_entry(Warp& w, uint32_t f, uint64_t e) {
   }
 }
 
-// Unit propagation to a fixpoint. Returns true on conflict.
+// Unit propagation to a fixpoint by one warp. Returns true on conflict.
 // Each round takes the trail literals assigned in the previous round (the
 // frontier) and spreads their occurrence entries over the 32 lanes:
 // The values of a conflicting instance are what this order of visits leaves.
@@ -151,5 +157,47 @@ __device__ bool close_rounds(Warp& w) {
       __syncwarp();
       if (*(volatile uint32_t*)&w.ws->conflict) return true;
     }
+  }
+}
+
+// Unit propagation to a fixpoint by the whole block. Returns true on conflict.
+// The next literal's list bounds are loaded before this one's entries are
+// evaluated, and its first entries before those of this one's are used up.
+__device__ __forceinline__ bool close_shared(Warp& w) {
+  const uint32_t groups = blockDim.x >> 3, sub = threadIdx.x & 7u;
+  uint32_t lo = 0;
+  for (;;) {
+    __syncthreads();
+    const uint32_t hi = *(volatile uint32_t*)&w.ws->tail;
+    const uint32_t bad = *(volatile uint32_t*)&w.ws->conflict;
+    __syncthreads();  // everyone has read the tail before it moves again
+    if (bad) return true;
+    if (lo >= hi) return false;
+    uint32_t p = lo + (threadIdx.x >> 3);
+    uint32_t f = 0, beg = 0, end = 0;
+    if (p < hi) {
+      f = WIDX(w, w.trail[p] ^ 1u, 2u * w.V, 4);
+      beg = __ldg(&w.occ[f]);
+      end = __ldg(&w.occ[f + 1]);
+    }
+    while (p < hi) {
+      uint32_t k = beg + sub;
+      uint64_t e = 0;
+      if (k < end) e = __ldg(&w.ent[WIDX(w, k, w.ent_end, 5)]);
+      const uint32_t f0 = f, end0 = end;
+      p += groups;
+      if (p < hi) {
+        f = WIDX(w, w.trail[p] ^ 1u, 2u * w.V, 4);
+        beg = __ldg(&w.occ[f]);
+        end = __ldg(&w.occ[f + 1]);
+      }
+      while (k < end0) {
+        const uint64_t e0 = e;
+        k += 8;
+        if (k < end0) e = __ldg(&w.ent[WIDX(w, k, w.ent_end, 5)]);
+        close_entry(w, f0, e0);
+      }
+    }
+    lo = hi;
   }
 }

@@ -12,11 +12,12 @@
 // the occurrences in shared memory; a scan over (literal, warp) turns the
 // counts into list offsets and per-warp cursors; pass 2 reads the clauses again
 // (from L2: an instance is a few 100 KB) and writes each entry where its warp's
-// cursor stands. A list is therefore in the order of the clauses' groups of 32,
-// the same in every run, and no count, cursor or normalised literal goes
-// through global memory. The ranges of one large instance need nothing from
-// each other: a block also counts the literals below its range, which is where
-// its first list begins.
+// cursor stands. A list is therefore in the order of the clauses' groups of 32
+// (within a group: first literals, then second, then third, each in the order
+// in which the SM serves a warp's shared-memory atomics), and no count, cursor
+// or normalised literal goes through global memory. The ranges of one large
+// instance need nothing from each other: a block also counts the literals below
+// its range, which is where its first list begins.
 
 // Header checks, scratch layout and launch shape of one call's preparation.
 struct Prep {
@@ -37,7 +38,7 @@ struct Prep {
   uint64_t* ent;       // [L]
   uint32_t* units;     // [C]
   uint32_t* nunits;    // [n]
-  uint32_t* flags;     // [n]
+  uint32_t* flags;     // [n] F_EMPTY, F_BAD
   int2* items;         // {instance, range} of each work item; NULL: item i is instance i
   uint32_t item_cap;
 };
@@ -173,44 +174,58 @@ __global__ void __launch_bounds__(1024) k_setup(Prep P, SearchInit I) {
   }
 }
 
-// One clause as a lane sees it: its literal range in the caller's CSR and, up
-// to length 3, its literals.
+// The clauses of one instance: literal slots [base, end) of the CSR.
+struct Slots {
+  int64_t base, end;
+};
+
+// One clause as a lane sees it: its first literal slot (from the instance's),
+// its length (0 past the last clause too) and, up to length 3, its literals.
 struct RawClause {
-  int64_t b, e;
+  uint32_t at, len;
+  bool bad;
   int32_t l[3];
 };
 
-__device__ __forceinline__ RawClause load_bounds(const Prep& P, int64_t c, int64_t c1) {
+__device__ __forceinline__ RawClause load_bounds(const Prep& P, const Slots& S, int64_t c,
+                                                 int64_t c1) {
   RawClause R;
-  R.b = R.e = 0;
+  R.at = R.len = 0;
+  R.bad = false;
   if (c < c1) {
-    R.b = __ldg(P.cb + c);
-    R.e = __ldg(P.cb + c + 1);
+    const int64_t b = __ldg(P.cb + c), e = __ldg(P.cb + c + 1);
+    R.bad = b < S.base || e < b || e > S.end;
+    if (!R.bad) {
+      R.at = (uint32_t)(b - S.base);
+      R.len = (uint32_t)(e - b);
+    }
   }
   return R;
 }
 
-__device__ __forceinline__ void load_literals(const Prep& P, RawClause& R) {
-  const int64_t len = R.b >= 0 && R.e <= P.L ? R.e - R.b : 0;
+__device__ __forceinline__ void load_literals(const int32_t* lits, RawClause& R) {
 #pragma unroll
-  for (int k = 0; k < 3; k++) R.l[k] = k < len ? __ldg(P.lits + R.b + k) : 0;
+  for (int k = 0; k < 3; k++) R.l[k] = k < R.len ? __ldg(lits + R.at + k) : 0;
 }
 
 // The warp's clauses [s0, s1) in groups of 32, fn(group start, lane's clause):
-// the literals of the next group and the bounds of the one after it are on
-// their way while a group is handled.
+// the literals of the next two groups and the bounds of the one after them are
+// on their way while a group is handled. lits: the instance's first literal.
 template <class Fn>
-__device__ __forceinline__ void each_group(const Prep& P, int64_t s0, int64_t s1, int lane,
-                                           Fn&& fn) {
-  RawClause R = load_bounds(P, s0 + lane, s1);
-  RawClause N = load_bounds(P, s0 + 32 + lane, s1);
-  load_literals(P, R);
+__device__ __forceinline__ void each_group(const Prep& P, const Slots& S, const int32_t* lits,
+                                           int64_t s0, int64_t s1, int lane, Fn&& fn) {
+  RawClause R = load_bounds(P, S, s0 + lane, s1);
+  RawClause N = load_bounds(P, S, s0 + 32 + lane, s1);
+  RawClause M = load_bounds(P, S, s0 + 64 + lane, s1);
+  load_literals(lits, R);
+  load_literals(lits, N);
   for (int64_t cs = s0; cs < s1; cs += 32) {
-    load_literals(P, N);
-    const RawClause M = load_bounds(P, cs + 64 + lane, s1);
+    load_literals(lits, M);
+    const RawClause Q = load_bounds(P, S, cs + 96 + lane, s1);
     fn(cs, R);
     R = N;
     N = M;
+    M = Q;
   }
 }
 
@@ -218,63 +233,31 @@ enum { CL_NONE, CL_SHORT, CL_UNIT, CL_LONG };
 
 // Normalise a clause: CL_SHORT with its 2 or 3 distinct codes in u, CL_UNIT
 // with u[0], CL_LONG (its codes are read from the CSR as they stand), CL_NONE
-// (no clause, a tautology, or one that raised F_EMPTY / F_BAD in f).
-__device__ __forceinline__ int classify(const Prep& P, const RawClause& R, bool valid, int V,
-                                        uint32_t u[3], int& nk, uint32_t& f) {
-  nk = 0;
-  if (!valid) return CL_NONE;
-  if (R.b < 0 || R.e < R.b || R.e > P.L) {
-    f |= F_BAD;
-    return CL_NONE;
-  }
-  const int64_t len = R.e - R.b;
-  if (len == 0) {
-    f |= F_EMPTY;
-    return CL_NONE;
-  }
-  if (len > 3) return CL_LONG;
-  bool bad = false, taut = false;
-#pragma unroll
-  for (int q = 0; q < 3; q++) {
-    if (q >= len) break;
-    const int32_t l = R.l[q];
-    bad |= l == 0 || l > V || l < -V;
-    const uint32_t x = code_of(l);
-    bool dup = false;
-#pragma unroll
-    for (int r = 0; r < 2; r++)
-      if (r < nk) {
-        dup |= u[r] == x;
-        taut |= u[r] == (x ^ 1u);
-      }
-    if (!dup) {
-      if (nk == 0) u[0] = x;
-      else if (nk == 1) u[1] = x;
-      else u[2] = x;
-      nk++;
-    }
-  }
-  if (bad) {
-    f |= F_BAD;
-    nk = 0;
-    return CL_NONE;
-  }
-  if (taut) {
-    nk = 0;
-    return CL_NONE;
-  }
-  if (nk == 1) {
-    nk = 0;
-    return CL_UNIT;
-  }
-  return CL_SHORT;
+// (no clause, an empty one, or a tautology).
+__device__ __forceinline__ int classify(const RawClause& R, uint32_t u[3], int& nk) {
+  const uint32_t x0 = code_of(R.l[0]), x1 = code_of(R.l[1]), x2 = code_of(R.l[2]);
+  const bool h1 = R.len > 1, h2 = R.len > 2;
+  const bool d1 = h1 && x1 == x0;               // a literal said before
+  const bool d2 = h2 && (x2 == x0 || x2 == x1);
+  const bool taut = (h1 && x1 == (x0 ^ 1u)) || (h2 && (x2 == (x0 ^ 1u) || x2 == (x1 ^ 1u)));
+  nk = (int)h1 - (int)d1 + (int)h2 - (int)d2 + 1;
+  u[0] = x0;
+  u[1] = h1 && !d1 ? x1 : x2;
+  u[2] = x2;
+  if (R.len > 3) return CL_LONG;
+  return R.len == 0 || taut ? CL_NONE : nk == 1 ? CL_UNIT : CL_SHORT;
 }
+
+// A literal of 0, or of a variable the instance does not have.
+__device__ __forceinline__ bool bad_literal(int32_t l, int V) { return l == 0 || l > V || l < -V; }
 
 // WARPS = 8 for batches whose literals fit one item (several blocks per SM),
 // 32 for larger ones (one block per SM; a large instance is cut into ranges).
-// Per item the clauses are read twice; the passes are bound by the latency of
-// their loads and shared-memory updates, which the loads issued ahead of their
-// group and the other warps cover.
+// Per item the clauses are read twice; the passes are bound by instruction
+// issue and by the latency of their loads and shared-memory updates, which the
+// loads issued ahead of their group and the other warps cover. (Ranks within a
+// group by __match_any_sync, about 380 cycles when all lanes differ, cost more
+// than the rest of pass 2.)
 template <int WARPS>
 __global__ void __launch_bounds__(32 * WARPS) k_prep(const __grid_constant__ Prep P) {
   extern __shared__ uint32_t smem[];
@@ -302,14 +285,16 @@ __global__ void __launch_bounds__(32 * WARPS) k_prep(const __grid_constant__ Pre
       continue;
     }
     const int32_t nv = P.nv[i], V = clamp_nv(nv, P.vmax);
-    const int64_t lbase = c0 < c1 ? P.cb[c0] : 0;
+    Slots slots{0, 0};
+    if (c0 < c1) slots = Slots{P.cb[c0], P.cb[c1]};
     const int64_t vb = P.vb[i];
     // occurrence offsets are 32-bit within an instance; the model must fit
-    if (nv != V || (c0 < c1 && P.cb[c1] - lbase >= (1LL << 32)) || vb < 0 ||
-        vb + (int64_t)V > P.total_vars) {
+    if (nv != V || slots.base < 0 || slots.end < slots.base || slots.end > P.L ||
+        slots.end - slots.base >= (1LL << 32) || vb < 0 || vb + (int64_t)V > P.total_vars) {
       if (first_range && threadIdx.x == 0) P.flags[i] = F_BAD;
       continue;
     }
+    const int32_t* const lits = P.lits + slots.base;
     const uint32_t lo = (uint32_t)item.y * P.range;
     const uint32_t hi = min(lo + P.range, 2u * (uint32_t)V);
     const uint32_t nl = hi - lo, nl2 = (nl + 1u) >> 1;
@@ -325,28 +310,34 @@ __global__ void __launch_bounds__(32 * WARPS) k_prep(const __grid_constant__ Pre
     uint32_t f = 0, below = 0, units = 0, wide = 0;
     auto count = [&](uint32_t x) {
       below += x < lo;
-      if (x >= lo && x < hi) {
-        const uint32_t sh = ((x - lo) & 1u) * 16u;
-        const uint32_t old = atomicAdd(&my_packed[(x - lo) >> 1], 1u << sh);
+      const uint32_t r = x - lo;
+      if (r < nl) {
+        const uint32_t sh = (r & 1u) * 16u;
+        const uint32_t old = atomicAdd(&my_packed[r >> 1], 1u << sh);
         wide |= ((old >> sh) & 0xffffu) == 0xffffu;
       }
     };
-    each_group(P, s0, s1, lane, [&](int64_t cs, const RawClause& R) {
+    each_group(P, slots, lits, s0, s1, lane, [&](int64_t cs, const RawClause& R) {
       uint32_t u[3];
       int nk;
-      const int kind = classify(P, R, cs + lane < s1, V, u, nk, f);
-      if (kind == CL_SHORT) {
+      const int kind = classify(R, u, nk);
+      bool bad = R.bad;
+#pragma unroll
+      for (int k = 0; k < 3; k++) bad |= k < R.len && R.len <= 3 && bad_literal(R.l[k], V);
+      if (bad) {
+        f |= F_BAD;
+      } else if (kind == CL_SHORT) {
         count(u[0]);
         count(u[1]);
         if (nk == 3) count(u[2]);
       } else if (kind == CL_LONG) {
-        bool bad = false;
-        for (int64_t q = R.b; q < R.e; q++) {
-          const int32_t l = __ldg(P.lits + q);
-          if (l == 0 || l > V || l < -V) bad = true;
+        for (uint32_t q = 0; q < R.len; q++) {
+          const int32_t l = __ldg(lits + R.at + q);
+          if (bad_literal(l, V)) f |= F_BAD;
           else count(code_of(l));
         }
-        if (bad) f |= F_BAD;
+      } else if (kind == CL_NONE && R.len == 0 && cs + lane < s1) {
+        f |= F_EMPTY;
       }
       units += __popc(__ballot_sync(FULL, kind == CL_UNIT));
     });
@@ -363,10 +354,15 @@ __global__ void __launch_bounds__(32 * WARPS) k_prep(const __grid_constant__ Pre
     f = s_flags;
     if (first_range && threadIdx.x == 0) P.flags[i] = f;
     if (f & F_BAD) continue;
-    // ---- scan: list begins, and each warp's cursor within each list ----
+    // ---- scan: where the lists begin, and each warp's cursor within each list ----
     uint32_t* const occ = P.occ_begin + P.occ_base[i];
+    auto head = [&](uint32_t r, uint32_t at) {  // literal lo + r's list begins at `at`
+      begin[r] = at;
+      occ[lo + r] = at;
+    };
     uint32_t run = s_below;
-    for (uint32_t k0 = 0; k0 < nl2; k0 += 32 * WARPS) {
+    const bool recount = s_wide != 0;  // a 16-bit count ran over: the counts are void
+    for (uint32_t k0 = 0; k0 < nl2 && !recount; k0 += 32 * WARPS) {
       const uint32_t k = k0 + threadIdx.x;
       uint32_t a = 0, b = 0;  // occurrences of codes lo + 2k, lo + 2k + 1
       if (k < nl2) {
@@ -382,45 +378,42 @@ __global__ void __launch_bounds__(32 * WARPS) k_prep(const __grid_constant__ Pre
       uint32_t total;
       const uint32_t at = run + block_exclusive(a + b, part, total);
       run += total;
-      if (k < nl2) {
-        begin[2 * k] = at;
-        occ[lo + 2 * k] = at;
-        if (2 * k + 1 < nl) {
-          begin[2 * k + 1] = at + a;
-          occ[lo + 2 * k + 1] = at + a;
-        }
+      if (k < nl2) {  // nl is even
+        head(2 * k, at);
+        head(2 * k + 1, at + a);
       }
     }
     __syncthreads();
     if (s_wide) {
       // more than 65,535 occurrences of a literal: 32-bit counts for the whole
       // block, and one warp fills the lists
-      for (uint32_t k = threadIdx.x; k < nl; k += 32 * WARPS) begin[k] = 0u;
+      uint32_t* const cnt32 = packed;  // [nl]: WARPS * nl2 words or more
+      for (uint32_t k = threadIdx.x; k < nl; k += 32 * WARPS) cnt32[k] = 0u;
       __syncthreads();
       for (int64_t c = c0 + threadIdx.x; c < c1; c += 32 * WARPS) {
-        RawClause Q = load_bounds(P, c, c1);
-        load_literals(P, Q);
-        uint32_t u[3], g = 0;
+        RawClause Q = load_bounds(P, slots, c, c1);
+        load_literals(lits, Q);
+        uint32_t u[3];
         int nk;
-        const int kind = classify(P, Q, true, V, u, nk, g);
-        const int64_t len = kind == CL_LONG ? Q.e - Q.b : nk;
-        for (int64_t q = 0; q < len; q++) {
-          const uint32_t x = kind == CL_LONG ? code_of(__ldg(P.lits + Q.b + q))
+        const int kind = classify(Q, u, nk);
+        const uint32_t len = kind == CL_LONG ? Q.len : kind == CL_SHORT ? (uint32_t)nk : 0u;
+        for (uint32_t q = 0; q < len; q++) {
+          const uint32_t x = kind == CL_LONG ? code_of(__ldg(lits + Q.at + q))
                                              : (q == 0 ? u[0] : q == 1 ? u[1] : u[2]);
-          if (x >= lo && x < hi) atomicAdd(&begin[x - lo], 1u);
+          if (x - lo < nl) atomicAdd(&cnt32[x - lo], 1u);
         }
       }
       __syncthreads();
       run = s_below;
       for (uint32_t k0 = 0; k0 < nl; k0 += 32 * WARPS) {
         const uint32_t k = k0 + threadIdx.x;
-        const uint32_t a = k < nl ? begin[k] : 0u;
+        const uint32_t a = k < nl ? cnt32[k] : 0u;
         uint32_t total;
         const uint32_t at = run + block_exclusive(a, part, total);
         run += total;
         if (k < nl) {
-          begin[k] = at;
-          occ[lo + k] = at;
+          head(k, at);
+          cnt32[k] = 0u;  // from here on the list's cursor
         }
       }
       __syncthreads();
@@ -438,52 +431,41 @@ __global__ void __launch_bounds__(32 * WARPS) k_prep(const __grid_constant__ Pre
     }
     if (one_warp && wib != 0) continue;
     // ---- pass 2: entries and unit literals ----
-    uint16_t* const cur = reinterpret_cast<uint16_t*>(my_packed);
-    uint64_t* const ent = P.ent + lbase;
+    uint64_t* const ent = P.ent + slots.base;
     const int64_t e1 = one_warp ? c1 : s1;
-    each_group(P, s0, e1, lane, [&](int64_t cs, const RawClause& R) {
-      uint32_t u[3], g = 0;
+    each_group(P, slots, lits, s0, e1, lane, [&](int64_t cs, const RawClause& R) {
+      uint32_t u[3];
       int nk;
-      const int kind = classify(P, R, cs + lane < e1, V, u, nk, g);
+      const int kind = classify(R, u, nk);
       if (first_range) {
         const uint32_t ub = __ballot_sync(FULL, kind == CL_UNIT);
         if (kind == CL_UNIT) P.units[c0 + nunit + __popc(ub & below_me)] = u[0];
         nunit += __popc(ub);
       }
-      // literal k of every clause of the group at once
-      auto place = [&](bool has, uint32_t x, uint64_t entry) {
-        has = has && x >= lo && x < hi;
-        if (!__any_sync(FULL, has)) return;
-        const uint32_t grp = __match_any_sync(FULL, has ? x : (0x80000000u | (uint32_t)lane));
-        const int leader = __ffs(grp) - 1;
-        uint32_t at = 0;
-        if (has && lane == leader) {
-          if (one_warp) {
-            at = begin[x - lo];
-            begin[x - lo] = at + __popc(grp);
-          } else {
-            const uint32_t used = cur[x - lo];
-            at = begin[x - lo] + used;
-            cur[x - lo] = (uint16_t)(used + __popc(grp));
-          }
+      // literal x of the lane's clause: its entry {a, b} at the list's next place
+      auto place = [&](bool has, uint32_t x, uint32_t a, uint32_t b) {
+        const uint32_t r = x - lo;
+        if (!has || r >= nl) return;
+        uint32_t p;
+        if (one_warp) {
+          p = atomicAdd(&packed[r], 1u);
+        } else {
+          const uint32_t sh = (r & 1u) * 16u;
+          p = (atomicAdd(&my_packed[r >> 1], 1u << sh) >> sh) & 0xffffu;
         }
-        at = __shfl_sync(FULL, at, leader);
-        if (has) ent[at + __popc(grp & below_me)] = entry;
-        __syncwarp();
+        ent[begin[r] + p] = (uint64_t)a | ((uint64_t)b << 32);
       };
       const bool sh = kind == CL_SHORT;
       const uint32_t third = nk == 3 ? u[2] : NONE;
-      place(sh, u[0], (uint64_t)u[1] | ((uint64_t)third << 32));
-      place(sh, u[1], (uint64_t)u[0] | ((uint64_t)third << 32));
-      place(sh && nk == 3, u[2], (uint64_t)u[0] | ((uint64_t)u[1] << 32));
+      place(sh, u[0], u[1], third);
+      place(sh, u[1], u[0], third);
+      place(sh && nk == 3, u[2], u[0], u[1]);
       if (__any_sync(FULL, kind == CL_LONG)) {
-        const uint32_t len = kind == CL_LONG ? (uint32_t)(R.e - R.b) : 0u;
+        const uint32_t len = kind == CL_LONG ? R.len : 0u;
         const uint32_t rounds = __reduce_max_sync(FULL, len);
-        const uint64_t entry = (uint64_t)(LONG_CLAUSE | (uint32_t)(cs + lane - c0));
-        for (uint32_t k = 0; k < rounds; k++) {
-          const bool has = k < len;
-          place(has, has ? code_of(__ldg(P.lits + R.b + k)) : 0u, entry);
-        }
+        for (uint32_t k = 0; k < rounds; k++)
+          place(k < len, k < len ? code_of(__ldg(lits + R.at + k)) : 0u,
+                LONG_CLAUSE | (uint32_t)(cs + lane - c0), 0u);
       }
     });
   }

@@ -231,8 +231,9 @@ struct Solve {
   uint32_t share_lbd;          // publish learned clauses of LBD <= this; 0: off
 };
 
-// Recent trail literals a warp keeps in shared memory (a power of two).
-constexpr uint32_t RING = 64;
+// Recent trail literals a warp keeps in shared memory (a power of two; the
+// clause-learning search keeps more, with their reasons: cdcl.cuh).
+constexpr uint32_t RING = 16;
 
 struct alignas(16) WarpShared {
   uint32_t tail, conflict;  // closures only: the searches keep theirs in registers
@@ -240,13 +241,14 @@ struct alignas(16) WarpShared {
   uint32_t pad[3];
   // ring[p mod RING] = trail[p] for the positions p in [head, tail) that are
   // at most RING below the tail: a propagation round reads its literals here
-  // instead of waiting for the global trail
+  // instead of waiting for the global trail (DPLL)
   uint32_t ring[RING];
   // per-job work counters (lane 0 updates them; kept out of registers)
   unsigned long long decisions, conflicts, props, visits, act_reads, undone;
-  // clause-learning profile (cycles of lane 0 per phase; counts)
-  unsigned long long cyc[8];
 };
+// The largest instance that fits an SM's shared memory beside this struct is part
+// of the interface.
+static_assert(sizeof(WarpShared) == 144, "per-warp shared memory");
 
 enum : uint32_t { LV_U = 0, LV_T = 1, LV_F = 2, LV_X = 3 };
 
@@ -266,6 +268,7 @@ struct Warp {
   uint32_t* trail;
   uint32_t* dstack;
   float* act;
+  unsigned long long* cyc; // clause learning: profile (cycles of lane 0 per phase; counts)
   int lane;
   int inst;
   uint32_t V;
@@ -311,19 +314,21 @@ __device__ __forceinline__ void warp_checks(Warp& w, Ctrl* c) {
 
 #include "closure.cuh"
 
-// Trail literal p of the current frontier.
-__device__ __forceinline__ uint32_t frontier_lit(const Warp& w, uint32_t p) {
-  return w.tail - p <= RING ? w.ws->ring[p & (RING - 1u)] : w.trail[p];
+// Trail literal p of the current frontier, from a ring of SIZE.
+template <uint32_t SIZE>
+__device__ __forceinline__ uint32_t frontier_lit(const Warp& w, const uint32_t* ring, uint32_t p) {
+  return w.tail - p <= SIZE ? ring[p & (SIZE - 1u)] : w.trail[p];
 }
 
 // Append the literals of the lanes with won set to the trail (all lanes): in
 // lane order, so no counter in memory is involved. Returns the lane's position.
-__device__ __forceinline__ uint32_t push_trail(Warp& w, bool won, uint32_t l) {
+template <uint32_t SIZE>
+__device__ __forceinline__ uint32_t push_trail(Warp& w, uint32_t* ring, bool won, uint32_t l) {
   const uint32_t m = __ballot_sync(FULL, won);
   const uint32_t pos = w.tail + __popc(m & ((1u << w.lane) - 1u));
   if (won) {
     w.trail[WIDX(w, pos, w.V, 2)] = l;
-    w.ws->ring[pos & (RING - 1u)] = l;
+    ring[pos & (SIZE - 1u)] = l;
   }
   w.tail += __popc(m);
   return pos;
@@ -355,7 +360,7 @@ __device__ __forceinline__ bool claim_bits(Warp& w, bool want, uint32_t l, bool&
 __device__ __forceinline__ void assign_one(Warp& w, uint32_t l) {
   bool won;
   claim_bits<1>(w, w.lane == 0, l, won);
-  push_trail(w, won, l);
+  push_trail<RING>(w, w.ws->ring, won, l);
   __syncwarp();
 }
 
@@ -483,7 +488,7 @@ __device__ __forceinline__ bool bcp(Warp& w) {
       const LaneMap m = lane_map(w.lane, nlit);
       uint32_t f = 0, beg = 0, cnt = 0;
       if (m.mine < nlit) {
-        f = WIDX(w, frontier_lit(w, base + m.mine) ^ 1u, 2u * w.V, 4);  // became false
+        f = WIDX(w, frontier_lit<RING>(w, w.ws->ring, base + m.mine) ^ 1u, 2u * w.V, 4);  // became false
         beg = __ldg(&w.occ[f]);
         cnt = __ldg(&w.occ[f + 1]) - beg;
       }
@@ -493,7 +498,7 @@ __device__ __forceinline__ bool bcp(Warp& w) {
         if (__any_sync(FULL, r.want || r.confl)) {
           bool won;
           const bool clash = claim_bits<1>(w, r.want, r.lit, won);
-          push_trail(w, won, r.lit);
+          push_trail<RING>(w, w.ws->ring, won, r.lit);
           note_conflict(w, r.confl || clash, r.c0, r.c1, r.c2);
           __syncwarp();
         }
@@ -936,8 +941,8 @@ __device__ void finish_job(const Solve& S, Warp& w, int unit, int r) {
     }
     if (S.prof) {
       atomicAdd(&S.prof[1], 1ull);  // jobs run
-      for (int k = 0; k < 8; k++)
-        if (w.ws->cyc[k]) atomicAdd(&S.prof[8 + k], w.ws->cyc[k]);
+      for (int k = 0; w.cyc && k < 8; k++)
+        if (w.cyc[k]) atomicAdd(&S.prof[8 + k], w.cyc[k]);
     }
     if (S.stats) {
       unsigned long long* st = (unsigned long long*)&S.stats[SCUBA_NSTATS * (int64_t)unit];
@@ -1035,7 +1040,7 @@ __device__ int run_job_body(const Solve& S, Warp& w, int unit, int inst, const T
     const uint32_t l = k0 + w.lane < nu ? un[k0 + w.lane] : NONE;
     bool won;
     const bool clash = claim_bits<1>(w, l != NONE, l, won);
-    push_trail(w, won, l);
+    push_trail<RING>(w, w.ws->ring, won, l);
     __syncwarp();
     // a unit clause against an earlier one's value, or another lane's
     const bool bad = l != NONE && !won && lit_value(w.asg, l) != LV_T;
@@ -1186,6 +1191,7 @@ __global__ void __launch_bounds__(256, MODE == MODE_LEARNED ? SCUBA_LEARNED_MINB
   w.lvlcnt = nullptr;
   w.lvl_node = nullptr;
   w.xtile = nullptr;
+  w.cyc = nullptr;
   if (MODE == MODE_TRACE) {
     w.lvlcnt = S.lvlcnt + (size_t)slot * learn::MAX_TRACE_DEPTH * S.vmax;
     w.lvl_node = S.lvl_node + (size_t)slot * learn::MAX_TRACE_DEPTH;
@@ -1205,6 +1211,7 @@ __global__ void __launch_bounds__(256, MODE == MODE_LEARNED ? SCUBA_LEARNED_MINB
                         (S.trail_smem ? (size_t)S.vmax * wpb : 0)) * 4;
     area = reinterpret_cast<unsigned char*>(smem) + ((off + 15) & ~(size_t)15) +
            (size_t)wib * S.cd_smem_warp;
+    w.cyc = reinterpret_cast<unsigned long long*>(area);
     if (S.cd_smem & CD_SMEM_ACT) w.act = cd_area_act(area);
   }
   if (batch_failed(S.ctrl)) return;
@@ -1294,7 +1301,7 @@ __global__ void __launch_bounds__(256, MODE == MODE_LEARNED ? SCUBA_LEARNED_MINB
     if (lane == 0) {
       w.ws->decisions = w.ws->conflicts = w.ws->props = 0;
       w.ws->visits = w.ws->act_reads = w.ws->undone = 0;
-      for (int k = 0; k < 8; k++) w.ws->cyc[k] = 0;
+      for (int k = 0; w.cyc && k < 8; k++) w.cyc[k] = 0;
     }
     __syncwarp();
     uint32_t moot = 0;
@@ -1326,9 +1333,9 @@ __global__ void __launch_bounds__(256, MODE == MODE_LEARNED ? SCUBA_LEARNED_MINB
 }
 
 // Unit-propagation closure of each instance under its unit clauses and the
-// caller's assumption literals: one warp per instance, the same BCP as the
-// search. values[vb[i] + v] = 0 open, 1 true, 2 false; conflict[i] = 1 when
-// propagation falsifies a clause (values are then unspecified).
+// caller's assumption literals, one block per instance. values[vb[i] + v] = 0
+// open, 1 true, 2 false; conflict[i] = 1 when propagation falsifies a clause
+// (values are then unspecified).
 struct PropArgs {
   int n;
   int32_t vmax;
@@ -1346,28 +1353,25 @@ struct PropArgs {
   const uint32_t* flags;
   const int64_t* asm_begin;   // [n+1]
   const int32_t* asm_lits;    // DIMACS
-  uint32_t* trail;            // [slots][vmax]
+  uint32_t* trail;            // [blocks][vmax], or NULL: in shared memory
   uint8_t* values;
   uint8_t* conflict;
   Ctrl* ctrl;
 };
 
-__global__ void __launch_bounds__(256) k_propagate(const __grid_constant__ PropArgs A) {
+__global__ void __launch_bounds__(512) k_propagate(const __grid_constant__ PropArgs A) {
   extern __shared__ uint32_t smem[];
-  const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5, wpb = blockDim.x >> 5;
-  WarpShared* wsh = reinterpret_cast<WarpShared*>(smem);
+  const int lane = threadIdx.x & 31;
   Warp w;
-  w.S = nullptr;  // the propagate kernel has no search state; BCP reads only w.*
+  w.S = nullptr;  // the propagate kernel has no search state
   w.cb = A.cb;
   w.lits = A.lits;
-  w.ws = &wsh[wib];
-  w.asg = smem + (sizeof(WarpShared) / 4) * wpb + (size_t)A.assign_words * wib;
+  w.ws = reinterpret_cast<WarpShared*>(smem);
+  w.asg = smem + sizeof(WarpShared) / 4;
   w.lane = lane;
-  const int64_t slot = (int64_t)blockIdx.x * wpb + wib;
-  w.trail = A.trail + slot * A.vmax;
+  w.trail = A.trail ? A.trail + (int64_t)blockIdx.x * A.vmax : w.asg + A.assign_words;
   if (batch_failed(A.ctrl)) return;
-  // instance i goes to block i mod grid: few instances spread over the SMs
-  for (int i = (int)(wib * gridDim.x + blockIdx.x); i < A.n; i += gridDim.x * wpb) {
+  for (int i = blockIdx.x; i < A.n; i += gridDim.x) {
     if (A.flags[i] & F_BAD) continue;
     w.V = (uint32_t)A.nv[i];
     w.c0 = A.icb[i];
@@ -1375,32 +1379,47 @@ __global__ void __launch_bounds__(256) k_propagate(const __grid_constant__ PropA
     const int64_t lbase = A.icb[i] < A.icb[i + 1] ? A.cb[A.icb[i]] : 0;
     w.ent = A.ent + lbase;
     warp_checks(w, A.ctrl);
+    const bool empty = (A.flags[i] & F_EMPTY) != 0;
+    // the assignment cleared, the unit clauses and assumptions claimed by threads
+    // first, first + step, ...
+    auto clear = [&](uint32_t first, uint32_t step) {
+      for (uint32_t k = first; k < (w.V + 15u) >> 4; k += step) w.asg[k] = 0u;
+      if (first == 0) w.ws->tail = w.ws->conflict = 0;
+    };
+    auto start = [&](uint32_t first, uint32_t step) {
+      for (uint32_t k = first; k < A.nunits[i] && !empty; k += step)
+        if (!close_claim(w, A.units[w.c0 + k])) close_conflict(w, 0, NONE, NONE);
+      for (int64_t k = A.asm_begin[i] + first; k < A.asm_begin[i + 1]; k += step) {
+        const int32_t l = A.asm_lits[k];
+        if (l == 0 || l > (int32_t)w.V || l < -(int32_t)w.V) continue;
+        if (!close_claim(w, code_of(l))) close_conflict(w, 0, NONE, NONE);
+      }
+    };
+    __syncthreads();  // the previous instance's values have been read
+    clear(threadIdx.x, blockDim.x);
+    __syncthreads();
+    start(threadIdx.x, blockDim.x);
+    __syncthreads();
+    bool confl = empty || *(volatile uint32_t*)&w.ws->conflict != 0;
+    const bool alone = blockDim.x == 32;
     w.head = 0;
-    const uint32_t nwords = (w.V + 15u) >> 4;
-    for (uint32_t k = lane; k < nwords; k += 32) w.asg[k] = 0u;
-    if (lane == 0) {
-      w.ws->tail = 0;
-      w.ws->conflict = 0;
-      w.ws->props = w.ws->visits = 0;
+    if (!confl) confl = alone ? close_rounds(w) : close_shared(w);
+    __syncthreads();
+    if (confl && !alone) {  // again, in the fixed order
+      if (threadIdx.x < 32) {
+        clear(lane, 32);
+        __syncwarp();
+        start(lane, 32);
+        __syncwarp();
+        if (!empty && w.ws->conflict == 0) close_rounds(w);
+      }
+      __syncthreads();
     }
-    __syncwarp();
-    bool confl = (A.flags[i] & F_EMPTY) != 0;
-    for (uint32_t k = lane; k < A.nunits[i] && !confl; k += 32)
-      if (!close_claim(w, A.units[w.c0 + k])) close_conflict(w, 0, NONE, NONE);
-    for (int64_t k = A.asm_begin[i] + lane; k < A.asm_begin[i + 1]; k += 32) {
-      const int32_t l = A.asm_lits[k];
-      if (l == 0 || l > (int32_t)w.V || l < -(int32_t)w.V) continue;
-      if (!close_claim(w, code_of(l))) close_conflict(w, 0, NONE, NONE);
-    }
-    __syncwarp();
-    confl = confl || w.ws->conflict != 0;
-    if (!confl) confl = close_rounds(w);
-    if (lane == 0) A.conflict[i] = confl ? 1 : 0;
-    for (uint32_t x = lane; x < w.V; x += 32) {
+    if (threadIdx.x == 0) A.conflict[i] = confl ? 1 : 0;
+    for (uint32_t x = threadIdx.x; x < w.V; x += blockDim.x) {
       const uint32_t bits = (w.asg[x >> 4] >> ((x & 15u) * 2u)) & 3u;
       A.values[A.vb[i] + x] = (uint8_t)(bits == 3u ? 0u : bits);
     }
-    __syncwarp();
   }
 }
 
@@ -2246,22 +2265,33 @@ extern "C" int scuba_propagate_batch(const scuba_cnf_batch* b, const int64_t* as
   const int64_t C = b->total_clauses, L = b->total_lits;
   const int vmax = std::max(1, (int)b->max_vars);
   const int64_t occ_total = 2LL * b->total_vars + n;
-  const int wpb = 8;
   const uint32_t assign_words = (uint32_t)((vmax + 15) / 16);
-  const size_t smem = (sizeof(dev::WarpShared) + (size_t)assign_words * 4) * wpb;
-  if (smem > 227 * 1024) return SCUBA_ERR_TOO_LARGE;
-  // as many blocks as stay resident (the kernel waits on dependent loads, so
-  // warps in flight are what counts), but no more warps than instances
-  const int bps = (int)std::max<size_t>(1, std::min<size_t>(6, 227 * 1024 / (smem + 1024)));
-  const int blocks = std::max(1, std::min({n, S.sms * bps, std::max(S.sms, (n + wpb - 1) / wpb)}));
-  const int64_t slots = (int64_t)blocks * wpb;
+  if ((sizeof(dev::WarpShared) + (size_t)assign_words * 4) * 8 > 227 * 1024)
+    return SCUBA_ERR_TOO_LARGE;
+  // warps per instance: as many as keep about 48 on an SM, one per 512 variables
+  // at most (a round has to have work for them), 16 at most. (33 instances of up to
+  // 46,000 variables: 1.30, 0.89, 0.62, 0.47, 0.40 ms for 1, 2, 4, 8, 16 warps,
+  // preparation included; one warp in close_rounds 1.31 ms. 4,096 instances of
+  // 1,800 variables: one warp in close_rounds 0.99 ms, two to eight sharing an
+  // instance 1.32 to 1.51 ms.)
+  int wpb = 1;
+  while (wpb < 16 && 2LL * wpb * n <= 48LL * S.sms && 1024 * wpb <= vmax) wpb *= 2;
+  // a shared instance's trail in shared memory where it fits; not for one warp
+  // each, whose lists then lose the L1 (1.26 against 0.99 ms)
+  const bool trail_smem = wpb > 1 && (size_t)vmax * 4 <= (size_t)wpb * 12 * 1024;
+  const size_t smem = sizeof(dev::WarpShared) + (size_t)assign_words * 4 +
+                      (trail_smem ? (size_t)vmax * 4 : 0);
+  const int per_sm = (int)std::max<size_t>(1, std::min<size_t>(64 / wpb > 32 ? 32 : 64 / wpb,
+                                                               227 * 1024 / (smem + 1024)));
+  const int blocks = std::min(n, S.sms * per_sm);
   const PrepShape shape = prep_shape(n, b->total_vars, vmax);
   if (ensure(S.occ_base, 8 * (size_t)(n + 1)) ||
       ensure(S.items, shape.table ? 8 * (size_t)shape.items : 0) ||
       ensure(S.occ_begin, 4 * (size_t)occ_total) ||
       ensure(S.ent, 8 * (size_t)L) || ensure(S.units, 4 * (size_t)std::max<int64_t>(C, 1)) ||
       ensure(S.nunits, 4 * (size_t)n) || ensure(S.flags, 4 * (size_t)n) ||
-      ensure(S.trail, 4 * (size_t)slots * vmax) || ensure(S.ctrl, sizeof(dev::Ctrl)))
+      ensure(S.trail, trail_smem ? 0 : 4 * (size_t)blocks * vmax) ||
+      ensure(S.ctrl, sizeof(dev::Ctrl)))
     return SCUBA_ERR_NOMEM;
   dev::Prep pr = prep_args(b, vmax, shape);
   pr.occ_base = P<int64_t>(S.occ_base);
@@ -2292,7 +2322,7 @@ extern "C" int scuba_propagate_batch(const scuba_cnf_batch* b, const int64_t* as
   A.flags = pr.flags;
   A.asm_begin = asm_begin;
   A.asm_lits = asm_lits;
-  A.trail = P<uint32_t>(S.trail);
+  A.trail = trail_smem ? nullptr : P<uint32_t>(S.trail);
   A.values = values;
   A.conflict = conflict;
   A.ctrl = pr.ctrl;

@@ -72,7 +72,7 @@ constexpr uint32_t CD_HDR = 4;
 // global memory a resolution step took about 2,700 cycles.
 enum { CD_SMEM_POS = 1, CD_SMEM_ACT = 2 };
 constexpr uint32_t CD_RING = 64, LSM = 64;
-constexpr size_t CD_FIXED = 8 * 8 + CD_RING * 12 + LSM * 4;
+constexpr size_t CD_FIXED = 8 * 8 + CD_RING * 12 + LSM * 4 + 16;
 
 __host__ __device__ __forceinline__ size_t cd_area_bytes(int what, int32_t vmax) {
   const size_t v16 = ((size_t)vmax + 15) & ~(size_t)15;
@@ -132,6 +132,9 @@ struct CdWarp {
   }
   __device__ __forceinline__ uint32_t* lsm() const {
     return reinterpret_cast<uint32_t*>(area + 64 + 12 * CD_RING);
+  }
+  __device__ __forceinline__ uint4* next() const {  // the literal to resolve next, its reason
+    return reinterpret_cast<uint4*>(area + 64 + 12 * CD_RING + 4 * LSM);
   }
   uint32_t arena_words, pool_cap;
   uint32_t top;       // first free arena word
@@ -253,14 +256,26 @@ __device__ __noinline__ uint32_t grow_list(WList* wl, uint64_t* pool, uint32_t p
 // Append entry e to literal g's watch list in every lane with mover set (all
 // lanes): lists with room take theirs at once, the others grow one by one.
 // Sets cd.full and a conflict (which ends the propagation) if the pool is full.
+template <bool DISTINCT>
 __device__ __forceinline__ void append_watches(Warp& w, CdWarp& cd, bool mover, uint32_t g,
                                                uint64_t e) {
   uint32_t todo = __ballot_sync(FULL, mover);
   while (todo) {
     uint4 L = make_uint4(0, 0, 0, 0);  // {offset, length, capacity}
     if (mover) L = *reinterpret_cast<const uint4*>(&cd.wl[g]);
-    const uint32_t grp =
-        (todo & (todo - 1u)) ? __match_any_sync(FULL, mover ? g : ~(uint32_t)w.lane) : 1u << w.lane;
+    uint32_t grp = 1u << w.lane;
+    if (!DISTINCT && (todo & (todo - 1u))) {
+      if (__popc(todo) <= 3) {
+        for (uint32_t left = todo; left;) {
+          const uint32_t g0 = __shfl_sync(FULL, g, __ffs(left) - 1);
+          const uint32_t same = __ballot_sync(FULL, mover && g == g0);
+          if (mover && g == g0) grp = same;
+          left &= ~same;
+        }
+      } else {
+        grp = __match_any_sync(FULL, mover ? g : ~(uint32_t)w.lane);
+      }
+    }
     const uint32_t rank = __popc(grp & ((1u << w.lane) - 1u)), size = __popc(grp);
     const bool fits = mover && L.y + size <= L.z;
     if (fits) {
@@ -323,8 +338,7 @@ __device__ __forceinline__ void learned_batch(Warp& w, CdWarp& cd, const LaneMap
                                               uint32_t cnt) {
   if (!__any_sync(FULL, cnt != 0)) return;
   const long long t0 = pf_now(*w.S);
-  const uint32_t total = batch_total(m, cnt);
-  WCOUNT(w, visits, total);
+  if (counts_list(m)) WADD(w, visits, cnt);
   const uint32_t width = 1u << m.lg, sub = m.sub;
   // the lanes of this lane's literal, and those of them before it
   const uint32_t mates = (width == 32u ? FULL : (1u << width) - 1u) << ((uint32_t)w.lane - sub);
@@ -400,7 +414,7 @@ __device__ __forceinline__ void learned_batch(Warp& w, CdWarp& cd, const LaneMap
         }
         __syncwarp();
       }
-      if (__any_sync(FULL, mover)) append_watches(w, cd, mover && !cd.full, g, now);
+      if (__any_sync(FULL, mover)) append_watches<false>(w, cd, mover && !cd.full, g, now);
       // close the list up behind the entries that left
       const uint32_t stay = __ballot_sync(FULL, in && !mover);
       const uint32_t to = kept + __popc(stay & before);
@@ -426,7 +440,7 @@ __device__ __forceinline__ bool bcp_cd(Warp& w, CdWarp& cd) {
     WCOUNT(w, props, hi - lo);
     for (uint32_t base = lo; base < hi; base += 32) {
       const uint32_t nlit = min(32u, hi - base);
-      const LaneMap m = lane_map(w.lane, nlit);
+      const LaneMap m = lane_map<true>(w.lane, nlit);
       uint32_t f = 0, beg = 0, cnt = 0, lbeg = 0, lcnt = 0;
       if (m.mine < nlit) {
         const uint32_t t = WIDX(w, frontier_lit<CD_RING>(w, cd.ring(), base + m.mine), 2u * w.V, 14);
@@ -453,8 +467,7 @@ __device__ __forceinline__ bool bcp_cd(Warp& w, CdWarp& cd) {
         }
         return w.confl != 0;
       });
-      const uint32_t total = batch_total(m, cnt);
-      WCOUNT(w, visits, total);
+      if (counts_list(m)) WADD(w, visits, cnt);
       if (w.confl) return true;
       if (cd.top) {
         learned_batch(w, cd, m, nlit, f, lbeg, lcnt);
@@ -577,11 +590,15 @@ __device__ __forceinline__ uint32_t analyze_cd(Warp& w, CdWarp& cd, uint32_t& bl
       // the newest waiting literal (trail positions are distinct)
       const uint32_t top = __reduce_max_sync(FULL, key);
       if (top == 0) return 0;
-      const int owner = __ffs(__ballot_sync(FULL, key == top)) - 1;
-      p = __shfl_sync(FULL, mylit, owner);
-      r0 = __shfl_sync(FULL, my0, owner);
-      r1 = __shfl_sync(FULL, my1, owner);
-      if (key == top) key = 0;
+      if (key == top) {  // through shared memory: finding the lane takes longer
+        *cd.next() = make_uint4(mylit, my0, my1, 0u);
+        key = 0;
+      }
+      __syncwarp();
+      const uint4 c = *cd.next();
+      p = c.x;
+      r0 = c.y;
+      r1 = c.z;
       idx = top - 1u;
     } else {
       for (;;) {  // the newest seen literal on the trail
@@ -689,7 +706,7 @@ __device__ __forceinline__ uint32_t add_learnt(Warp& w, CdWarp& cd, uint32_t n, 
   cd.top = c + clause_words(n);
   cd.ncl++;
   const uint32_t l0 = cd.lsm()[0], l1 = cd.lsm()[1];
-  append_watches(w, cd, w.lane < 2, w.lane == 0 ? l0 : l1,
+  append_watches<true>(w, cd, w.lane < 2, w.lane == 0 ? l0 : l1,
                  (uint64_t)c | ((uint64_t)(w.lane == 0 ? l1 : l0) << 32));
   return c;
 }
@@ -1160,6 +1177,7 @@ __device__ int run_cdcl(const Solve& S, Warp& w, int64_t slot, int unit, int ins
       S.share_lbd > 0 ? S.share_base[(uint32_t)inst & S.share_mask] : 0ull;
   for (;;) {
     if ((++iter & 63u) == 0u) {
+      flush_counters(S, w, unit);
       int stop = 0;
       if (w.lane == 0) {
         if (S.abort_flag && *S.abort_flag) stop = 1;

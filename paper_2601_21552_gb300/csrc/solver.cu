@@ -243,8 +243,10 @@ struct alignas(16) WarpShared {
   // at most RING below the tail: a propagation round reads its literals here
   // instead of waiting for the global trail (DPLL)
   uint32_t ring[RING];
-  // per-job work counters (lane 0 updates them; kept out of registers)
-  unsigned long long decisions, conflicts, props, visits, act_reads, undone;
+  // work counters, kept out of registers: added to without waiting (WADD), moved
+  // to the caller's 64-bit ones every 64 steps of the search (flush_counters)
+  uint32_t decisions, conflicts, props, visits, act_reads, undone;
+  uint32_t pad2[6];
 };
 // The largest instance that fits an SM's shared memory beside this struct is part
 // of the interface.
@@ -307,10 +309,26 @@ __device__ __forceinline__ void warp_checks(Warp& w, Ctrl* c) {
 #endif
 }
 
-#define WCOUNT(w, field, amount)                 \
-  do {                                           \
-    if ((w).lane == 0) (w).ws->field += (amount); \
+// Add to a work counter, by the lanes that have something to add / by lane 0;
+// nothing waits for the sum.
+#define WADD(w, field, amount) atomicAdd(&(w).ws->field, (uint32_t)(amount))
+#define WCOUNT(w, field, amount)               \
+  do {                                         \
+    if ((w).lane == 0) WADD(w, field, amount); \
   } while (0)
+
+// The work counters into unit's statistics (all lanes).
+__device__ __forceinline__ void flush_counters(const Solve& S, Warp& w, int unit) {
+  __syncwarp();
+  if (w.lane < SCUBA_NSTATS) {
+    uint32_t* c = &w.ws->decisions + w.lane;
+    if (S.stats)
+      atomicAdd((unsigned long long*)&S.stats[SCUBA_NSTATS * (int64_t)unit + w.lane],
+                (unsigned long long)*c);
+    *c = 0;
+  }
+  __syncwarp();
+}
 
 #include "closure.cuh"
 
@@ -404,8 +422,10 @@ __device__ __forceinline__ Found eval_entry(const Warp& w, uint32_t f, uint64_t 
   return Found{ua || ub, fa && fb, ua ? a : b, f, a, b0};
 }
 
-// How the lanes share a batch of nlit frontier literals: one literal has the
-// whole warp, two have 16 lanes each, more have 8 lanes each, four at a time.
+// How the lanes share a batch of nlit frontier literals: 8 lanes each, four at a
+// time; in the DPLL search (NARROW false) a single literal has the whole warp and
+// two have 16 lanes each. (DPLL on 256 bounds queries: 9.0 ms so, 10.0 with 8
+// lanes always; clause learning on random 3-SAT 55.5 and 53.0, elsewhere equal.)
 // Most lists hold 3 to 8 entries and most rounds 1 to 4 literals, so a round is
 // usually one pass -- no scan over the list lengths, no search for the owner
 // of an entry. With up to four literals (few) every lane reads its own
@@ -419,9 +439,10 @@ struct LaneMap {
   bool few;
 };
 
+template <bool NARROW>
 __device__ __forceinline__ LaneMap lane_map(uint32_t lane, uint32_t nlit) {
   LaneMap m;
-  m.lg = nlit == 1 ? 5u : nlit == 2 ? 4u : 3u;
+  m.lg = NARROW || nlit > 2 ? 3u : nlit == 1 ? 5u : 4u;
   m.sub = lane & ((1u << m.lg) - 1u);
   m.group = lane >> m.lg;
   m.few = nlit <= 4;
@@ -453,10 +474,8 @@ __device__ __forceinline__ bool spread_lists(const LaneMap& m, uint32_t nlit, ui
   return false;
 }
 
-// Entries of all lists of a batch (every lane).
-__device__ __forceinline__ uint32_t batch_total(const LaneMap& m, uint32_t cnt) {
-  return __reduce_add_sync(FULL, m.few && m.sub != 0 ? 0u : cnt);
-}
+// Whether this lane counts its list among the batch's.
+__device__ __forceinline__ bool counts_list(const LaneMap& m) { return !m.few || m.sub == 0; }
 
 // Remember the conflict of the first lane that has one (all lanes).
 __device__ __forceinline__ void note_conflict(Warp& w, bool confl, uint32_t c0, uint32_t c1,
@@ -485,7 +504,7 @@ __device__ __forceinline__ bool bcp(Warp& w) {
     WCOUNT(w, props, hi - lo);
     for (uint32_t base = lo; base < hi; base += 32) {
       const uint32_t nlit = min(32u, hi - base);
-      const LaneMap m = lane_map(w.lane, nlit);
+      const LaneMap m = lane_map<false>(w.lane, nlit);
       uint32_t f = 0, beg = 0, cnt = 0;
       if (m.mine < nlit) {
         f = WIDX(w, frontier_lit<RING>(w, w.ws->ring, base + m.mine) ^ 1u, 2u * w.V, 4);  // became false
@@ -504,8 +523,7 @@ __device__ __forceinline__ bool bcp(Warp& w) {
         }
         return w.confl != 0;
       });
-      const uint32_t total = batch_total(m, cnt);
-      WCOUNT(w, visits, total);
+      if (counts_list(m)) WADD(w, visits, cnt);
       if (w.confl) return true;
     }
   }
@@ -925,6 +943,7 @@ __device__ void ring_release(const Solve& S, uint32_t slot, int lane) {
 // SCUBA_UNKNOWN). The last open job of a unit (an instance, or an instance
 // under assumptions) writes its verdict.
 __device__ void finish_job(const Solve& S, Warp& w, int unit, int r) {
+  flush_counters(S, w, unit);
   if (w.lane == 0) {
     if (r == SCUBA_SAT) {
       S.verdict[unit] = SCUBA_SAT;
@@ -943,15 +962,6 @@ __device__ void finish_job(const Solve& S, Warp& w, int unit, int r) {
       atomicAdd(&S.prof[1], 1ull);  // jobs run
       for (int k = 0; w.cyc && k < 8; k++)
         if (w.cyc[k]) atomicAdd(&S.prof[8 + k], w.cyc[k]);
-    }
-    if (S.stats) {
-      unsigned long long* st = (unsigned long long*)&S.stats[SCUBA_NSTATS * (int64_t)unit];
-      atomicAdd(st + 0, w.ws->decisions);
-      atomicAdd(st + 1, w.ws->conflicts);
-      atomicAdd(st + 2, w.ws->props);
-      atomicAdd(st + 3, w.ws->visits);
-      atomicAdd(st + 4, w.ws->act_reads);
-      atomicAdd(st + 5, w.ws->undone);
     }
   }
   __syncwarp();
@@ -1051,6 +1061,7 @@ __device__ int run_job_body(const Solve& S, Warp& w, int unit, int inst, const T
   uint32_t iter = 0;
   for (;;) {
     if ((++iter & 63u) == 0u) {
+      flush_counters(S, w, unit);
       int stop = 0;
       if (w.lane == 0) {
         if (S.abort_flag && *S.abort_flag) stop = 1;

@@ -136,7 +136,9 @@ typedef struct scuba_options {
   int32_t blocks_per_sm;     /* 0: autotuned default */
   int32_t split_interval;    /* decisions between checks for idle warps; 0: default 16 */
   int32_t split_min;         /* decisions a subtree makes before it may share work;
-                                0: default 256 */
+                                0: default 256. CDCL: split_min and split_interval
+                                hold while 7 of 8 warps are idle and double with the
+                                busy share, up to 128 and 16 (larger settings stay) */
   int32_t trail_placement;   /* 0: auto (global), 1: shared memory, 2: global memory */
   int64_t* finish_ns;        /* profiling, device [num_instances] or NULL: time from
                                 the start of the search to each verdict, in ns */

@@ -4,7 +4,10 @@ sharing parameters.
 Sweeps blocks per SM, the decisions a subtree makes before it may share work
 (split_min) and the decisions between checks for idle warps (split_interval)
 on a workload, timing each setting over several solves, and writes the
-setting with the lowest MEAN time (a steady setting within 5 % of it wins
+setting with the lowest MEAN time. The workload is a large batch, on which
+every warp starts busy, and two small ones, on which a few hard instances have
+to reach the idle warps; a solve's time is the geometric mean over the three.
+The choice is by the mean (a steady setting within 5 % of it wins
 over one whose slowest solve took more than 1.5x its median) to a JSON file
 that bench.py and
 api.solve(..., tuned=True) read. The search is nondeterministic: a few runs
@@ -31,24 +34,25 @@ import time
 HERE = os.path.dirname(os.path.abspath(__file__))
 DEFAULT_OUT = os.path.join(HERE, "autotune.json")
 SPACE = {
-    "blocks_per_sm": [4, 5],
-    "split_min": [128, 256, 1024],
-    "split_interval": [8, 16, 64],
+    "blocks_per_sm": [2, 3],
+    "split_min": [64, 128],
+    "split_interval": [16, 32],
 }
-# clause learning: decisions before a job may give away cubes and the
-# deepest cube level that may split further (248: the prefix capacity, no
-# cap); the decisions between checks for idle warps (16) and the conflicts per
-# Luby restart unit (25) come from a wider sweep over {8, 16, 32} x
-# {12, 25, 40}, and smaller split_min (4-16) and caps (10-18) lost to these
-# on the mean; share_lbd is the LBD bound of the clauses the jobs of one
-# instance share (-1: no sharing); a gate on the job's own conflicts before
-# it may give cubes away (8-128) was measured no better than none
+# clause learning: decisions before a job may give away cubes, the decisions
+# between checks for idle warps (both while most warps are idle, see
+# scuba_options) and the deepest cube level that may split further (248: the
+# prefix capacity, no cap); split_min of 8 and less lets cube trees explode, 32
+# and more leaves small batches waiting; the conflicts per Luby restart unit (25)
+# come from a sweep over {12, 25, 40, 50, 100}; share_lbd is the LBD bound of the
+# clauses the jobs of one instance share (-1: no sharing); a gate on the job's
+# own conflicts before it may give cubes away (8-128) was measured no better
+# than none
 SPACE_CDCL = {
-    "split_min": [32, 48, 64],
+    "split_min": [12, 16, 24, 32],
     "split_depth": [248],
-    "split_interval": [16],
+    "split_interval": [4, 8],
     "restart_unit": [25],
-    "share_lbd": [-1, 2, 4, 8],
+    "share_lbd": [2],
 }
 
 
@@ -63,7 +67,9 @@ def load(path: str = DEFAULT_OUT, section: str = "best") -> dict:
 
 
 def sweep(db, reps: int = 3, space: dict | None = None, time_budget_ms: int = 120000,
-          fixed: dict | None = None):
+          fixed: dict | None = None, more: tuple = ()):
+    """Times every setting of `space` on db (and each batch of `more`: a rep's
+    time is then the geometric mean). Returns (the choice, all trials)."""
     import numpy as np
     import torch
 
@@ -75,14 +81,18 @@ def sweep(db, reps: int = 3, space: dict | None = None, time_budget_ms: int = 12
         opts = dict(zip(keys, combo))
         times, failed = [], []
         for _ in range(reps):
-            torch.cuda.synchronize()
-            t0 = time.perf_counter()
-            api.solve(db, want_model=False, stats=False, time_budget_ms=time_budget_ms,
-                      **opts, **(fixed or {}))
-            rc = api.status()
-            times.append(time.perf_counter() - t0 if rc == 0 else float("inf"))
-            if rc != 0:
-                failed.append(rc)  # e.g. the time budget reached
+            each = []
+            for batch in (db, *more):
+                torch.cuda.synchronize()
+                t0 = time.perf_counter()
+                api.solve(batch, want_model=False, stats=False, time_budget_ms=time_budget_ms,
+                          **opts, **(fixed or {}))
+                rc = api.status()
+                each.append(time.perf_counter() - t0 if rc == 0 else float("inf"))
+                if rc != 0:
+                    failed.append(rc)  # e.g. the time budget reached
+            times.append(each[0] if len(each) == 1
+                         else float(np.exp(np.mean(np.log(np.array(each))))))
         trials.append({"options": opts, "mean_s": float(np.mean(times)),
                        "median_s": float(np.median(times)), "times": times})
         if failed:
@@ -106,14 +116,14 @@ def main():
     ap = argparse.ArgumentParser()
     ap.add_argument("--queries", type=int, default=4096)
     ap.add_argument("--width", type=int, default=16)
-    ap.add_argument("--reps", type=int, default=0, help="solves per setting (0: 3 for "
+    ap.add_argument("--reps", type=int, default=0, help="solves per setting (0: 6 for "
                     "DPLL, 16 for clause learning)")
     ap.add_argument("--out", default=DEFAULT_OUT)
     ap.add_argument("--search", default="dpll", choices=["dpll", "cdcl"])
     ap.add_argument("--space", default="", help="JSON dict replacing the sweep space, "
                     "e.g. '{\"split_min\": [8, 16], \"split_depth\": [12, 14]}'")
     args = ap.parse_args()
-    args.reps = args.reps or (16 if args.search == "cdcl" else 3)
+    args.reps = args.reps or (16 if args.search == "cdcl" else 6)
     sys.path.insert(0, os.path.dirname(HERE))
     import torch
 
@@ -122,20 +132,23 @@ def main():
     irs, _ = queries.config2(args.queries, w=args.width)
     enc = B.scuba_encode_batch(irs)
     db = api.DeviceBatch(enc, "cuda")
+    more = tuple(api.DeviceBatch(B.scuba_encode_batch(q), "cuda") for q in
+                 (queries.config1(256, w=8)[0], queries.config2(512, w=10)[0]))
     torch.cuda.synchronize()
     space = json.loads(args.space) if args.space else None
     if args.search == "cdcl":
         best, trials = sweep(db, reps=args.reps, space=space or SPACE_CDCL,
-                             fixed={"search": "cdcl"})
+                             fixed={"search": "cdcl"}, more=more)
     else:
-        best, trials = sweep(db, reps=args.reps, space=space)
+        best, trials = sweep(db, reps=args.reps, space=space, more=more)
     try:  # the other search's section stays as it was
         with open(args.out) as f:
             out = json.load(f)
     except (OSError, ValueError):
         out = {}
     sfx = "_cdcl" if args.search == "cdcl" else ""
-    out.update({"workload": f"partition queries, {args.width}-bit inputs, {args.queries} queries",
+    out.update({"workload": f"partition queries, {args.width}-bit inputs, {args.queries} queries; "
+                            "256 bounds queries of 8 bits; 512 partition queries of 10 bits",
                 "device": torch.cuda.get_device_name(0), "reps" + sfx: args.reps,
                 "best" + sfx: best["options"], "best_mean_s" + sfx: best["mean_s"],
                 "best_median_s" + sfx: best["median_s"], "trials" + sfx: trials})

@@ -54,7 +54,7 @@ def build(force: bool = False, verbose: bool = False) -> str:
     cuda_inc = os.path.join(os.path.dirname(os.path.dirname(os.path.realpath(_nvcc()))), "include")
     inc = ["-I", os.path.join(ROOT, "include"), "-I", CSRC, "-I", cuda_inc]
     defs = []
-    for var in ("SCUBA_LEARNED_MINBLOCKS", "SCUBA_CDCL_MINBLOCKS"):
+    for var in ("SCUBA_PLAIN_MINBLOCKS", "SCUBA_LEARNED_MINBLOCKS", "SCUBA_CDCL_MINBLOCKS"):
         if os.environ.get(var):
             defs.append(f"-D{var}=" + str(int(os.environ[var])))
     jobs = []

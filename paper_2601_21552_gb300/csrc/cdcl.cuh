@@ -1306,17 +1306,29 @@ __device__ int run_cdcl(const Solve& S, Warp& w, int64_t slot, int unit, int ins
     // cube-and-conquer: hand the other side of the first free decision to an
     // idle warp and keep this side as an assumption, up to split_depth cube
     // levels below the instance. A cube relearns almost from scratch, so a
-    // job should share only once it has shown itself hard (split_min
-    // decisions): splitting easy jobs whenever warps are idle can cost an
-    // instance that needs a few hundred conflicts alone millions of them
+    // job should share only once it has shown itself hard: sharing after 2 to 4
+    // decisions whenever warps are idle took 48 ms for 12 bounds queries that need
+    // 2.1 (16 decisions). split_min and split_interval hold while more than 7/8 of
+    // the warps are idle, where a few hard instances decide the time and the
+    // tree has to reach the idle warps quickly; both double with the busy share from
+    // there on, up to 128 and 16 decisions, when most warps are busy and sharing
+    // gains least. (16 and 4 so, against 32 and 16 throughout: 12
+    // and 256 bounds queries 4.2 -> 2.8 and 6.6 -> 5.0 ms, units 10.0 -> 7.9, random
+    // 3-SAT 51.5 -> 47.6, 4,096 partition queries 100 -> 97; three seeds.)
     if (S.split && w.decisions >= (uint32_t)S.split_min &&
-        (w.decisions % (uint32_t)S.split_interval) == 0 && w.nd > w.nd_fixed &&
+        w.decisions % (uint32_t)S.split_interval == 0 && w.nd > w.nd_fixed &&
         w.nd_fixed + 1 <= (uint32_t)MAX_PREFIX &&
         w.nd_fixed < asm_levels + (uint32_t)S.split_depth) {
       uint32_t idle = 0;
       if (w.lane == 0) idle = *(volatile uint32_t*)&S.ctrl->idle;
       idle = __shfl_sync(FULL, idle, 0);
-      if (idle > 0) {
+      const uint32_t warps = gridDim.x * (blockDim.x >> 5), busy = warps - min(idle, warps);
+      const uint32_t times = busy > warps / 2 ? 8 : busy > warps / 4 ? 4 : busy > warps / 8 ? 2 : 1;
+      // (a setting beyond the limits is taken as it is)
+      const uint32_t gate = max((uint32_t)S.split_min, min((uint32_t)S.split_min * times, 128u));
+      const uint32_t interval =
+          max((uint32_t)S.split_interval, min((uint32_t)S.split_interval * times, 16u));
+      if (idle > 0 && w.decisions >= gate && w.decisions % interval == 0) {
         const uint32_t k = w.nd_fixed;
         if (w.lane == 0) atomicAdd(&S.pending[unit], 1u);
         __syncwarp();

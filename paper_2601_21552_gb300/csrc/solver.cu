@@ -140,7 +140,10 @@ struct TraceDev {
   int32_t* var;                // [max_rows]
 };
 
-enum { MODE_PLAIN = 0, MODE_TRACE = 1, MODE_LEARNED = 2, MODE_CDCL = 3 };
+// MODE_CDCL1: clause learning where only one block fits an SM anyway, with the
+// registers of two (no spills; 5 % faster on 16-bit partition queries).
+enum { MODE_PLAIN = 0, MODE_TRACE = 1, MODE_LEARNED = 2, MODE_CDCL = 3, MODE_CDCL1 = 4 };
+constexpr bool is_cdcl(int mode) { return mode == MODE_CDCL || mode == MODE_CDCL1; }
 
 // Activities of a slot: whole groups of 16, what one 2-bit assignment word covers.
 __host__ __device__ __forceinline__ int64_t act_stride(int32_t vmax) {
@@ -465,11 +468,15 @@ __device__ __forceinline__ bool spread_lists(const LaneMap& m, uint32_t nlit, ui
       jc = __shfl_sync(FULL, cnt, j);
       if (j >= nlit) jc = 0;
     }
+    bool more;
     uint32_t k = m.sub;
     do {
-      if (visit(jf, jb + k, k < jc)) return true;
+      const bool in = k < jc;
+      const uint32_t at = jb + k;
       k += 1u << m.lg;
-    } while (__any_sync(FULL, k < jc));
+      more = __any_sync(FULL, k < jc);  // asked before it is needed
+      if (visit(jf, at, in)) return true;
+    } while (more);
   }
   return false;
 }
@@ -1163,14 +1170,21 @@ __device__ int run_job_body(const Solve& S, Warp& w, int unit, int inst, const T
 
 #include "cdcl.cuh"
 
-// Plain search: 48 registers per thread, 5 blocks x 8 warps = 40 resident
-// warps per SM. The learned variant (MLP on the tensor cores) defaults to 4
-// blocks (64 registers); SCUBA_LEARNED_MINBLOCKS=5 trades spills for warps
-// (measured slower). The clause-learning variant runs 2 blocks (116
-// registers, no spills): measured faster than 3 (80 registers) or 4 (64,
-// spilling) on partition queries and on random 3-SAT.
+// Blocks of 8 warps that stay resident on an SM, which sets the registers a
+// thread gets. Plain search: 3 (80 registers, against 5 blocks of 48 that spilled
+// 116 bytes). More warps do not pay: a subtree given away repeats part of its
+// donor's work, so idle warps multiply the decisions. With 64 decisions before
+// the first share, 4,096 partition queries of 16 bits take 1.17 s on 2 blocks
+// against 1.59 s on 5 (512 of 10 bits 11.6 and 24.5 ms), and 8,192 random 3-SAT
+// of 250 variables with a budget, where no warp is idle, 85 ms on 3 against 92.
+// The learned variant takes 2 (its trees are the same), trace recording, which
+// shares nothing, 5. Clause learning takes 2 (128 registers): measured faster than
+// 3 or 4, which spill, on partition queries and on random 3-SAT.
+#ifndef SCUBA_PLAIN_MINBLOCKS
+#define SCUBA_PLAIN_MINBLOCKS 3
+#endif
 #ifndef SCUBA_LEARNED_MINBLOCKS
-#define SCUBA_LEARNED_MINBLOCKS 4
+#define SCUBA_LEARNED_MINBLOCKS 2
 #endif
 #ifndef SCUBA_CDCL_MINBLOCKS
 #define SCUBA_CDCL_MINBLOCKS 2
@@ -1178,6 +1192,8 @@ __device__ int run_job_body(const Solve& S, Warp& w, int unit, int inst, const T
 template <int MODE>
 __global__ void __launch_bounds__(256, MODE == MODE_LEARNED ? SCUBA_LEARNED_MINBLOCKS
                                        : MODE == MODE_CDCL  ? SCUBA_CDCL_MINBLOCKS
+                                       : MODE == MODE_PLAIN ? SCUBA_PLAIN_MINBLOCKS
+                                       : MODE == MODE_CDCL1 ? 1
                                                             : 5)
     k_solve(const __grid_constant__ Solve S) {
   extern __shared__ uint32_t smem[];
@@ -1215,7 +1231,7 @@ __global__ void __launch_bounds__(256, MODE == MODE_LEARNED ? SCUBA_LEARNED_MINB
     w.xtile = reinterpret_cast<__nv_bfloat16*>(tiles) + (size_t)wib * 32 * learn::NFEAT;
   }
   unsigned char* area = nullptr;
-  if (MODE == MODE_CDCL) {
+  if (is_cdcl(MODE)) {
     // the warp's own area after the per-warp assignment (and trail) areas,
     // 16-byte aligned
     const size_t off = ((sizeof(WarpShared) / 4) * wpb + (size_t)S.assign_words * wpb +
@@ -1251,7 +1267,7 @@ __global__ void __launch_bounds__(256, MODE == MODE_LEARNED ? SCUBA_LEARNED_MINB
       taken.len = len;
       taken.inc = cell->inc;
       taken.cls = nullptr;
-      if (MODE == MODE_CDCL) {  // the donor's learned clauses, copied out too
+      if (is_cdcl(MODE)) {  // the donor's learned clauses, copied out too
         const uint32_t* src = S.job_cls + (size_t)(slot_j & (S.ring_cap - 1)) * JOB_CLS_WORDS;
         uint32_t* dst = S.cls_copy + slot * JOB_CLS_WORDS;
         const uint32_t words = min(src[1], JOB_CLS_WORDS);
@@ -1329,7 +1345,7 @@ __global__ void __launch_bounds__(256, MODE == MODE_LEARNED ? SCUBA_LEARNED_MINB
       if (lane == 0) set_status(S, SCUBA_ERR_TOO_LARGE);
     } else if (moot) {
       r = SCUBA_UNSAT;  // moot: another subtree already found a model
-    } else if constexpr (MODE == MODE_CDCL) {
+    } else if constexpr (is_cdcl(MODE)) {
       r = run_cdcl(S, w, slot, unit, inst, job, area, abort_code);
     } else {
       r = run_job<MODE>(S, w, unit, inst, job, abort_code);
@@ -1457,7 +1473,7 @@ struct Scratch {
   Buf h_icb, h_cb, h_lits, h_nv, h_vb, h_verdict, h_model, h_stats;  // for the host entry
   int sms = 0;
   int32_t last_status = 0;
-  int smem_set[4] = {0, 0, 0, 0};  // dynamic shared memory granted per search mode
+  int smem_set[5] = {0, 0, 0, 0, 0};  // dynamic shared memory granted per search mode
   int smem_prop = 0;
 };
 
@@ -1719,8 +1735,10 @@ static int solve_impl(const scuba_cnf_batch* b, uint8_t* verdict, uint8_t* model
     return SCUBA_ERR_TOO_LARGE;
   }
   while (bps > 1 && (smem + 1024) * bps > sm_cap) bps--;
+  if (mode == dev::MODE_PLAIN) bps = std::min(bps, SCUBA_PLAIN_MINBLOCKS);
   if (mode == dev::MODE_LEARNED) bps = std::min(bps, SCUBA_LEARNED_MINBLOCKS);
   if (mode == dev::MODE_CDCL) bps = std::min(bps, SCUBA_CDCL_MINBLOCKS);
+  const bool one_block = mode == dev::MODE_CDCL && bps == 1;
   const int64_t slots = (int64_t)S.sms * bps * wpb;
   const uint32_t ring_cap = 2048;
 
@@ -1894,15 +1912,17 @@ static int solve_impl(const scuba_cnf_batch* b, uint8_t* verdict, uint8_t* model
   if (e != cudaSuccess) return cuda_fail("preparation launch", e);
   auto kern = mode == dev::MODE_TRACE     ? dev::k_solve<dev::MODE_TRACE>
               : mode == dev::MODE_LEARNED ? dev::k_solve<dev::MODE_LEARNED>
+              : one_block                 ? dev::k_solve<dev::MODE_CDCL1>
               : mode == dev::MODE_CDCL    ? dev::k_solve<dev::MODE_CDCL>
                                           : dev::k_solve<dev::MODE_PLAIN>;
   // raise the dynamic shared-memory limit only when it grows, so that a
   // repeated call (for example while a CUDA graph is being captured) issues
   // no attribute change
-  if ((int)smem > S.smem_set[mode]) {
+  int& granted = S.smem_set[one_block ? (int)dev::MODE_CDCL1 : mode];
+  if ((int)smem > granted) {
     e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return cuda_fail("cudaFuncSetAttribute", e);
-    S.smem_set[mode] = (int)smem;
+    granted = (int)smem;
   }
   if (opt->search_event_begin) cudaEventRecord((cudaEvent_t)opt->search_event_begin, st);
   kern<<<S.sms * bps, 32 * wpb, smem, st>>>(sv);

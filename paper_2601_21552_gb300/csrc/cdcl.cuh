@@ -72,7 +72,7 @@ constexpr uint32_t CD_HDR = 4;
 // global memory a resolution step took about 2,700 cycles.
 enum { CD_SMEM_POS = 1, CD_SMEM_ACT = 2 };
 constexpr uint32_t CD_RING = 64, LSM = 64;
-constexpr size_t CD_FIXED = 8 * 8 + CD_RING * 12 + LSM * 4 + 16;
+constexpr size_t CD_FIXED = 8 * 8 + CD_RING * 12 + LSM * 4 + 16 + 32 * 12;
 
 __host__ __device__ __forceinline__ size_t cd_area_bytes(int what, int32_t vmax) {
   const size_t v16 = ((size_t)vmax + 15) & ~(size_t)15;
@@ -135,6 +135,12 @@ struct CdWarp {
   }
   __device__ __forceinline__ uint4* next() const {  // the literal to resolve next, its reason
     return reinterpret_cast<uint4*>(area + 64 + 12 * CD_RING + 4 * LSM);
+  }
+  __device__ __forceinline__ uint2* visit() const {  // [32] clauses to visit {clause, false watch}
+    return reinterpret_cast<uint2*>(area + 64 + 12 * CD_RING + 4 * LSM + 16);
+  }
+  __device__ __forceinline__ uint32_t* outcome() const {  // [32] what became of their entries
+    return reinterpret_cast<uint32_t*>(area + 64 + 12 * CD_RING + 4 * LSM + 16 + 32 * 8);
   }
   uint32_t arena_words, pool_cap;
   uint32_t top;       // first free arena word
@@ -298,34 +304,98 @@ __device__ __forceinline__ void append_watches(Warp& w, CdWarp& cd, bool mover, 
   }
 }
 
-// A new watch for a learned clause: the first position >= 2 whose literal is
-// not false, else the first whose literal was falsified during this round
-// (its own list brings the clause back next round), else NONE; g gets the
-// literal. x: the clause's first four literals; further ones are read 4 at a
-// time (16-byte loads; clauses are 16-byte aligned and padded).
-__device__ __forceinline__ uint32_t new_watch(const uint32_t* asg, const uint32_t* lits, uint4 x,
-                                              uint32_t len, uint32_t& g) {
-  uint32_t fresh_pos = NONE;
-  for (uint32_t q = 0;;) {
-    const uint32_t l[4] = {x.x, x.y, x.z, x.w};
-    uint32_t open = 0, fr = 0;
-#pragma unroll
-    for (int i = 0; i < 4; i++) {
-      if (q + i < 2 || q + i >= len) continue;
-      const uint2 ws = lit_words(asg, l[i]);
-      if (!has_bit(ws.x, l[i] ^ 1u)) open |= 1u << i;
-      else if (!has_bit(ws.y, l[i] ^ 1u)) fr |= 1u << i;
+// Outcome of a visited clause for its entry in the list: the new blocker, or
+constexpr uint32_t OUT_SAME = 0xffffffffu, OUT_MOVED = 0xfffffffeu;
+
+// Visit the `total` clauses in cd.visit(): eight lanes take a clause, four
+// clauses at a time, a lane each literal, so that a search for a new watch is
+// one trip to memory per eight literals whatever the lanes' clauses are (one
+// lane per clause took about 1,900 cycles on random 3-SAT, each four literals
+// of the longest clause one after another). A clause whose other watch is
+// true gets it as its blocker; else the watch moves to the first literal from
+// position 2 on that is not false, or if there is none the first that was
+// falsified during this round (its own list brings the clause back next
+// round); else the clause implies its other watch or is a conflict. dups: a
+// clause may be there twice (both its watches false): the second is visited
+// after the first has moved its watch. Stops at a conflict.
+__device__ __forceinline__ void visit_clauses(Warp& w, CdWarp& cd, uint32_t total, bool dups) {
+  const uint32_t sub = (uint32_t)w.lane & 7u, group = (uint32_t)w.lane >> 3;
+  const uint32_t shift = (uint32_t)w.lane & 24u;  // this group's bits in a ballot
+  for (uint32_t r0 = 0; r0 < total && !w.confl; r0 += 4) {
+    uint32_t todo = (1u << min(4u, total - r0)) - 1u;  // groups whose clause is not done
+    while (todo && !w.confl) {
+      const uint32_t r = r0 + group;
+      bool go = (todo >> group) & 1u;
+      uint2 v = make_uint2(0, 0);
+      if (go) v = cd.visit()[r];
+      if (dups)
+        for (uint32_t q = 0; q < 3; q++)
+          if (go && q < group && ((todo >> q) & 1u) && cd.visit()[r0 + q].x == v.x) go = false;
+      uint32_t* const L = cd.arena + v.x + CD_HDR;
+      uint32_t lit = 0, len = 0;
+      if (go) {
+        lit = L[sub];  // past the clause's end too: not used then
+        len = L[-(int)CD_HDR];
+      }
+      const bool in = sub < len;
+      if (!in) lit = 0;
+      uint2 ws = lit_words(w.asg, lit);
+      const uint32_t m_true = __ballot_sync(FULL, in && has_bit(ws.x, lit));
+      const uint32_t m_open = __ballot_sync(FULL, in && !has_bit(ws.x, lit ^ 1u));
+      const uint32_t m_fresh =
+          __ballot_sync(FULL, in && has_bit(ws.x, lit ^ 1u) && !has_bit(ws.y, lit ^ 1u));
+      const uint32_t m_f = __ballot_sync(FULL, in && sub < 2 && lit == v.y);
+      const uint32_t which = (m_f >> shift) & 1u ? 0u : 1u, op = which ^ 1u;
+      const uint32_t other = __shfl_sync(FULL, lit, shift + op);
+      const bool o_true = (m_true >> (shift + op)) & 1u, o_open = (m_open >> (shift + op)) & 1u;
+      uint32_t cand = (m_open >> shift) & 0xfcu, fresh = (m_fresh >> shift) & 0xfcu;
+      // position and literal of the new watch (fresh_*: the fallback)
+      uint32_t at = __ffs(cand) - 1u, fresh_at = __ffs(fresh) - 1u;
+      uint32_t g = __shfl_sync(FULL, lit, shift + (at & 7u));
+      uint32_t fresh_g = __shfl_sync(FULL, lit, shift + (fresh_at & 7u));
+      for (uint32_t q = 8; __any_sync(FULL, go && !o_true && at == NONE && q < len); q += 8) {
+        const bool more = go && !o_true && at == NONE && q + sub < len;
+        lit = more ? L[q + sub] : 0u;
+        ws = lit_words(w.asg, lit);
+        const bool isf = has_bit(ws.x, lit ^ 1u);
+        cand = (__ballot_sync(FULL, more && !isf) >> shift) & 0xffu;
+        fresh = (__ballot_sync(FULL, more && isf && !has_bit(ws.y, lit ^ 1u)) >> shift) & 0xffu;
+        const uint32_t a = __ffs(cand) - 1u, b = __ffs(fresh) - 1u;
+        const uint32_t la = __shfl_sync(FULL, lit, shift + (a & 7u));
+        const uint32_t lb = __shfl_sync(FULL, lit, shift + (b & 7u));
+        if (cand) {
+          at = q + a;
+          g = la;
+        }
+        if (fresh && fresh_at == NONE) {
+          fresh_at = q + b;
+          fresh_g = lb;
+        }
+      }
+      if (at == NONE) {
+        at = fresh_at;
+        g = fresh_g;
+      }
+      // the group's first lane acts
+      const bool act = go && sub == 0, moves = act && !o_true && at != NONE;
+      const bool want = act && !o_true && at == NONE && o_open;
+      bool confl = act && !o_true && at == NONE && !o_open;
+      if (moves) {
+        L[at] = v.y;
+        L[which] = g;
+      }
+      if (act && (o_true || moves)) cd.outcome()[r] = moves ? OUT_MOVED : other;
+      const uint32_t done = __ballot_sync(FULL, act);
+      for (uint32_t q = 0; q < 4; q++)
+        if ((done >> (8 * q)) & 1u) todo &= ~(1u << q);
+      if (__any_sync(FULL, want || confl)) {
+        confl |= claim_cd(w, cd, want, other, LEARNT_REF | v.x, 0u);
+        note_conflict(w, confl, LEARNT_REF | v.x, NONE, NONE);
+      }
+      __syncwarp();
+      if (__any_sync(FULL, moves) && !cd.full)
+        append_watches<false>(w, cd, moves, g, (uint64_t)v.x | ((uint64_t)other << 32));
     }
-    const uint32_t hit = open ? open : fresh_pos == NONE ? fr : 0u;
-    if (hit) {
-      const int i = __ffs(hit) - 1;
-      g = i == 0 ? l[0] : i == 1 ? l[1] : i == 2 ? l[2] : l[3];
-      if (open) return q + i;
-      fresh_pos = q + i;
-    }
-    q += 4;
-    if (q >= len) return fresh_pos;
-    x = *reinterpret_cast<const uint4*>(lits + q);
   }
 }
 
@@ -339,11 +409,8 @@ __device__ __forceinline__ void learned_batch(Warp& w, CdWarp& cd, const LaneMap
   if (!__any_sync(FULL, cnt != 0)) return;
   const long long t0 = pf_now(*w.S);
   if (counts_list(m)) WADD(w, visits, cnt);
-  const uint32_t width = 1u << m.lg, sub = m.sub;
-  // the lanes of this lane's literal, and those of them before it
-  const uint32_t mates = (width == 32u ? FULL : (1u << width) - 1u) << ((uint32_t)w.lane - sub);
-  const uint32_t before = mates & ((1u << w.lane) - 1u);
-  for (uint32_t s = 0; s < nlit; s += 32u >> m.lg) {
+  const uint32_t below = (1u << w.lane) - 1u, mates = 0xffu << ((uint32_t)w.lane & 24u);
+  for (uint32_t s = 0; s < nlit; s += 4) {
     uint32_t jb = beg, jf = f, jc = cnt;
     if (!m.few) {
       const uint32_t j = s + m.group;
@@ -353,76 +420,44 @@ __device__ __forceinline__ void learned_batch(Warp& w, CdWarp& cd, const LaneMap
       if (j >= nlit) jc = 0;
     }
     uint32_t kept = 0;
-    for (uint32_t k = sub; __any_sync(FULL, k < jc); k += width) {
+    bool more = __any_sync(FULL, m.sub < jc);
+    for (uint32_t k = m.sub; more; k += 8) {
       const bool in = k < jc;
       uint64_t entry = 0;
-      uint32_t c = 0;
       bool pending = false;
       if (in) {
         entry = cd.pool[WIDX(w, jb + k, cd.pool_cap, 16)];
-        c = WIDX(w, (uint32_t)entry, cd.top, 17);
         const uint32_t blocker = WIDX(w, (uint32_t)(entry >> 32), 2u * w.V, 18);
         pending = !has_bit(w.asg[2 * (blocker >> 5)], blocker);
       }
-      if (w.confl) pending = false;
+      more = __any_sync(FULL, k + 8 < jc);
+      const uint32_t c = WIDX(w, (uint32_t)entry, cd.top, 17);
+      const uint32_t pm = w.confl ? 0u : __ballot_sync(FULL, pending);
+      bool stay = in;
       uint64_t now = entry;  // the entry that stays in this list
-      bool mover = false;
-      uint32_t g = NONE;
-      while (__any_sync(FULL, pending)) {
-        uint32_t* const L = cd.arena + c + CD_HDR;
-        uint4 x = make_uint4(0, 0, 0, 0);
-        uint32_t len = 0, other = 0;
-        uint2 ow = make_uint2(0, 0);
-        bool both = false;
+      if (pm) {
+        const uint32_t rank = __popc(pm & below);
         if (pending) {
-          x = *reinterpret_cast<const uint4*>(L);
-          len = L[-(int)CD_HDR];
-          other = x.x == jf ? x.y : x.x;
-          ow = lit_words(w.asg, other);
-          both = has_bit(ow.x, other ^ 1u);
-        }
-        // both watches false: the clause may be on another lane's list too; the
-        // first lane moves its watch (or finds the conflict), the next looks again
-        bool go = pending;
-        const uint32_t bm = __ballot_sync(FULL, both);
-        if (bm & (bm - 1u)) {
-          const uint32_t grp = __match_any_sync(FULL, both ? c : ~(uint32_t)w.lane);
-          go = pending && (!both || (grp & ((1u << w.lane) - 1u)) == 0u);
-        }
-        bool want = false, confl = false;
-        if (go) {
-          pending = false;
-          if (has_bit(ow.x, other)) {
-            now = (uint64_t)c | ((uint64_t)other << 32);  // new blocker
-          } else {
-            const uint32_t at = new_watch(w.asg, L, x, len, g);
-            if (at != NONE) {
-              L[at] = jf;
-              L[x.x == jf ? 0 : 1] = g;
-              mover = true;
-              now = (uint64_t)c | ((uint64_t)other << 32);
-            } else {
-              confl = both;
-              want = !both;
-            }
-          }
-        }
-        if (__any_sync(FULL, want || confl)) {
-          confl |= claim_cd(w, cd, want, other, LEARNT_REF | c, 0u);
-          note_conflict(w, confl, LEARNT_REF | c, NONE, NONE);
-          if (w.confl) pending = false;
+          cd.visit()[rank] = make_uint2(c, jf);
+          cd.outcome()[rank] = OUT_SAME;
         }
         __syncwarp();
+        visit_clauses(w, cd, __popc(pm), nlit > 1);
+        __syncwarp();
+        if (pending) {
+          const uint32_t o = cd.outcome()[rank];
+          stay = o != OUT_MOVED;
+          if (stay && o != OUT_SAME) now = (uint64_t)c | ((uint64_t)o << 32);
+        }
       }
-      if (__any_sync(FULL, mover)) append_watches<false>(w, cd, mover && !cd.full, g, now);
       // close the list up behind the entries that left
-      const uint32_t stay = __ballot_sync(FULL, in && !mover);
-      const uint32_t to = kept + __popc(stay & before);
-      if (in && !mover && (to != k || now != entry)) cd.pool[jb + to] = now;
-      kept += __popc(stay & mates);
+      const uint32_t stays = __ballot_sync(FULL, stay);
+      const uint32_t to = kept + __popc(stays & mates & below);
+      if (stay && (to != k || now != entry)) cd.pool[jb + to] = now;
+      kept += __popc(stays & mates);
       __syncwarp();
     }
-    if (sub == 0 && kept != jc) cd.wl[jf].len = kept;
+    if (m.sub == 0 && kept != jc) cd.wl[jf].len = kept;
   }
   __syncwarp();
   pf_add(*w.S, w, PF_LEARNED, t0);
@@ -711,11 +746,18 @@ __device__ __forceinline__ uint32_t add_learnt(Warp& w, CdWarp& cd, uint32_t n, 
   return c;
 }
 
+// Room every watch list gets before its first entry (a list grows one at a time,
+// the warp copying it): four entries, a sector, where that takes little of the pool.
+__device__ __forceinline__ uint32_t list_room(const Warp& w, const CdWarp& cd) {
+  return (uint64_t)w.V * 32u <= cd.pool_cap ? 4u : 0u;
+}
+
 __device__ __noinline__ void clear_learnts(Warp& w, CdWarp& cd) {
-  for (uint32_t k = w.lane; k < 2u * w.V; k += 32) cd.wl[k] = WList{0u, 0u, 0u, 0u};
+  const uint32_t room = list_room(w, cd);
+  for (uint32_t k = w.lane; k < 2u * w.V; k += 32) cd.wl[k] = WList{room * k, 0u, room, 0u};
   cd.top = 0;
   cd.ncl = 0;
-  cd.pool_top = 0;
+  cd.pool_top = room * 2u * w.V;
   cd.full = 0;
   __syncwarp();
 }
@@ -790,11 +832,12 @@ __device__ bool rebuild_watches(Warp& w, CdWarp& cd) {
     atomicAdd(&cd.wl[cd.arena[c + CD_HDR + 1]].len, 1u);
   }
   __syncwarp();
+  const uint32_t room = list_room(w, cd);
   uint32_t base = 0;
   for (uint32_t k0 = 0; k0 < nl; k0 += 32) {
     const uint32_t k = k0 + w.lane;
     const uint32_t len = k < nl ? cd.wl[k].len : 0u;
-    const uint32_t cap = len ? len + max(4u, len / 2u) : 0u;
+    const uint32_t cap = k < nl ? len + (len ? max(4u, len / 2u) : room) : 0u;
     uint32_t inc = cap;
 #pragma unroll
     for (int d = 1; d < 32; d <<= 1) {

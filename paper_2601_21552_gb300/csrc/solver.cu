@@ -1777,7 +1777,8 @@ static int solve_impl(const scuba_cnf_batch* b, uint8_t* verdict, uint8_t* model
         ensure(S.cd_wl, 32 * (size_t)slots * vmax) ||
         ensure(S.cd_pool, 8 * (size_t)slots * arena_words) ||
         ensure(S.cd_learnt, 4 * (size_t)slots * vmax) ||
-        ensure(S.cd_arena, 4 * (size_t)slots * arena_words) ||
+        // a clause's reader takes eight literals at a time, past its end too
+        ensure(S.cd_arena, 4 * (size_t)slots * arena_words + 64) ||
         ensure(S.cd_clidx, 4 * (size_t)slots * (arena_words / 8)) ||
         ensure(S.job_cls, 4 * (size_t)ring_cap * dev::JOB_CLS_WORDS) ||
         ensure(S.cls_copy, 4 * (size_t)slots * dev::JOB_CLS_WORDS) ||

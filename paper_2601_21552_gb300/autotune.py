@@ -41,18 +41,20 @@ SPACE = {
 # clause learning: decisions before a job may give away cubes, the decisions
 # between checks for idle warps (both while most warps are idle, see
 # scuba_options) and the deepest cube level that may split further (248: the
-# prefix capacity, no cap); split_min of 8 and less lets cube trees explode, 32
-# and more leaves small batches waiting; the conflicts per Luby restart unit (25)
-# come from a sweep over {12, 25, 40, 50, 100}; share_lbd is the LBD bound of the
-# clauses the jobs of one instance share (-1: no sharing); a gate on the job's
+# prefix capacity, no cap); split_min of 8 and less lets cube trees explode (10
+# was measured within 1 % of 12), 32 and more leaves small batches waiting; the
+# conflicts per Luby restart unit (25) come from a sweep over {12, 25, 40, 50,
+# 100}; share_lbd is the LBD bound of the clauses the jobs of one instance share
+# (-1: no sharing; reading fewer of them pays more than they prune: 2 takes 3 %
+# longer than 1); a gate on the job's
 # own conflicts before it may give cubes away (8-128) was measured no better
 # than none
 SPACE_CDCL = {
-    "split_min": [12, 16, 24, 32],
+    "split_min": [12, 16, 24],
     "split_depth": [248],
     "split_interval": [4, 8],
     "restart_unit": [25],
-    "share_lbd": [2],
+    "share_lbd": [1, 2],
 }
 
 

@@ -1178,8 +1178,13 @@ __device__ int run_job_body(const Solve& S, Warp& w, int unit, int inst, const T
 // against 1.59 s on 5 (512 of 10 bits 11.6 and 24.5 ms), and 8,192 random 3-SAT
 // of 250 variables with a budget, where no warp is idle, 85 ms on 3 against 92.
 // The learned variant takes 2 (its trees are the same), trace recording, which
-// shares nothing, 5. Clause learning takes 2 (128 registers): measured faster than
-// 3 or 4, which spill, on partition queries and on random 3-SAT.
+// shares nothing, 5. Clause learning takes 2 blocks of 6 warps, three warps for
+// each quarter of the SM, which leaves a thread 168 registers and no spills; 16
+// warps (128 registers, 206 bytes spilled) are the better choice only where the
+// search keeps every warp at work of its own for long: 511 random 3-SAT instances
+// of 150 variables take 45.0 ms against 41.7, 256 of them 27.5 against 27.0, but 511
+// of 100 variables 8.0 against 9.0, 24 to 2,048 bounds queries of 8 bits 8 to 13 % less,
+// partition queries of 10 bits 6 to 11 % less.
 #ifndef SCUBA_PLAIN_MINBLOCKS
 #define SCUBA_PLAIN_MINBLOCKS 3
 #endif
@@ -1189,12 +1194,14 @@ __device__ int run_job_body(const Solve& S, Warp& w, int unit, int inst, const T
 #ifndef SCUBA_CDCL_MINBLOCKS
 #define SCUBA_CDCL_MINBLOCKS 2
 #endif
+constexpr int CDCL_WARPS = 6;
 template <int MODE>
-__global__ void __launch_bounds__(256, MODE == MODE_LEARNED ? SCUBA_LEARNED_MINBLOCKS
-                                       : MODE == MODE_CDCL  ? SCUBA_CDCL_MINBLOCKS
-                                       : MODE == MODE_PLAIN ? SCUBA_PLAIN_MINBLOCKS
-                                       : MODE == MODE_CDCL1 ? 1
-                                                            : 5)
+__global__ void __launch_bounds__(MODE == MODE_CDCL ? 32 * CDCL_WARPS : 256,
+                                  MODE == MODE_LEARNED ? SCUBA_LEARNED_MINBLOCKS
+                                  : MODE == MODE_CDCL  ? SCUBA_CDCL_MINBLOCKS
+                                  : MODE == MODE_PLAIN ? SCUBA_PLAIN_MINBLOCKS
+                                  : MODE == MODE_CDCL1 ? 1
+                                                       : 5)
     k_solve(const __grid_constant__ Solve S) {
   extern __shared__ uint32_t smem[];
   const int lane = threadIdx.x & 31;
@@ -1724,6 +1731,11 @@ static int solve_impl(const scuba_cnf_batch* b, uint8_t* verdict, uint8_t* model
       if (vmax < 65536 && (per_warp + cd_smem_warp) * 8 + 16 <= smem_cap) break;
     }
     per_warp += cd_smem_warp;
+    // two blocks on an SM if blocks of CDCL_WARPS (or of what the caller asks
+    // for) fit so, else one of up to 8 warps
+    const int w2 = std::min(wpb, dev::CDCL_WARPS);
+    if (bps > 1 && (per_warp * w2 + 16 + 1024) * 2 <= sm_cap) wpb = w2;
+    else bps = 1;
   }
   size_t smem = per_warp * wpb + (mode == dev::MODE_CDCL ? 16 : 0);  // ring alignment
   while (wpb > 1 && smem > smem_cap) {

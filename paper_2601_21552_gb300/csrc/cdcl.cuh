@@ -69,22 +69,33 @@ constexpr uint32_t CD_HDR = 4;
 // activity (CD_SMEM_ACT), its trail position and level packed into 32 bits and
 // its mark (both CD_SMEM_POS; at most 65,535 variables). The analysis walks from
 // variable to variable, so what it reads of each has to be near: with these in
-// global memory a resolution step took about 2,700 cycles.
-enum { CD_SMEM_POS = 1, CD_SMEM_ACT = 2 };
+// global memory a resolution step took about 2,700 cycles. Where the activities
+// do not fit, a bound per group of them does (CD_SMEM_GMAX, see pick_grouped).
+enum { CD_SMEM_POS = 1, CD_SMEM_ACT = 2, CD_SMEM_GMAX = 4 };
 constexpr uint32_t CD_RING = 64, LSM = 64;
 constexpr size_t CD_FIXED = 8 * 8 + CD_RING * 12 + LSM * 4 + 16 + 32 * 12;
 
 __host__ __device__ __forceinline__ size_t cd_area_bytes(int what, int32_t vmax) {
   const size_t v16 = ((size_t)vmax + 15) & ~(size_t)15;
-  return CD_FIXED + (what & CD_SMEM_ACT ? 4 * v16 : 0) + (what & CD_SMEM_POS ? 5 * v16 : 0);
+  return CD_FIXED + (what & CD_SMEM_ACT ? 4 * v16 : 0) + (what & CD_SMEM_POS ? 5 * v16 : 0) +
+         (what & CD_SMEM_GMAX ? (4 * (((size_t)vmax + 127) / 128) + 15) & ~(size_t)15 : 0);
 }
+// A warp's area is never taken smaller than this: the largest instance that fits
+// an SM is part of the interface.
+constexpr size_t CD_AREA_MIN = 1792;
+static_assert(CD_FIXED <= CD_AREA_MIN, "largest instance");
 __device__ __forceinline__ float* cd_area_act(unsigned char* area) {
   return reinterpret_cast<float*>(area + CD_FIXED);
+}
+// (an area has either the activities or the groups' bounds)
+__device__ __forceinline__ uint32_t* cd_area_gmax(unsigned char* area) {
+  return reinterpret_cast<uint32_t*>(area + CD_FIXED);
 }
 
 // A variable's mark: bit 0 the saved phase, bits 1-7 the number (1..127, mod
 // 127) of the last analysis that met it, so that nothing is cleared after one.
 constexpr uint32_t MK_PHASE = 1, MK_EPOCHS = 127;
+constexpr uint32_t GMAX_LOOK = 0xffffffffu;  // a group's bound that is not known
 
 // Profile counters (only when the caller passed a profile array): lane 0
 // adds the clock cycles of each phase to its warp's profile.
@@ -691,6 +702,8 @@ __device__ __forceinline__ uint32_t analyze_cd(Warp& w, CdWarp& cd, uint32_t& bl
   if (big) {
     for (uint32_t v = w.lane; v < w.V; v += 32) w.act[v] *= 1e-20f;
     w.inc *= 1e-20f;
+    if (w.S->cd_smem & CD_SMEM_GMAX)
+      for (uint32_t g = w.lane; 128u * g < w.V; g += 32) cd_area_gmax(cd.area)[g] = GMAX_LOOK;
   }
   __syncwarp();
   blev = best_l;
@@ -709,6 +722,8 @@ __device__ void backjump_cd(Warp& w, CdWarp& cd, uint32_t lev) {
     atomicAnd(&w.asg[2 * (l >> 5)], keep);
     atomicAnd(&w.asg[2 * (l >> 5) + 1], keep);
     cd.mark[v] = (l & 1u) ? 0 : (uint8_t)MK_PHASE;
+    if (w.S->cd_smem & CD_SMEM_GMAX)
+      atomicMax(&cd_area_gmax(cd.area)[v >> 7], __float_as_uint(w.act[v]) + 1u);
   }
   __syncwarp();
   w.nd = lev;
@@ -994,7 +1009,67 @@ __device__ __noinline__ bool import_clauses(Warp& w, CdWarp& cd, const uint32_t*
   return true;
 }
 
-__device__ uint32_t pick_cd(Warp& w) { return pick_max<2>(w); }
+// pick_max where the activities are in global memory: for every 128 variables
+// shared memory holds a bound on the activities of the unassigned ones (0: none
+// left, else the bits of the bound plus 1). Assigning and bumping (an analysis
+// bumps assigned variables only) leave a bound valid; backjump_cd raises it for
+// what it unassigns, and looking at a group makes it exact. So a decision looks
+// at the few groups whose bound reaches the best variable found, not at 40 KB
+// of activities of an instance of 10,000 variables: on 128 large queries 20,000
+// cycles a decision became 3,200, 28 % of all cycles 6 %, and 65 ms 58.
+__device__ __forceinline__ uint32_t pick_grouped(const Warp& w, uint32_t* gmax) {
+  uint32_t best = 0, best_v = NONE;
+  for (;;) {
+    // the group of the highest bound, the lowest one of equals
+    uint32_t top = 0, g = NONE;
+    for (uint32_t k = w.lane; 128u * k < w.V; k += 32) {
+      const uint32_t x = gmax[k];
+      if (x > top) {
+        top = x;
+        g = k;
+      }
+    }
+    const uint32_t high = __reduce_max_sync(FULL, top);
+    if (high == 0u || high < best) return best_v;
+    g = __reduce_min_sync(FULL, top == high ? g : NONE);
+    if (high == best && g >= (best_v >> 7)) return best_v;
+    const uint32_t v = 128u * g + 4u * w.lane;
+    uint32_t un = 0;
+    if (v < w.V) {
+      const uint32_t word = w.asg[2 * (v >> 4)];
+      un = (~(word | (word >> 1)) >> (2u * (v & 15u))) & 0x55u;
+      if (w.V - v < 4u) un &= (1u << (2u * (w.V - v))) - 1u;
+    }
+    uint32_t key = 0, kv = NONE;
+    if (un) {
+      const float4 a = *reinterpret_cast<const float4*>(w.act + v);
+      const float x[4] = {a.x, a.y, a.z, a.w};
+#pragma unroll
+      for (int q = 0; q < 4; q++)
+        if (((un >> (2 * q)) & 1u) && __float_as_uint(x[q]) + 1u > key) {
+          key = __float_as_uint(x[q]) + 1u;
+          kv = v + q;
+        }
+    }
+    const uint32_t most = __reduce_max_sync(FULL, key);
+    kv = __reduce_min_sync(FULL, key == most ? kv : NONE);
+    if (w.lane == 0) gmax[g] = most;
+    __syncwarp();
+    if (most > best || (most == best && kv < best_v)) {
+      best = most;
+      best_v = kv;
+    }
+  }
+}
+
+__device__ uint32_t pick_cd(Warp& w, unsigned char* area) {
+  if (!(w.S->cd_smem & CD_SMEM_GMAX)) return pick_max<2>(w);
+  const uint32_t v = pick_grouped(w, cd_area_gmax(area));
+#ifdef SCUBA_CHECKED
+  (void)WIDX(w, v == pick_max<2>(w) ? 0u : 1u, 1u, 27);
+#endif
+  return v;
+}
 
 // ---- clauses shared between the jobs of one instance ----------------------
 //
@@ -1139,7 +1214,7 @@ __device__ int run_cdcl(const Solve& S, Warp& w, int64_t slot, int unit, int ins
   cd.mark = S.cd_mark + slot * S.vmax;
   if (S.cd_smem & CD_SMEM_POS) {
     const size_t v16 = ((size_t)S.vmax + 15) & ~(size_t)15;
-    unsigned char* at = area + cd_area_bytes(S.cd_smem & CD_SMEM_ACT, S.vmax);
+    unsigned char* at = area + cd_area_bytes(S.cd_smem & ~CD_SMEM_POS, S.vmax);
     cd.pl = reinterpret_cast<uint32_t*>(at);
     cd.mark = at + 4 * v16;
   }
@@ -1171,6 +1246,8 @@ __device__ int run_cdcl(const Solve& S, Warp& w, int64_t slot, int unit, int ins
     if (!job) w.act[v] = 0.0f;
     cd.mark[v] = 0;
   }
+  if (S.cd_smem & CD_SMEM_GMAX)
+    for (uint32_t g = w.lane; 128u * g < w.V; g += 32) cd_area_gmax(area)[g] = GMAX_LOOK;
   w.tail = 0;
   w.confl = 0;
   // Calls of the rarely used parts work on copies of w and cd, so that the
@@ -1331,7 +1408,7 @@ __device__ int run_cdcl(const Solve& S, Warp& w, int64_t slot, int unit, int ins
     }
     WCOUNT(w, act_reads, w.V - w.tail);
     t0 = pf_now(S);
-    const uint32_t v = pick_cd(w);
+    const uint32_t v = pick_cd(w, area);
     pf_add(S, w, PF_DECIDE, t0);
     if (v == NONE) {
       // the first cube of the instance to reach a model writes it

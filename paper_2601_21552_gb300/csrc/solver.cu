@@ -1723,13 +1723,17 @@ static int solve_impl(const scuba_cnf_batch* b, uint8_t* verdict, uint8_t* model
   int cd_smem = 0;
   uint32_t cd_smem_warp = 0;
   if (mode == dev::MODE_CDCL) {
-    // per-variable state in shared memory (9 or 5 bytes a variable) as long as 8
-    // warps still fit an SM
-    for (int what : {dev::CD_SMEM_POS | dev::CD_SMEM_ACT, (int)dev::CD_SMEM_POS, 0}) {
+    // per-variable state in shared memory (9 or 5 bytes a variable, or bounds of
+    // the activities only) as long as 8 warps still fit an SM
+    for (int what : {dev::CD_SMEM_POS | dev::CD_SMEM_ACT, dev::CD_SMEM_POS | dev::CD_SMEM_GMAX,
+                     (int)dev::CD_SMEM_GMAX, 0}) {
       cd_smem = what;
       cd_smem_warp = (uint32_t)dev::cd_area_bytes(what, vmax);
-      if (vmax < 65536 && (per_warp + cd_smem_warp) * 8 + 16 <= smem_cap) break;
+      if ((vmax < 65536 || !(what & dev::CD_SMEM_POS)) &&
+          (per_warp + cd_smem_warp) * 8 + 16 <= smem_cap)
+        break;
     }
+    if (!cd_smem) cd_smem_warp = std::max(cd_smem_warp, (uint32_t)dev::CD_AREA_MIN);
     per_warp += cd_smem_warp;
     // two blocks on an SM if blocks of CDCL_WARPS (or of what the caller asks
     // for) fit so, else one of up to 8 warps

@@ -25,18 +25,21 @@
 //    of the clause (the other watch when the entry was made) whose truth
 //    settles the clause without reading it. After the static occurrence
 //    entries of each frontier batch, the watchers of every literal in the
-//    batch are spread over the 32 lanes like the static entries. A clause
-//    can sit on two lists of one pass only when both its watches are false;
-//    the second lane then waits until the first has moved its watch. Moved
-//    watches are appended to their new lists all at once (the warp copies a
-//    list when it grows) and a list closes up while it is read.
+//    batch are spread over the 32 lanes like the static entries, and the
+//    clauses whose blocker is not true are visited by eight lanes each. A
+//    clause can sit on two lists of one pass only when both its watches are
+//    false; its second visit then waits until the first has moved its watch.
+//    Moved watches are appended to their new lists all at once (the warp
+//    copies a list when it grows) and a list closes up while it is read.
 //  * Conflict analysis resolves the falsified clause with the reasons of
 //    current-level literals, newest first on the trail, until one
 //    current-level literal (the first UIP) is left; the lanes take the
 //    literals of each clause, and the next literal to resolve is the newest
 //    of the waiting ones, each kept in a lane's registers (a warp-wide
 //    backward scan of the trail if more than 32 wait). Every variable met is
-//    bumped.
+//    bumped. (Dropping the literals that the rest of the clause implies, a lane
+//    per literal, saved 2 % of the conflicts on partition queries and 7 % on
+//    random 3-SAT, and cost as much as it saved or more.)
 //  * Hard instances are shared cube-and-conquer style through the DPLL mode's
 //    job ring: a busy warp that sees idle warps gives away the negation of
 //    its first free decision, together with the assumptions above it, as a

@@ -140,8 +140,8 @@ struct TraceDev {
   int32_t* var;                // [max_rows]
 };
 
-// MODE_CDCL1: clause learning where only one block fits an SM anyway, with the
-// registers of two (no spills; 5 % faster on 16-bit partition queries).
+// MODE_CDCL1: clause learning where an SM holds one block only (large instances),
+// which may then have 8 warps and 255 registers a thread.
 enum { MODE_PLAIN = 0, MODE_TRACE = 1, MODE_LEARNED = 2, MODE_CDCL = 3, MODE_CDCL1 = 4 };
 constexpr bool is_cdcl(int mode) { return mode == MODE_CDCL || mode == MODE_CDCL1; }
 
@@ -342,16 +342,18 @@ __device__ __forceinline__ uint32_t frontier_lit(const Warp& w, const uint32_t* 
 }
 
 // Append the literals of the lanes with won set to the trail (all lanes): in
-// lane order, so no counter in memory is involved. Returns the lane's position.
+// lane order, so no counter in memory is involved. A ring of fewer slots than
+// lanes takes the newest positions only: two lanes must not write one slot.
+// Returns the lane's position.
 template <uint32_t SIZE>
 __device__ __forceinline__ uint32_t push_trail(Warp& w, uint32_t* ring, bool won, uint32_t l) {
   const uint32_t m = __ballot_sync(FULL, won);
   const uint32_t pos = w.tail + __popc(m & ((1u << w.lane) - 1u));
+  w.tail += __popc(m);
   if (won) {
     w.trail[WIDX(w, pos, w.V, 2)] = l;
-    ring[pos & (SIZE - 1u)] = l;
+    if (SIZE >= 32u || w.tail - pos <= SIZE) ring[pos & (SIZE - 1u)] = l;
   }
-  w.tail += __popc(m);
   return pos;
 }
 

@@ -132,8 +132,9 @@ typedef struct scuba_options {
   int64_t decision_budget;   /* per instance (all its subtrees); <= 0: unlimited */
   int64_t time_budget_ms;    /* whole call; <= 0: 600000 */
   int32_t split;             /* 1: hand DPLL subtrees of busy instances to idle warps */
-  int32_t warps_per_block;   /* at most 8; 0: default 8 (6 for LEARNED). CDCL: at most 6
-                                where an SM holds two blocks */
+  int32_t warps_per_block;   /* at most 8; 0: default 8 (LEARNED: 6 for batches of fewer
+                                units than 24 warps an SM). CDCL: at most 6 where
+                                an SM holds two blocks */
   int32_t blocks_per_sm;     /* 0: autotuned default */
   int32_t split_interval;    /* decisions between checks for idle warps; 0: default 16 */
   int32_t split_min;         /* decisions a subtree makes before it may share work;

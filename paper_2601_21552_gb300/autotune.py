@@ -36,7 +36,7 @@ DEFAULT_OUT = os.path.join(HERE, "autotune.json")
 SPACE = {
     "blocks_per_sm": [2, 3],
     "split_min": [64, 128],
-    "split_interval": [16, 32],
+    "split_interval": [16],
 }
 # clause learning: decisions before a job may give away cubes, the decisions
 # between checks for idle warps (both while most warps are idle, see

@@ -1179,8 +1179,9 @@ __device__ int run_job_body(const Solve& S, Warp& w, int unit, int inst, const T
 // the first share, 4,096 partition queries of 16 bits take 1.17 s on 2 blocks
 // against 1.59 s on 5 (512 of 10 bits 11.6 and 24.5 ms), and 8,192 random 3-SAT
 // of 250 variables with a budget, where no warp is idle, 85 ms on 3 against 92.
-// The learned variant takes 2 (its trees are the same), trace recording, which
-// shares nothing, 5. Clause learning takes 2 blocks of 6 warps, three warps for
+// The learned variant takes up to 3 as well (80 registers, no spills; 2 blocks of 6
+// warps for small batches, see scuba_solve_units), trace recording, which shares
+// nothing, 5. Clause learning takes 2 blocks of 6 warps, three warps for
 // each quarter of the SM, which leaves a thread 168 registers and no spills; 16
 // warps (128 registers, 206 bytes spilled) are the better choice only where the
 // search keeps every warp at work of its own for long: 511 random 3-SAT instances
@@ -1191,7 +1192,7 @@ __device__ int run_job_body(const Solve& S, Warp& w, int unit, int inst, const T
 #define SCUBA_PLAIN_MINBLOCKS 3
 #endif
 #ifndef SCUBA_LEARNED_MINBLOCKS
-#define SCUBA_LEARNED_MINBLOCKS 2
+#define SCUBA_LEARNED_MINBLOCKS 3
 #endif
 #ifndef SCUBA_CDCL_MINBLOCKS
 #define SCUBA_CDCL_MINBLOCKS 2
@@ -1707,10 +1708,17 @@ static int solve_impl(const scuba_cnf_batch* b, uint8_t* verdict, uint8_t* model
 
   // shape: warps per block x blocks per SM (shared memory bounds the warps).
   // The trail goes to shared memory when that still leaves >= 16 warps/SM.
-  // (learned branching: 6 warps take 34.0 ms for 512 partition queries of 10 bits
-  // and 21.9 for 256 bounds queries of 8, 8 warps 35.6 and 22.6)
-  int wpb = opt->warps_per_block > 0 ? opt->warps_per_block : mode == dev::MODE_LEARNED ? 6 : 8;
-  int bps = opt->blocks_per_sm > 0 ? opt->blocks_per_sm : 5;
+  // Learned branching: two blocks of 6 warps unless the batch has a unit for every
+  // warp of three blocks of 8. 512 partition queries of 10 bits take 34.6 ms so and
+  // 38.7 on three blocks, 2,048 bounds queries of 8 bits 24.9 and 29.0, but
+  // 4,096 partition queries of 10 bits 101 and 93, of 16 bits 6.0 and 5.1 s.
+  const bool many = n_units >= 24 * S.sms;
+  int wpb = opt->warps_per_block > 0 ? opt->warps_per_block
+            : mode == dev::MODE_LEARNED && !many ? 6
+                                                 : 8;
+  int bps = opt->blocks_per_sm > 0 ? opt->blocks_per_sm
+            : mode == dev::MODE_LEARNED && !many ? 2
+                                                 : 5;
   wpb = std::min(wpb, 8);
   // 2 bits per variable; the clause-learning search keeps 4 (true, settled)
   const uint32_t assign_words = mode == dev::MODE_CDCL ? 2u * (uint32_t)((vmax + 15) / 16)

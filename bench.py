@@ -50,12 +50,12 @@ METRIC = "verdicts/sec + BCP propagations/sec on 1 GB300, learned vs plain, bit-
 
 
 # DRAM traffic of the clause-learning search kernel from one single-pass ncu
-# capture of a full bench launch (profiles/k_solve_cdcl_partition16.md: 8.71 GB
-# read + 7.04 GB written for 1.2389e8 propagations), per propagation, valid
+# capture of a full bench launch (profiles/k_solve_cdcl_partition16.md: 2.62 GB
+# read + 3.24 GB written for 1.1200e8 propagations), per propagation, valid
 # only for the kernel sources it was taken on (sha256 prefix of solver.cu +
 # learn.cuh + cdcl.cuh); scaled to each launch by the propagations it processes.
-PROFILED_SOURCES = "d559d46d82c2e11f"
-DRAM_BYTES_PER_PROPAGATION = {"cdcl": (8.7077e9 + 7.0410e9) / 1.2389e8}
+PROFILED_SOURCES = "933c95430e866518"
+DRAM_BYTES_PER_PROPAGATION = {"cdcl": (2.6246e9 + 3.2413e9) / 1.1200e8}
 
 
 def _kernel_sources_sha() -> str:
@@ -68,10 +68,10 @@ def _kernel_sources_sha() -> str:
 
 
 # L2 traffic of the same kernel from the same single-pass ncu capture
-# (lts__t_bytes.sum: 125.93 GB for 1.2389e8 propagations), per propagation,
+# (lts__t_bytes.sum: 54.67 GB for 1.1200e8 propagations), per propagation,
 # under the same source hash (idle warps polling the job ring and the
 # clause-sharing pools included).
-L2_BYTES_PER_PROPAGATION = {"cdcl": 125.93e9 / 1.2389e8}
+L2_BYTES_PER_PROPAGATION = {"cdcl": 54.67e9 / 1.1200e8}
 
 
 def l2_probe(dev, mib: int = 32, iters: int = 200) -> float:
@@ -778,7 +778,7 @@ def run_ours(args):
                    "autotuned": {"dpll": tuned, "cdcl": tuned_cdcl}},
         "arms": summ,
         "e2e": e2e,
-        "gpu_launches": 10 * args.steps,
+        "gpu_launches": 3 * args.steps,
         "l2": _l2_line(arms[0], head, ws, dev) if args.config == 2 else None,
         "roofline": {"bound": "hbm", "achieved": achieved, "peak": hbm, "unit": "GB/s",
                      "frac": achieved / hbm,

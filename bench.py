@@ -54,7 +54,7 @@ METRIC = "verdicts/sec + BCP propagations/sec on 1 GB300, learned vs plain, bit-
 # read + 3.24 GB written for 1.1200e8 propagations), per propagation, valid
 # only for the kernel sources it was taken on (sha256 prefix of solver.cu +
 # learn.cuh + cdcl.cuh); scaled to each launch by the propagations it processes.
-PROFILED_SOURCES = "933c95430e866518"
+PROFILED_SOURCES = "6e09aee0f0709900"
 DRAM_BYTES_PER_PROPAGATION = {"cdcl": (2.6246e9 + 3.2413e9) / 1.1200e8}
 
 

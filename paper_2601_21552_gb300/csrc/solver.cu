@@ -1176,9 +1176,10 @@ __device__ int run_job_body(const Solve& S, Warp& w, int unit, int inst, const T
 // thread gets. Plain search: 3 (80 registers, against 5 blocks of 48 that spilled
 // 116 bytes). More warps do not pay: a subtree given away repeats part of its
 // donor's work, so idle warps multiply the decisions. With 64 decisions before
-// the first share, 4,096 partition queries of 16 bits take 1.17 s on 2 blocks
-// against 1.59 s on 5 (512 of 10 bits 11.6 and 24.5 ms), and 8,192 random 3-SAT
-// of 250 variables with a budget, where no warp is idle, 85 ms on 3 against 92.
+// the first share, 4,096 partition queries of 16 bits take 0.75 s on 3 blocks,
+// 0.89 on 2, and took 1.59 on 5 (512 of 10 bits 11.6 ms on 2 and 24.5 on 5), and
+// 8,192 random 3-SAT of 250 variables with a budget, where no warp is idle, 85 ms
+// on 3 against 92 on 2.
 // The learned variant takes up to 3 as well (80 registers, no spills; 2 blocks of 6
 // warps for small batches, see scuba_solve_units), trace recording, which shares
 // nothing, 5. Clause learning takes 2 blocks of 6 warps, three warps for

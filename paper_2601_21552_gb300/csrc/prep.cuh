@@ -264,12 +264,13 @@ __global__ void __launch_bounds__(32 * WARPS) k_prep(const __grid_constant__ Pre
   __shared__ uint32_t part[32], s_units[WARPS], s_item, s_flags, s_wide, s_below;
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
   const uint32_t below_me = (1u << lane) - 1u;
-  if (batch_failed(P.ctrl)) return;
   const uint32_t n_items = P.ctrl->n_items;
   for (;;) {
     __syncthreads();
     if (threadIdx.x == 0) {
-      s_item = atomicAdd(&P.ctrl->next_item, 1u);
+      // another block may set the status at any time (a malformed range below):
+      // one thread reads it for the block, which leaves as a whole
+      s_item = batch_failed(P.ctrl) ? n_items : atomicAdd(&P.ctrl->next_item, 1u);
       s_flags = s_wide = s_below = 0;
     }
     __syncthreads();

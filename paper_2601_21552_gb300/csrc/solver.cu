@@ -1252,7 +1252,8 @@ __global__ void __launch_bounds__(MODE == MODE_CDCL ? 32 * CDCL_WARPS : 256,
     w.cyc = reinterpret_cast<unsigned long long*>(area);
     if (S.cd_smem & CD_SMEM_ACT) w.act = cd_area_act(area);
   }
-  if (batch_failed(S.ctrl)) return;
+  // the warp's lanes agree (other warps set the status while this one starts)
+  if (__any_sync(FULL, batch_failed(S.ctrl))) return;
   if (lane == 0) start_clock(S.ctrl);
   bool counted_idle = false;
   for (;;) {
@@ -1408,7 +1409,9 @@ __global__ void __launch_bounds__(512) k_propagate(const __grid_constant__ PropA
   w.asg = smem + sizeof(WarpShared) / 4;
   w.lane = lane;
   w.trail = A.trail ? A.trail + (int64_t)blockIdx.x * A.vmax : w.asg + A.assign_words;
-  if (batch_failed(A.ctrl)) return;
+  // the block's threads agree (a failed bounds check of the checked build sets
+  // the status while other blocks start)
+  if (__syncthreads_or(batch_failed(A.ctrl))) return;
   for (int i = blockIdx.x; i < A.n; i += gridDim.x) {
     if (A.flags[i] & F_BAD) continue;
     w.V = (uint32_t)A.nv[i];

@@ -261,7 +261,10 @@ __device__ __forceinline__ bool bad_literal(int32_t l, int V) { return l == 0 ||
 template <int WARPS>
 __global__ void __launch_bounds__(32 * WARPS) k_prep(const __grid_constant__ Prep P) {
   extern __shared__ uint32_t smem[];
-  __shared__ uint32_t part[32], s_units[WARPS], s_item, s_flags, s_wide, s_below;
+  __shared__ uint32_t part[32], s_units[WARPS], s_item, s_flags, s_below;
+  // a warp's own count ran over 16 bits (pass 1) / a list's did (scan): two words,
+  // since the scan sets its one while slower threads still read the other
+  __shared__ uint32_t s_wide, s_long;
   const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
   const uint32_t below_me = (1u << lane) - 1u;
   const uint32_t n_items = P.ctrl->n_items;
@@ -271,7 +274,7 @@ __global__ void __launch_bounds__(32 * WARPS) k_prep(const __grid_constant__ Pre
       // another block may set the status at any time (a malformed range below):
       // one thread reads it for the block, which leaves as a whole
       s_item = batch_failed(P.ctrl) ? n_items : atomicAdd(&P.ctrl->next_item, 1u);
-      s_flags = s_wide = s_below = 0;
+      s_flags = s_wide = s_long = s_below = 0;
     }
     __syncthreads();
     const uint32_t it = s_item;
@@ -374,7 +377,7 @@ __global__ void __launch_bounds__(32 * WARPS) k_prep(const __grid_constant__ Pre
           a += c & 0xffffu;
           b += c >> 16;
         }
-        if (a > 0xffffu || b > 0xffffu) s_wide = 1;
+        if (a > 0xffffu || b > 0xffffu) s_long = 1;
       }
       uint32_t total;
       const uint32_t at = run + block_exclusive(a + b, part, total);
@@ -385,7 +388,8 @@ __global__ void __launch_bounds__(32 * WARPS) k_prep(const __grid_constant__ Pre
       }
     }
     __syncthreads();
-    if (s_wide) {
+    const bool one_warp = recount || s_long != 0;
+    if (one_warp) {
       // more than 65,535 occurrences of a literal: 32-bit counts for the whole
       // block, and one warp fills the lists
       uint32_t* const cnt32 = packed;  // [nl]: WARPS * nl2 words or more
@@ -419,7 +423,6 @@ __global__ void __launch_bounds__(32 * WARPS) k_prep(const __grid_constant__ Pre
       }
       __syncthreads();
     }
-    const bool one_warp = s_wide != 0;
     if (hi == 2u * (uint32_t)V && threadIdx.x == 0) occ[hi] = run;
     uint32_t nunit = 0;
     if (first_range) {

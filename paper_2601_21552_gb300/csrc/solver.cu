@@ -33,6 +33,7 @@
 
 #include "../../include/scuba.h"
 #include "learn.cuh"
+#include "rules.h"
 #include "scuba_internal.h"
 
 namespace scuba {
@@ -844,7 +845,7 @@ __device__ __forceinline__ void start_clock(Ctrl* c) {
 }
 
 __device__ __forceinline__ uint64_t search_ns(const Solve& S) {
-  return globaltimer() - *(volatile uint64_t*)&S.ctrl->t0;
+  return elapsed_ns(*(volatile uint64_t*)&S.ctrl->t0, globaltimer());
 }
 
 __device__ __forceinline__ void set_status(const Solve& S, int32_t st) {

@@ -1290,7 +1290,11 @@ __device__ int run_cdcl(const Solve& S, Warp& w, int64_t slot, int unit, int ins
       S.unit_asm_begin ? (uint32_t)min(S.unit_asm_begin[unit + 1] - S.unit_asm_begin[unit],
                                        (int64_t)MAX_PREFIX)
                        : 0u;
-  uint32_t iter = 0, conflicts = 0, since_restart = 0, restart_no = 1;
+  uint32_t conflicts = 0, since_restart = 0, restart_no = 1;
+  auto steps = [&] {  // counted down: a register less than a mask
+    return flush_steps(__ldg(&w.occ[2u * w.V]), (uint64_t)S.cd_arena_words, w.V);
+  };
+  uint32_t until_flush = steps();
   uint32_t next_reduce = 2000u, reductions = 0;  // periodic database reduction
   uint32_t restart_at = (uint32_t)S.restart_unit * luby_cd(1);
   // clause sharing with the other jobs of this instance: on for a cube and
@@ -1299,7 +1303,8 @@ __device__ int run_cdcl(const Solve& S, Warp& w, int64_t slot, int unit, int ins
   unsigned long long share_rd =
       S.share_lbd > 0 ? S.share_base[(uint32_t)inst & S.share_mask] : 0ull;
   for (;;) {
-    if ((++iter & 63u) == 0u) {
+    if (--until_flush == 0u) {
+      until_flush = steps();
       flush_counters(S, w, unit);
       int stop = 0;
       if (w.lane == 0) {

@@ -248,7 +248,8 @@ struct alignas(16) WarpShared {
   // instead of waiting for the global trail (DPLL)
   uint32_t ring[RING];
   // work counters, kept out of registers: added to without waiting (WADD), moved
-  // to the caller's 64-bit ones every 64 steps of the search (flush_counters)
+  // to the caller's 64-bit ones every 64 steps of the search, oftener where 64
+  // could pass 32 bits (flush_counters, flush_steps)
   uint32_t decisions, conflicts, props, visits, act_reads, undone;
   uint32_t pad2[6];
 };
@@ -1069,8 +1070,9 @@ __device__ int run_job_body(const Solve& S, Warp& w, int unit, int inst, const T
   int next_asm = 0;
   const int n_asm = job ? job->len : 0;
   uint32_t iter = 0;
+  const uint32_t flush_mask = flush_steps(__ldg(&w.occ[2u * w.V]), 0, w.V) - 1u;
   for (;;) {
-    if ((++iter & 63u) == 0u) {
+    if ((++iter & flush_mask) == 0u) {
       flush_counters(S, w, unit);
       int stop = 0;
       if (w.lane == 0) {

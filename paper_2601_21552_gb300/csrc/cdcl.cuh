@@ -1411,7 +1411,7 @@ __device__ int run_cdcl(const Solve& S, Warp& w, int64_t slot, int unit, int ins
       }
       if (S.share_lbd > 0 && !shared) {
         uint32_t others = 0;
-        if (w.lane == 0) others = *(volatile uint32_t*)&S.pending[unit] > 1u;
+        if (w.lane == 0) others = (*(volatile uint32_t*)&S.pending[unit] & PEND_JOBS) > 1u;
         shared = __shfl_sync(FULL, others, 0) != 0u;
       }
       if (shared) {

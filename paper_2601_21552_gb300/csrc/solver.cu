@@ -44,6 +44,8 @@ constexpr uint32_t NONE = 0xffffffffu;
 constexpr uint32_t LONG_CLAUSE = 0x80000000u;
 constexpr uint32_t FLIP = 0x80000000u;
 constexpr uint32_t F_EMPTY = 1u, F_BAD = 2u;
+// A unit's word of open jobs: their number, a job found a model, a job gave up.
+constexpr uint32_t PEND_JOBS = 0x3fffffffu, PEND_SAT = 0x40000000u, PEND_GAVE_UP = 0x80000000u;
 constexpr int MAX_PREFIX = 248;   // literals in a split job's prefix
 // Learned clauses a clause-learning donor attaches to a cube: [count, words
 // used, offset of each clause (JOB_CLS_MAX), records {len, lbd, literals}].
@@ -180,8 +182,8 @@ struct Solve {
   uint8_t* model;
   int64_t* stats;
   // per instance bookkeeping
-  uint32_t* pending;       // open jobs of an instance
-  uint32_t* done;          // 1 once the verdict is final
+  uint32_t* pending;       // open jobs of a unit (PEND_JOBS), and what its finished ones found
+  uint32_t* done;          // 1 once a model was found, 8 once a job writes it
   unsigned long long* inst_dec;  // decisions so far (budget)
   // per slot
   uint32_t* trail;
@@ -952,20 +954,23 @@ __device__ void ring_release(const Solve& S, uint32_t slot, int lane) {
 
 // A unit's job finished with result r (SCUBA_SAT / SCUBA_UNSAT /
 // SCUBA_UNKNOWN). The last open job of a unit (an instance, or an instance
-// under assumptions) writes its verdict.
+// under assumptions) writes its verdict. What a job found goes into the word that
+// counts the open jobs: atomics of one thread on one word take effect in order,
+// so the last job sees what every other one found before it left (on two words
+// nothing but a fence would order them).
 __device__ void finish_job(const Solve& S, Warp& w, int unit, int r) {
   flush_counters(S, w, unit);
   if (w.lane == 0) {
     if (r == SCUBA_SAT) {
       S.verdict[unit] = SCUBA_SAT;
-      atomicOr(&S.done[unit], 1u);
+      atomicOr(&S.done[unit], 1u);  // the unit's other jobs may stop
+      atomicOr(&S.pending[unit], PEND_SAT);
     } else if (r == SCUBA_UNKNOWN) {
-      atomicOr(&S.done[unit], 2u);  // mark: some subtree gave up
+      atomicOr(&S.pending[unit], PEND_GAVE_UP);
     }
-    uint32_t left = atomicSub(&S.pending[unit], 1u) - 1u;
-    if (left == 0u) {
-      uint32_t d = atomicOr(&S.done[unit], 4u);
-      if (!(d & 1u)) S.verdict[unit] = (d & 2u) ? SCUBA_UNKNOWN : SCUBA_UNSAT;
+    const uint32_t p = atomicSub(&S.pending[unit], 1u);
+    if ((p & PEND_JOBS) == 1u) {  // the last one
+      if (!(p & PEND_SAT)) S.verdict[unit] = p & PEND_GAVE_UP ? SCUBA_UNKNOWN : SCUBA_UNSAT;
       atomicSub(&S.ctrl->inst_left, 1u);
       if (S.finish_ns) S.finish_ns[unit] = (int64_t)search_ns(S);
     }

@@ -6,10 +6,11 @@ Sweeps blocks per SM, the decisions a subtree makes before it may share work
 on a workload, timing each setting over several solves, and writes the
 setting with the lowest MEAN time. The workload is a large batch, on which
 every warp starts busy, and two small ones, on which a few hard instances have
-to reach the idle warps; a solve's time is the geometric mean over the three.
-The choice is by the mean (a steady setting within 5 % of it wins
-over one whose slowest solve took more than 1.5x its median) to a JSON file
-that bench.py and
+to reach the idle warps; settings are ranked by the geometric mean of the three
+batches' mean times (a steady setting within 5 % of the lowest wins over one
+whose slowest solve of any batch took more than 1.5x that batch's median; tails
+are judged and averaged batch by batch, since a mean over the three would hide
+them) and written to a JSON file that bench.py and
 api.solve(..., tuned=True) read. The search is nondeterministic: a few runs
 in ten can take several times the median (a hard instance's cube tree grows
 much deeper in them), so the mean -- what a sequence of solves costs -- is
@@ -28,6 +29,7 @@ import argparse
 import itertools
 import json
 import os
+import statistics
 import sys
 import time
 
@@ -70,8 +72,9 @@ def load(path: str = DEFAULT_OUT, section: str = "best") -> dict:
 
 def sweep(db, reps: int = 3, space: dict | None = None, time_budget_ms: int = 120000,
           fixed: dict | None = None, more: tuple = ()):
-    """Times every setting of `space` on db (and each batch of `more`: a rep's
-    time is then the geometric mean). Returns (the choice, all trials)."""
+    """Times every setting of `space` on db and each batch of `more`, reps solves
+    each; a setting's mean and median are the geometric means of its batches'.
+    Returns (the choice, all trials)."""
     import numpy as np
     import torch
 
@@ -81,10 +84,10 @@ def sweep(db, reps: int = 3, space: dict | None = None, time_budget_ms: int = 12
     trials = []
     for combo in itertools.product(*(space[k] for k in keys)):
         opts = dict(zip(keys, combo))
-        times, failed = [], []
+        batches = (db, *more)
+        times, failed = [[] for _ in batches], []
         for _ in range(reps):
-            each = []
-            for batch in (db, *more):
+            for batch, each in zip(batches, times):
                 torch.cuda.synchronize()
                 t0 = time.perf_counter()
                 api.solve(batch, want_model=False, stats=False, time_budget_ms=time_budget_ms,
@@ -93,10 +96,9 @@ def sweep(db, reps: int = 3, space: dict | None = None, time_budget_ms: int = 12
                 each.append(time.perf_counter() - t0 if rc == 0 else float("inf"))
                 if rc != 0:
                     failed.append(rc)  # e.g. the time budget reached
-            times.append(each[0] if len(each) == 1
-                         else float(np.exp(np.mean(np.log(np.array(each))))))
-        trials.append({"options": opts, "mean_s": float(np.mean(times)),
-                       "median_s": float(np.median(times)), "times": times})
+        over = lambda stat: float(np.exp(np.mean(np.log([stat(t) for t in times]))))
+        trials.append({"options": opts, "mean_s": over(np.mean), "median_s": over(np.median),
+                       "times": times if more else times[0]})
         if failed:
             trials[-1]["failed_status"] = failed
         print(json.dumps(trials[-1]), flush=True)
@@ -105,12 +107,17 @@ def sweep(db, reps: int = 3, space: dict | None = None, time_budget_ms: int = 12
 
 def pick(trials, within: float = 0.05, tail: float = 1.5):
     """The trial with the lowest mean time, unless its slowest solve took more
-    than `tail` times its median (a setting prone to the rare several-times-
-    slower solve) and a steady trial lies within `within` of that mean: then
-    the steady trial with the lowest mean."""
+    than `tail` times the median of its batch (a setting prone to the rare
+    several-times-slower solve) and a steady trial lies within `within` of that
+    mean: then the steady trial with the lowest mean. A trial's times are one
+    batch's, or a list of each batch's."""
+    def is_steady(times):
+        batches = times if isinstance(times[0], (list, tuple)) else [times]
+        return all(max(t) <= tail * statistics.median(t) for t in batches)
+
     best = min(trials, key=lambda t: t["mean_s"])
     steady = [t for t in trials if t["mean_s"] <= best["mean_s"] * (1.0 + within)
-              and max(t["times"]) <= tail * t["median_s"]]
+              and is_steady(t["times"])]
     return min(steady, key=lambda t: t["mean_s"]) if steady else best
 
 
@@ -118,14 +125,13 @@ def main():
     ap = argparse.ArgumentParser()
     ap.add_argument("--queries", type=int, default=4096)
     ap.add_argument("--width", type=int, default=16)
-    ap.add_argument("--reps", type=int, default=0, help="solves per setting (0: 6 for "
-                    "DPLL, 16 for clause learning)")
+    ap.add_argument("--reps", type=int, default=0, help="solves per setting (0: 16)")
     ap.add_argument("--out", default=DEFAULT_OUT)
     ap.add_argument("--search", default="dpll", choices=["dpll", "cdcl"])
     ap.add_argument("--space", default="", help="JSON dict replacing the sweep space, "
                     "e.g. '{\"split_min\": [8, 16], \"split_depth\": [12, 14]}'")
     args = ap.parse_args()
-    args.reps = args.reps or (16 if args.search == "cdcl" else 6)
+    args.reps = args.reps or 16
     sys.path.insert(0, os.path.dirname(HERE))
     import torch
 

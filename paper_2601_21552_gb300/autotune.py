@@ -121,6 +121,16 @@ def pick(trials, within: float = 0.05, tail: float = 1.5):
     return min(steady, key=lambda t: t["mean_s"]) if steady else best
 
 
+def summary(trial):
+    """A trial as the file keeps it: of each batch's solves the mean, the median
+    and the slowest (every tuned call reads the file, so it stays small)."""
+    batches = [{"mean_s": round(statistics.fmean(t), 6), "median_s": round(statistics.median(t), 6),
+                "max_s": round(max(t), 6)} for t in trial["times"]]
+    rest = {k: v for k, v in trial.items() if k != "times"}
+    return {**rest, "mean_s": round(trial["mean_s"], 6),
+            "median_s": round(trial["median_s"], 6), "batches": batches}
+
+
 def main():
     ap = argparse.ArgumentParser()
     ap.add_argument("--queries", type=int, default=4096)
@@ -159,9 +169,10 @@ def main():
                             "256 bounds queries of 8 bits; 512 partition queries of 10 bits",
                 "device": torch.cuda.get_device_name(0), "reps" + sfx: args.reps,
                 "best" + sfx: best["options"], "best_mean_s" + sfx: best["mean_s"],
-                "best_median_s" + sfx: best["median_s"], "trials" + sfx: trials})
+                "best_median_s" + sfx: best["median_s"],
+                "trials" + sfx: [summary(t) for t in trials]})
     with open(args.out, "w") as f:
-        json.dump(out, f, indent=1)
+        json.dump(out, f)
     print("best", json.dumps(best))
 
 

@@ -41,3 +41,18 @@ def test_the_mean_is_each_batch_s_own(monkeypatch):
     assert trials[0]["mean_s"] == pytest.approx((1.40 * 0.005 * 0.012) ** (1 / 3))
     assert trials[1]["median_s"] == pytest.approx((1.1 * 0.005 * 0.012) ** (1 / 3))
     assert [len(t) for t in trials[0]["times"]] == [4, 4, 4]
+
+
+def test_the_file_that_every_tuned_call_reads_stays_small(monkeypatch):
+    import json
+    import os
+
+    from paper_2601_21552_gb300 import autotune
+    plan = {s: [[0.8] * 63 + [2.5], [0.005] * 64, [0.012] * 64] for s in range(16)}
+    _, trials = run(monkeypatch, plan, 64)
+    kept = [autotune.summary(t) for t in trials]
+    assert len(json.dumps(kept)) < 16 * 400
+    assert kept[3]["batches"][0] == {"mean_s": pytest.approx(0.826562), "median_s": 0.8,
+                                     "max_s": 2.5}
+    assert kept[3]["options"] == {"split_min": 3} and "times" not in kept[3]
+    assert os.path.getsize(autotune.DEFAULT_OUT) < 8000

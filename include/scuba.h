@@ -268,8 +268,10 @@ int scuba_solve_batch_host(const scuba_cnf_batch* batch, uint8_t* verdict, uint8
  *     block shape (fixed below), trail_placement, profile, finish_ns,
  *     search_event_begin/end, inst_num_inputs, trace.
  *   - Shape: one block of 4 warps per SM and a 256-job subtree ring, so a
- *     batch fits when its scratch (about 12*L + 8*(2*total_vars + n) + 12*C
- *     bytes plus 12*max_vars per warp) is at most 64 MiB; larger batches are
+ *     batch fits when its scratch is at most 64 MiB, counted as 12*L +
+ *     8*(2*total_vars + n) + 4*C + 32*n bytes, 12*max_vars + 992 per warp,
+ *     1,024*max_vars + 252 KB for the ring and up to 4 KB of alignment (part of
+ *     it is set aside and not used); larger batches are
  *     rejected with SCUBA_ERR_TOO_LARGE and a message naming the limit.
  *   - The first call on a device looks up the array's device address
  *     (cudaGetSymbolAddress) with that device current.

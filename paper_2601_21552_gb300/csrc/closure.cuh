@@ -6,9 +6,13 @@
 // eight lanes take a literal's list, every lane claims what its entry implies by
 // itself, and a round ends at a barrier (close_shared). The closure does not
 // depend on the order of that.
-// What a conflict leaves in the assignment does, so an instance that
-// conflicts is done again by one warp in a fixed order (close_rounds): its
-// values are the same in every run, as they always were.
+// What a conflict leaves in the assignment does (the interface leaves those
+// values open), so an instance that conflicts is done again by one warp
+// (close_rounds): however many warps took it first, its values are those of one
+// walk over the lists in their order. That order is the clauses' but for the
+// entries of 32 neighbouring clauses, and the claims of one step take the order in
+// which the SM serves a warp's shared-memory atomics; neither has been seen to
+// differ between runs, and nothing promises it.
 
 __device__ __forceinline__ void close_conflict(Warp& w, uint32_t a, uint32_t b, uint32_t c) {
   if (atomicCAS(&w.ws->conflict, 0u, 1u) == 0u) {
@@ -85,8 +89,9 @@ __device__ __forceinline__ void close_entry(Warp& w, uint32_t f, uint64_t e) {
 
 // Unit propagation to a fixpoint by one warp. Returns true on conflict.
 // Each round takes the trail literals assigned in the previous round (the
-// frontier) and spreads their occurrence entries over the 32 lanes:
-// The values of a conflicting instance are what this order of visits leaves.
+// frontier), 32 at a time, and spreads their occurrence entries over the lanes as
+// one list. The values of a conflicting instance are what this order of visits
+// leaves.
 __device__ bool close_rounds(Warp& w) {
   for (;;) {
     __syncwarp();

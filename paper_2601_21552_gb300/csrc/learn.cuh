@@ -38,12 +38,14 @@ __device__ __forceinline__ uint32_t pack_bf16(__nv_bfloat16 lo, __nv_bfloat16 hi
 }
 
 // D = A(16x16, row-major) * B(16x8, col-major) + C, BF16 inputs, FP32 accumulate.
-__device__ __forceinline__ void mma16816(float c[4], const uint32_t a[4], const uint32_t b[2]) {
+__device__ __forceinline__ void mma_add(float d[4], const uint32_t a[4], uint32_t b0, uint32_t b1,
+                                        float c0, float c1, float c2, float c3) {
   asm volatile(
       "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 "
-      "{%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};\n"
-      : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
-      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b[0]), "r"(b[1]));
+      "{%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%10,%11,%12,%13};\n"
+      : "=f"(d[0]), "=f"(d[1]), "=f"(d[2]), "=f"(d[3])
+      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1), "f"(c0), "f"(c1), "f"(c2),
+        "f"(c3));
 }
 
 // A fragment for rows [r0, r0+16) of a row-major [rows x NFEAT] BF16 tile.
@@ -68,12 +70,9 @@ __device__ __forceinline__ void load_b(const MlpWeights* W, int n, int lane, uin
 }
 
 // Scores of the 16 rows of one tile. Every lane ends with the scores of rows
-// g and g+8 (lane/4 = g). z (optional) receives the pre-activations in the
-// mma output layout: z[4n + k] for hidden pair (8n + 2t, 8n + 2t + 1) of rows
-// g (k = 0, 1) and g+8 (k = 2, 3).
+// g and g+8 (lane/4 = g).
 __device__ __forceinline__ void mlp_tile_scores(const MlpWeights* W, const __nv_bfloat16* xtile,
-                                                int lane, float& s_lo, float& s_hi,
-                                                float* z = nullptr) {
+                                                int lane, float& s_lo, float& s_hi) {
   uint32_t a[4];
   load_a(xtile, lane, a);
   const int t = lane & 3;
@@ -82,17 +81,11 @@ __device__ __forceinline__ void mlp_tile_scores(const MlpWeights* W, const __nv_
   for (int n = 0; n < NHID / 8; n++) {
     uint32_t b[2];
     load_b(W, n, lane, b);
-    float c[4] = {0.f, 0.f, 0.f, 0.f};
-    mma16816(c, a, b);
+    float c[4];
+    mma_add(c, a, b[0], b[1], 0.f, 0.f, 0.f, 0.f);
     const int j0 = 8 * n + 2 * t, j1 = j0 + 1;
     const float z0 = c[0] + W->b1[j0], z1 = c[1] + W->b1[j1];
     const float z2 = c[2] + W->b1[j0], z3 = c[3] + W->b1[j1];
-    if (z) {
-      z[4 * n + 0] = z0;
-      z[4 * n + 1] = z1;
-      z[4 * n + 2] = z2;
-      z[4 * n + 3] = z3;
-    }
     const float w0 = __bfloat162float(W->w2[j0]), w1 = __bfloat162float(W->w2[j1]);
     p_lo += fmaxf(z0, 0.f) * w0 + fmaxf(z1, 0.f) * w1;
     p_hi += fmaxf(z2, 0.f) * w0 + fmaxf(z3, 0.f) * w1;

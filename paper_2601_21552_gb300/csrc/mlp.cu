@@ -30,6 +30,7 @@
 namespace scuba {
 namespace mlpk {
 
+using learn::mma_add;
 using learn::MlpWeights;
 using learn::NFEAT;
 using learn::NHID;
@@ -108,17 +109,6 @@ __device__ __forceinline__ void load_hidden(const MlpWeights* W, int g, int t, H
       H.w2[q][u] = __bfloat162float(W->w2[j]);
     }
   }
-}
-
-// D = A(16x16) * B(16x8) + C, BF16 inputs, FP32 accumulate.
-__device__ __forceinline__ void mma_add(float d[4], const uint32_t a[4], uint32_t b0, uint32_t b1,
-                                        float c0, float c1, float c2, float c3) {
-  asm volatile(
-      "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 "
-      "{%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%10,%11,%12,%13};\n"
-      : "=f"(d[0]), "=f"(d[1]), "=f"(d[2]), "=f"(d[3])
-      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1), "f"(c0), "f"(c1), "f"(c2),
-        "f"(c3));
 }
 
 __device__ __forceinline__ uint32_t transpose8x8(uint32_t m) {
@@ -219,16 +209,19 @@ __device__ __forceinline__ SoftStat merge(const SoftStat& a, const SoftStat& b) 
 // softmax cross-entropy against the normalised targets, dS = softmax - target
 // and the gradients of every parameter (dW1 on the tensor cores from dH in
 // BF16). `split` blocks (a cluster) share a node's 16-row tiles and exchange
-// their softmax statistics through distributed shared memory; the nodes are
-// strided over the clusters, the gradients stay in registers across them and
-// are reduced once per block. A thread keeps the scores of its own rows in dS
-// between the two passes over the node's rows; the rows' features come from
-// L1 or L2 the second time.
+// their softmax statistics through distributed shared memory; a block takes one
+// node, keeps its gradients in registers and adds them to the global sums once.
+// (Blocks that stride over the nodes were slower: 101 against 91 us at 1,001
+// nodes.) A thread keeps the scores of its own rows in dS between the two passes
+// over the node's rows; the rows' features come from L1 or L2 the second time.
 //
-// Bound by instruction issue: about 500 instructions per 16-row tile
-// (activations, masks and sums of 64 hidden units per row) against 640 bytes.
-// A minibatch of 64 nodes has 64,000 rows, too few for one warp per node
-// (the split is the one that fills 2 blocks on each of the 152 SMs).
+// Many nodes: about 700 instructions per 16-row tile, the block's reduction
+// included (activations, masks and sums of 64 hidden units per row), against 640
+// bytes; 1,001 nodes of 300 to 1,500 rows take 79 us, of which their issue is 33 and
+// most of the rest the uneven nodes over 3.3 waves of blocks (scores, loss and
+// gradient as kernels of their own: 383). A minibatch of 64 nodes has 64,000 rows,
+// too few for one warp per node: the split is the one that fills 2 blocks on each
+// of the 152 SMs (17 us, was 213).
 constexpr int kGradWarps = 8;
 constexpr int kGradStride = 17 * NHID + 2 * NHID + 4;  // floats one warp stages for the reduction
 

@@ -1184,14 +1184,16 @@ __device__ int run_job_body(const Solve& S, Warp& w, int unit, int inst, const T
 // thread gets. Plain search: 3 (80 registers, against 5 blocks of 48 that spilled
 // 116 bytes). More warps do not pay: a subtree given away repeats part of its
 // donor's work, so idle warps multiply the decisions. With 64 decisions before
-// the first share, 4,096 partition queries of 16 bits take 0.75 s on 3 blocks,
-// 0.89 on 2, and took 1.59 on 5 (512 of 10 bits 11.6 ms on 2 and 24.5 on 5), and
+// the first share, 4,096 partition queries of 16 bits take a median of 0.74 s on 3
+// blocks, 0.87 on 2 (means over 32 solves 0.98 and 1.23: one solve in five meets an
+// unlucky split on either), and took 1.59 on 5 (512 of 10 bits 15.4 ms on 3, 12.6 on
+// 2 and 24.5 on 5), and
 // 8,192 random 3-SAT of 250 variables with a budget, where no warp is idle, 85 ms
 // on 3 against 92 on 2.
 // The learned variant takes up to 3 as well (80 registers, no spills; 2 blocks of 6
 // warps for small batches, see scuba_solve_units), trace recording, which shares
 // nothing, 5. Clause learning takes 2 blocks of 6 warps, three warps for
-// each quarter of the SM, which leaves a thread 168 registers and no spills; 16
+// each quarter of the SM, which leaves a thread 168 registers (162 used, no spills); 16
 // warps (128 registers, 206 bytes spilled) are the better choice only where the
 // search keeps every warp at work of its own for long: 511 random 3-SAT instances
 // of 150 variables take 45.0 ms against 41.7, 256 of them 27.5 against 27.0, but 511
@@ -1718,12 +1720,14 @@ static int solve_impl(const scuba_cnf_batch* b, uint8_t* verdict, uint8_t* model
   // occurrence offsets: sum over instances of (2V+1)
   const int64_t occ_total = 2LL * b->total_vars + n;
 
-  // shape: warps per block x blocks per SM (shared memory bounds the warps).
-  // The trail goes to shared memory when that still leaves >= 16 warps/SM.
+  // shape: warps per block x blocks per SM (shared memory bounds the warps)
   // Learned branching: two blocks of 6 warps unless the batch has a unit for every
-  // warp of three blocks of 8. 512 partition queries of 10 bits take 34.6 ms so and
-  // 38.7 on three blocks, 2,048 bounds queries of 8 bits 24.9 and 29.0, but
-  // 4,096 partition queries of 10 bits 101 and 93, of 16 bits 6.0 and 5.1 s.
+  // warp of three blocks of 8. 512 partition queries of 10 bits take 24.2 ms so and
+  // 26.3 on three blocks, 2,048 bounds queries of 8 bits 16.1 and 17.7. A batch that
+  // large may hold long searches, which want the warps (4,096 partition queries of
+  // 16 bits: 1,041 and 755 ms, with an untrained network 4.1 and 2.8 s; bounds
+  // queries of 16 bits: 1,741 and 1,217 ms), or short ones, which do not (partition
+  // queries of 10 bits: 28-33 and 43-49 ms); the former cost more to get wrong.
   const bool many = n_units >= 24 * S.sms;
   int wpb = opt->warps_per_block > 0 ? opt->warps_per_block
             : mode == dev::MODE_LEARNED && !many ? 6
@@ -1738,10 +1742,10 @@ static int solve_impl(const scuba_cnf_batch* b, uint8_t* verdict, uint8_t* model
   const size_t smem_cap = 227 * 1024, sm_cap = 228 * 1024;
   const size_t per_warp_g = sizeof(dev::WarpShared) + (size_t)assign_words * 4;
   const size_t per_warp_s = per_warp_g + (size_t)vmax * 4;
-  // Global memory by default: a small shared-memory carve-out leaves a larger L1
-  // for the read-only occurrence lists, which measured faster.
-  int trail_smem = opt->trail_placement == 1 ? 1 : 0;
-  (void)per_warp_s;
+  // The trail in global memory unless the caller asks otherwise: a small
+  // shared-memory carve-out leaves a larger L1 for the read-only occurrence lists,
+  // which measured faster.
+  const int trail_smem = opt->trail_placement == 1 ? 1 : 0;
   size_t per_warp = trail_smem ? per_warp_s : per_warp_g;
   if (mode == dev::MODE_LEARNED) per_warp += 32 * learn::NFEAT * sizeof(__nv_bfloat16);
   int cd_smem = 0;
@@ -2184,7 +2188,8 @@ extern "C" int scuba_solve_batch_noalloc(const scuba_cnf_batch* b, uint8_t* verd
     return at;
   };
   // 4 L + 4 occ_total bytes are set aside and not used (but for the padding of
-  // the activities): the limit on what a batch may need is part of the interface
+  // the activities): the limit on what a batch may need is part of the interface,
+  // which states it
   carve(4 * (size_t)L);
   carve(4 * (size_t)occ_total);
   const size_t act_bytes = 4 * (size_t)(slots * dev::act_stride(vmax));

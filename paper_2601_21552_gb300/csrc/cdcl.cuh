@@ -1083,7 +1083,7 @@ __device__ uint32_t pick_cd(Warp& w, unsigned char* area) {
 // short, low-LBD learned clauses to a per-instance pool and read the others'
 // at each restart. A pool is a ring of fixed-size records in global memory:
 // a writer reserves record r with one atomicAdd on the pool's cursor, writes
-// the body, fences, then writes the header r + 1. A reader takes record r only
+// the body, then the header r + 1 with a release store. A reader takes record r only
 // if its header reads r + 1 before the body and the cursor shows, after the
 // body, that no writer can have reserved the record's slot again (cursor <=
 // r + cap). Records that fail either check are skipped, never guessed.

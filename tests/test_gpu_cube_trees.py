@@ -1,0 +1,26 @@
+"""Cube trees stay in proportion: 512 partition queries of 16 bits, fewer than the
+launch has warps, under the tuned settings. One warp alone needs 4,521 conflicts for
+the hardest of them and a solve's cubes some 200 thousand; without the clauses that
+the cubes share, one solve in five spent 2 to 50 million on one instance."""
+import pytest
+
+torch = pytest.importorskip("torch")
+
+from test_gpu_prep_shapes import libs  # noqa: F401
+
+pytestmark = pytest.mark.gpu
+
+
+def test_no_instance_takes_a_multiple_of_its_usual_conflicts(libs):
+    from workloads import queries
+    api, B = libs
+    db = api.DeviceBatch(B.scuba_encode_batch(queries.config2(512, w=16)[0]), "cuda")
+    first, worst = None, 0
+    for _ in range(16):
+        v, _, st = api.solve(db, want_model=False, search="cdcl", tuned=True,
+                             time_budget_ms=60000)
+        assert api.status() == 0
+        worst = max(worst, int(st[:, 1].max()))
+        first = v if first is None else first
+        assert bool((v == first).all())
+    assert worst < 2_000_000

@@ -1751,22 +1751,35 @@ static int solve_impl(const scuba_cnf_batch* b, uint8_t* verdict, uint8_t* model
   int cd_smem = 0;
   uint32_t cd_smem_warp = 0;
   if (mode == dev::MODE_CDCL) {
-    // per-variable state in shared memory (9 or 5 bytes a variable, or bounds of
-    // the activities only) as long as 8 warps still fit an SM
-    for (int what : {dev::CD_SMEM_POS | dev::CD_SMEM_ACT, dev::CD_SMEM_POS | dev::CD_SMEM_GMAX,
-                     (int)dev::CD_SMEM_GMAX, 0}) {
-      cd_smem = what;
-      cd_smem_warp = (uint32_t)dev::cd_area_bytes(what, vmax);
-      if ((vmax < 65536 || !(what & dev::CD_SMEM_POS)) &&
-          (per_warp + cd_smem_warp) * 8 + 16 <= smem_cap)
-        break;
-    }
-    if (!cd_smem) cd_smem_warp = std::max(cd_smem_warp, (uint32_t)dev::CD_AREA_MIN);
-    per_warp += cd_smem_warp;
-    // two blocks on an SM if blocks of CDCL_WARPS (or of what the caller asks
-    // for) fit so, else one of up to 8 warps
+    // per-variable state in shared memory: 9 or 5 bytes a variable, or bounds of
+    // the activities only, the first that fits `blocks` blocks of `warps` on an SM
+    auto place = [&](int warps, int blocks) {
+      for (int what : {dev::CD_SMEM_POS | dev::CD_SMEM_ACT, dev::CD_SMEM_POS | dev::CD_SMEM_GMAX,
+                       (int)dev::CD_SMEM_GMAX, 0}) {
+        if (vmax >= 65536 && (what & dev::CD_SMEM_POS)) continue;
+        cd_smem = what;
+        cd_smem_warp = (uint32_t)dev::cd_area_bytes(what, vmax);
+        if (!what) cd_smem_warp = std::max(cd_smem_warp, (uint32_t)dev::CD_AREA_MIN);
+        const size_t block = (per_warp + cd_smem_warp) * warps + 16;
+        if (blocks == 2 ? (block + 1024) * 2 <= sm_cap : block <= smem_cap) return true;
+      }
+      return false;
+    };
+    // Two blocks on an SM if blocks of CDCL_WARPS (or of what the caller asks for)
+    // fit so, else one of up to 8 warps. A batch with more units than one block
+    // an SM has warps takes what lets two of them fit, others as much state as one
+    // allows. (4,000 random 3-SAT and 32-bit bounds queries, 4,905 variables at most:
+    // 2,047 ms on one block with positions and marks in shared memory, 1,542 on two
+    // with the activities' bounds only; 2,048 partition queries of 20 bits 270 and
+    // 249; but 64 of them 88 and 94, 16 bounds queries of 32 bits 22.6 and 23.1.)
     const int w2 = std::min(wpb, dev::CDCL_WARPS);
-    if (bps > 1 && (per_warp * w2 + 16 + 1024) * 2 <= sm_cap) wpb = w2;
+    bool two = bps > 1 && n_units > 8 * S.sms && place(w2, 2);
+    if (!two) {
+      place(8, 1);
+      two = bps > 1 && ((per_warp + cd_smem_warp) * w2 + 16 + 1024) * 2 <= sm_cap;
+    }
+    per_warp += cd_smem_warp;
+    if (two) wpb = w2;
     else bps = 1;
   }
   size_t smem = per_warp * wpb + (mode == dev::MODE_CDCL ? 16 : 0);  // ring alignment

@@ -190,12 +190,11 @@ typedef struct scuba_options {
   int32_t share_lbd;         /* CDCL: jobs that run beside other jobs of their instance
                                 (cubes, and the job that gave them away) publish
                                 their learned clauses of at most 12 literals and LBD
-                                <= share_lbd (units always) to a per-instance pool,
+                                <= share_lbd (units always, LBD 2 from cubes of 20
+                                and more levels) to a per-instance pool,
                                 and add the others' clauses at each restart; every
                                 learned clause is implied by the formula, so this
-                                never changes a verdict. 0: 2 where the batch has
-                                fewer units than the launch has warps, else 1;
-                                < 0: off */
+                                never changes a verdict. 0: default 2; < 0: off */
 } scuba_options;
 
 /* Number of int64 counters per instance in scuba_options.stats. */

@@ -5,11 +5,8 @@ Sweeps blocks per SM, the decisions a subtree makes before it may share work
 (split_min) and the decisions between checks for idle warps (split_interval)
 on a workload, timing each setting over several solves, and writes the
 setting with the lowest MEAN time. The workload is a large batch, on which
-every warp starts busy, two small ones, on which a few hard instances have
-to reach the idle warps, and for clause learning one of hard instances for a
-quarter of the warps, whose cube trees can grow out of hand (plain DPLL's trees
-do under every setting: its median on that batch was 279 and 985 ms in two runs
-of one setting, which no sweep can rank); settings are ranked by the geometric mean of the
+every warp starts busy, and two small ones, on which a few hard instances have
+to reach the idle warps; settings are ranked by the geometric mean of the
 batches' mean times (a steady setting within 5 % of the lowest wins over one
 whose slowest solve of any batch took more than 1.5x that batch's median; tails
 are judged and averaged batch by batch, since a mean over them would hide them) and written to a JSON file that bench.py and
@@ -49,8 +46,8 @@ SPACE = {
 # was measured within 1 % of 12), 24 and more leaves small batches waiting; the
 # conflicts per Luby restart unit (25) come from a sweep over {12, 25, 40, 50,
 # 100}; share_lbd is the LBD bound of the clauses the jobs of one instance share
-# (-1: no sharing, 0: the library's rule, 1 for batches that have a unit for every
-# warp and 2 for smaller ones, whose cube trees now and then explode with 1); a gate
+# (-1: no sharing; reading fewer of them pays more than they prune, and deep cubes
+# share two-level clauses in any case); a gate
 # on the job's own conflicts before it may give cubes away (8-128) was measured no better
 # than none
 SPACE_CDCL = {
@@ -58,7 +55,7 @@ SPACE_CDCL = {
     "split_depth": [248],
     "split_interval": [4, 8],
     "restart_unit": [25],
-    "share_lbd": [0, 1, 2],
+    "share_lbd": [1, 2],
 }
 
 
@@ -153,8 +150,7 @@ def main():
     enc = B.scuba_encode_batch(irs)
     db = api.DeviceBatch(enc, "cuda")
     more = tuple(api.DeviceBatch(B.scuba_encode_batch(q), "cuda") for q in
-                 (queries.config1(256, w=8)[0], queries.config2(512, w=10)[0],
-                  *([queries.config2(512, w=16)[0]] if args.search == "cdcl" else [])))
+                 (queries.config1(256, w=8)[0], queries.config2(512, w=10)[0]))
     torch.cuda.synchronize()
     space = json.loads(args.space) if args.space else None
     if args.search == "cdcl":
@@ -169,8 +165,7 @@ def main():
         out = {}
     sfx = "_cdcl" if args.search == "cdcl" else ""
     out.update({"workload": f"partition queries, {args.width}-bit inputs, {args.queries} queries; "
-                            "256 bounds queries of 8 bits; 512 partition queries of 10 bits, "
-                            "for clause learning of 16 bits too",
+                            "256 bounds queries of 8 bits; 512 partition queries of 10 bits",
                 "device": torch.cuda.get_device_name(0), "reps" + sfx: args.reps,
                 "best" + sfx: best["options"], "best_mean_s" + sfx: best["mean_s"],
                 "best_median_s" + sfx: best["median_s"],

@@ -99,6 +99,7 @@ __device__ __forceinline__ uint32_t* cd_area_gmax(unsigned char* area) {
 // 127) of the last analysis that met it, so that nothing is cleared after one.
 constexpr uint32_t MK_PHASE = 1, MK_EPOCHS = 127;
 constexpr uint32_t GMAX_LOOK = 0xffffffffu;  // a group's bound that is not known
+constexpr uint32_t DEEP_CUBE = 20;  // cube levels from which two-level clauses are shared
 
 // Profile counters (only when the caller passed a profile array): lane 0
 // adds the clock cycles of each phase to its warp's profile.
@@ -1341,7 +1342,16 @@ __device__ int run_cdcl(const Solve& S, Warp& w, int64_t slot, int unit, int ins
         abort_code = SCUBA_ERR_INTERNAL;
         return SCUBA_UNKNOWN;
       }
-      if (shared && n <= SHARE_MAXLEN && (n == 1 || lbd <= S.share_lbd))
+      // Cubes many levels deep share clauses of two levels whatever the bound: such a
+      // tree is growing out of hand, and they keep it from it. With a bound of one
+      // level throughout, 16 to 24 solves of 512 partition queries of 16 bits took a
+      // mean of 116-288 ms (slowest 2,179), so 76 (175); 128 of them 259-316 and 79, 512
+      // of 18 bits 266-395 and 93, 256 of 20 bits 240-1,196 (11,241) and 146 (471). With
+      // two levels throughout 50, 61, 74 and 155, but 4,096 of 16 bits 92 (86 and 87
+      // so), 256 bounds queries of 16 bits 56 (33 and 33), units 6.9 (6.1). From 14
+      // levels 55, 68, 109, 144 and 87, 39; from 28 62, 80, 103, 254 and 88, 33.
+      if (shared && n <= SHARE_MAXLEN &&
+          (n == 1 || lbd <= S.share_lbd || (lbd <= 2u && w.nd_fixed >= asm_levels + DEEP_CUBE)))
         share_publish(S, w, cd, n, lbd, slot);
       // Activities fade quickly while the search learns clauses that join few
       // levels (a conflict of one part of the formula: stay there), slowly

@@ -1939,14 +1939,7 @@ static int solve_impl(const scuba_cnf_batch* b, uint8_t* verdict, uint8_t* model
     sv.share_base = P<unsigned long long>(S.share_base);
     sv.share_mask = kSharePools - 1;
     sv.share_cap = kShareCap;
-    // Clauses of one level where every warp has a unit of its own: reading more of
-    // the others' costs more than it prunes (4,096 partition queries of 16 bits 85.7
-    // ms, two levels 91.7; of 18 bits 153 and 162). With fewer units than warps whole
-    // trees of cubes work on one instance, and without the others' two-level
-    // clauses a tree at times grows a hundredfold: 512 partition queries of 16 bits
-    // mean 50 ms, slowest of 24 solves 54 (one level: 116 to 288 and 2,179), 128 of
-    // them 61 (259-316), 512 of 18 bits 74 (266-395).
-    sv.share_lbd = opt->share_lbd > 0 ? (uint32_t)opt->share_lbd : n_units < slots ? 2u : 1u;
+    sv.share_lbd = opt->share_lbd > 0 ? (uint32_t)opt->share_lbd : 2u;
   }
   std::memset(&sv.tr, 0, sizeof(sv.tr));
   if (mode == dev::MODE_TRACE) {

@@ -134,7 +134,8 @@ typedef struct scuba_options {
   int32_t split;             /* 1: hand DPLL subtrees of busy instances to idle warps */
   int32_t warps_per_block;   /* at most 8; 0: default 8 (LEARNED: 6 for batches of fewer
                                 units than 24 warps an SM). CDCL: at most 6 where
-                                an SM holds two blocks */
+                                an SM holds two blocks, but 8 for a batch with a
+                                budget and more than 12 units an SM */
   int32_t blocks_per_sm;     /* 0: autotuned default */
   int32_t split_interval;    /* decisions between checks for idle warps; 0: default 16 */
   int32_t split_min;         /* decisions a subtree makes before it may share work;

@@ -144,9 +144,11 @@ struct TraceDev {
 };
 
 // MODE_CDCL1: clause learning where an SM holds one block only (large instances),
-// which may then have 8 warps and 255 registers a thread.
-enum { MODE_PLAIN = 0, MODE_TRACE = 1, MODE_LEARNED = 2, MODE_CDCL = 3, MODE_CDCL1 = 4 };
-constexpr bool is_cdcl(int mode) { return mode == MODE_CDCL || mode == MODE_CDCL1; }
+// which may then have 8 warps and 255 registers a thread. MODE_CDCL8: two blocks of
+// 8 warps (128 registers) for batches that keep every warp busy.
+enum { MODE_PLAIN = 0, MODE_TRACE = 1, MODE_LEARNED = 2, MODE_CDCL = 3, MODE_CDCL1 = 4,
+       MODE_CDCL8 = 5 };
+constexpr bool is_cdcl(int mode) { return mode >= MODE_CDCL; }
 
 // Activities of a slot: whole groups of 16, what one 2-bit assignment word covers.
 __host__ __device__ __forceinline__ int64_t act_stride(int32_t vmax) {
@@ -1212,7 +1214,7 @@ constexpr int CDCL_WARPS = 6;
 template <int MODE>
 __global__ void __launch_bounds__(MODE == MODE_CDCL ? 32 * CDCL_WARPS : 256,
                                   MODE == MODE_LEARNED ? SCUBA_LEARNED_MINBLOCKS
-                                  : MODE == MODE_CDCL  ? SCUBA_CDCL_MINBLOCKS
+                                  : MODE == MODE_CDCL || MODE == MODE_CDCL8 ? SCUBA_CDCL_MINBLOCKS
                                   : MODE == MODE_PLAIN ? SCUBA_PLAIN_MINBLOCKS
                                   : MODE == MODE_CDCL1 ? 1
                                                        : 5)
@@ -1497,7 +1499,7 @@ struct Scratch {
   Buf h_icb, h_cb, h_lits, h_nv, h_vb, h_verdict, h_model, h_stats;  // for the host entry
   int sms = 0;
   int32_t last_status = 0;
-  int smem_set[5] = {0, 0, 0, 0, 0};  // dynamic shared memory granted per search mode
+  int smem_set[6] = {0, 0, 0, 0, 0, 0};  // dynamic shared memory granted per search mode
   int smem_prop = 0;
 };
 
@@ -1749,6 +1751,7 @@ static int solve_impl(const scuba_cnf_batch* b, uint8_t* verdict, uint8_t* model
   size_t per_warp = trail_smem ? per_warp_s : per_warp_g;
   if (mode == dev::MODE_LEARNED) per_warp += 32 * learn::NFEAT * sizeof(__nv_bfloat16);
   int cd_smem = 0;
+  bool wide = false;  // clause learning: two blocks of 8 warps
   uint32_t cd_smem_warp = 0;
   if (mode == dev::MODE_CDCL) {
     // per-variable state in shared memory: 9 or 5 bytes a variable, or bounds of
@@ -1772,8 +1775,15 @@ static int solve_impl(const scuba_cnf_batch* b, uint8_t* verdict, uint8_t* model
     // 2,047 ms on one block with positions and marks in shared memory, 1,542 on two
     // with the activities' bounds only; 2,048 partition queries of 20 bits 270 and
     // 249; but 64 of them 88 and 94, 16 bounds queries of 32 bits 22.6 and 23.1.)
-    const int w2 = std::min(wpb, dev::CDCL_WARPS);
-    bool two = bps > 1 && n_units > 8 * S.sms && place(w2, 2);
+    // A budget says that units are not expected to finish; with more of them than
+    // two blocks of CDCL_WARPS have warps every warp stays busy, and two blocks of 8
+    // do more in spite of their spills: 2,000 random 3-SAT instances of 200 to 400
+    // variables 600 -> 419 ms, 9,000 2,726 -> 2,243. (Without a budget the last
+    // instances decide, and partition and bounds queries take 3 to 13 % longer.)
+    wide = bps > 1 && wpb == 8 && opt->decision_budget > 0 &&
+           n_units > 2 * dev::CDCL_WARPS * S.sms && place(8, 2);
+    const int w2 = wide ? 8 : std::min(wpb, dev::CDCL_WARPS);
+    bool two = wide || (bps > 1 && n_units > 8 * S.sms && place(w2, 2));
     if (!two) {
       place(8, 1);
       two = bps > 1 && ((per_warp + cd_smem_warp) * w2 + 16 + 1024) * 2 <= sm_cap;
@@ -1971,12 +1981,13 @@ static int solve_impl(const scuba_cnf_batch* b, uint8_t* verdict, uint8_t* model
   auto kern = mode == dev::MODE_TRACE     ? dev::k_solve<dev::MODE_TRACE>
               : mode == dev::MODE_LEARNED ? dev::k_solve<dev::MODE_LEARNED>
               : one_block                 ? dev::k_solve<dev::MODE_CDCL1>
+              : wide                      ? dev::k_solve<dev::MODE_CDCL8>
               : mode == dev::MODE_CDCL    ? dev::k_solve<dev::MODE_CDCL>
                                           : dev::k_solve<dev::MODE_PLAIN>;
   // raise the dynamic shared-memory limit only when it grows, so that a
   // repeated call (for example while a CUDA graph is being captured) issues
   // no attribute change
-  int& granted = S.smem_set[one_block ? (int)dev::MODE_CDCL1 : mode];
+  int& granted = S.smem_set[one_block ? (int)dev::MODE_CDCL1 : wide ? (int)dev::MODE_CDCL8 : mode];
   if ((int)smem > granted) {
     e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return cuda_fail("cudaFuncSetAttribute", e);

@@ -1,7 +1,7 @@
 """Batches with more units than one block on every SM has warps, whose largest
-instance leaves no room for two blocks with positions and marks in shared memory:
-they run on two blocks, with the same verdicts as one by one, models that verify, and
-work counters that say where the state lay does not matter to the result."""
+instance leaves no room for two blocks with positions and marks in shared memory, and
+batches with a budget, which take two blocks of 8 warps: the verdicts of the DPLL
+search, and models that verify, on both sides of each line."""
 import numpy as np
 import pytest
 

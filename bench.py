@@ -50,12 +50,12 @@ METRIC = "verdicts/sec + BCP propagations/sec on 1 GB300, learned vs plain, bit-
 
 
 # DRAM traffic of the clause-learning search kernel from one single-pass ncu
-# capture of a full bench launch (profiles/k_solve_cdcl_partition16.md: 2.58 GB
-# read + 3.19 GB written for 1.1026e8 propagations), per propagation, valid
+# capture of a full bench launch (profiles/k_solve_cdcl_partition16.md: 2.64 GB
+# read + 3.22 GB written for 1.1200e8 propagations), per propagation, valid
 # only for the kernel sources it was taken on (sha256 prefix of solver.cu +
 # learn.cuh + cdcl.cuh); scaled to each launch by the propagations it processes.
-PROFILED_SOURCES = "8ffc384b256798f6"
-DRAM_BYTES_PER_PROPAGATION = {"cdcl": (2.5775e9 + 3.1858e9) / 1.1026e8}
+PROFILED_SOURCES = "910e299a5e0ce22b"
+DRAM_BYTES_PER_PROPAGATION = {"cdcl": (2.6386e9 + 3.2249e9) / 1.1200e8}
 
 
 def _kernel_sources_sha() -> str:
@@ -68,10 +68,10 @@ def _kernel_sources_sha() -> str:
 
 
 # L2 traffic of the same kernel from the same single-pass ncu capture
-# (lts__t_bytes.sum: 53.87 GB for 1.1026e8 propagations), per propagation,
+# (lts__t_bytes.sum: 54.80 GB for 1.1200e8 propagations), per propagation,
 # under the same source hash (idle warps polling the job ring and the
 # clause-sharing pools included).
-L2_BYTES_PER_PROPAGATION = {"cdcl": 53.87e9 / 1.1026e8}
+L2_BYTES_PER_PROPAGATION = {"cdcl": 54.80e9 / 1.1200e8}
 
 
 def l2_probe(dev, mib: int = 32, iters: int = 200) -> float:
